@@ -540,3 +540,177 @@ _RUN = {"sparsify": _run_sparsify, "alg1": _run_alg1, "train": _run_train, "forw
 
 def run(state):
     return _RUN[state["kind"]](state)
+
+
+# ---------------------------------------------------------------------------------------------
+# the same outputs in 64 bits, in plain torch
+# ---------------------------------------------------------------------------------------------
+
+def exact(case, seed):
+    """What `run` returns, computed in fp64 on the inputs of `prepare`.  Kept lists and what is gathered by them follow the
+    fp32 scores (a near-tie may fall either way), so they have no value here."""
+    with torch.no_grad():
+        if case["kind"] in ("sparsify", "alg1"):
+            return _exact_scores(case, seed)
+        s = prepare(case, seed)
+        if case["kind"] == "attention":
+            return _exact_attention(case, s)
+        return _exact_block(case, s)
+
+
+def _exact_scores(c, seed):
+    t, _ = _dense_model(c, _Gen(seed))
+    sq = lambda x, cols: (x * x).sum(0 if cols else 1)       # over the axis that is not shared
+    cols_in, cols_out = not c["linear"], c["linear"]
+    up, imp = [], []
+    for l in range(c["layers"]):
+        x = {nm: t[nm][l] for nm in t}
+        for a, b, cols_b, n_seg in (("q", "k", cols_in, c["heads"]), ("v", "o", cols_out, c["heads"]), ("1", "2", cols_out, 1)):
+            w1 = x["w" + a].double()
+            if a == "1" and "w1b" in x:
+                w1 = w1 * x["w1b"].double()
+            c1, c2 = sq(w1, cols_in).view(n_seg, -1), sq(x["w" + b].double(), cols_b).view(n_seg, -1)
+            n = c1.shape[1]
+            rope = c["rope"] if a == "q" else "none"
+            if rope == "none":
+                raw = c1.sqrt() * c2.sqrt()
+                ups = raw / raw.norm(dim=1, keepdim=True)
+            else:                                          # the unit is a rotation pair, counted once
+                fold = (lambda v: v.view(n_seg, 2, n // 2).sum(1)) if rope == "half" else (lambda v: v.view(n_seg, n // 2, 2).sum(2))
+                raw = fold(c1).sqrt() * fold(c2).sqrt()
+                u = raw / raw.norm(dim=1, keepdim=True)
+                ups = u.repeat(1, 2) if rope == "half" else u.repeat_interleave(2, dim=1)
+            mean = lambda nm, cols: sq(x[nm].double(), cols).view(n_seg, -1).sum(1) * n_seg / x[nm].numel()
+            m1 = mean("g" + a, cols_in)
+            if a == "1" and "g1b" in x:
+                m1 = 0.5 * (m1 + mean("g1b", cols_in))
+            up.append(ups.reshape(-1))
+            imp.append(0.5 * (m1 + mean("g" + b, cols_b)) / (c["batch"] * c["seq"]))
+    r = {"scores": torch.cat(up), "importance": torch.cat(imp), "out": None}
+    r["kept" if c["kind"] == "sparsify" else "chosen"] = None
+    return r
+
+
+def _blocks16(counts):
+    """First column and width of every head's block, widths rounded up to 16."""
+    out, at = [], 0
+    for n in counts:
+        w = -(-n // 16) * 16
+        out.append((at, w))
+        at += w
+    return out
+
+
+def _exact_core(c, q, k, v, scale, d_ctx=None):
+    """softmax(scale q k^T) v of one sequence and head in fp64, its log-sum-exp, and the three gradients."""
+    z = scale * (q @ k.t())
+    if c["causal"]:
+        i = torch.arange(c["seq"], device=z.device)
+        z = z.masked_fill(i[None, :] > i[:, None], -math.inf)
+    lse = torch.logsumexp(z, 1)
+    p = torch.exp(z - lse[:, None])
+    ctx = p @ v
+    if d_ctx is None:
+        return ctx, lse, None
+    ds = p * (d_ctx @ v.t() - (d_ctx * ctx).sum(1, keepdim=True)) * scale
+    return ctx, lse, (ds @ k, ds.t() @ q, p.t() @ d_ctx)
+
+
+def _exact_attention(c, s):
+    kq, kv = _kv_counts(c)
+    rep = c["heads"] // len(kq)
+    qb, ob = _blocks16([n for n in kq for _ in range(rep)]), _blocks16([n for n in kv for _ in range(rep)])
+    kb, vb = _blocks16(kq), _blocks16(kv)
+    S, T = c["seq"], c["batch"] * c["seq"]
+    r = {nm: torch.zeros(s[nm].shape, dtype=torch.float64, device=DEV) for nm in ("Ctx", "dQ", "dK", "dV")}
+    lse = torch.zeros((c["heads"], T), dtype=torch.float64, device=DEV)
+    for b in range(c["batch"]):
+        rows = slice(b * S, (b + 1) * S)
+        for h in range(c["heads"]):
+            cut = lambda blk: slice(blk[0], blk[0] + blk[1])
+            q, o, k, v = cut(qb[h]), cut(ob[h]), cut(kb[h // rep]), cut(vb[h // rep])
+            ctx, l, (dq, dk, dv) = _exact_core(c, s["Q"][rows, q].double(), s["K"][rows, k].double(), s["V"][rows, v].double(),
+                                               s["scale"], s["dCtx"][rows, o].double())
+            r["Ctx"][rows, o], lse[h, rows], r["dQ"][rows, q] = ctx, l, dq
+            r["dK"][rows, k] += dk
+            r["dV"][rows, v] += dv
+    r["lse"] = lse.view(-1)
+    return r
+
+
+def _exact_block(c, s):
+    train, attn, S = c["kind"] == "train", s["attn"], c["seq"]
+    n_qk, n_vo, k, lin = s["n_qk"], s["n_vo"], s["k"], c["linear"]
+    w, x = s["w"], s["x"].double()
+    real = {"wq": n_qk, "wk": n_qk, "wv": n_vo, "wo": n_vo, "w1": k, "w1b": k, "w2": k}
+    rows = {nm for nm in real if (nm in ("wo", "w2")) != lin}   # stored with the shared index as the slow axis
+    W = {nm: (w[nm].double().t() if nm in rows else w[nm].double())[:, :real[nm]] for nm in real if nm in w}   # d_m x n
+    bias = lambda nm, n: w[nm][:n].double() if nm in w else 0.0
+    Q, K, V = x @ W["wq"] + bias("bq", n_qk), x @ W["wk"] + bias("bk", n_qk), x @ W["wv"] + bias("bv", n_vo)
+    qk, vo, _ = _counts(c)
+    heads = [(slice(a, a + m), slice(e, e + n)) for (a, m), (e, n) in zip(_blocks16(qk), _blocks16(vo))]
+
+    def cores(d_ctx):
+        ctx = torch.zeros_like(V)
+        g = [torch.zeros_like(Q), torch.zeros_like(K), torch.zeros_like(V)]
+        for b in range(c["batch"]):
+            r = slice(b * S, (b + 1) * S)
+            for i, o in heads:
+                ctx[r, o], _, d = _exact_core(c, Q[r, i], K[r, i], V[r, o], s["scale"], None if d_ctx is None else d_ctx[r, o])
+                if d is not None:
+                    g[0][r, i], g[1][r, i], g[2][r, o] = d
+        return ctx, g
+
+    d_ctx = s["dOut"].double() @ W["wo"] if train else None
+    if attn:
+        ctx, grads = cores(d_ctx)
+    else:
+        ctx, grads = s["Ctx"].double(), [s[nm].double() for nm in ("dQ", "dK", "dV")] if train else None
+    out = {"Out": ctx @ W["wo"].t() + bias("bo", x.shape[1])}
+    F = torch.nn.functional
+    H = x @ W["w1"] + bias("b1", k)
+    if c["ffn"] == "swiglu":
+        Hb = x @ W["w1b"]
+        sg = torch.sigmoid(H)
+        A, dact = H * sg * Hb, None
+    else:
+        A = F.gelu(H, approximate="tanh" if c["ffn"] == "gelu_tanh" else "none")
+    out["Y"] = A @ W["w2"].t() + bias("b2", x.shape[1])
+    if attn:
+        out["Ctx"] = ctx
+    if not train:
+        return out
+    dY = s["dY"].double()
+    dA = dY @ W["w2"]
+    if c["ffn"] == "swiglu":
+        dH, dHb = dA * Hb * sg * (1 + H * (1 - sg)), dA * H * sg
+    elif c["ffn"] == "gelu":
+        dH = dA * (0.5 * (1 + torch.erf(H / math.sqrt(2.0))) + H * torch.exp(-0.5 * H * H) / math.sqrt(2.0 * math.pi))
+    else:
+        t = torch.tanh(math.sqrt(2.0 / math.pi) * (H + 0.044715 * H ** 3))
+        dH = dA * (0.5 * (1 + t) + 0.5 * H * (1 - t * t) * math.sqrt(2.0 / math.pi) * (1 + 3 * 0.044715 * H * H))
+
+    def stored(nm, g, like):                                    # d_m x n -> as the weight's gradient is stored
+        g = g.t() if nm in rows else g
+        r = torch.zeros(like.shape, dtype=torch.float64, device=DEV)
+        r[:, :g.shape[1]] = g
+        return r
+
+    f, xt = s["ffn"], x.t()
+    out.update({"dCtx": d_ctx, "dW1": stored("w1", xt @ dH, f["dW1"]), "dW2": stored("w2", dY.t() @ A, f["dW2"])})
+    dX = dH @ W["w1"].t()
+    if c["ffn"] == "swiglu":
+        out["dW1b"] = stored("w1b", xt @ dHb, f["dW1b"])
+        dX += dHb @ W["w1b"].t()
+    elif s["bias"]:
+        out["db1"] = dH.sum(0)
+    for nm, g in zip(("wq", "wk", "wv"), grads):
+        dX += g @ W[nm].t()
+        out["d" + nm] = stored(nm, xt @ g, s["grads"][nm])
+        if s["bias"] and not (nm == "wk" and attn):
+            out["db" + nm[1]] = F.pad(g.sum(0), (0, s["grads"]["b" + nm[1]].numel() - g.shape[1]))
+    out["dX"] = dX
+    out["dwo"] = stored("wo", s["dOut"].double().t() @ ctx, s["grads"]["wo"])
+    if s["bias"]:
+        out["db2"], out["dbo"] = dY.sum(0), s["dOut"].double().sum(0)
+    return out
