@@ -23,6 +23,34 @@ inline int64_t mat_cols(const ecospa_mat_t& m, int64_t D) { return m.layout == E
 
 #ifdef __CUDACC__
 
+// Programmatic stream serialization.  A kernel launched with launch_pdl may be placed while the previous kernel of the
+// stream drains; it touches no memory that a kernel writes before pdl_wait(), which returns when every earlier kernel of
+// the stream is complete and its writes are visible.  pdl_start() lets the next kernel do the same with this one.
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename Params>
+ecospa_status_t launch_pdl(void (*kernel)(Params), dim3 grid, int threads, cudaStream_t stream, const Params& p, const char* name,
+                           size_t dyn_smem = 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = dyn_smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
+    if (e != cudaSuccess) {
+        set_cuda_error(e, name);
+        cudaGetLastError();
+        return ECOSPA_ERR_CUDA;
+    }
+    return check_launch(name);
+}
+
 __device__ __forceinline__ uint4 ldg_stream16(const void* p) {
     uint4 v;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"

@@ -24,42 +24,50 @@ constexpr int kThreads = 256;
 // ------------------------------------------------------------------------------------------------
 // helper kernels
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) cast_f32_bf16_kernel(const float* __restrict__ in, int64_t ld_in,
-                                                                 uint16_t* __restrict__ out, int64_t ld_out, int64_t rows,
-                                                                 int64_t cols, int64_t cols_out) {
-    // one thread per 4 output columns; columns [cols, cols_out) are zero-filled
-    const int64_t per_row = (cols_out + 3) / 4;
-    const int64_t total = rows * per_row;
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(kThreads) + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * kThreads) {
-        const int64_t r = i / per_row, c = (i % per_row) * 4;
-        for (int e = 0; e < 4; ++e) {
-            if (c + e < cols_out) {
-                const float v = (c + e < cols) ? in[r * ld_in + c + e] : 0.f;
-                __nv_bfloat16 b = __float2bfloat16_rn(v);
-                out[r * ld_out + c + e] = *reinterpret_cast<uint16_t*>(&b);
-            }
-        }
-    }
+// fp32 -> bf16 staging of every operand of a call in one launch.  Bound by launch latency at the sizes of a small fp32
+// block (a 512 x 256 operand is 0.5 MB: 0.1 us of memory time): one launch per operand was 23 launches of 2 us, each
+// with its gap, in a training step of that block (188 us); one per call with its set-up under the tail of the previous
+// kernel, 164 us in all (the same passes, timed in turn).  A thread takes 8 output columns: two 16-byte loads and one 16-byte store where the pitches allow
+// (a staged row is a whole number of 8 columns, the columns past the operand's own are zero).
+constexpr int kMaxCasts = 8;
+struct CastJob {
+    const float* in;
+    uint16_t* out;
+    int64_t ld_in, cols;
+    int64_t groups;          // 8-column groups of the matrix = rows * per_row
+    int32_t per_row, vec_ok;
+    int32_t blk_start, n_blk;
+};
+struct CastParams {
+    CastJob job[kMaxCasts];
+    int32_t n_jobs, pad_;
+};
+__device__ __forceinline__ uint32_t cast_pair(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
 }
-
-// These helpers are launched with programmatic stream serialization, like the GEMM engine: their blocks may be
-// placed while the previous kernel drains, and touch no global memory before pdl_wait().
-__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <typename Params>
-cudaError_t launch_pdl(void (*kernel)(Params), dim3 grid, cudaStream_t stream, const Params& p) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+__global__ void __launch_bounds__(kThreads) cast_f32_bf16_kernel(const __grid_constant__ CastParams P) {
+    pdl_start();
+    pdl_wait();
+    int ji = 0;
+    while (ji + 1 < P.n_jobs && static_cast<int>(blockIdx.x) >= P.job[ji + 1].blk_start) ++ji;
+    const CastJob& J = P.job[ji];
+    for (int64_t i = (blockIdx.x - J.blk_start) * static_cast<int64_t>(kThreads) + threadIdx.x; i < J.groups;
+         i += static_cast<int64_t>(J.n_blk) * kThreads) {
+        const int64_t r = i / J.per_row, c = (i % J.per_row) * 8;
+        const float* src = J.in + r * J.ld_in + c;
+        float v[8];
+        if (J.vec_ok && c + 8 <= J.cols) {
+            const uint4 a = *reinterpret_cast<const uint4*>(src), b = *reinterpret_cast<const uint4*>(src + 4);
+            v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y); v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
+            v[4] = __uint_as_float(b.x); v[5] = __uint_as_float(b.y); v[6] = __uint_as_float(b.z); v[7] = __uint_as_float(b.w);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = c + e < J.cols ? src[e] : 0.f;
+        }
+        *reinterpret_cast<uint4*>(J.out + i * 8) =
+            make_uint4(cast_pair(v[0], v[1]), cast_pair(v[2], v[3]), cast_pair(v[4], v[5]), cast_pair(v[6], v[7]));
+    }
 }
 
 // Column sums (bias gradients) of up to two bf16 matrices with the same number of rows, two launches:
@@ -226,6 +234,8 @@ struct Ctx {
     Arena arena;
     int dtype = ECOSPA_BF16;  // of the model (activations, weights, outputs)
     ecospa_status_t st = ECOSPA_OK;
+    CastParams casts = {};    // operands of an fp32 model still to be staged (run_ops launches them)
+    int cast_blocks = 0;
 };
 
 // A (rows x cols, pitch ld) matrix of the model dtype as a bf16 Stored operand (staged if fp32).
@@ -246,11 +256,20 @@ Stored as_bf16(Ctx& cx, const void* p, int64_t rows, int64_t cols, int64_t ld) {
         cx.st = ECOSPA_ERR_WORKSPACE;
         return s;
     }
-    const int64_t total = rows * ((ldo + 3) / 4);
-    const int grid = static_cast<int>(std::min<int64_t>(ceil_div(total, kThreads), 148 * 16));
-    cast_f32_bf16_kernel<<<grid, kThreads, 0, cx.stream>>>(static_cast<const float*>(p), ld, static_cast<uint16_t*>(buf), ldo,
-                                                           rows, cols, ldo);
-    cx.st = check_launch("cast_f32_bf16_kernel");
+    if (cx.casts.n_jobs == kMaxCasts) {
+        cx.st = ECOSPA_ERR_UNSUPPORTED;   // (no call has that many operands)
+        return s;
+    }
+    CastJob& J = cx.casts.job[cx.casts.n_jobs++];
+    J.in = static_cast<const float*>(p);
+    J.out = static_cast<uint16_t*>(buf);
+    J.ld_in = ld; J.cols = cols;
+    J.per_row = static_cast<int32_t>(ldo / 8);
+    J.groups = rows * J.per_row;
+    J.vec_ok = aligned16(p) && ld % 4 == 0;
+    J.n_blk = static_cast<int32_t>(std::min<int64_t>(ceil_div(J.groups, kThreads), 148 * 8));
+    J.blk_start = cx.cast_blocks;
+    cx.cast_blocks += J.n_blk;
     s.ptr = buf; s.rows = rows; s.cols = cols; s.ld = ldo;
     return s;
 }
@@ -267,6 +286,17 @@ Stored scratch_bf16(Ctx& cx, int64_t rows, int64_t cols) {
     }
     s.ptr = buf; s.rows = rows; s.cols = cols; s.ld = ld;
     return s;
+}
+
+// The launch of a call's (first) products, after the staging of its operands.
+ecospa_status_t run_ops(Ctx& cx, const GemmOp* ops, int n_ops) {
+    if (cx.casts.n_jobs > 0) {
+        const ecospa_status_t st = launch_pdl(cast_f32_bf16_kernel, dim3(cx.cast_blocks), kThreads, cx.stream, cx.casts,
+                                              "cast_f32_bf16_kernel");
+        cx.casts.n_jobs = cx.cast_blocks = 0;
+        if (st != ECOSPA_OK) return st;
+    }
+    return launch_grouped_gemm(ops, n_ops, cx.stream);
 }
 
 // Column sums of up to three bf16 matrices with the same row count.  colsum_plan takes the scratch of the chunk
@@ -307,14 +337,7 @@ const ColsumParams& colsum_begin(Ctx& cx, const ColsumParams& P) {
     if (cx.st != ECOSPA_OK || P.n_jobs == 0) return P;
     int tiles = 0;
     for (int i = 0; i < P.n_jobs; ++i) tiles += P.job[i].col_tiles;
-    const cudaError_t e = launch_pdl(colsum_partial_kernel, dim3(tiles, P.chunks), cx.stream, P);
-    if (e != cudaSuccess) {
-        set_cuda_error(e, "colsum_partial_kernel launch");
-        cudaGetLastError();
-        cx.st = ECOSPA_ERR_CUDA;
-        return P;
-    }
-    cx.st = check_launch("colsum_partial_kernel");
+    cx.st = launch_pdl(colsum_partial_kernel, dim3(tiles, P.chunks), kThreads, cx.stream, P, "colsum_partial_kernel");
     return P;
 }
 
@@ -485,14 +508,7 @@ void finish(Ctx& cx, const PendingReduce* red, int n_red, const ColsumParams& cs
     P.red_blocks = blocks;
     for (int i = 0; i < cs.n_jobs; ++i) blocks += static_cast<int>(round_up32(cs.job[i].cols) / 32);
     if (blocks == 0) return;
-    const cudaError_t e = launch_pdl(post_kernel, dim3(blocks), cx.stream, P);
-    if (e != cudaSuccess) {
-        set_cuda_error(e, "post_kernel launch");
-        cudaGetLastError();
-        cx.st = ECOSPA_ERR_CUDA;
-        return;
-    }
-    cx.st = check_launch("post_kernel");
+    cx.st = launch_pdl(post_kernel, dim3(blocks), kThreads, cx.stream, P, "post_kernel");
 }
 
 }  // namespace
@@ -532,7 +548,7 @@ extern "C" ecospa_status_t ecospa_coupled_qk_fwd(const void* X, int64_t ldx, int
     ops[n_ops++] = proj_op(Xs, weight_bf16(cx, wq_c, d_m, n), mn_over_other(wq_c), T, d_m, n, bq_c, Qc, ld_out, cx.dtype);
     if (wk_c) ops[n_ops++] = proj_op(Xs, weight_bf16(cx, wk_c, d_m, n), mn_over_other(wk_c), T, d_m, n, bk_c, Kc, ld_out, cx.dtype);
     if (cx.st != ECOSPA_OK) return cx.st;
-    return launch_grouped_gemm(ops, n_ops, cx.stream);
+    return run_ops(cx, ops, n_ops);
 }
 
 extern "C" ecospa_status_t ecospa_coupled_qk_bwd(const void* X, int64_t ldx, int64_t T, int64_t d_m,
@@ -575,7 +591,7 @@ extern "C" ecospa_status_t ecospa_coupled_qk_bwd(const void* X, int64_t ldx, int
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
     const ColsumParams cs = colsum_plan(cx, dQs, dbq_c, dKs, wk_c ? dbk_c : nullptr);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = launch_grouped_gemm(ops, n_ops, cx.stream)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
     finish(cx, red, 2, colsum_begin(cx, cs));
     return cx.st;
 }
@@ -604,7 +620,7 @@ extern "C" ecospa_status_t ecospa_coupled_vo_fwd_o(const void* Ctxm, int64_t ld_
     op.epi = EPI_STORE; op.C = Out; op.ldc = ld_out; op.out_f32 = cx.dtype == ECOSPA_F32;
     op.bias = bo; op.bias_f32 = cx.dtype == ECOSPA_F32;
     if (cx.st != ECOSPA_OK) return cx.st;
-    return launch_grouped_gemm(&op, 1, cx.stream);
+    return run_ops(cx, &op, 1);
 }
 
 extern "C" ecospa_status_t ecospa_coupled_vo_bwd(const void* X, int64_t ldx, const void* Ctxm, int64_t ld_ctx, int64_t T,
@@ -647,7 +663,7 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd(const void* X, int64_t ldx, con
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
     const ColsumParams cs = colsum_plan(cx, dVs, dbv_c, dOs, dbo);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = launch_grouped_gemm(ops, n_ops, cx.stream)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
     finish(cx, red, 2, colsum_begin(cx, cs));
     return cx.st;
 }
@@ -672,7 +688,7 @@ extern "C" ecospa_status_t ecospa_coupled_qkv_fwd(const void* X, int64_t ldx, in
     ops[1] = proj_op(Xs, weight_bf16(cx, wk_c, d_m, n_qk), mn_over_other(wk_c), T, d_m, n_qk, bk_c, Kc, ld_qk, cx.dtype);
     ops[2] = proj_op(Xs, weight_bf16(cx, wv_c, d_m, n_vo), mn_over_other(wv_c), T, d_m, n_vo, bv_c, Vc, ld_v, cx.dtype);
     if (cx.st != ECOSPA_OK) return cx.st;
-    return launch_grouped_gemm(ops, 3, cx.stream);
+    return run_ops(cx, ops, 3);
 }
 
 // Backward of the three projections in one launch: dW_Q^c, dW_K^c, dW_V^c (split over the tokens when they
@@ -716,7 +732,7 @@ extern "C" ecospa_status_t ecospa_coupled_qkv_bwd(const void* X, int64_t ldx, in
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = cx.dtype == ECOSPA_F32; dx.accumulate = accumulate_dX != 0;
     const ColsumParams cs = colsum_plan(cx, dQs, dbq_c, dKs, dbk_c, dVs, dbv_c);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = launch_grouped_gemm(ops, n_ops, cx.stream)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
     finish(cx, red, 3, colsum_begin(cx, cs));
     return cx.st;
 }
@@ -747,7 +763,7 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd_o(const void* Ctxm, int64_t ld_
     dc.epi = EPI_STORE; dc.C = dCtx; dc.ldc = ld_dctx; dc.out_f32 = cx.dtype == ECOSPA_F32;
     const ColsumParams cs = colsum_plan(cx, dOs, dbo);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = launch_grouped_gemm(ops, n_ops, cx.stream)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
     finish(cx, &red, 1, colsum_begin(cx, cs));
     return cx.st;
 }
@@ -800,8 +816,8 @@ extern "C" ecospa_status_t ecospa_coupled_ffn_fwd(const void* X, int64_t ldx, in
     down.bias = b2; down.bias_f32 = f32;
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = validate_gemm_ops(&up, 1)) != ECOSPA_OK || (st = validate_gemm_ops(&down, 1)) != ECOSPA_OK) return st;
-    if ((st = launch_grouped_gemm(&up, 1, cx.stream)) != ECOSPA_OK) return st;
-    return launch_grouped_gemm(&down, 1, cx.stream);
+    if ((st = run_ops(cx, &up, 1)) != ECOSPA_OK) return st;
+    return run_ops(cx, &down, 1);
 }
 
 extern "C" ecospa_status_t ecospa_coupled_ffn_bwd(const void* X, int64_t ldx, int64_t T, int64_t d_m, int32_t act,
@@ -870,8 +886,8 @@ extern "C" ecospa_status_t ecospa_coupled_ffn_bwd(const void* X, int64_t ldx, in
     const ColsumParams cs = colsum_plan(cx, dYs, db2, dH, sw ? nullptr : db1_c);
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = validate_gemm_ops(ops, n_ops)) != ECOSPA_OK || (st = validate_gemm_ops(ops2, n_ops2)) != ECOSPA_OK) return st;
-    if ((st = launch_grouped_gemm(ops, n_ops, cx.stream)) != ECOSPA_OK) return st;
-    if ((st = launch_grouped_gemm(ops2, n_ops2, cx.stream)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops2, n_ops2)) != ECOSPA_OK) return st;
     finish(cx, red, 3, colsum_begin(cx, cs));
     return cx.st;
 }

@@ -1,0 +1,61 @@
+"""Sizes at the edges of the kernels' forms, against the CPU oracle or plain indexing: segment widths around one warp's and
+one block's share, kept lists whose source span is dense, sparse or unaligned, products of one 128 x 128 tile and around the
+number of tiles at which CTA pairs take over, fp32 operands with ragged pitches."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2511_11641_b200 import binding as B
+from paper_2511_11641_b200 import block as BL
+from paper_2511_11641_b200 import layers as L
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _rel(got, want):
+    return float(np.linalg.norm(got.double().cpu().numpy() - want) / max(np.linalg.norm(want), 1e-30))
+
+
+@pytest.mark.parametrize("T,d_m,k", [(1, 64, 1), (127, 72, 31), (128, 128, 64), (129, 136, 65), (300, 264, 129), (1100, 512, 1032), (1664, 1536, 1408)])
+@pytest.mark.parametrize("act", [B.ACT_GELU_ERF, B.ACT_SWIGLU])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("lin", [False, True])
+def test_ffn_tiles(T, d_m, k, act, dtype, lin):
+    """Forward and backward of products from less than one 128 x 128 tile to more tiles than SMs (where the launch changes from
+    single CTAs to pairs); the fp32 operands also come with a pitch that is not a multiple of four.  Bound: bf16 operands,
+    fp32 sums, saved activations rounded to bf16 (2e-2, as in test_gpu_layers)."""
+    g = torch.Generator(device=DEV).manual_seed(T)
+    sw = act == B.ACT_SWIGLU
+    odd = 1 if dtype == torch.float32 else 0
+    mat = lambda r, c, pitch, std: (torch.randn(r, pitch, generator=g, device=DEV) * std).to(dtype)[:, :c]
+    X, dY = mat(T, d_m, d_m + 2 * odd, 1.0), mat(T, d_m, d_m + 3 * odd, 1.0)
+    kp = BL.pad8(k, 2)
+    wmat = lambda rows_shared: mat(k, d_m, d_m + odd, 0.1) if rows_shared else mat(d_m, kp, kp + odd, 0.1)
+    w1, w2 = wmat(lin), wmat(not lin)
+    w1b = wmat(lin) if sw else None
+    buf = L.ffn_buffers(T, d_m, k, act, dtype, DEV, transposed=lin)
+    lay = {"w_in_layout": int(lin), "w_out_layout": int(not lin)}
+    L.ffn_fwd_bwd(X, dY, act, w1, w2, k, buf, w1bc=w1b, bias_grads=not sw, **lay)
+    B.ecospa_device_status()
+    d = lambda w, rows: w.double().t() if rows else w.double()[:, :k]      # d_m x k
+    W1, W2, x, dy = d(w1, lin), d(w2, not lin), X.double(), dY.double()
+    H, dA = x @ W1, dy @ W2
+    if sw:
+        Hb, s = x @ d(w1b, lin), torch.sigmoid(H)
+        A, dH, dHb = H * s * Hb, dA * Hb * s * (1 + H * (1 - s)), dA * H * s
+        dX = dH @ W1.t() + dHb @ d(w1b, lin).t()
+    else:
+        A = torch.nn.functional.gelu(H)
+        dH = dA * (0.5 * (1 + torch.erf(H / 2 ** 0.5)) + H * torch.exp(-0.5 * H * H) / (2 * np.pi) ** 0.5)
+        dX = dH @ W1.t()
+    st = lambda gw, rows: (gw.t() if rows else gw).cpu().numpy()
+    cut = lambda t, rows: t if rows else t[:, :k]
+    errs = {"Y": _rel(buf["Y"], (A @ W2.t()).cpu().numpy()), "dX": _rel(buf["dX"], dX.cpu().numpy()),
+            "dW1": _rel(cut(buf["dW1"], lin), st(x.t() @ dH, lin)), "dW2": _rel(cut(buf["dW2"], not lin), st(dy.t() @ A, not lin))}
+    if sw:
+        errs["dW1b"] = _rel(cut(buf["dW1b"], lin), st(x.t() @ dHb, lin))
+    else:
+        errs["db1"], errs["db2"] = _rel(buf["db1"], dH.sum(0).cpu().numpy()), _rel(buf["db2"], dy.sum(0).cpu().numpy())
+    assert max(errs.values()) <= 2e-2, errs
