@@ -14,6 +14,31 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("every,n_kept", [(1, 255), (1, 3000), (2, 256), (2, 1500), (5, 257), (9, 300), (40, 75), (1, 1)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_gather_spans(dtype, every, n_kept, shift):
+    """Shared-cols tensors: spans of 256 outputs that are staged four, two or one row ahead, or too wide to be; "no index"
+    entries; an input that does not start on a 16-byte boundary; row counts around a tile's."""
+    r = np.random.default_rng(every * 1000 + n_kept)
+    D = 3000
+    idx = np.sort(r.choice(np.arange(0, D, every), n_kept, replace=False)).astype(np.int32)
+    idx[r.random(n_kept) < 0.02] = -1
+    kept = torch.from_numpy(idx).to(DEV)
+    jobs, outs, ins = [], [], []
+    for rows in (1, 15, 17, 130):
+        t = torch.randn(rows + 1, D + 8, device=DEV).to(dtype)[:rows, shift:shift + D]
+        o = torch.full((rows, BL.pad8(n_kept, t.element_size())), 7.0, dtype=dtype, device=DEV)
+        jobs.append(B.gather(t, o, B.SHARED_COLS, kept, n_kept, D))
+        ins.append(t)
+        outs.append(o)
+    B.ecospa_compact_tensors(jobs)
+    at = torch.from_numpy(np.maximum(idx, 0)).long().to(DEV)
+    for t, o in zip(ins, outs):
+        want = torch.where(kept[None, :] >= 0, t[:, at], torch.zeros((), dtype=dtype, device=DEV))
+        assert torch.equal(o[:, :n_kept], want) and not o[:, n_kept:].any()
+
+
 def _rel(got, want):
     return float(np.linalg.norm(got.double().cpu().numpy() - want) / max(np.linalg.norm(want), 1e-30))
 
