@@ -22,7 +22,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxJobs = 400;      // per launch; 72 B each -> 28.8 KB of kernel parameters (limit 32764)
-constexpr int kMaxPairs = 256;     // per finalize launch; 64 B each
+constexpr int kMaxPairs = 256;     // per finalize launch; 80 B each
 constexpr int kRowTile = 32;       // shared-rows tile: rows per CTA
 constexpr int kUnroll = 4;
 
@@ -56,12 +56,14 @@ struct PairDesc {
     const float* gs2;
     int32_t n_seg, seg_len;
     int32_t d_off;      // offset of this pair in upsilon / raw
-    int32_t seg_start;  // first global segment index (also offset into fisher)
+    int32_t seg_start;  // first segment of this launch that is the pair's (offset into fisher)
+    int32_t blk_start;  // first block of this launch that is the pair's
     float inv_numel1, inv_numel2;
     int32_t rope;       // ecospa_rope_t: the scored unit is a rotation pair of shared indices
     int16_t rep1, rep2; // heads stacked per segment on the W_1 / W_2 side (grouped-query attention); 1 = ordinary pair
+    int32_t pad_;
 };
-static_assert(sizeof(PairDesc) == 72, "pair descriptor size");
+static_assert(sizeof(PairDesc) == 80, "pair descriptor size");
 
 struct FinalizeParams {
     int32_t n_pairs;
@@ -226,6 +228,7 @@ __device__ __forceinline__ void rows_tile(const SumsqJob& J, int local) {
 
 __global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__ SumsqParams P) {
     __shared__ float smem[kWarps * (256 + 4)];
+    pdl_start();
     const int tile = blockIdx.x;
     const int ji = find_owner(P.n_jobs, tile, [&](int i) { return P.jobs[i].tile_start; });
     const SumsqJob& J = P.jobs[ji];
@@ -239,96 +242,228 @@ __global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__
 
 // stat[c] = sum over chunks of partial[chunk][c], chunk order fixed.
 __global__ void __launch_bounds__(kThreads) reduce_kernel(const __grid_constant__ SumsqParams P) {
+    pdl_start();
     const int blk = blockIdx.x;
     const int ji = find_owner(P.n_jobs, blk, [&](int i) { return P.jobs[i].red_start; });
     const SumsqJob& J = P.jobs[ji];
     const int c = (blk - J.red_start) * kThreads + threadIdx.x;
+    pdl_wait();
     if (J.n_chunks <= 1 || c >= J.D) return;
     float s = 0.f;
     for (int k = 0; k < J.n_chunks; ++k) s += J.partial[static_cast<int64_t>(k) * J.D + c];
     J.stat[c] = s;
 }
 
-__global__ void __launch_bounds__(kThreads) finalize_kernel(const __grid_constant__ FinalizeParams P) {
-    __shared__ float scratch[kWarps];
-    const int seg = blockIdx.x;
-    const int pi = find_owner(P.n_pairs, seg, [&](int i) { return P.pairs[i].seg_start; });
-    const PairDesc& Q = P.pairs[pi];
-    const int s = seg - Q.seg_start;
-    const int base = s * Q.seg_len;
-    if (Q.rep1 > 1 || Q.rep2 > 1) {
-        // Grouped heads: the statistic of index j on a stacked side is the sum over the group's heads, in head order.
-        auto stacked = [&](const float* v, int rep, int j) {
-            float t = 0.f;
-            for (int r = 0; r < rep; ++r) t += v[(s * rep + r) * Q.seg_len + j];
-            return t;
-        };
-        float ss = 0.f;
-        for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-            const float r = sqrtf(stacked(Q.c1, Q.rep1, j)) * sqrtf(stacked(Q.c2, Q.rep2, j));
-            ss = fmaf(r, r, ss);
-        }
-        const float nrm = sqrtf(block_sum<kWarps>(ss, scratch));
-        for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-            const float r = sqrtf(stacked(Q.c1, Q.rep1, j)) * sqrtf(stacked(Q.c2, Q.rep2, j));
-            if (P.raw) P.raw[Q.d_off + base + j] = r;
-            P.upsilon[Q.d_off + base + j] = nrm > 0.f ? __fdiv_rn(r, nrm) : 0.f;
-        }
-        if (P.fisher) {
-            float a = 0.f, b = 0.f;
-            for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-                a += stacked(Q.gs1, Q.rep1, j);
-                b += stacked(Q.gs2, Q.rep2, j);
-            }
-            a = block_sum<kWarps>(a, scratch);
-            b = block_sum<kWarps>(b, scratch);
-            if (threadIdx.x == 0)
-                P.fisher[seg] = static_cast<float>(0.5 * (static_cast<double>(a) * Q.inv_numel1 + static_cast<double>(b) * Q.inv_numel2) *
-                                                   P.inv_n_samples);
-        }
+// Scores and importance of the segments, from the per-index sums.  The work is a few operations per index; what bounds it is
+// the latency of the loads, so everything is laid out for few dependent rounds of them:
+//   segments of up to kNarrow indices (heads): one warp each, kFinWarps to a block; an index or a few per lane, no barrier.
+//   wider segments (FFN): two blocks of kFinThreads each, one for the scores and one for the importance (they share
+//   nothing), several independent loads per thread in flight, the scores kept in shared memory between the two passes.
+// One 256-thread block per segment, which walked an 11008-wide segment in 43 dependent rounds and three passes, took
+// 30 us on the FFN segment of one 4096 / 11008 layer (now 12) and 22 us on 22 layers of 2048 / 5632 (now 9).
+// The sums keep one order for every width, that of 256 virtual threads: virtual thread t adds indices t, t + 256, ... in turn,
+// then 32 neighbours are added as a shuffle tree and the eight results in turn.  (A narrow segment has one index per virtual
+// thread, so its warp goes straight to the trees.)
+constexpr int kFinThreads = 512;
+constexpr int kFinWarps = kFinThreads / 32;
+constexpr int kNarrow = 256;
+constexpr int kFinPass = 22 * kFinThreads;        // scores of a wide segment that shared memory holds at a time
+
+// What the scores of a pair are taken from: single indices, rotation pairs of indices, or indices summed over grouped heads.
+// A compile-time choice, so that the loads of an unrolled loop stand free of branches and go out together.
+enum : int { kSingle = 0, kRotation = 1, kGrouped = 2 };
+
+// The statistic of index j of segment seg (grouped heads: over the `rep` heads that the segment stacks, in head order).
+template <int MODE>
+__device__ __forceinline__ float stat_of(const float* v, int rep, int64_t seg, int n, int j) {
+    if (MODE != kGrouped) return v[seg * n + j];
+    float t = 0.f;
+    for (int r = 0; r < rep; ++r) t += v[(seg * rep + r) * n + j];
+    return t;
+}
+// The two sums of squares behind the raw score of index j: its own column's / row's, or those of its rotation pair (both
+// members get the pair's value; the pair is counted once in the normaliser).  raw = sqrt(x) * sqrt(y); kept apart from the
+// square roots, whose branches would hold back the loads of an unrolled loop.
+template <int MODE>
+__device__ __forceinline__ void norms_of(const PairDesc& Q, int64_t seg, int n, int j, float& x, float& y) {
+    if (MODE != kRotation) {
+        x = stat_of<MODE>(Q.c1, Q.rep1, seg, n, j);
+        y = stat_of<MODE>(Q.c2, Q.rep2, seg, n, j);
         return;
     }
-    const float* c1 = Q.c1 + base;
-    const float* c2 = Q.c2 + base;
+    const int half = n >> 1;
+    const bool inter = Q.rope == ECOSPA_ROPE_INTERLEAVED;
+    const int a = inter ? (j & ~1) : (j < half ? j : j - half);
+    const int b = inter ? (a | 1) : a + half;
+    const float* c1 = Q.c1 + seg * n;
+    const float* c2 = Q.c2 + seg * n;
+    x = c1[a] + c1[b];
+    y = c2[a] + c2[b];
+}
+__device__ __forceinline__ float importance(const PairDesc& Q, float a, float ab, float b, double inv_n_samples) {
+    double t1 = static_cast<double>(a) * Q.inv_numel1;
+    if (Q.gs1b) t1 = 0.5 * (t1 + static_cast<double>(ab) * Q.inv_numel1);
+    const double t2 = static_cast<double>(b) * Q.inv_numel2;
+    return static_cast<float>(0.5 * (t1 + t2) * inv_n_samples);
+}
 
-    // raw score of index j: its own column/row norms, or those of its rotation pair (both members get the
-    // pair's value; the pair is counted once in the normaliser)
-    const int half = Q.seg_len >> 1;
-    auto raw_of = [&](int j) -> float {
-        if (Q.rope == ECOSPA_ROPE_NONE) return sqrtf(c1[j]) * sqrtf(c2[j]);
-        const int a = Q.rope == ECOSPA_ROPE_INTERLEAVED ? (j & ~1) : (j < half ? j : j - half);
-        const int b = Q.rope == ECOSPA_ROPE_INTERLEAVED ? (a | 1) : a + half;
-        return sqrtf(c1[a] + c1[b]) * sqrtf(c2[a] + c2[b]);
+// A warp, a segment of at most 32 * TREES indices.
+template <int MODE, int TREES>
+__device__ __forceinline__ void finalize_narrow(const FinalizeParams& P, const PairDesc& Q, int seg) {
+    const int lane = threadIdx.x & 31, n = Q.seg_len;
+    const bool with_fisher = P.fisher != nullptr, with_up = Q.gs1b != nullptr;
+    float r[TREES], y[TREES], g1[TREES], g1b[TREES], g2[TREES];
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        const int j = min(32 * i + lane, n - 1);          // (lanes past the end read the last index and add nothing)
+        norms_of<MODE>(Q, seg, n, j, r[i], y[i]);
+        g1[i] = with_fisher ? stat_of<MODE>(Q.gs1, Q.rep1, seg, n, j) : 0.f;
+        g1b[i] = with_fisher && with_up ? Q.gs1b[static_cast<int64_t>(seg) * n + j] : 0.f;
+        g2[i] = with_fisher ? stat_of<MODE>(Q.gs2, Q.rep2, seg, n, j) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        r[i] = sqrtf(r[i]) * sqrtf(y[i]);
+        if (32 * i + lane >= n) r[i] = g1[i] = g1b[i] = g2[i] = 0.f;
+    }
+    float total = 0.f, a = 0.f, ab = 0.f, b = 0.f;
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        total += warp_sum(fmaf(r[i], r[i], 0.f));
+        a += warp_sum(g1[i]);
+        ab += warp_sum(g1b[i]);
+        b += warp_sum(g2[i]);
+    }
+    const float nrm = sqrtf(MODE == kRotation ? 0.5f * total : total);
+    const int64_t out = Q.d_off + static_cast<int64_t>(seg) * n;
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        const int j = 32 * i + lane;
+        if (j < n) {
+            if (P.raw) P.raw[out + j] = r[i];
+            P.upsilon[out + j] = nrm > 0.f ? __fdiv_rn(r[i], nrm) : 0.f;
+        }
+    }
+    if (with_fisher && lane == 0) P.fisher[Q.seg_start + seg] = importance(Q, a, ab, b, P.inv_n_samples);
+}
+
+// Wide segments.  The loops stay rolled: a block runs them once, so straight-line code would wait for its instructions.
+// Ends a sum of 256 virtual threads (threads first ... first + 255 of the block hold one each).
+__device__ __forceinline__ float end_wide_sum(float acc, int first, float* scratch) {
+    acc = warp_sum(acc);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += scratch[(first >> 5) + w];
+    return t;
+}
+template <int MODE>
+__device__ __forceinline__ void scores_wide(const FinalizeParams& P, const PairDesc& Q, int seg, float* buf, float* scratch) {
+    const int n = Q.seg_len, tid = threadIdx.x;
+    const int64_t out = Q.d_off + static_cast<int64_t>(seg) * n;
+    // buf[j - base] = raw score of index j of a pass
+    auto compute = [&](int base, int end) {
+#pragma unroll 1
+        for (int j0 = base + tid; j0 < end; j0 += 4 * kFinThreads) {
+            float x[4], y[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) norms_of<MODE>(Q, seg, n, min(j0 + i * kFinThreads, end - 1), x[i], y[i]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int j = j0 + i * kFinThreads;
+                const float r = sqrtf(x[i]) * sqrtf(y[i]);
+                if (j < end) buf[j - base] = r;
+            }
+        }
     };
-    float ss = 0.f;
-    for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-        const float r = raw_of(j);
-        ss = fmaf(r, r, ss);
-    }
-    const float total = block_sum<kWarps>(ss, scratch);
-    const float nrm = sqrtf(Q.rope == ECOSPA_ROPE_NONE ? total : 0.5f * total);
-    for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-        const float r = raw_of(j);
-        if (P.raw) P.raw[Q.d_off + base + j] = r;
-        P.upsilon[Q.d_off + base + j] = nrm > 0.f ? __fdiv_rn(r, nrm) : 0.f;
-    }
-    if (P.fisher) {
-        float a = 0.f, ab = 0.f, b = 0.f;
-        for (int j = threadIdx.x; j < Q.seg_len; j += kThreads) {
-            a += Q.gs1[base + j];
-            if (Q.gs1b) ab += Q.gs1b[base + j];
-            b += Q.gs2[base + j];
-        }
-        a = block_sum<kWarps>(a, scratch);
-        ab = block_sum<kWarps>(ab, scratch);
-        b = block_sum<kWarps>(b, scratch);
-        if (threadIdx.x == 0) {
-            double t1 = static_cast<double>(a) * Q.inv_numel1;
-            if (Q.gs1b) t1 = 0.5 * (t1 + static_cast<double>(ab) * Q.inv_numel1);
-            const double t2 = static_cast<double>(b) * Q.inv_numel2;
-            P.fisher[seg] = static_cast<float>(0.5 * (t1 + t2) * P.inv_n_samples);
+    float acc = 0.f;
+#pragma unroll 1
+    for (int base = 0; base < n; base += kFinPass) {
+        const int end = min(n, base + kFinPass);
+        if (base > 0) __syncthreads();                       // the previous pass has been added
+        compute(base, end);
+        __syncthreads();
+        if (tid < 256) {
+#pragma unroll 8
+            for (int j = tid; j < end - base; j += 256) acc = fmaf(buf[j], buf[j], acc);
         }
     }
+    const float total = end_wide_sum(acc, 0, scratch);
+    const float nrm = sqrtf(MODE == kRotation ? 0.5f * total : total);
+#pragma unroll 1
+    for (int base = 0; base < n; base += kFinPass) {
+        const int end = min(n, base + kFinPass);
+        if (n > kFinPass) {                                  // (the buffer holds the last pass only)
+            __syncthreads();
+            compute(base, end);
+            __syncthreads();
+        }
+#pragma unroll 2
+        for (int j = base + tid; j < end; j += kFinThreads) {
+            const float r = buf[j - base];
+            if (P.raw) P.raw[out + j] = r;
+            P.upsilon[out + j] = nrm > 0.f ? __fdiv_rn(r, nrm) : 0.f;
+        }
+    }
+}
+// Virtual thread vt's sum of a statistic.
+template <int MODE>
+__device__ __forceinline__ float virtual_sum(const float* v, int rep, int seg, int n, int vt) {
+    float s = 0.f;
+#pragma unroll 1
+    for (int j0 = vt; j0 < n; j0 += 8 * 256) {
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = stat_of<MODE>(v, rep, seg, n, min(j0 + 256 * i, n - 1));
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (j0 + 256 * i < n) s += x[i];
+    }
+    return s;
+}
+template <int MODE>
+__device__ __forceinline__ void importance_wide(const FinalizeParams& P, const PairDesc& Q, int seg, float* scratch) {
+    // threads 0-255: W_1's sum, then the up projection's; threads 256-511: W_2's
+    const int n = Q.seg_len, tid = threadIdx.x;
+    const bool first = tid < 256;
+    const float s = virtual_sum<MODE>(first ? Q.gs1 : Q.gs2, first ? Q.rep1 : Q.rep2, seg, n, tid & 255);
+    const float s_up = first && Q.gs1b ? virtual_sum<kSingle>(Q.gs1b, 1, seg, n, tid) : 0.f;
+    const float a = end_wide_sum(s, 0, scratch);
+    const float b = end_wide_sum(s, 256, scratch);
+    const float ab = end_wide_sum(s_up, 0, scratch);
+    if (tid == 0) P.fisher[Q.seg_start + seg] = importance(Q, a, ab, b, P.inv_n_samples);
+}
+
+// A block's share of a pair: kFinWarps narrow segments, or the scores or the importance of one wide segment.
+template <int MODE>
+__device__ __forceinline__ void finalize_pair(const FinalizeParams& P, const PairDesc& Q, int local, float* buf, float* scratch) {
+    const int n = Q.seg_len;
+    if (n <= kNarrow) {
+        const int seg = local * kFinWarps + (threadIdx.x >> 5);
+        if (seg >= Q.n_seg) return;
+        if (n <= 64) finalize_narrow<MODE, 2>(P, Q, seg);
+        else if (n <= 128) finalize_narrow<MODE, 4>(P, Q, seg);
+        else finalize_narrow<MODE, kNarrow / 32>(P, Q, seg);
+        return;
+    }
+    if (P.fisher && (local & 1)) importance_wide<MODE>(P, Q, local >> 1, scratch);
+    else scores_wide<MODE>(P, Q, P.fisher ? local >> 1 : local, buf, scratch);
+}
+
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const __grid_constant__ FinalizeParams P) {
+    __shared__ float buf[kFinPass];
+    __shared__ float scratch[kFinWarps];
+    pdl_start();
+    const int blk = blockIdx.x;
+    const int pi = find_owner(P.n_pairs, blk, [&](int i) { return P.pairs[i].blk_start; });
+    const PairDesc& Q = P.pairs[pi];
+    const int local = blk - Q.blk_start;
+    pdl_wait();
+    if (Q.rep1 > 1 || Q.rep2 > 1) finalize_pair<kGrouped>(P, Q, local, buf, scratch);
+    else if (Q.rope != ECOSPA_ROPE_NONE) finalize_pair<kRotation>(P, Q, local, buf, scratch);
+    else finalize_pair<kSingle>(P, Q, local, buf, scratch);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -497,8 +632,7 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
         ecospa_status_t st = check_launch("sumsq_kernel");
         if (st != ECOSPA_OK) return st;
         if (red > 0) {
-            reduce_kernel<<<red, kThreads, 0, stream>>>(sp);
-            if ((st = check_launch("reduce_kernel")) != ECOSPA_OK) return st;
+            if ((st = launch_pdl(reduce_kernel, red, kThreads, stream, sp, "reduce_kernel")) != ECOSPA_OK) return st;
         }
     }
 
@@ -508,7 +642,7 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
     int32_t d_off = 0, seg_off = 0;
     int p = 0;
     while (p < n_pairs) {
-        int np = 0, segs = 0;
+        int np = 0, segs = 0, blocks = 0;
         const int32_t seg_base = seg_off;
         for (; p < n_pairs && np < kMaxPairs; ++p, ++np) {
             const ecospa_pair_t& pr = pairs[p];
@@ -527,6 +661,8 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             Q.rope = pr.rope;
             Q.d_off = d_off;
             Q.seg_start = segs;
+            Q.blk_start = blocks;
+            blocks += pr.seg_len <= kNarrow ? static_cast<int>(ceil_div(pr.n_seg, kFinWarps)) : pr.n_seg * (grads ? 2 : 1);
             Q.rep1 = static_cast<int16_t>(std::max(1, pr.w1_rep));
             Q.rep2 = static_cast<int16_t>(std::max(1, pr.w2_rep));
             Q.inv_numel1 = static_cast<float>(1.0 / (static_cast<double>(pr.w1.other_dim) * pr.seg_len * Q.rep1));
@@ -540,8 +676,7 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
         fp.raw = raw;
         fp.fisher = fisher ? fisher + seg_base : nullptr;
         fp.inv_n_samples = 1.0 / n_samples;
-        finalize_kernel<<<segs, kThreads, 0, stream>>>(fp);
-        ecospa_status_t st = check_launch("finalize_kernel");
+        const ecospa_status_t st = launch_pdl(finalize_kernel, blocks, kFinThreads, stream, fp, "finalize_kernel");
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;

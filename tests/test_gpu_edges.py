@@ -14,6 +14,33 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 65, 128, 129, 256, 257, 512, 513, 11264, 11265, 23000])
+@pytest.mark.parametrize("rope", [B.ROPE_NONE, B.ROPE_HALF])
+def test_score_segment_widths(n, rope):
+    """Up to 256 indices a warp, above it two blocks, above 11264 in passes; beside a group of another width."""
+    if rope and n % 2:
+        pytest.skip("rotation pairs need an even width")
+    g = torch.Generator().manual_seed(n)
+    segs, d_m = 3, 16
+    w = {k: torch.randn(d_m, segs * n, generator=g) for k in ("w1", "w2", "g1", "g2")}
+    v = {k: torch.randn(d_m, 2 * 40, generator=g) for k in ("w1", "w2", "g1", "g2")}
+    dev = lambda t: {k: x.to(DEV) for k, x in t.items()}
+    wd, vd = dev(w), dev(v)
+    ps = [B.pair(B.PAIR_PLAIN, segs, n, wd["w1"], wd["w2"], 0, 0, g1=wd["g1"], g2=wd["g2"], rope=rope),
+          B.pair(B.PAIR_PLAIN, 2, 40, vd["w1"], vd["w2"], 0, 0, g1=vd["g1"], g2=vd["g2"])]
+    ups, fis = torch.empty(segs * n + 80, device=DEV), torch.empty(segs + 2, device=DEV)
+    raw, only = torch.empty_like(ups), torch.empty_like(ups)
+    B.ecospa_score_pairs(ps, 7.0, ups, raw, fis)
+    B.ecospa_score_pairs(ps, 7.0, only)                       # without importance: one block per wide segment
+    assert torch.equal(ups, only)
+    raw_o, ups_o = O.score_pair(w["w1"], w["w2"], 0, 0, segs, n, rope=rope)
+    raw_v, ups_v = O.score_pair(v["w1"], v["w2"], 0, 0, 2, 40)
+    for got, a, b in ((ups, ups_o, ups_v), (raw, raw_o, raw_v)):
+        np.testing.assert_allclose(got.double().cpu().numpy(), np.concatenate([a.ravel(), b.ravel()]), rtol=1e-5, atol=1e-7)
+    want = np.concatenate([O.fisher_pair(w["g1"], w["g2"], 0, 0, segs, n, 7.0).ravel(), O.fisher_pair(v["g1"], v["g2"], 0, 0, 2, 40, 7.0).ravel()])
+    np.testing.assert_allclose(fis.double().cpu().numpy(), want, rtol=1e-5)
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("every,n_kept", [(1, 255), (1, 3000), (2, 256), (2, 1500), (5, 257), (9, 300), (40, 75), (1, 1)])
 @pytest.mark.parametrize("shift", [0, 1])
