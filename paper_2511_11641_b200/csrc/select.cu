@@ -1,9 +1,8 @@
 // Aligned top-k per segment (Definition 1 applied to the lowest-scored indices).
 //
-// One CTA per segment.  The k-th largest score is found by a 4-pass radix select over an
-// order-preserving 32-bit key; the kept indices are then emitted in ascending order with a
-// block-wide stream compaction, taking equal-to-threshold scores lowest index first.  The score
-// vector of a segment (<= 44 KB at the shapes of interest) is re-read from L1/L2 in each pass.
+// The k-th largest score of a segment is found over an order-preserving 32-bit key (bit by bit with ballots for a segment
+// that a warp holds in registers, by counting into parts of a shrinking range of keys for a wider one); the kept indices are then emitted in ascending
+// order, taking equal-to-threshold scores lowest index first.  
 
 #include <vector>
 
@@ -24,6 +23,8 @@ struct SelPair {
     int32_t d_off;      // offset of the pair's scores in upsilon, and base added to nothing: kept
                         // indices are relative to the pair group (segment offset included)
     int32_t rope;       // ecospa_rope_t: units of two shared indices are ranked and kept together
+    int32_t blk_start;  // select_kernel: first block of the launch that is the pair's,
+    int32_t seg_first, n_seg;   // and the pair's segments of the launch
 };
 
 struct SelectParams {
@@ -46,141 +47,261 @@ __device__ __forceinline__ uint32_t order_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// ROPE = false: no pair group of the launch has rotation pairs (the common case, compiled without the unit logic).
-template <bool ROPE>
-__global__ void __launch_bounds__(kThreads) select_kernel(const __grid_constant__ SelectParams P) {
-    __shared__ int hist[256];
-    __shared__ int warp_tot[kWarps];
-    __shared__ uint32_t sh_prefix;
-    __shared__ int sh_want, sh_cnt_eq;
+// Segments of up to kNarrow indices (heads) take a warp each, kSelWarps to a block; wider ones (FFN) a block of kSelThreads
+// that keeps its keys in shared memory.  The scores of a model are a few hundred KB at most: what bounds the
+// kernel is the chain of dependent steps of its longest segment.  One 256-thread block per segment, one score per thread and
+// round, four barriers a round, took 27 us on the FFN segment of one 4096 / 11008 layer (now 14) and 20 us on 22 layers of 2048 / 5632 (now 13).
+constexpr int kSelThreads = 512;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kNarrow = 256;
+constexpr int kSelPass = 22 * kSelThreads;       // keys of a wide segment that shared memory holds at a time
 
-    const int seg = blockIdx.x;
+// What a segment needs: its scores (unit u at stride * u), how many units there are and stay, where the kept list goes.
+struct SegView {
+    const float* sc;
+    int n, k, stride, rope, first, out0;
+    int32_t* kept;
+    __device__ __forceinline__ uint32_t key(int j) const { return order_key(sc[static_cast<int64_t>(j) * stride]); }
+    __device__ __forceinline__ void emit(int j, int pos) const {
+        if (rope == ECOSPA_ROPE_NONE) {
+            kept[out0 + pos] = first + j;
+        } else if (rope == ECOSPA_ROPE_INTERLEAVED) {           // members 2j, 2j + 1
+            kept[out0 + 2 * pos] = first + 2 * j;
+            kept[out0 + 2 * pos + 1] = first + 2 * j + 1;
+        } else {                                                // members j, j + seg_len/2: both halves ascending
+            kept[out0 + pos] = first + j;
+            kept[out0 + k + pos] = first + n + j;
+        }
+    }
+};
+// Opens segment `seg` of the launch (one thread, `writer`, notes its offset).
+__device__ __forceinline__ SegView open_segment(const SelectParams& P, const SelPair& Q, int seg, bool writer) {
+    SegView V;
+    const int seg_len = Q.seg_len, seg_in_pair = seg - Q.seg_start;
+    // With rotation pairs the ranked units are the seg_len/2 pairs; both members carry the pair's score, so
+    // unit u is read at index 2u (interleaved pairs) or u (pairs of the two halves).
+    V.rope = Q.rope;
+    V.n = Q.rope ? seg_len >> 1 : seg_len;
+    V.stride = Q.rope == ECOSPA_ROPE_INTERLEAVED ? 2 : 1;
+    V.first = seg_in_pair * seg_len;                            // kept indices are shared indices of the pair group
+    V.sc = P.upsilon + Q.d_off + static_cast<int64_t>(seg_in_pair) * seg_len;
+    V.out0 = P.k_dev ? Q.d_off + seg_in_pair * seg_len : P.out_off[seg];
+    const int k_idx = P.k_dev ? min(max(P.k_dev[P.seg_base + seg], 0), seg_len) : P.out_off[seg + 1] - V.out0;
+    V.k = Q.rope ? k_idx >> 1 : k_idx;
+    V.kept = P.kept;
+    if (P.seg_offsets && writer) {
+        P.seg_offsets[P.seg_base + seg] = V.out0;
+        if (P.is_last && seg == P.n_segs - 1) P.seg_offsets[P.seg_base + seg + 1] = V.out0 + k_idx;
+    }
+    return V;
+}
+
+// A warp, at most 32 * TREES units.  The key of the k-th largest is the largest value that at least k keys reach: built bit
+// by bit with ballots, the keys in registers.  (TREES is a compile-time count: a ballot under a condition costs more than
+// the ballot.)
+template <int TREES>
+__device__ __forceinline__ void select_narrow(const SegView& V, int lane) {
+    const int n = V.n, k = V.k;
+    uint32_t key[TREES];
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        key[i] = V.key(min(32 * i + lane, n - 1));
+        if (32 * i + lane >= n) key[i] = 0u;                // (below every threshold that is tried)
+    }
+    uint32_t thr = 0;
+#pragma unroll 4
+    for (int bit = 31; bit >= 0; --bit) {
+        const uint32_t t = thr | (1u << bit);
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < TREES; ++i) c += __popc(__ballot_sync(0xffffffffu, key[i] >= t));
+        if (c >= k) thr = t;
+    }
+    unsigned bg[TREES], be[TREES];
+    int above = 0;
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        const bool in = 32 * i + lane < n;
+        bg[i] = __ballot_sync(0xffffffffu, in && key[i] > thr);
+        be[i] = __ballot_sync(0xffffffffu, in && key[i] == thr);
+        above += __popc(bg[i]);
+    }
+    const int want = k - above;             // units equal to the threshold that stay, lowest index first
+    const unsigned before = (1u << lane) - 1u;
+    int run_gt = 0, run_eq = 0;
+#pragma unroll
+    for (int i = 0; i < TREES; ++i) {
+        const int eq_before = run_eq + __popc(be[i] & before);
+        const bool gt = (bg[i] >> lane) & 1u, eq = (be[i] >> lane) & 1u;
+        if (gt || (eq && eq_before < want)) V.emit(32 * i + lane, run_gt + __popc(bg[i] & before) + min(eq_before, want));
+        run_gt += __popc(bg[i]);
+        run_eq += __popc(be[i]);
+    }
+}
+
+// A block, any number of units.  The key of the k-th largest is found by narrowing a range of keys: the range is cut into
+// up to kBins equal parts, the keys are counted per part, and the part that holds the k-th largest is the next range.
+// Starting from the smallest and the largest key spreads the counting over the bins (the scores of a segment share their
+// leading bits: counting by fixed digits sends most of them to one bin).  The keys are kept in shared memory, kSelPass at a
+// time; the loops stay rolled, because a block runs them a few times only and would wait for straight-line code.
+constexpr int kBins = kSelThreads;
+struct WideShared {
+    uint32_t key[kSelPass];
+    int hist[kBins];
+    uint32_t lo, hi;
+    int want;
+    uint32_t warp_a[kSelWarps], warp_b[kSelWarps];
+};
+__device__ __forceinline__ void select_wide(const SegView& V, WideShared& S) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = V.n, k = V.k;
+    const bool held = n <= kSelPass;
+    auto load = [&](int base) {                                 // S.key[j - base] = key of unit j
+        __syncthreads();
+        const int end = min(n, base + kSelPass);
+#pragma unroll 1
+        for (int j0 = base + tid; j0 < end; j0 += 4 * kSelThreads) {
+            uint32_t t[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) t[i] = V.key(min(j0 + i * kSelThreads, end - 1));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (j0 + i * kSelThreads < end) S.key[j0 + i * kSelThreads - base] = t[i];
+        }
+        __syncthreads();
+    };
+    uint32_t lo = ~0u, hi = 0u;
+#pragma unroll 1
+    for (int base = 0; base < n; base += kSelPass) {
+        load(base);
+        const int m = min(n - base, kSelPass);
+#pragma unroll 4
+        for (int j = tid; j < m; j += kSelThreads) {
+            lo = min(lo, S.key[j]);
+            hi = max(hi, S.key[j]);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        S.warp_a[warp] = lo;
+        S.warp_b[warp] = hi;
+    }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, S.warp_a[lane % kSelWarps]);
+    hi = __reduce_max_sync(0xffffffffu, S.warp_b[lane % kSelWarps]);
+    int want = k;                           // the k-th largest is the want-th largest of the keys in [lo, hi]
+#pragma unroll 1
+    while (lo < hi) {
+        const int shift = max(0, 23 - __clz(hi - lo));          // (hi - lo) >> shift < kBins
+        S.hist[tid] = 0;
+        __syncthreads();
+#pragma unroll 1
+        for (int base = 0; base < n; base += kSelPass) {
+            if (!held) load(base);
+            const int m = min(n - base, kSelPass);
+#pragma unroll 4
+            for (int j = tid; j < m; j += kSelThreads) {
+                const uint32_t key = S.key[j];
+                if (key - lo <= hi - lo) atomicAdd(&S.hist[(key - lo) >> shift], 1);
+            }
+        }
+        __syncthreads();
+        const int bin = kBins - 1 - tid, own = S.hist[bin];     // (a bin per thread, descending)
+        int incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) S.warp_a[warp] = static_cast<uint32_t>(incl);
+        __syncthreads();
+        incl += static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? S.warp_a[lane] : 0u));
+        if (incl - own < want && want <= incl) {
+            const uint32_t first = lo + (static_cast<uint32_t>(bin) << shift), last = (1u << shift) - 1u;
+            S.lo = first;
+            S.hi = hi - first < last ? hi : first + last;       // (first + last may not fit 32 bits)
+            S.want = want - (incl - own);
+        }
+        __syncthreads();
+        lo = S.lo;
+        hi = S.hi;
+        want = S.want;
+    }
+    const uint32_t thr = lo;                // key of the k-th largest; the first `want` units equal to it stay
+    // ascending order: a thread takes `own` neighbouring units (an odd number: no bank conflicts) as two bit masks, the counts
+    // before it come from a scan over the block, and the list is put together in shared memory so that it leaves in whole lines
+    int run_gt = 0, run_eq = 0;
+#pragma unroll 1
+    for (int base = 0; base < n; base += kSelPass) {
+        if (!held) load(base);
+        const int m = min(n - base, kSelPass), own = ((m + kSelThreads - 1) / kSelThreads) | 1, j0 = tid * own;
+        static_assert(kSelPass / kSelThreads <= 30, "one bit per unit");
+        uint32_t gt = 0, eq = 0;
+        const int cnt = min(max(m - j0, 0), own);
+#pragma unroll 4
+        for (int i = 0; i < cnt; ++i) {
+            const uint32_t key = S.key[j0 + i];
+            gt |= (key > thr ? 1u : 0u) << i;
+            eq |= (key == thr ? 1u : 0u) << i;
+        }
+        const uint32_t mine = static_cast<uint32_t>(__popc(gt)) | (static_cast<uint32_t>(__popc(eq)) << 16);
+        uint32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) S.warp_a[warp] = incl;
+        __syncthreads();                                        // (every key of the pass has been read, too)
+        const uint32_t all = S.warp_a[lane % kSelWarps];
+        const uint32_t before = incl - mine + __reduce_add_sync(0xffffffffu, lane < warp ? all : 0u);
+        const uint32_t total = __reduce_add_sync(0xffffffffu, lane < kSelWarps ? all : 0u);
+        const int eq_before = run_eq + static_cast<int>(before >> 16);
+        for (int drop = __popc(eq) - max(0, want - eq_before); drop > 0; --drop) eq &= ~(0x80000000u >> __clz(eq));   // lowest index first
+        const int first_pos = run_gt + min(run_eq, want);       // of this pass
+        int pos = run_gt + static_cast<int>(before & 0xffffu) + min(eq_before, want) - first_pos;
+        for (uint32_t sel = gt | eq; sel; sel &= sel - 1) S.key[pos++] = static_cast<uint32_t>(base + j0 + __ffs(sel) - 1);
+        __syncthreads();
+        run_gt += static_cast<int>(total & 0xffffu);
+        run_eq += static_cast<int>(total >> 16);
+        const int n_pass = run_gt + min(run_eq, want) - first_pos;
+#pragma unroll 2
+        for (int p = tid; p < n_pass; p += kSelThreads) V.emit(static_cast<int>(S.key[p]), first_pos + p);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_constant__ SelectParams P) {
+    __shared__ WideShared S;
+    pdl_start();
+    const int blk = blockIdx.x;
     int lo = 0, hi = P.n_pairs - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (P.pairs[mid].seg_start <= seg) lo = mid; else hi = mid - 1;
+        if (P.pairs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
     }
     const SelPair& Q = P.pairs[lo];
-    const int seg_len = Q.seg_len;
-    const int seg_in_pair = seg - Q.seg_start;
-    // With rotation pairs the ranked units are the seg_len/2 pairs; both members carry the pair's score, so
-    // unit u is read at index 2u (interleaved pairs) or u (pairs of the two halves).
-    const int rope = ROPE ? Q.rope : ECOSPA_ROPE_NONE;
-    const int n = rope ? seg_len >> 1 : seg_len;
-    const int stride = rope == ECOSPA_ROPE_INTERLEAVED ? 2 : 1;
-    const float* sc = P.upsilon + Q.d_off + static_cast<int64_t>(seg_in_pair) * seg_len;
-    const int out0 = P.k_dev ? Q.d_off + seg_in_pair * seg_len : P.out_off[seg];
-    const int k_idx = P.k_dev ? min(max(P.k_dev[P.seg_base + seg], 0), seg_len) : P.out_off[seg + 1] - out0;
-    const int k = rope ? k_idx >> 1 : k_idx;     // units to keep
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-    if (P.seg_offsets && tid == 0) {
-        P.seg_offsets[P.seg_base + seg] = out0;
-        if (P.is_last && seg == P.n_segs - 1) P.seg_offsets[P.seg_base + seg + 1] = out0 + k_idx;
+    pdl_wait();
+    if (Q.seg_len <= kNarrow) {
+        const int i = (blk - Q.blk_start) * kSelWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (i >= Q.n_seg) return;
+        const SegView V = open_segment(P, Q, Q.seg_first + i, lane == 0);
+        if (V.k <= 0) return;
+        if (V.n <= 64) select_narrow<2>(V, lane);
+        else if (V.n <= 128) select_narrow<4>(V, lane);
+        else select_narrow<kNarrow / 32>(V, lane);
+        return;
     }
-    if (k <= 0) return;
-
-    // ---- radix select: key of the k-th largest element
-    uint32_t prefix = 0, mask = 0;
-    int want = k, cnt_eq = 0;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        hist[tid] = 0;
-        __syncthreads();
-        for (int j = tid; j < n; j += kThreads) {
-            const uint32_t key = order_key(__ldg(sc + j * stride));
-            if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
-        }
-        __syncthreads();
-        if (warp == 0) {
-            // lane l owns bins 255-8l ... 248-8l (descending)
-            int local[8], s = 0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                local[b] = hist[255 - 8 * lane - b];
-                s += local[b];
-            }
-            int incl = s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const int excl = incl - s;
-            if (excl < want && want <= incl) {
-                int cum = excl;
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    if (cum < want && want <= cum + local[b]) {
-                        sh_prefix = prefix | (static_cast<uint32_t>(255 - 8 * lane - b) << shift);
-                        sh_want = want - cum;
-                        sh_cnt_eq = local[b];
-                    }
-                    cum += local[b];
-                }
-            }
-        }
-        __syncthreads();
-        prefix = sh_prefix;
-        want = sh_want;
-        cnt_eq = sh_cnt_eq;
-        mask |= 255u << shift;
-        __syncthreads();
-    }
-    const uint32_t thr = prefix;            // key of the k-th largest
-    const bool all_eq = (want == cnt_eq);   // every element equal to the threshold is kept
-
-    // ---- emit ascending: key > thr, plus the first `want` elements with key == thr
-    const int seg_first = seg_in_pair * seg_len;  // kept indices are shared indices of the pair group
-    int run_eq = 0, run_out = 0;
-    for (int base = 0; base < n; base += kThreads) {
-        const int j = base + tid;
-        uint32_t key = 0;
-        bool valid = j < n;
-        if (valid) key = order_key(__ldg(sc + j * stride));
-        const bool gt = valid && key > thr;
-        const bool eq = valid && key == thr;
-        bool sel;
-        if (all_eq) {
-            sel = gt || eq;
-        } else {
-            const unsigned beq = __ballot_sync(0xffffffffu, eq);
-            if (lane == 0) warp_tot[warp] = __popc(beq);
-            __syncthreads();
-            int rank = run_eq + __popc(beq & ((1u << lane) - 1u));
-            int tot = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                if (w < warp) rank += warp_tot[w];
-                tot += warp_tot[w];
-            }
-            run_eq += tot;
-            sel = gt || (eq && rank < want);
-            __syncthreads();
-        }
-        const unsigned bs = __ballot_sync(0xffffffffu, sel);
-        if (lane == 0) warp_tot[warp] = __popc(bs);
-        __syncthreads();
-        int pos = run_out + __popc(bs & ((1u << lane) - 1u));
-        int tot = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            if (w < warp) pos += warp_tot[w];
-            tot += warp_tot[w];
-        }
-        run_out += tot;
-        if (sel && pos < k) {
-            if (rope == ECOSPA_ROPE_NONE) {
-                P.kept[out0 + pos] = seg_first + j;
-            } else if (rope == ECOSPA_ROPE_INTERLEAVED) {           // members 2j, 2j + 1
-                P.kept[out0 + 2 * pos] = seg_first + 2 * j;
-                P.kept[out0 + 2 * pos + 1] = seg_first + 2 * j + 1;
-            } else {                                                // members j, j + seg_len/2: both halves ascending
-                P.kept[out0 + pos] = seg_first + j;
-                P.kept[out0 + k + pos] = seg_first + n + j;
-            }
-        }
-        __syncthreads();
-    }
+    const SegView V = open_segment(P, Q, Q.seg_first + (blk - Q.blk_start), threadIdx.x == 0);
+    if (V.k > 0) select_wide(V, S);
+}
+// Adds the pair's segments of a launch (those from `seg_first` on) to the launch's blocks.
+inline int select_blocks(SelPair& Q, int seg_first, int n_seg, int blk_start) {
+    Q.seg_first = seg_first;
+    Q.n_seg = n_seg;
+    Q.blk_start = blk_start;
+    return blk_start + (Q.seg_len <= kNarrow ? (n_seg + kSelWarps - 1) / kSelWarps : n_seg);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -216,6 +337,8 @@ struct ThresholdParams {
 __global__ void __launch_bounds__(kThreads) threshold_count_kernel(const __grid_constant__ ThresholdParams P) {
     __shared__ double scratch[kWarps];
     __shared__ uint32_t sh_max[kWarps];
+    pdl_start();
+    pdl_wait();
     const int seg = blockIdx.x;
     int lo_p = 0, hi_p = P.n_pairs - 1;
     while (lo_p < hi_p) {
@@ -345,6 +468,8 @@ struct PackParams {
     int32_t src[kPackSegs], dst[kPackSegs], k[kPackSegs], add[kPackSegs];
 };
 __global__ void __launch_bounds__(128) pack_kept_kernel(const __grid_constant__ PackParams P) {
+    pdl_start();
+    pdl_wait();
     const int s = blockIdx.x;
     for (int i = threadIdx.x; i < P.k[s]; i += blockDim.x) P.out[P.dst[s] + i] = P.slots[P.src[s] + i] + P.add[s];
 }
@@ -352,6 +477,8 @@ __global__ void __launch_bounds__(128) pack_kept_kernel(const __grid_constant__ 
 // Kept list with padded segments: the k[s] entries of segment s, then -1 ("no index") up to its padded count
 // (carried in the `add` slot of the parameters).
 __global__ void __launch_bounds__(128) pad_kept_kernel(const __grid_constant__ PackParams P) {
+    pdl_start();
+    pdl_wait();
     const int s = blockIdx.x;
     for (int i = threadIdx.x; i < P.add[s]; i += blockDim.x) P.out[P.dst[s] + i] = i < P.k[s] ? P.slots[P.src[s] + i] : -1;
 }
@@ -374,8 +501,7 @@ extern "C" ecospa_status_t ecospa_pad_kept(const int32_t* kept, const int32_t* s
         for (int i = 0; i < n; ++i) {
             pp.src[i] = src[base + i]; pp.dst[i] = dst[base + i]; pp.k[i] = k[base + i]; pp.add[i] = k_padded[base + i];
         }
-        pad_kept_kernel<<<n, 128, 0, static_cast<cudaStream_t>(stream)>>>(pp);
-        const ecospa_status_t st = check_launch("pad_kept_kernel");
+        const ecospa_status_t st = launch_pdl(pad_kept_kernel, n, 128, static_cast<cudaStream_t>(stream), pp, "pad_kept_kernel");
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
@@ -393,8 +519,7 @@ extern "C" ecospa_status_t ecospa_pack_kept(const int32_t* slots, const int32_t*
         for (int i = 0; i < n; ++i) {
             pp.src[i] = src[base + i]; pp.dst[i] = dst[base + i]; pp.k[i] = k[base + i]; pp.add[i] = add[base + i];
         }
-        pack_kept_kernel<<<n, 128, 0, static_cast<cudaStream_t>(stream)>>>(pp);
-        const ecospa_status_t st = check_launch("pack_kept_kernel");
+        const ecospa_status_t st = launch_pdl(pack_kept_kernel, n, 128, static_cast<cudaStream_t>(stream), pp, "pack_kept_kernel");
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
@@ -427,7 +552,7 @@ static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* 
     int p = 0, s_in_p = 0;          // walk position: pair, segment inside pair
     int32_t d_off = 0, out = 0, seg_global = 0;
     while (p < n_pairs) {
-        int np = 0, ns = 0;
+        int np = 0, ns = 0, blocks = 0;
         sp.seg_base = seg_global;
         // a pair can be split across launches; each launch sees it as a pair starting at s_in_p
         while (p < n_pairs && np < kMaxPairs && ns < kMaxSegs) {
@@ -437,6 +562,7 @@ static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* 
             Q.seg_len = seg_len[p];
             Q.d_off = d_off;
             Q.rope = rope ? rope[p] : ECOSPA_ROPE_NONE;
+            blocks = select_blocks(Q, ns, take, blocks);
             for (int s = 0; s < take; ++s) {
                 sp.out_off[ns++] = out;
                 out += k_per_seg[seg_global++];
@@ -456,11 +582,7 @@ static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* 
         sp.n_pairs = np;
         sp.n_segs = ns;
         sp.is_last = (p >= n_pairs) ? 1 : 0;
-        bool any_rope = false;
-        for (int i = 0; i < np; ++i) any_rope = any_rope || sp.pairs[i].rope != ECOSPA_ROPE_NONE;
-        if (any_rope) select_kernel<true><<<ns, kThreads, 0, stream>>>(sp);
-        else select_kernel<false><<<ns, kThreads, 0, stream>>>(sp);
-        ecospa_status_t st = check_launch("select_kernel");
+        const ecospa_status_t st = launch_pdl(select_kernel, blocks, kSelThreads, stream, sp, "select_kernel");
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
@@ -504,7 +626,7 @@ extern "C" ecospa_status_t ecospa_select_aligned_threshold(const float* upsilon,
     int p = 0, s_in_p = 0;
     int32_t d_off = 0, seg_global = 0;
     while (p < n_pairs) {
-        int np = 0, ns = 0;
+        int np = 0, ns = 0, blocks = 0;
         const int32_t seg_base = seg_global;
         while (p < n_pairs && np < kMaxPairs && ns < kMaxSegs) {
             const int take = std::min(n_seg[p] - s_in_p, kMaxSegs - ns);
@@ -513,6 +635,7 @@ extern "C" ecospa_status_t ecospa_select_aligned_threshold(const float* upsilon,
             Q.seg_len = seg_len[p];
             Q.d_off = d_off;
             Q.rope = rope ? rope[p] : ECOSPA_ROPE_NONE;
+            blocks = select_blocks(Q, ns, take, blocks);
             tp.pairs[np] = Q;
             ++np;
             ns += take;
@@ -527,18 +650,13 @@ extern "C" ecospa_status_t ecospa_select_aligned_threshold(const float* upsilon,
         tp.upsilon = upsilon; tp.chosen = chosen; tp.k_out = k_out;
         tp.theta = theta; tp.l1 = l1 ? 1 : 0; tp.k_min = k_min;
         tp.n_pairs = np; tp.seg_base = seg_base;
-        threshold_count_kernel<<<ns, kThreads, 0, stream>>>(tp);
-        ecospa_status_t st = check_launch("threshold_count_kernel");
+        ecospa_status_t st = launch_pdl(threshold_count_kernel, ns, kThreads, stream, tp, "threshold_count_kernel");
         if (st != ECOSPA_OK) return st;
         // the fixed-count selection, with the counts just written and one slot of seg_len entries per segment
         sp.upsilon = upsilon; sp.kept = kept; sp.seg_offsets = nullptr;
         sp.n_pairs = np; sp.n_segs = ns; sp.seg_base = seg_base; sp.is_last = 0;
         sp.k_dev = k_out;
-        bool any_rope = false;
-        for (int i = 0; i < np; ++i) any_rope = any_rope || sp.pairs[i].rope != ECOSPA_ROPE_NONE;
-        if (any_rope) select_kernel<true><<<ns, kThreads, 0, stream>>>(sp);
-        else select_kernel<false><<<ns, kThreads, 0, stream>>>(sp);
-        if ((st = check_launch("select_kernel")) != ECOSPA_OK) return st;
+        if ((st = launch_pdl(select_kernel, blocks, kSelThreads, stream, sp, "select_kernel")) != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
 }

@@ -41,6 +41,21 @@ def test_score_segment_widths(n, rope):
     np.testing.assert_allclose(fis.double().cpu().numpy(), want, rtol=1e-5)
 
 
+@pytest.mark.parametrize("n", [1, 2, 32, 33, 64, 65, 128, 129, 256, 257, 511, 513, 1024, 11264, 11265, 23000])
+@pytest.mark.parametrize("values", ["normal", "ties", "wide"])
+def test_select_segment_widths(n, values):
+    """Every count from one to all at the edges of the two forms; few distinct values; values from zero and denormals to inf."""
+    r = np.random.default_rng(n)
+    ks = sorted({1, min(2, n), n // 2, n - 1, n} - {0})
+    u = {"normal": lambda: np.abs(r.standard_normal(n)), "ties": lambda: r.integers(0, 4, n) * 0.25,
+         "wide": lambda: np.where(r.random(n) < 0.1, r.choice([0.0, np.inf, 1e-42, 3e38], n), 10.0 ** r.uniform(-30, 30, n))}[values]
+    ups = np.concatenate([u() for _ in ks]).astype(np.float32)
+    kept, offs = torch.empty(sum(ks), dtype=torch.int32, device=DEV), torch.empty(len(ks) + 1, dtype=torch.int32, device=DEV)
+    B.ecospa_select_aligned_topk(torch.from_numpy(ups).to(DEV), [len(ks)], [n], ks, kept, offs)
+    assert np.array_equal(kept.cpu().numpy(), O.select_topk(ups, len(ks), n, ks))
+    assert np.array_equal(offs.cpu().numpy(), np.concatenate([[0], np.cumsum(ks)]))
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("every,n_kept", [(1, 255), (1, 3000), (2, 256), (2, 1500), (5, 257), (9, 300), (40, 75), (1, 1)])
 @pytest.mark.parametrize("shift", [0, 1])
