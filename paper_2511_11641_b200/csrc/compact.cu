@@ -6,6 +6,7 @@
 //   (every sector of the input row holds a kept element at moderate sparsity), the writes of a warp are whole lines.
 // Pad columns [n_kept, round_up(n_kept, 16 bytes)) of shared-cols outputs are zero-filled.
 
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -16,7 +17,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxJobs = 400;
+// Jobs per launch, as kernel parameters; the small form is for a block or two of a model (a launch costs the host more, the
+// larger its parameters).
+constexpr int kMaxJobs = 400, kFewJobs = 32;
 constexpr int kColTile = 256;  // shared-cols tile: output columns per CTA
 constexpr int kRowTile = 32;   // shared-rows tile: output rows per CTA
 
@@ -34,10 +37,11 @@ struct GatherJob {
 };
 static_assert(sizeof(GatherJob) == 64, "job descriptor size");
 
+template <int CAP>
 struct GatherParams {
     int32_t n_jobs;
     int32_t col_rows;        // rows per shared-cols tile
-    GatherJob jobs[kMaxJobs];
+    GatherJob jobs[CAP];
 };
 
 // shared-cols tile: kColTile output columns of `rows_per_tile` rows; a warp takes every eighth row.  What bounds the work is
@@ -207,7 +211,8 @@ __device__ __forceinline__ void rows_tile(const GatherJob& J, int local) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 4) gather_kernel(const __grid_constant__ GatherParams P) {
+template <int CAP>
+__global__ void __launch_bounds__(kThreads, 4) gather_kernel(const __grid_constant__ GatherParams<CAP> P) {
     extern __shared__ __align__(16) uint8_t stage_all[];
     pdl_start();
     const int tile = blockIdx.x;
@@ -266,7 +271,7 @@ ecospa_status_t compact_impl(const ecospa_gather_t* jobs, int32_t n_jobs, cudaSt
         ecospa_status_t st = validate_job(jobs[i]);
         if (st != ECOSPA_OK) return st;
     }
-    static thread_local GatherParams gp;
+    static thread_local GatherParams<kMaxJobs> gp;
     // Rows per shared-cols tile: as many as leave four rounds of resident blocks (a tile's start costs a few dependent
     // loads, so long tiles are cheaper), at least two per warp.
     int64_t rows = 0;
@@ -311,8 +316,17 @@ ecospa_status_t compact_impl(const ecospa_gather_t* jobs, int32_t n_jobs, cudaSt
         }
         if (nj == 0) continue;
         gp.n_jobs = nj;
-        const ecospa_status_t st = launch_pdl(gather_kernel, tiles, kThreads, stream, gp, "gather_kernel",
-                                              any_cols ? kWarps * kStageBytes : 0);
+        const size_t smem = any_cols ? kWarps * kStageBytes : 0;
+        ecospa_status_t st;
+        if (nj <= kFewJobs) {
+            GatherParams<kFewJobs> few;
+            few.n_jobs = nj;
+            few.col_rows = col_rows;
+            std::copy(gp.jobs, gp.jobs + nj, few.jobs);
+            st = launch_pdl(gather_kernel<kFewJobs>, tiles, kThreads, stream, few, "gather_kernel", smem);
+        } else {
+            st = launch_pdl(gather_kernel<kMaxJobs>, tiles, kThreads, stream, gp, "gather_kernel", smem);
+        }
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;

@@ -48,8 +48,6 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kTmemCols = 512;
 constexpr int kMaxSeg = 3;
-constexpr int kOperandMaps = 3 * kMaxSeg;   // per K segment: one A map and two B (half) maps
-constexpr int kMapsPerOp = kOperandMaps + 3; // + one store map per output (C, C2, C3)
 constexpr int kEpiSlotBytes = 32 * 32 * 2;  // one 32-row x 64-byte staging image; a warp owns two (= one 32 x 128-byte image)
 constexpr int kEpiBytes = kEpiWarps * 2 * kEpiSlotBytes;
 constexpr int kSmemBytes = kRingBytes + kEpiBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
@@ -80,18 +78,27 @@ struct DevProblem {
     int64_t ldc, ldh;
 };
 
-constexpr int kMaxOrder = 2048;              // entries of the explicit tile schedule
 constexpr uint16_t kNoTile = 0xffff;
-struct GemmParams {
-    alignas(64) CUtensorMap maps[kMaxGemmOps * kMapsPerOp];
-    DevProblem prob[kMaxGemmOps];
+struct GemmHead {
     // Worker w runs, in round i, tile order[w + i * workers] (kNoTile = nothing) when use_order is set,
     // otherwise tile w + i * workers.
-    uint16_t order[kMaxOrder];
     int32_t n_problems, total_tiles, rounds, use_order;
     int* status;
     unsigned long long wait_limit_ns;   // every mbarrier wait of the launch gives up after this long
 };
+// Kernel parameters in two sizes: what a launch costs the host grows with them (measured with an idle queue, a call of the
+// score kernels with 29 KB took 43-79 us for three launches and takes 16 with 1.7 KB).  Most launches fit the small form (a call's operands, one map each); the large one is for
+// weight gradients split over the tokens and for schedules of many tiles.
+template <int MAPS, int OPS, int ORDER>
+struct GemmParams {
+    static constexpr int kMaps = MAPS, kOps = OPS, kOrder = ORDER;
+    alignas(64) CUtensorMap maps[MAPS];
+    DevProblem prob[OPS];
+    GemmHead head;
+    uint16_t order[ORDER];               // the explicit tile schedule
+};
+using LargeParams = GemmParams<72, kMaxGemmOps, 2048>;
+using SmallParams = GemmParams<20, 5, 512>;
 
 __device__ int g_gemm_status = 0;
 
@@ -497,13 +504,14 @@ __device__ __forceinline__ void staged_load32_finish(uint32_t buf, const uint4 (
 }
 
 // tile of worker `worker` in round `i`, or -1
-__device__ __forceinline__ int scheduled_tile(const GemmParams& P, int worker, int n_workers, int i) {
+template <typename Params>
+__device__ __forceinline__ int scheduled_tile(const Params& P, int worker, int n_workers, int i) {
     const int pos = worker + i * n_workers;
-    if (P.use_order) {
+    if (P.head.use_order) {
         const int t = P.order[pos];
         return t == kNoTile ? -1 : t;
     }
-    return pos < P.total_tiles ? pos : -1;
+    return pos < P.head.total_tiles ? pos : -1;
 }
 
 // v[i] += bias of column i, where lane i of the warp holds that column's bias
@@ -512,19 +520,20 @@ __device__ __forceinline__ void add_bias32(float (&v)[32], float b) {
     for (int i = 0; i < 32; ++i) v[i] += __shfl_sync(0xffffffffu, b, i);
 }
 
-__device__ __forceinline__ const DevProblem& find_problem(const GemmParams& P, int tile) {
+template <typename Params>
+__device__ __forceinline__ const DevProblem& find_problem(const Params& P, int tile) {
     int pi = 0;
 #pragma unroll
-    for (int i = 1; i < kMaxGemmOps; ++i)
-        if (i < P.n_problems && P.prob[i].tile_start <= tile) pi = i;
+    for (int i = 1; i < Params::kOps; ++i)
+        if (i < P.head.n_problems && P.prob[i].tile_start <= tile) pi = i;
     return P.prob[pi];
 }
 
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-template <bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant__ GemmParams P) {
+template <bool PAIR, typename Params>
+__global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant__ Params P) {
     constexpr int kSub = 2;                                  // 64-deep k-blocks per pipeline stage
     constexpr int kStages = PAIR ? 3 : 2;
     constexpr int kBLocal = PAIR ? kBHalf : kBStage;        // B bytes this CTA holds per k-block
@@ -565,7 +574,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const int tile0 = P.rounds > 0 ? scheduled_tile(P, worker, n_workers, 0) : -1;
+        const int tile0 = P.head.rounds > 0 ? scheduled_tile(P, worker, n_workers, 0) : -1;
         if (tile0 >= 0) {
             // warm the descriptors of the first tile while TMEM is allocated and the CTAs meet
             const DevProblem& Q0 = find_problem(P, tile0);
@@ -596,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int round = 0; ok && round < P.rounds; ++round) {
+            for (int round = 0; ok && round < P.head.rounds; ++round) {
                 const int tile = scheduled_tile(P, worker, n_workers, round);
                 if (tile < 0) continue;
                 const DevProblem& Q = find_problem(P, tile);
@@ -608,7 +617,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                 const int kb_lo = seg ? Q.kb_end[seg - 1] : 0, kb_hi = Q.kb_end[seg];
                 for (int kb0 = kb_lo; kb0 < kb_hi; kb0 += kSub) {
                     const int nsub = min(kSub, kb_hi - kb0);
-                    if (!(ok = mbar_wait<PAIR>(empty_bar(stage), phase ^ 1u, abort_flag, 1, P.status, P.wait_limit_ns))) break;
+                    if (!(ok = mbar_wait<PAIR>(empty_bar(stage), phase ^ 1u, abort_flag, 1, P.head.status, P.head.wait_limit_ns))) break;
                     // "big" operands arrive as one box holding both k-blocks (zero-filled past the end of K)
                     const bool a_big = PAIR && Q.a_big[seg], b_big = PAIR && Q.b_big[seg];
                     const uint32_t tx = (a_big ? kSub : nsub) * kAStage + (b_big ? kSub : nsub) * kBLocal;
@@ -721,20 +730,20 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             uint32_t phase = 0;
             int it = 0;
             bool ok = true;
-            for (int round = 0; ok && round < P.rounds; ++round) {
+            for (int round = 0; ok && round < P.head.rounds; ++round) {
                 const int tile = scheduled_tile(P, worker, n_workers, round);
                 if (tile < 0) continue;
                 const DevProblem& Q = find_problem(P, tile);
                 const int acc = it & 1;
                 const uint32_t acc_phase = (it >> 1) & 1u;
-                if (!(ok = mbar_wait<PAIR>(tempty_bar(acc), acc_phase ^ 1u, abort_flag, 2, P.status, P.wait_limit_ns))) break;
+                if (!(ok = mbar_wait<PAIR>(tempty_bar(acc), acc_phase ^ 1u, abort_flag, 2, P.head.status, P.head.wait_limit_ns))) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 for (int seg = 0; ok && seg < kMaxSeg; ++seg) {
                 const int kb_lo = seg ? Q.kb_end[seg - 1] : 0, kb_hi = Q.kb_end[seg];
                 for (int kb0 = kb_lo; kb0 < kb_hi; kb0 += kSub) {
                     const int nsub = min(kSub, kb_hi - kb0);
-                    if (!(ok = mbar_wait<PAIR>(full_bar(stage), phase, abort_flag, 3, P.status, P.wait_limit_ns))) break;
+                    if (!(ok = mbar_wait<PAIR>(full_bar(stage), phase, abort_flag, 3, P.head.status, P.head.wait_limit_ns))) break;
                     tc_fence_after();
 #pragma unroll
                     for (int sub = 0; sub < kSub; ++sub) {
@@ -782,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         const uint32_t buf_out = sEpi + ew * 2 * kEpiSlotBytes, buf_in = buf_out + kEpiSlotBytes;
         int it = 0;
         bool ok = true;
-        for (int round = 0; ok && round < P.rounds; ++round) {
+        for (int round = 0; ok && round < P.head.rounds; ++round) {
             const int tile = scheduled_tile(P, worker, n_workers, round);
             if (tile < 0) continue;
             const DevProblem& Q = find_problem(P, tile);
@@ -818,7 +827,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                                              : __uint_as_float(static_cast<uint32_t>(static_cast<const unsigned short*>(Q.bias)[col]) << 16);
                 }
             }
-            if (!(ok = mbar_wait<PAIR>(tfull_bar(acc), acc_phase, abort_flag, 4, P.status, P.wait_limit_ns))) break;
+            if (!(ok = mbar_wait<PAIR>(tfull_bar(acc), acc_phase, abort_flag, 4, P.head.status, P.head.wait_limit_ns))) break;
             tc_fence_after();
             const uint32_t t_row = tmem_base + acc * BN + (static_cast<uint32_t>(quad * 32) << 16);
             const bool warp_rows = m_warp < QM;          // any row of this warp inside the output
@@ -1127,6 +1136,9 @@ DeviceState g_dev[kMaxDevices];
 int g_pair_mode = 1;   // 1: CTA pairs (cta_group::2) whenever an op has more than one 128-row tile; 0: never
 std::atomic<unsigned long long> g_wait_limit_ns{kDefaultWaitLimitNs};
 
+template <typename Params>
+cudaError_t allow_smem(void (*kernel)(Params)) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); }
+
 // State of the current device (set up on first use), or nullptr with *st set.
 DeviceState* gemm_setup(ecospa_status_t* st_out) {
     int dev = 0;
@@ -1142,8 +1154,10 @@ DeviceState* gemm_setup(ecospa_status_t* st_out) {
     DeviceState& D = g_dev[dev];
     std::call_once(D.once, [&D, dev] {
         cudaError_t e = cudaDeviceGetAttribute(&D.num_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<false, SmallParams>);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<false, LargeParams>);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<true, SmallParams>);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<true, LargeParams>);
         if (const char* v = std::getenv("ECOSPA_GEMM_PAIR")) g_pair_mode = std::atoi(v);
         if (e == cudaSuccess) {
             // the tile schedule is static, so only as many pairs as can run at the same time are launched
@@ -1159,7 +1173,7 @@ DeviceState* gemm_setup(ecospa_status_t* st_out) {
             cfg.attrs = attr;
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<true>, &cfg) == cudaSuccess && n > 0) D.max_pairs = n;
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<true, LargeParams>, &cfg) == cudaSuccess && n > 0) D.max_pairs = n;
             else cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaGetSymbolAddress(reinterpret_cast<void**>(&D.status_ptr), g_gemm_status);
@@ -1177,36 +1191,128 @@ DeviceState* gemm_setup(ecospa_status_t* st_out) {
 // plain stride (worker w takes w, w + workers, ...) can leave one worker with several long tiles, so the
 // tiles are handed out longest first to the least-loaded worker (ties: lowest worker) and the result is
 // written as a table; with many tiles per worker the stride is balanced enough and needs no table.
-void build_schedule(GemmParams& gp, int workers) {
-    const int tiles = gp.total_tiles;
-    gp.use_order = 0;
-    gp.rounds = static_cast<int32_t>(ceil_div(tiles, workers));
-    if (tiles <= workers || tiles > kMaxOrder || tiles >= kNoTile) return;
-    static thread_local int64_t load[256];
+void build_schedule(LargeParams& gp, int workers) {
+    const int tiles = gp.head.total_tiles;
+    gp.head.use_order = 0;
+    gp.head.rounds = static_cast<int32_t>(ceil_div(tiles, workers));
+    if (tiles <= workers || tiles > LargeParams::kOrder || tiles >= kNoTile) return;
+    // workers as a binary heap by (load, worker): the top is the least loaded one, the lowest of those with equal loads
+    static thread_local uint64_t heap[256];
     static thread_local int32_t len[256];
     static thread_local uint16_t lists[256][64];
     if (workers > 256) return;
-    for (int w = 0; w < workers; ++w) load[w] = len[w] = 0;
+    for (int w = 0; w < workers; ++w) {
+        heap[w] = static_cast<uint64_t>(w);
+        len[w] = 0;
+    }
     int max_len = 0;
     int pi = 0;
     for (int t = 0; t < tiles; ++t) {
-        while (pi + 1 < gp.n_problems && gp.prob[pi + 1].tile_start <= t) ++pi;
+        while (pi + 1 < gp.head.n_problems && gp.prob[pi + 1].tile_start <= t) ++pi;
         // main loop, or the epilogue where that is the longer of the two (measured, in k-block times), + a fixed share
         static const int kEpiCost[7] = {5, 14, 14, 16, 20, 20, 26};
         const int64_t cost = std::max<int64_t>(gp.prob[pi].kblocks, kEpiCost[gp.prob[pi].epi]) + 4;
-        int best = 0;
-        for (int w = 1; w < workers; ++w)
-            if (load[w] < load[best]) best = w;
+        const int best = static_cast<int>(heap[0] & 0xff);
         if (len[best] >= 64) return;                       // not expected; keep the stride
         lists[best][len[best]++] = static_cast<uint16_t>(t);
-        load[best] += cost;
         max_len = std::max(max_len, static_cast<int>(len[best]));
+        const uint64_t key = heap[0] + (static_cast<uint64_t>(cost) << 8);
+        int i = 0;                                         // sift the new load down
+        for (int c = 1; c < workers; c = 2 * i + 1) {
+            if (c + 1 < workers && heap[c + 1] < heap[c]) ++c;
+            if (heap[c] >= key) break;
+            heap[i] = heap[c];
+            i = c;
+        }
+        heap[i] = key;
     }
-    if (static_cast<int64_t>(max_len) * workers > kMaxOrder) return;
+    if (static_cast<int64_t>(max_len) * workers > LargeParams::kOrder) return;
     for (int i = 0; i < max_len; ++i)
         for (int w = 0; w < workers; ++w) gp.order[w + i * workers] = i < len[w] ? lists[w][i] : kNoTile;
-    gp.rounds = max_len;
-    gp.use_order = 1;
+    gp.head.rounds = max_len;
+    gp.head.use_order = 1;
+}
+
+// The maps of a launch: operands that several products (or both halves of a tile) share get one map.
+struct MapTable {
+    struct Key {
+        const void* ptr;
+        int64_t rows, cols, ld;
+        int form;
+    };
+    static constexpr int kOutput = 16;                     // (no operand form has this value)
+    LargeParams& gp;
+    Key key[LargeParams::kMaps];
+    int n = 0;
+    explicit MapTable(LargeParams& g) : gp(g) {}
+    int find(const Stored& m, int form) const {
+        for (int i = 0; i < n; ++i)
+            if (key[i].ptr == m.ptr && key[i].rows == m.rows && key[i].cols == m.cols && key[i].ld == m.ld && key[i].form == form) return i;
+        return -1;
+    }
+    CUtensorMap* next() { return n < LargeParams::kMaps ? &gp.maps[n] : nullptr; }
+    int add(const Stored& m, int form) {
+        key[n] = Key{m.ptr, m.rows, m.cols, m.ld, form};
+        return n++;
+    }
+};
+enum OperandForm { FORM_PLAIN = 0, FORM_3D = 1, FORM_BIG = 2 };   // how a stage's box is fetched, see the encoders
+// Map of operand m (K-major or MN-major) in the widest form that it and the launch's mode allow; box_rows: of the plain
+// K-major form.
+ecospa_status_t operand_map(MapTable& T, const Stored& m, bool mn, bool pair, int box_rows, bool allow_3d, int* map, int* form) {
+    // what tells the maps of one tensor apart: form, orientation and, for the plain K-major form, the box
+    auto tag = [&](int f) { return 4 * f + (mn ? 2 : 0) + (f == FORM_PLAIN && !mn && box_rows != 128 ? 1 : 0); };
+    for (int f = pair ? FORM_BIG : FORM_3D; f >= FORM_PLAIN; --f) {
+        if (f == FORM_3D && !allow_3d) continue;
+        const int id = T.find(m, tag(f));
+        if (id >= 0) {
+            *map = id;
+            *form = f;
+            return ECOSPA_OK;
+        }
+    }
+    CUtensorMap* out = T.next();
+    if (!out) return ECOSPA_ERR_UNSUPPORTED;               // (not reached by the library's own calls)
+    if (pair && encode_map_big(out, m, mn)) *form = FORM_BIG;
+    else if (allow_3d && mn && encode_map_mn3d(out, m)) *form = FORM_3D;
+    else {
+        const ecospa_status_t st = encode_map(out, m, mn ? 64 : box_rows);
+        if (st != ECOSPA_OK) return st;
+        *form = FORM_PLAIN;
+    }
+    *map = T.add(m, tag(*form));
+    return ECOSPA_OK;
+}
+
+template <bool PAIR, typename Params>
+cudaError_t launch_form(const Params& gp, int workers, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(PAIR ? 2 * workers : workers);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = PAIR ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, gemm_kernel<PAIR, Params>, gp);
+}
+template <bool PAIR>
+cudaError_t launch_smallest_form(const LargeParams& gp, int n_maps, int workers, cudaStream_t stream) {
+    const int n_order = gp.head.use_order ? gp.head.rounds * workers : 0;
+    if (n_maps > SmallParams::kMaps || gp.head.n_problems > SmallParams::kOps || n_order > SmallParams::kOrder)
+        return launch_form<PAIR>(gp, workers, stream);
+    static thread_local SmallParams sp;
+    std::memcpy(sp.maps, gp.maps, n_maps * sizeof(CUtensorMap));
+    std::memcpy(sp.prob, gp.prob, gp.head.n_problems * sizeof(DevProblem));
+    sp.head = gp.head;
+    std::memcpy(sp.order, gp.order, n_order * sizeof(uint16_t));
+    return launch_form<PAIR>(sp, workers, stream);
 }
 
 }  // namespace
@@ -1263,7 +1369,8 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     }
     const int tile_m = pair ? 2 * BM : BM;
 
-    static thread_local GemmParams gp;
+    static thread_local LargeParams gp;
+    MapTable T(gp);
     int tiles = 0;
     for (int oi = 0; oi < n_ops; ++oi) {
         const GemmOp& op = ops[order[oi]];
@@ -1303,24 +1410,22 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
             // a range that stops before the end of the stored tensor must end on a k-block boundary
             if (k_end < (ks.a_mn ? a.rows : a.cols) && ks.K % BK) return ECOSPA_ERR_INVALID;
             if (ks.a_mn ? (a.rows < k_end || a.cols != op.M) : (a.rows != op.M || a.cols < k_end)) return ECOSPA_ERR_INVALID;
-            const int mi = oi * kMapsPerOp;
-            Q.a_big[s] = pair && encode_map_big(&gp.maps[mi + 3 * s], a, ks.a_mn);
-            Q.a_3d[s] = !Q.a_big[s] && ks.a_mn && encode_map_mn3d(&gp.maps[mi + 3 * s], a);
-            if (!Q.a_big[s] && !Q.a_3d[s] && (st = encode_map(&gp.maps[mi + 3 * s], a, ks.a_mn ? 64 : 128)) != ECOSPA_OK) return st;
-            Q.map_a[s] = static_cast<uint8_t>(mi + 3 * s);
+            int map = 0, form = 0;
+            if ((st = operand_map(T, a, ks.a_mn, pair, 128, true, &map, &form)) != ECOSPA_OK) return st;
+            Q.map_a[s] = static_cast<uint8_t>(map);
+            Q.a_big[s] = form == FORM_BIG;
+            Q.a_3d[s] = form == FORM_3D;
             for (int h = 0; h < 2; ++h) {
                 const Stored& b = (swiglu && h == 1) ? ks.b[1] : ks.b[0];
                 if (ks.b_mn ? (b.rows < k_end || b.cols != op.N) : (b.rows != op.N || b.cols < k_end)) return ECOSPA_ERR_INVALID;
-                const bool bb = pair && encode_map_big(&gp.maps[mi + 3 * s + 1 + h], b, ks.b_mn);
-                const bool b3 = !bb && ks.b_mn && encode_map_mn3d(&gp.maps[mi + 3 * s + 1 + h], b);
+                if ((st = operand_map(T, b, ks.b_mn, pair, 128, true, &map, &form)) != ECOSPA_OK) return st;
+                Q.map_b[s][h] = static_cast<uint8_t>(map);
                 if (h == 0) {
-                    Q.b_big[s] = bb;
-                    Q.b_3d[s] = b3;
-                } else if (bb != (Q.b_big[s] != 0) || b3 != (Q.b_3d[s] != 0)) {
+                    Q.b_big[s] = form == FORM_BIG;
+                    Q.b_3d[s] = form == FORM_3D;
+                } else if ((form == FORM_BIG) != (Q.b_big[s] != 0) || (form == FORM_3D) != (Q.b_3d[s] != 0)) {
                     return ECOSPA_ERR_UNSUPPORTED;   // both halves take the same path
                 }
-                if (!bb && !b3 && (st = encode_map(&gp.maps[mi + 3 * s + 1 + h], b, ks.b_mn ? 64 : 128)) != ECOSPA_OK) return st;
-                Q.map_b[s][h] = static_cast<uint8_t>(mi + 3 * s + 1 + h);
             }
             Q.a_mn[s] = ks.a_mn;
             Q.b_mn[s] = ks.b_mn;
@@ -1333,9 +1438,11 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
             const bool wide = op.epi == EPI_STORE || op.epi == EPI_GELU_ERF || op.epi == EPI_GELU_TANH;
             void* outs[3] = {op.C, op.C2, op.C3};
             for (int o = 0; o < 3; ++o) {
-                Q.map_c[o] = static_cast<uint8_t>(oi * kMapsPerOp + kOperandMaps + o);
                 if (!outs[o]) continue;
-                if ((st = encode_out_map(&gp.maps[Q.map_c[o]], outs[o], op.M, op.N, op.ldc, op.out_f32, wide)) != ECOSPA_OK) return st;
+                CUtensorMap* out = T.next();
+                if (!out) return ECOSPA_ERR_UNSUPPORTED;
+                if ((st = encode_out_map(out, outs[o], op.M, op.N, op.ldc, op.out_f32, wide)) != ECOSPA_OK) return st;
+                Q.map_c[o] = static_cast<uint8_t>(T.add(Stored(), MapTable::kOutput));   // (never shared)
             }
         }
         for (int s2 = op.n_kseg; s2 < kMaxSeg; ++s2) Q.kb_end[s2] = Q.kblocks;
@@ -1344,27 +1451,13 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
         Q.tile_start = tiles;
         tiles += Q.tiles_m * Q.tiles_n;
     }
-    gp.n_problems = n_ops;
-    gp.total_tiles = tiles;
-    gp.status = dev->status_ptr;
-    gp.wait_limit_ns = g_wait_limit_ns.load(std::memory_order_relaxed);
+    gp.head.n_problems = n_ops;
+    gp.head.total_tiles = tiles;
+    gp.head.status = dev->status_ptr;
+    gp.head.wait_limit_ns = g_wait_limit_ns.load(std::memory_order_relaxed);
     const int workers = pair ? std::min(tiles, g_max_pairs) : std::min(tiles, g_num_sms);
     build_schedule(gp, workers);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pair ? 2 * workers : workers);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pair ? 2 : 1;
-    const cudaError_t e = pair ? cudaLaunchKernelEx(&cfg, gemm_kernel<true>, gp) : cudaLaunchKernelEx(&cfg, gemm_kernel<false>, gp);
+    const cudaError_t e = pair ? launch_smallest_form<true>(gp, T.n, workers, stream) : launch_smallest_form<false>(gp, T.n, workers, stream);
     if (e != cudaSuccess) {
         set_cuda_error(e, "gemm_kernel launch");
         cudaGetLastError();

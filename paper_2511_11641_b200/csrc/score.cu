@@ -21,8 +21,10 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxJobs = 400;      // per launch; 72 B each -> 28.8 KB of kernel parameters (limit 32764)
-constexpr int kMaxPairs = 256;     // per finalize launch; 80 B each
+// Jobs / pairs per launch, as kernel parameters (limit 32764 bytes).  What a launch costs the host grows with the size of its
+// parameters, so there is a small form of each kernel for a block or two of a model besides the form for a whole model.
+constexpr int kMaxJobs = 400, kFewJobs = 24;      // 72 B each
+constexpr int kMaxPairs = 256, kFewPairs = 16;    // 80 B each
 constexpr int kRowTile = 32;       // shared-rows tile: rows per CTA
 constexpr int kUnroll = 4;
 
@@ -42,10 +44,11 @@ struct SumsqJob {
 };
 static_assert(sizeof(SumsqJob) == 72, "job descriptor size");
 
+template <int CAP>
 struct SumsqParams {
     int32_t n_jobs;
     int32_t pad_;
-    SumsqJob jobs[kMaxJobs];
+    SumsqJob jobs[CAP];
 };
 
 struct PairDesc {
@@ -65,14 +68,18 @@ struct PairDesc {
 };
 static_assert(sizeof(PairDesc) == 80, "pair descriptor size");
 
-struct FinalizeParams {
+struct FinalizeOut {
     int32_t n_pairs;
     int32_t pad_;
     float* upsilon;
     float* raw;
     float* fisher;
     double inv_n_samples;
-    PairDesc pairs[kMaxPairs];
+};
+template <int CAP>
+struct FinalizeParams {
+    FinalizeOut out;
+    PairDesc pairs[CAP];
 };
 
 // Largest i with start(i) <= x.
@@ -226,7 +233,8 @@ __device__ __forceinline__ void rows_tile(const SumsqJob& J, int local) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__ SumsqParams P) {
+template <int CAP>
+__global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__ SumsqParams<CAP> P) {
     __shared__ float smem[kWarps * (256 + 4)];
     pdl_start();
     const int tile = blockIdx.x;
@@ -241,7 +249,8 @@ __global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__
 }
 
 // stat[c] = sum over chunks of partial[chunk][c], chunk order fixed.
-__global__ void __launch_bounds__(kThreads) reduce_kernel(const __grid_constant__ SumsqParams P) {
+template <int CAP>
+__global__ void __launch_bounds__(kThreads) reduce_kernel(const __grid_constant__ SumsqParams<CAP> P) {
     pdl_start();
     const int blk = blockIdx.x;
     const int ji = find_owner(P.n_jobs, blk, [&](int i) { return P.jobs[i].red_start; });
@@ -309,7 +318,7 @@ __device__ __forceinline__ float importance(const PairDesc& Q, float a, float ab
 
 // A warp, a segment of at most 32 * TREES indices.
 template <int MODE, int TREES>
-__device__ __forceinline__ void finalize_narrow(const FinalizeParams& P, const PairDesc& Q, int seg) {
+__device__ __forceinline__ void finalize_narrow(const FinalizeOut& P, const PairDesc& Q, int seg) {
     const int lane = threadIdx.x & 31, n = Q.seg_len;
     const bool with_fisher = P.fisher != nullptr, with_up = Q.gs1b != nullptr;
     float r[TREES], y[TREES], g1[TREES], g1b[TREES], g2[TREES];
@@ -360,7 +369,7 @@ __device__ __forceinline__ float end_wide_sum(float acc, int first, float* scrat
     return t;
 }
 template <int MODE>
-__device__ __forceinline__ void scores_wide(const FinalizeParams& P, const PairDesc& Q, int seg, float* buf, float* scratch) {
+__device__ __forceinline__ void scores_wide(const FinalizeOut& P, const PairDesc& Q, int seg, float* buf, float* scratch) {
     const int n = Q.seg_len, tid = threadIdx.x;
     const int64_t out = Q.d_off + static_cast<int64_t>(seg) * n;
     // buf[j - base] = raw score of index j of a pass
@@ -424,7 +433,7 @@ __device__ __forceinline__ float virtual_sum(const float* v, int rep, int seg, i
     return s;
 }
 template <int MODE>
-__device__ __forceinline__ void importance_wide(const FinalizeParams& P, const PairDesc& Q, int seg, float* scratch) {
+__device__ __forceinline__ void importance_wide(const FinalizeOut& P, const PairDesc& Q, int seg, float* scratch) {
     // threads 0-255: W_1's sum, then the up projection's; threads 256-511: W_2's
     const int n = Q.seg_len, tid = threadIdx.x;
     const bool first = tid < 256;
@@ -438,7 +447,7 @@ __device__ __forceinline__ void importance_wide(const FinalizeParams& P, const P
 
 // A block's share of a pair: kFinWarps narrow segments, or the scores or the importance of one wide segment.
 template <int MODE>
-__device__ __forceinline__ void finalize_pair(const FinalizeParams& P, const PairDesc& Q, int local, float* buf, float* scratch) {
+__device__ __forceinline__ void finalize_pair(const FinalizeOut& P, const PairDesc& Q, int local, float* buf, float* scratch) {
     const int n = Q.seg_len;
     if (n <= kNarrow) {
         const int seg = local * kFinWarps + (threadIdx.x >> 5);
@@ -452,18 +461,19 @@ __device__ __forceinline__ void finalize_pair(const FinalizeParams& P, const Pai
     else scores_wide<MODE>(P, Q, P.fisher ? local >> 1 : local, buf, scratch);
 }
 
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const __grid_constant__ FinalizeParams P) {
+template <int CAP>
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const __grid_constant__ FinalizeParams<CAP> P) {
     __shared__ float buf[kFinPass];
     __shared__ float scratch[kFinWarps];
     pdl_start();
     const int blk = blockIdx.x;
-    const int pi = find_owner(P.n_pairs, blk, [&](int i) { return P.pairs[i].blk_start; });
+    const int pi = find_owner(P.out.n_pairs, blk, [&](int i) { return P.pairs[i].blk_start; });
     const PairDesc& Q = P.pairs[pi];
     const int local = blk - Q.blk_start;
     pdl_wait();
-    if (Q.rep1 > 1 || Q.rep2 > 1) finalize_pair<kGrouped>(P, Q, local, buf, scratch);
-    else if (Q.rope != ECOSPA_ROPE_NONE) finalize_pair<kRotation>(P, Q, local, buf, scratch);
-    else finalize_pair<kSingle>(P, Q, local, buf, scratch);
+    if (Q.rep1 > 1 || Q.rep2 > 1) finalize_pair<kGrouped>(P.out, Q, local, buf, scratch);
+    else if (Q.rope != ECOSPA_ROPE_NONE) finalize_pair<kRotation>(P.out, Q, local, buf, scratch);
+    else finalize_pair<kSingle>(P.out, Q, local, buf, scratch);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -557,6 +567,14 @@ size_t plan_stats(const ecospa_pair_t* pairs, int n_pairs, bool grads, std::vect
     return off;
 }
 
+template <int CAP>
+ecospa_status_t launch_sums(const SumsqParams<CAP>& sp, int tiles, int reduce_blocks, cudaStream_t stream) {
+    sumsq_kernel<CAP><<<tiles, kThreads, 0, stream>>>(sp);
+    const ecospa_status_t st = check_launch("sumsq_kernel");
+    if (st != ECOSPA_OK || reduce_blocks == 0) return st;
+    return launch_pdl(reduce_kernel<CAP>, reduce_blocks, kThreads, stream, sp, "reduce_kernel");
+}
+
 bool mat_aligned(const ecospa_mat_t& m) {
     return aligned16(m.ptr) && (m.ld * elem_bytes(m.dtype)) % 16 == 0;
 }
@@ -594,7 +612,7 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
     float* ws = static_cast<float*>(workspace);
 
     // --- sumsq + reduce, in launches of at most kMaxJobs jobs
-    static thread_local SumsqParams sp;
+    static thread_local SumsqParams<kMaxJobs> sp;
     size_t si = 0;
     while (si < stats.size()) {
         int nj = 0, tiles = 0, red = 0;
@@ -628,16 +646,20 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             if (J.n_chunks > 1) red += static_cast<int>(ceil_div(J.D, kThreads));
         }
         sp.n_jobs = nj;
-        sumsq_kernel<<<tiles, kThreads, 0, stream>>>(sp);
-        ecospa_status_t st = check_launch("sumsq_kernel");
-        if (st != ECOSPA_OK) return st;
-        if (red > 0) {
-            if ((st = launch_pdl(reduce_kernel, red, kThreads, stream, sp, "reduce_kernel")) != ECOSPA_OK) return st;
+        ecospa_status_t st;
+        if (nj <= kFewJobs) {
+            SumsqParams<kFewJobs> few;
+            few.n_jobs = nj;
+            std::copy(sp.jobs, sp.jobs + nj, few.jobs);
+            st = launch_sums(few, tiles, red, stream);
+        } else {
+            st = launch_sums(sp, tiles, red, stream);
         }
+        if (st != ECOSPA_OK) return st;
     }
 
     // --- finalize, in launches of at most kMaxPairs pairs
-    static thread_local FinalizeParams fp;
+    static thread_local FinalizeParams<kMaxPairs> fp;
     size_t stat_i = 0;
     int32_t d_off = 0, seg_off = 0;
     int p = 0;
@@ -671,12 +693,20 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             segs += pr.n_seg;
             seg_off += pr.n_seg;
         }
-        fp.n_pairs = np;
-        fp.upsilon = upsilon;
-        fp.raw = raw;
-        fp.fisher = fisher ? fisher + seg_base : nullptr;
-        fp.inv_n_samples = 1.0 / n_samples;
-        const ecospa_status_t st = launch_pdl(finalize_kernel, blocks, kFinThreads, stream, fp, "finalize_kernel");
+        fp.out.n_pairs = np;
+        fp.out.upsilon = upsilon;
+        fp.out.raw = raw;
+        fp.out.fisher = fisher ? fisher + seg_base : nullptr;
+        fp.out.inv_n_samples = 1.0 / n_samples;
+        ecospa_status_t st;
+        if (np <= kFewPairs) {
+            FinalizeParams<kFewPairs> few;
+            few.out = fp.out;
+            std::copy(fp.pairs, fp.pairs + np, few.pairs);
+            st = launch_pdl(finalize_kernel<kFewPairs>, blocks, kFinThreads, stream, few, "finalize_kernel");
+        } else {
+            st = launch_pdl(finalize_kernel<kMaxPairs>, blocks, kFinThreads, stream, fp, "finalize_kernel");
+        }
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;

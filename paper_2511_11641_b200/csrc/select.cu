@@ -4,7 +4,7 @@
 // that a warp holds in registers, by counting into parts of a shrinking range of keys for a wider one); the kept indices are then emitted in ascending
 // order, taking equal-to-threshold scores lowest index first.  
 
-#include <vector>
+#include <algorithm>
 
 #include "common.cuh"
 
@@ -14,8 +14,10 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxSegs = 4096;   // per launch (16 KB of offsets)
-constexpr int kMaxPairs = 256;   // per launch
+// Segments and pairs per launch, as kernel parameters; the small forms are for a block or two of a model (a launch costs the
+// host more, the larger its parameters).
+constexpr int kMaxSegs = 4096, kFewSegs = 256;   // 4 B of offsets each
+constexpr int kMaxPairs = 256, kFewPairs = 16;
 
 struct SelPair {
     int32_t seg_start;  // first segment (within this launch) of the pair
@@ -27,7 +29,7 @@ struct SelPair {
     int32_t seg_first, n_seg;   // and the pair's segments of the launch
 };
 
-struct SelectParams {
+struct SelectHead {
     const float* upsilon;
     int32_t* kept;
     int32_t* seg_offsets;   // may be null; global prefix sums of k
@@ -36,8 +38,12 @@ struct SelectParams {
     int32_t is_last;        // this launch writes the final seg_offsets entry
     const int32_t* k_dev;   // non-null: kept counts are read from the device (indexed by global segment) and
                             // segment s of a pair writes at the pair's score offset + s * seg_len
-    SelPair pairs[kMaxPairs];
-    int32_t out_off[kMaxSegs + 1];  // global offsets into kept
+};
+template <int PAIRS, int SEGS>
+struct SelectParams {
+    SelectHead head;
+    SelPair pairs[PAIRS];
+    int32_t out_off[SEGS + 1];  // global offsets into kept
 };
 
 // fp32 -> uint32 whose unsigned order is the float order; -0 and +0 map to the same key.
@@ -75,7 +81,7 @@ struct SegView {
     }
 };
 // Opens segment `seg` of the launch (one thread, `writer`, notes its offset).
-__device__ __forceinline__ SegView open_segment(const SelectParams& P, const SelPair& Q, int seg, bool writer) {
+__device__ __forceinline__ SegView open_segment(const SelectHead& P, const int32_t* out_off, const SelPair& Q, int seg, bool writer) {
     SegView V;
     const int seg_len = Q.seg_len, seg_in_pair = seg - Q.seg_start;
     // With rotation pairs the ranked units are the seg_len/2 pairs; both members carry the pair's score, so
@@ -85,8 +91,8 @@ __device__ __forceinline__ SegView open_segment(const SelectParams& P, const Sel
     V.stride = Q.rope == ECOSPA_ROPE_INTERLEAVED ? 2 : 1;
     V.first = seg_in_pair * seg_len;                            // kept indices are shared indices of the pair group
     V.sc = P.upsilon + Q.d_off + static_cast<int64_t>(seg_in_pair) * seg_len;
-    V.out0 = P.k_dev ? Q.d_off + seg_in_pair * seg_len : P.out_off[seg];
-    const int k_idx = P.k_dev ? min(max(P.k_dev[P.seg_base + seg], 0), seg_len) : P.out_off[seg + 1] - V.out0;
+    V.out0 = P.k_dev ? Q.d_off + seg_in_pair * seg_len : out_off[seg];
+    const int k_idx = P.k_dev ? min(max(P.k_dev[P.seg_base + seg], 0), seg_len) : out_off[seg + 1] - V.out0;
     V.k = Q.rope ? k_idx >> 1 : k_idx;
     V.kept = P.kept;
     if (P.seg_offsets && writer) {
@@ -272,11 +278,12 @@ __device__ __forceinline__ void select_wide(const SegView& V, WideShared& S) {
     }
 }
 
-__global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_constant__ SelectParams P) {
+template <int PAIRS, int SEGS>
+__global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_constant__ SelectParams<PAIRS, SEGS> P) {
     __shared__ WideShared S;
     pdl_start();
     const int blk = blockIdx.x;
-    int lo = 0, hi = P.n_pairs - 1;
+    int lo = 0, hi = P.head.n_pairs - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (P.pairs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
@@ -286,15 +293,26 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     if (Q.seg_len <= kNarrow) {
         const int i = (blk - Q.blk_start) * kSelWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
         if (i >= Q.n_seg) return;
-        const SegView V = open_segment(P, Q, Q.seg_first + i, lane == 0);
+        const SegView V = open_segment(P.head, P.out_off, Q, Q.seg_first + i, lane == 0);
         if (V.k <= 0) return;
         if (V.n <= 64) select_narrow<2>(V, lane);
         else if (V.n <= 128) select_narrow<4>(V, lane);
         else select_narrow<kNarrow / 32>(V, lane);
         return;
     }
-    const SegView V = open_segment(P, Q, Q.seg_first + (blk - Q.blk_start), threadIdx.x == 0);
+    const SegView V = open_segment(P.head, P.out_off, Q, Q.seg_first + (blk - Q.blk_start), threadIdx.x == 0);
     if (V.k > 0) select_wide(V, S);
+}
+using SelectAll = SelectParams<kMaxPairs, kMaxSegs>;
+using SelectFew = SelectParams<kFewPairs, kFewSegs>;
+ecospa_status_t launch_select(const SelectAll& sp, int blocks, cudaStream_t stream) {
+    const int np = sp.head.n_pairs, ns = sp.head.n_segs;
+    if (np > kFewPairs || ns > kFewSegs) return launch_pdl(select_kernel<kMaxPairs, kMaxSegs>, blocks, kSelThreads, stream, sp, "select_kernel");
+    SelectFew few;
+    few.head = sp.head;
+    std::copy(sp.pairs, sp.pairs + np, few.pairs);
+    if (!sp.head.k_dev) std::copy(sp.out_off, sp.out_off + ns + 1, few.out_off);
+    return launch_pdl(select_kernel<kFewPairs, kFewSegs>, blocks, kSelThreads, stream, few, "select_kernel");
 }
 // Adds the pair's segments of a launch (those from `seg_first` on) to the launch's blocks.
 inline int select_blocks(SelPair& Q, int seg_first, int n_seg, int blk_start) {
@@ -458,29 +476,50 @@ __global__ void __launch_bounds__(1024) choose_pairs_kernel(const float* __restr
     }
 }
 
-// Packs the per-segment slots of the variable-count selection into one ascending list per pair group:
-// out[dst[s] + i] = slots[src[s] + i] + add[s] for i < k[s].
-constexpr int kPackSegs = 512;
+// One list out of per-segment lists, a block per segment.  PAD = false: packs the per-segment slots of the variable-count
+// selection into one ascending list per pair group, out[dst[s] + i] = slots[src[s] + i] + add[s] for i < k[s].
+// PAD = true: kept list with padded segments, the k[s] entries of segment s, then -1 ("no index") up to add[s] entries.
+template <int CAP>
 struct PackParams {
     const int32_t* slots;
     int32_t* out;
-    int32_t n;
-    int32_t src[kPackSegs], dst[kPackSegs], k[kPackSegs], add[kPackSegs];
+    int32_t src[CAP], dst[CAP], k[CAP], add[CAP];
 };
-__global__ void __launch_bounds__(128) pack_kept_kernel(const __grid_constant__ PackParams P) {
+template <bool PAD, int CAP>
+__global__ void __launch_bounds__(128) pack_kept_kernel(const __grid_constant__ PackParams<CAP> P) {
     pdl_start();
     pdl_wait();
-    const int s = blockIdx.x;
-    for (int i = threadIdx.x; i < P.k[s]; i += blockDim.x) P.out[P.dst[s] + i] = P.slots[P.src[s] + i] + P.add[s];
+    const int s = blockIdx.x, k = P.k[s], n = PAD ? P.add[s] : k;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        if (PAD) P.out[P.dst[s] + i] = i < k ? P.slots[P.src[s] + i] : -1;
+        else P.out[P.dst[s] + i] = P.slots[P.src[s] + i] + P.add[s];
+    }
 }
 
-// Kept list with padded segments: the k[s] entries of segment s, then -1 ("no index") up to its padded count
-// (carried in the `add` slot of the parameters).
-__global__ void __launch_bounds__(128) pad_kept_kernel(const __grid_constant__ PackParams P) {
-    pdl_start();
-    pdl_wait();
-    const int s = blockIdx.x;
-    for (int i = threadIdx.x; i < P.add[s]; i += blockDim.x) P.out[P.dst[s] + i] = i < P.k[s] ? P.slots[P.src[s] + i] : -1;
+template <bool PAD, int CAP>
+ecospa_status_t launch_pack(const int32_t* slots, const int32_t* src, const int32_t* dst, const int32_t* k, const int32_t* add, int n,
+                            int32_t* out, cudaStream_t stream) {
+    static thread_local PackParams<CAP> pp;
+    pp.slots = slots; pp.out = out;
+    std::copy(src, src + n, pp.src);
+    std::copy(dst, dst + n, pp.dst);
+    std::copy(k, k + n, pp.k);
+    std::copy(add, add + n, pp.add);
+    return launch_pdl(pack_kept_kernel<PAD, CAP>, n, 128, stream, pp, PAD ? "pad_kept_kernel" : "pack_kept_kernel");
+}
+// As few launches as the parameters allow, each in the smallest form that holds its segments.
+template <bool PAD>
+ecospa_status_t launch_packs(const int32_t* slots, const int32_t* src, const int32_t* dst, const int32_t* k, const int32_t* add, int n_segs,
+                             int32_t* out, cudaStream_t stream) {
+    constexpr int kMost = 2000, kSome = 512, kFew = 64;      // 16 B each
+    ecospa_status_t st = ECOSPA_OK;
+    for (int b = 0; b < n_segs && st == ECOSPA_OK; b += kMost) {
+        const int n = std::min(kMost, n_segs - b);
+        if (n <= kFew) st = launch_pack<PAD, kFew>(slots, src + b, dst + b, k + b, add + b, n, out, stream);
+        else if (n <= kSome) st = launch_pack<PAD, kSome>(slots, src + b, dst + b, k + b, add + b, n, out, stream);
+        else st = launch_pack<PAD, kMost>(slots, src + b, dst + b, k + b, add + b, n, out, stream);
+    }
+    return st;
 }
 
 }  // namespace
@@ -494,17 +533,7 @@ extern "C" ecospa_status_t ecospa_pad_kept(const int32_t* kept, const int32_t* s
     if (!kept || !src || !dst || !k || !k_padded || !out || n_segs < 1) return ECOSPA_ERR_INVALID;
     for (int i = 0; i < n_segs; ++i)
         if (src[i] < 0 || dst[i] < 0 || k[i] < 0 || k_padded[i] < k[i]) return ECOSPA_ERR_INVALID;
-    static thread_local PackParams pp;
-    for (int base = 0; base < n_segs; base += kPackSegs) {
-        const int n = std::min(kPackSegs, n_segs - base);
-        pp.slots = kept; pp.out = out; pp.n = n;
-        for (int i = 0; i < n; ++i) {
-            pp.src[i] = src[base + i]; pp.dst[i] = dst[base + i]; pp.k[i] = k[base + i]; pp.add[i] = k_padded[base + i];
-        }
-        const ecospa_status_t st = launch_pdl(pad_kept_kernel, n, 128, static_cast<cudaStream_t>(stream), pp, "pad_kept_kernel");
-        if (st != ECOSPA_OK) return st;
-    }
-    return ECOSPA_OK;
+    return launch_packs<true>(kept, src, dst, k, k_padded, n_segs, out, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" ecospa_status_t ecospa_pack_kept(const int32_t* slots, const int32_t* src, const int32_t* dst, const int32_t* k,
@@ -512,17 +541,7 @@ extern "C" ecospa_status_t ecospa_pack_kept(const int32_t* slots, const int32_t*
     if (!slots || !src || !dst || !k || !add || !out || n_segs < 1) return ECOSPA_ERR_INVALID;
     for (int i = 0; i < n_segs; ++i)
         if (src[i] < 0 || dst[i] < 0 || k[i] < 0) return ECOSPA_ERR_INVALID;
-    static thread_local PackParams pp;
-    for (int base = 0; base < n_segs; base += kPackSegs) {
-        const int n = std::min(kPackSegs, n_segs - base);
-        pp.slots = slots; pp.out = out; pp.n = n;
-        for (int i = 0; i < n; ++i) {
-            pp.src[i] = src[base + i]; pp.dst[i] = dst[base + i]; pp.k[i] = k[base + i]; pp.add[i] = add[base + i];
-        }
-        const ecospa_status_t st = launch_pdl(pack_kept_kernel, n, 128, static_cast<cudaStream_t>(stream), pp, "pack_kept_kernel");
-        if (st != ECOSPA_OK) return st;
-    }
-    return ECOSPA_OK;
+    return launch_packs<false>(slots, src, dst, k, add, n_segs, out, static_cast<cudaStream_t>(stream));
 }
 
 static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* n_seg, const int32_t* seg_len,
@@ -548,12 +567,12 @@ static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* 
     }
     if (total_d > INT32_MAX || total_k > INT32_MAX) return ECOSPA_ERR_UNSUPPORTED;
 
-    static thread_local SelectParams sp;
+    static thread_local SelectAll sp;
     int p = 0, s_in_p = 0;          // walk position: pair, segment inside pair
     int32_t d_off = 0, out = 0, seg_global = 0;
     while (p < n_pairs) {
         int np = 0, ns = 0, blocks = 0;
-        sp.seg_base = seg_global;
+        sp.head.seg_base = seg_global;
         // a pair can be split across launches; each launch sees it as a pair starting at s_in_p
         while (p < n_pairs && np < kMaxPairs && ns < kMaxSegs) {
             const int take = std::min(n_seg[p] - s_in_p, kMaxSegs - ns);
@@ -575,14 +594,14 @@ static ecospa_status_t select_fixed_counts(const float* upsilon, const int32_t* 
             }
         }
         sp.out_off[ns] = out;
-        sp.upsilon = upsilon;
-        sp.kept = kept;
-        sp.k_dev = nullptr;
-        sp.seg_offsets = seg_offsets;
-        sp.n_pairs = np;
-        sp.n_segs = ns;
-        sp.is_last = (p >= n_pairs) ? 1 : 0;
-        const ecospa_status_t st = launch_pdl(select_kernel, blocks, kSelThreads, stream, sp, "select_kernel");
+        sp.head.upsilon = upsilon;
+        sp.head.kept = kept;
+        sp.head.k_dev = nullptr;
+        sp.head.seg_offsets = seg_offsets;
+        sp.head.n_pairs = np;
+        sp.head.n_segs = ns;
+        sp.head.is_last = (p >= n_pairs) ? 1 : 0;
+        const ecospa_status_t st = launch_select(sp, blocks, stream);
         if (st != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
@@ -622,7 +641,7 @@ extern "C" ecospa_status_t ecospa_select_aligned_threshold(const float* upsilon,
     if (total_d > INT32_MAX) return ECOSPA_ERR_UNSUPPORTED;
 
     static thread_local ThresholdParams tp;
-    static thread_local SelectParams sp;
+    static thread_local SelectAll sp;
     int p = 0, s_in_p = 0;
     int32_t d_off = 0, seg_global = 0;
     while (p < n_pairs) {
@@ -653,10 +672,10 @@ extern "C" ecospa_status_t ecospa_select_aligned_threshold(const float* upsilon,
         ecospa_status_t st = launch_pdl(threshold_count_kernel, ns, kThreads, stream, tp, "threshold_count_kernel");
         if (st != ECOSPA_OK) return st;
         // the fixed-count selection, with the counts just written and one slot of seg_len entries per segment
-        sp.upsilon = upsilon; sp.kept = kept; sp.seg_offsets = nullptr;
-        sp.n_pairs = np; sp.n_segs = ns; sp.seg_base = seg_base; sp.is_last = 0;
-        sp.k_dev = k_out;
-        if ((st = launch_pdl(select_kernel, blocks, kSelThreads, stream, sp, "select_kernel")) != ECOSPA_OK) return st;
+        sp.head.upsilon = upsilon; sp.head.kept = kept; sp.head.seg_offsets = nullptr;
+        sp.head.n_pairs = np; sp.head.n_segs = ns; sp.head.seg_base = seg_base; sp.head.is_last = 0;
+        sp.head.k_dev = k_out;
+        if ((st = launch_select(sp, blocks, stream)) != ECOSPA_OK) return st;
     }
     return ECOSPA_OK;
 }
