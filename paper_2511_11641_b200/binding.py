@@ -8,6 +8,7 @@ or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import List, Optional, Sequence, Tuple
@@ -87,8 +88,32 @@ def _dtype_code(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+# Marshalling.  A call on a small block is all host time, so the per-element and per-call work of building argument lists
+# stays out of the interpreter: integer lists go through array.array, descriptor lists through one bytes.join (measured on
+# lists of a 24-layer model: 768 segments 0.67 -> 0.05 ms, 480 gather jobs 0.18 -> 0.026 ms).
+
+def _i32(v) -> array.array:
+    try:
+        return array.array("i", v)
+    except TypeError:                      # (values that are not integers by type)
+        return array.array("i", [int(x) for x in v])
+
+
+def _addr(a: array.array) -> int:
+    return a.buffer_info()[0]
+
+
+def _structs(kind, items):
+    """The descriptors side by side in memory (anything that passes as their address)."""
+    if set(map(type, items)) == {kind}:
+        return b"".join(items)
+    return (kind * len(items))(*items)
+
+
 def _stream(stream) -> C.c_void_p:
     if stream is None:
+        if torch.cuda.is_initialized():
+            return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
         stream = torch.cuda.current_stream()
     return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
@@ -118,41 +143,33 @@ def pair(kind: int, n_seg: int, seg_len: int, w1, w2, layout1: int, layout2: int
     return p
 
 
-def _pair_array(pairs: Sequence[Pair]):
-    arr = (Pair * len(pairs))(*pairs)
-    return arr
-
-
 def ecospa_score_workspace_bytes(pairs: Sequence[Pair]) -> int:
-    arr = _pair_array(pairs)
-    return int(lib().ecospa_score_workspace_bytes(C.addressof(arr), len(pairs)))
+    arr = _structs(Pair, pairs)
+    return int(lib().ecospa_score_workspace_bytes(arr, len(pairs)))
 
 
 def ecospa_score_pairs(pairs: Sequence[Pair], n_samples: float, upsilon: torch.Tensor,
                        raw: Optional[torch.Tensor] = None, fisher: Optional[torch.Tensor] = None,
                        workspace: Optional[torch.Tensor] = None, stream=None) -> None:
     """upsilon/raw: fp32 [sum D]; fisher: fp32 [sum n_seg] or None; workspace: uint8 device buffer."""
-    arr = _pair_array(pairs)
+    arr = _structs(Pair, pairs)
     if workspace is None:
         workspace = torch.empty(ecospa_score_workspace_bytes(pairs), dtype=torch.uint8, device=upsilon.device)
-    st = lib().ecospa_score_pairs(C.addressof(arr), len(pairs), float(n_samples), _ptr(upsilon), _ptr(raw),
+    st = lib().ecospa_score_pairs(arr, len(pairs), float(n_samples), _ptr(upsilon), _ptr(raw),
                                   _ptr(fisher), _ptr(workspace), workspace.numel(), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_score_pairs")
 
 
 def ecospa_score_pair_static_max_bytes() -> int:
-    f = lib().ecospa_score_pair_static_max_bytes
-    f.restype = C.c_size_t
+    f = _fn("ecospa_score_pair_static_max_bytes")
     return int(f())
 
 
 def ecospa_score_pair_static(p: Pair, n_samples: float, upsilon: torch.Tensor, raw: Optional[torch.Tensor] = None,
                              fisher: Optional[torch.Tensor] = None, stream=None) -> None:
     """Scores of one pair group using the library's built-in scratch array; allocates nothing."""
-    f = lib().ecospa_score_pair_static
-    f.restype = C.c_int
-    f.argtypes = [C.c_void_p, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+    f = _fn("ecospa_score_pair_static")
     st = f(C.addressof(p), float(n_samples), _ptr(upsilon), _ptr(raw), _ptr(fisher), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_score_pair_static")
@@ -162,12 +179,12 @@ def ecospa_select_aligned_topk(upsilon: torch.Tensor, n_seg: Sequence[int], seg_
                                k_per_seg: Sequence[int], kept: torch.Tensor,
                                seg_offsets: Optional[torch.Tensor] = None, stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg = (C.c_int32 * n_pairs)(*n_seg)
-    a_slen = (C.c_int32 * n_pairs)(*seg_len)
-    a_k = (C.c_int32 * len(k_per_seg))(*k_per_seg)
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
+    assert len(a_slen) == n_pairs
+    a_k = _i32(k_per_seg)
     assert len(k_per_seg) == sum(n_seg)
     assert kept.dtype == torch.int32 and kept.numel() >= sum(k_per_seg)
-    st = lib().ecospa_select_aligned_topk(_ptr(upsilon), C.addressof(a_nseg), C.addressof(a_slen), C.addressof(a_k),
+    st = lib().ecospa_select_aligned_topk(_ptr(upsilon), _addr(a_nseg), _addr(a_slen), _addr(a_k),
                                           n_pairs, _ptr(kept), _ptr(seg_offsets), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_select_aligned_topk")
@@ -177,16 +194,14 @@ def ecospa_select_rotation_pairs(upsilon: torch.Tensor, n_seg: Sequence[int], se
                                  k_per_seg: Sequence[int], rope: Sequence[int], kept: torch.Tensor,
                                  seg_offsets: Optional[torch.Tensor] = None, stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg = (C.c_int32 * n_pairs)(*n_seg)
-    a_slen = (C.c_int32 * n_pairs)(*seg_len)
-    a_rope = (C.c_int32 * n_pairs)(*rope)
-    a_k = (C.c_int32 * len(k_per_seg))(*k_per_seg)
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
+    assert len(a_slen) == n_pairs
+    a_rope = _i32(rope)
+    a_k = _i32(k_per_seg)
     assert len(k_per_seg) == sum(n_seg) and len(rope) == n_pairs
     assert kept.dtype == torch.int32 and kept.numel() >= sum(k_per_seg)
-    fn = lib().ecospa_select_rotation_pairs
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p]
-    st = fn(_ptr(upsilon), C.addressof(a_nseg), C.addressof(a_slen), C.addressof(a_k), C.addressof(a_rope), n_pairs,
+    fn = _fn("ecospa_select_rotation_pairs")
+    st = fn(_ptr(upsilon), _addr(a_nseg), _addr(a_slen), _addr(a_k), _addr(a_rope), n_pairs,
             _ptr(kept), _ptr(seg_offsets), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_select_rotation_pairs")
@@ -196,12 +211,9 @@ def ecospa_pack_kept(slots: torch.Tensor, src: Sequence[int], dst: Sequence[int]
                      out: torch.Tensor, stream=None) -> None:
     n = len(src)
     assert len(dst) == n and len(k) == n and len(add) == n and slots.dtype == torch.int32 and out.dtype == torch.int32
-    arr = lambda v: (C.c_int32 * n)(*v)
-    a_src, a_dst, a_k, a_add = arr(src), arr(dst), arr(k), arr(add)
-    fn = lib().ecospa_pack_kept
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]
-    st = fn(_ptr(slots), C.addressof(a_src), C.addressof(a_dst), C.addressof(a_k), C.addressof(a_add), n, _ptr(out),
+    a_src, a_dst, a_k, a_add = _i32(src), _i32(dst), _i32(k), _i32(add)
+    fn = _fn("ecospa_pack_kept")
+    st = fn(_ptr(slots), _addr(a_src), _addr(a_dst), _addr(a_k), _addr(a_add), n, _ptr(out),
             _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_pack_kept")
@@ -209,9 +221,7 @@ def ecospa_pack_kept(slots: torch.Tensor, src: Sequence[int], dst: Sequence[int]
 
 def ecospa_choose_pairs(fisher: torch.Tensor, m: int, chosen: torch.Tensor, stream=None) -> None:
     assert fisher.dtype == torch.float32 and chosen.dtype == torch.int32 and chosen.numel() >= fisher.numel()
-    fn = lib().ecospa_choose_pairs
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p]
+    fn = _fn("ecospa_choose_pairs")
     st = fn(_ptr(fisher), fisher.numel(), int(m), _ptr(chosen), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_choose_pairs")
@@ -222,16 +232,14 @@ def ecospa_select_aligned_threshold(upsilon: torch.Tensor, n_seg: Sequence[int],
                                     chosen: Optional[torch.Tensor] = None, rope: Optional[Sequence[int]] = None,
                                     stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg = (C.c_int32 * n_pairs)(*n_seg)
-    a_slen = (C.c_int32 * n_pairs)(*seg_len)
-    a_rope = (C.c_int32 * n_pairs)(*rope) if rope is not None else None
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
+    assert len(a_slen) == n_pairs
+    a_rope = _i32(rope) if rope is not None else None
+    assert a_rope is None or len(a_rope) == n_pairs
     assert kept.dtype == torch.int32 and kept.numel() >= sum(a * b for a, b in zip(n_seg, seg_len))
     assert k_out.dtype == torch.int32 and k_out.numel() >= sum(n_seg)
-    fn = lib().ecospa_select_aligned_threshold
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_double, C.c_int32, C.c_int32, C.c_void_p,
-                   C.c_void_p, C.c_void_p, C.c_void_p]
-    st = fn(_ptr(upsilon), C.addressof(a_nseg), C.addressof(a_slen), C.addressof(a_rope) if a_rope is not None else None,
+    fn = _fn("ecospa_select_aligned_threshold")
+    st = fn(_ptr(upsilon), _addr(a_nseg), _addr(a_slen), _addr(a_rope) if a_rope is not None else None,
             n_pairs, float(theta), int(bool(l1)), int(k_min), _ptr(chosen), _ptr(kept), _ptr(k_out), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_select_aligned_threshold")
@@ -244,19 +252,17 @@ def gather(inp: torch.Tensor, out: torch.Tensor, layout: int, kept: torch.Tensor
 
 
 def ecospa_compact_tensors(jobs: Sequence[Gather], stream=None) -> None:
-    arr = (Gather * len(jobs))(*jobs)
-    st = lib().ecospa_compact_tensors(C.addressof(arr), len(jobs), _stream(stream))
+    arr = _structs(Gather, jobs)
+    st = lib().ecospa_compact_tensors(arr, len(jobs), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_compact_tensors")
 
 
 def ecospa_compact_tensors_inplace(jobs: Sequence[Gather], stream=None) -> None:
     """Jobs whose output is their input (same pointer and pitch): the kept part moves to the front."""
-    arr = (Gather * len(jobs))(*jobs)
-    fn = lib().ecospa_compact_tensors_inplace
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_int32, C.c_void_p]
-    st = fn(C.addressof(arr), len(jobs), _stream(stream))
+    arr = _structs(Gather, jobs)
+    fn = _fn("ecospa_compact_tensors_inplace")
+    st = fn(arr, len(jobs), _stream(stream))
     if st != 0:
         raise EcospaError(st, "ecospa_compact_tensors_inplace")
 
@@ -282,7 +288,7 @@ def ecospa_compact_pair(p: Pair, kept: torch.Tensor, n_kept: int, w1_out: torch.
 # compacted-pair forward / backward
 # ---------------------------------------------------------------------------------------------
 
-_LAYER_SIGS = {
+_SIGS = {
     "ecospa_proj_workspace_bytes": (C.c_size_t, [C.c_int64, C.c_int64, C.c_int64, C.c_int32]),
     "ecospa_ffn_workspace_bytes": (C.c_size_t, [C.c_int64, C.c_int64, C.c_int64, C.c_int32, C.c_int32]),
     "ecospa_coupled_qk_fwd": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_int64, C.c_void_p, C.c_void_p, C.c_int64,
@@ -321,6 +327,34 @@ _LAYER_SIGS = {
                                           C.c_int64, C.c_void_p, C.c_int64, C.c_int32, C.c_void_p, C.c_int64, C.c_void_p,
                                           C.c_void_p, C.c_size_t, C.c_void_p]),
     "ecospa_device_status": (C.c_int, [C.c_void_p, C.c_void_p]),
+    "ecospa_score_pair_static_max_bytes": (C.c_size_t, []),
+    "ecospa_score_pair_static": (C.c_int, [C.c_void_p, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "ecospa_select_rotation_pairs": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32,
+                                               C.c_void_p, C.c_void_p, C.c_void_p]),
+    "ecospa_pack_kept": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p,
+                                   C.c_void_p]),
+    "ecospa_choose_pairs": (C.c_int, [C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p]),
+    "ecospa_select_aligned_threshold": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_double,
+                                                  C.c_int32, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "ecospa_compact_tensors_inplace": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p]),
+    "ecospa_attn_workspace_bytes": (C.c_size_t, [C.c_int64, C.c_int64, C.c_int32]),
+    "ecospa_coupled_attn_fwd": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_int64, C.c_int64,
+                                          C.c_void_p, C.c_float, C.c_int32, C.c_void_p, C.c_int64, C.c_void_p, C.c_void_p]),
+    "ecospa_coupled_attn_bwd": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64,
+                                          C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_float,
+                                          C.c_int32, C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_void_p,
+                                          C.c_size_t, C.c_void_p]),
+    "ecospa_pad_kept": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p,
+                                  C.c_void_p]),
+    "ecospa_launch_count": (C.c_uint64, []),
+    "ecospa_set_device_wait_limit_ns": (C.c_int, [C.c_uint64]),
+    "ecospa_gemm_resident_pairs": (C.c_int32, []),
+    "ecospa_alg1_workspace_bytes": (C.c_size_t, [C.c_void_p, C.c_int32]),
+    "ecospa_alg1_offsets": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p]),
+    "ecospa_alg1_plan": (C.c_int, [C.c_void_p, C.c_int32, C.c_double, C.c_int32, C.c_double, C.c_int32, C.c_int32,
+                                   C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p]),
+    "ecospa_alg1_apply": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t,
+                                    C.c_void_p]),
 }
 _sigs_done = False
 
@@ -329,7 +363,7 @@ def _fn(name: str):
     global _sigs_done
     l = lib()
     if not _sigs_done:
-        for n, (res, args) in _LAYER_SIGS.items():
+        for n, (res, args) in _SIGS.items():
             f = getattr(l, n)
             f.restype, f.argtypes = res, args
         _sigs_done = True
@@ -520,19 +554,14 @@ def heads(qk_off: Sequence[int], qk_w: Sequence[int], vo_off: Sequence[int], vo_
 
 
 def ecospa_attn_workspace_bytes(batch: int, seq: int, n_heads: int) -> int:
-    f = lib().ecospa_attn_workspace_bytes
-    f.restype = C.c_size_t
-    f.argtypes = [C.c_int64, C.c_int64, C.c_int32]
+    f = _fn("ecospa_attn_workspace_bytes")
     return int(f(batch, seq, n_heads))
 
 
 def ecospa_coupled_attn_fwd(Qc, Kc, Vc, batch: int, seq: int, hd: Heads, scale: float, causal: bool, Ctx, lse,
                             stream=None) -> None:
     """Ctx_h = softmax(scale * Q_h K_h^T) V_h per sequence and head; lse: fp32 [n_heads * T]."""
-    f = lib().ecospa_coupled_attn_fwd
-    f.restype = C.c_int
-    f.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_int64, C.c_int64, C.c_void_p, C.c_float,
-                  C.c_int32, C.c_void_p, C.c_int64, C.c_void_p, C.c_void_p]
+    f = _fn("ecospa_coupled_attn_fwd")
     assert Qc.stride(0) == Kc.stride(0)
     _check(f(Qc.data_ptr(), Kc.data_ptr(), Qc.stride(0), Vc.data_ptr(), Vc.stride(0), batch, seq, C.addressof(hd),
              float(scale), int(bool(causal)), Ctx.data_ptr(), Ctx.stride(0), lse.data_ptr(), _stream(stream)),
@@ -541,11 +570,7 @@ def ecospa_coupled_attn_fwd(Qc, Kc, Vc, batch: int, seq: int, hd: Heads, scale: 
 
 def ecospa_coupled_attn_bwd(Qc, Kc, Vc, Ctx, dCtx, lse, batch: int, seq: int, hd: Heads, scale: float, causal: bool,
                             dQc, dKc, dVc, workspace, stream=None) -> None:
-    f = lib().ecospa_coupled_attn_bwd
-    f.restype = C.c_int
-    f.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_void_p, C.c_int64,
-                  C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_float, C.c_int32, C.c_void_p, C.c_void_p, C.c_int64,
-                  C.c_void_p, C.c_int64, C.c_void_p, C.c_size_t, C.c_void_p]
+    f = _fn("ecospa_coupled_attn_bwd")
     assert Qc.stride(0) == Kc.stride(0) and dQc.stride(0) == dKc.stride(0)
     wp, wb = _ws(workspace)
     _check(f(Qc.data_ptr(), Kc.data_ptr(), Qc.stride(0), Vc.data_ptr(), Vc.stride(0), Ctx.data_ptr(), Ctx.stride(0),
@@ -558,12 +583,9 @@ def ecospa_pad_kept(kept: torch.Tensor, src: Sequence[int], dst: Sequence[int], 
                     k_padded: Sequence[int], out: torch.Tensor, stream=None) -> None:
     n = len(src)
     assert len(dst) == n and len(k) == n and len(k_padded) == n and kept.dtype == torch.int32 and out.dtype == torch.int32
-    arr = lambda v: (C.c_int32 * n)(*[int(x) for x in v])
-    a_src, a_dst, a_k, a_kp = arr(src), arr(dst), arr(k), arr(k_padded)
-    fn = lib().ecospa_pad_kept
-    fn.restype = C.c_int
-    fn.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]
-    _check(fn(_ptr(kept), C.addressof(a_src), C.addressof(a_dst), C.addressof(a_k), C.addressof(a_kp), n, _ptr(out),
+    a_src, a_dst, a_k, a_kp = _i32(src), _i32(dst), _i32(k), _i32(k_padded)
+    fn = _fn("ecospa_pad_kept")
+    _check(fn(_ptr(kept), _addr(a_src), _addr(a_dst), _addr(a_k), _addr(a_kp), n, _ptr(out),
               _stream(stream)), "ecospa_pad_kept")
 
 
@@ -589,21 +611,15 @@ def group(w1, w2, layout1: int, layout2: int, widths: Sequence[int], w1b=None, g
     return g
 
 
-def _alg1(name, restype, argtypes):
-    f = getattr(lib(), name)
-    f.restype, f.argtypes = restype, argtypes
-    return f
-
-
 def ecospa_alg1_workspace_bytes(groups: Sequence[Group]) -> int:
-    arr = (Group * len(groups))(*groups)
-    return int(_alg1("ecospa_alg1_workspace_bytes", C.c_size_t, [C.c_void_p, C.c_int32])(C.addressof(arr), len(groups)))
+    arr = _structs(Group, groups)
+    return int(_fn("ecospa_alg1_workspace_bytes")(arr, len(groups)))
 
 
 def ecospa_alg1_offsets(groups: Sequence[Group]) -> List[int]:
-    arr = (Group * len(groups))(*groups)
+    arr = _structs(Group, groups)
     out = (C.c_int64 * 6)()
-    _check(_alg1("ecospa_alg1_offsets", C.c_int, [C.c_void_p, C.c_int32, C.c_void_p])(C.addressof(arr), len(groups), C.addressof(out)),
+    _check(_fn("ecospa_alg1_offsets")(arr, len(groups), C.addressof(out)),
            "ecospa_alg1_offsets")
     return [int(v) for v in out]
 
@@ -611,44 +627,38 @@ def ecospa_alg1_offsets(groups: Sequence[Group]) -> List[int]:
 def ecospa_alg1_plan(groups: Sequence[Group], n_samples: float, n_choose: int, theta: float, l1: bool, k_min: int,
                      workspace: torch.Tensor, stream=None) -> List[int]:
     """Returns the new width of every pair of every group (synchronises the stream)."""
-    arr = (Group * len(groups))(*groups)
+    arr = _structs(Group, groups)
     n = sum(g.n_pairs for g in groups)
     k = (C.c_int32 * n)()
-    f = _alg1("ecospa_alg1_plan", C.c_int, [C.c_void_p, C.c_int32, C.c_double, C.c_int32, C.c_double, C.c_int32, C.c_int32,
-                                            C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p])
-    _check(f(C.addressof(arr), len(groups), float(n_samples), int(n_choose), float(theta), int(bool(l1)), int(k_min),
+    f = _fn("ecospa_alg1_plan")
+    _check(f(arr, len(groups), float(n_samples), int(n_choose), float(theta), int(bool(l1)), int(k_min),
              workspace.data_ptr(), workspace.numel(), C.addressof(k), _stream(stream)), "ecospa_alg1_plan")
     return list(k)
 
 
 def ecospa_alg1_apply(groups: Sequence[Group], k: Sequence[int], out: Optional[Sequence[Group]], workspace: torch.Tensor,
                       in_place: bool = False, stream=None) -> None:
-    arr = (Group * len(groups))(*groups)
-    oarr = (Group * len(out))(*out) if out is not None else None
-    ka = (C.c_int32 * len(k))(*[int(v) for v in k])
-    f = _alg1("ecospa_alg1_apply", C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t,
-                                             C.c_void_p])
-    _check(f(C.addressof(arr), len(groups), C.addressof(ka), C.addressof(oarr) if oarr is not None else None,
+    arr = _structs(Group, groups)
+    oarr = _structs(Group, out) if out is not None else None
+    ka = _i32(k)
+    f = _fn("ecospa_alg1_apply")
+    _check(f(arr, len(groups), _addr(ka), oarr,
              int(bool(in_place)), workspace.data_ptr(), workspace.numel(), _stream(stream)), "ecospa_alg1_apply")
 
 
 def ecospa_launch_count() -> int:
-    f = lib().ecospa_launch_count
-    f.restype = C.c_uint64
+    f = _fn("ecospa_launch_count")
     return int(f())
 
 
 def ecospa_set_device_wait_limit_ns(ns: int) -> None:
     """How long a device-side wait of the layer kernels may last before the kernel gives up (default 2 s)."""
-    f = lib().ecospa_set_device_wait_limit_ns
-    f.restype = C.c_int
-    f.argtypes = [C.c_uint64]
+    f = _fn("ecospa_set_device_wait_limit_ns")
     _check(f(int(ns)), "ecospa_set_device_wait_limit_ns")
 
 
 def ecospa_gemm_resident_pairs() -> int:
-    f = lib().ecospa_gemm_resident_pairs
-    f.restype = C.c_int32
+    f = _fn("ecospa_gemm_resident_pairs")
     return int(f())
 
 
