@@ -1,6 +1,7 @@
 // Grouped persistent bf16 GEMM for sm_100a: TMA -> shared memory ring -> tcgen05.mma (fp32 accumulators
 // in TMEM, double buffered) -> fused epilogues.  Two forms of the same kernel:
-//   single  cta_group::1, one CTA per SM computes 128x256 tiles (2 stages of 2 x (16 KB A + 32 KB B))
+//   single  cta_group::1, one CTA per SM computes 128x128 tiles (3 stages of 2 x (16 KB A + 16 KB B)): launches that
+//           such tiles fill in one round
 //   pair    cta_group::2, a cluster of two CTAs computes 256x256 tiles: each CTA loads its 128 rows of A
 //           and its half of B (3 stages of 2 x (16 KB + 16 KB)), the leader CTA issues the MMAs for both,
 //           so every SM fetches a third less operand data per flop.  Every CTA issues its own loads: the
@@ -37,16 +38,21 @@ namespace ecospa {
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64;
-constexpr int kAStage = BM * BK * 2;        // 16 KB
-constexpr int kBStage = BN * BK * 2;        // 32 KB
-constexpr int kBHalf = kBStage / 2;
-constexpr int kRingBytes = 4 * (kAStage + kBStage);   // = 6 * (kAStage + kBHalf) = 192 KB
-constexpr int kMaxStages = 6;
+constexpr int BM = 128, BK = 64;
+constexpr int kAStage = BM * BK * 2;        // 16 KB: 128 rows of A
+constexpr int kBStage = 128 * BK * 2;       // 16 KB: 128 columns of B (a pair's CTA holds half of the tile's 256)
+constexpr int kSub = 2;                     // 64-deep k-blocks per pipeline stage
+constexpr int kStages = 3;
+constexpr int kRingBytes = kStages * kSub * (kAStage + kBStage);   // 192 KB
+// Tile of a worker, by form: rows and columns.
+template <bool PAIR>
+struct TileShape {
+    static constexpr int kM = PAIR ? 2 * BM : BM, kN = PAIR ? 256 : 128;
+    static constexpr int kTmemCols = 2 * kN;               // two accumulators
+};
 constexpr int kAtomBytes = 64 * 64 * 2;     // one 64x64 bf16 swizzle atom of an MN-major operand
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kTmemCols = 512;
 constexpr int kMaxSeg = 3;
 constexpr int kEpiSlotBytes = 32 * 32 * 2;  // one 32-row x 64-byte staging image; a warp owns two (= one 32 x 128-byte image)
 constexpr int kEpiBytes = kEpiWarps * 2 * kEpiSlotBytes;
@@ -58,7 +64,7 @@ struct DevProblem {
     int32_t kb_end[kMaxSeg];     // cumulative k-blocks: segment s covers [kb_end[s-1], kb_end[s])
     int32_t kblocks;             // k-blocks of all segments
     int32_t tiles_m, tiles_n, tile_start;
-    int32_t n_per_tile;          // output columns per tile: 256, or 128 hidden units for EPI_SWIGLU
+    int32_t n_per_tile;          // output columns per tile: the tile's, or half as many hidden units for EPI_SWIGLU
     int32_t half1_n_off;         // n-coordinate of B half 1 relative to half 0
     int32_t epi;
     int32_t k_off[kMaxSeg];      // first contraction index of each segment
@@ -534,10 +540,9 @@ __device__ __forceinline__ const DevProblem& find_problem(const Params& P, int t
 // ------------------------------------------------------------------------------------------------
 template <bool PAIR, typename Params>
 __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant__ Params P) {
-    constexpr int kSub = 2;                                  // 64-deep k-blocks per pipeline stage
-    constexpr int kStages = PAIR ? 3 : 2;
-    constexpr int kBLocal = PAIR ? kBHalf : kBStage;        // B bytes this CTA holds per k-block
-    constexpr int kTileM = PAIR ? 2 * BM : BM;               // rows of one scheduled tile
+    constexpr int kTileM = TileShape<PAIR>::kM, kTileN = TileShape<PAIR>::kN;
+    constexpr int kTmemCols = TileShape<PAIR>::kTmemCols;
+    constexpr int kHalfN = kTileN / 2;                       // columns of an epilogue warp
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;       // 1024-byte aligned stage memory
@@ -546,8 +551,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     const uint32_t sEpi = base + kRingBytes;
     uint8_t* tail = smem + kRingBytes + kEpiBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);        // full[S], empty[S], tmem_full[2], tmem_empty[2]
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + (2 * kMaxStages + 4) * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + (2 * kMaxStages + 4) * 8 + 8);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + (2 * kStages + 4) * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + (2 * kStages + 4) * 8 + 8);
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
@@ -620,7 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     if (!(ok = mbar_wait<PAIR>(empty_bar(stage), phase ^ 1u, abort_flag, 1, P.head.status, P.head.wait_limit_ns))) break;
                     // "big" operands arrive as one box holding both k-blocks (zero-filled past the end of K)
                     const bool a_big = PAIR && Q.a_big[seg], b_big = PAIR && Q.b_big[seg];
-                    const uint32_t tx = (a_big ? kSub : nsub) * kAStage + (b_big ? kSub : nsub) * kBLocal;
+                    const uint32_t tx = (a_big ? kSub : nsub) * kAStage + (b_big ? kSub : nsub) * kBStage;
                     if (PAIR) {
                         if (leader) mbar_expect_tx(full_bar(stage), 2 * tx);   // both CTAs' bytes
                     } else {
@@ -641,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                             }
                         }
                         if (b_big) {
-                            const uint32_t dst = sB + stage * kSub * kBLocal;
+                            const uint32_t dst = sB + stage * kSub * kBStage;
                             const CUtensorMap* mb = &P.maps[Q.map_b[seg][cta_rank]];
                             const int nc = n0 + static_cast<int>(cta_rank) * Q.half1_n_off;
                             if (!Q.b_mn[seg]) {
@@ -658,7 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     if (sub >= nsub) break;
                     const int kb = kb0 + sub;
                     const int k0 = (kb - kb_lo) * BK + Q.k_off[seg];
-                    const uint32_t a_dst = sA + (stage * kSub + sub) * kAStage, b_dst = sB + (stage * kSub + sub) * kBLocal;
+                    const uint32_t a_dst = sA + (stage * kSub + sub) * kAStage, b_dst = sB + (stage * kSub + sub) * kBStage;
                     const CUtensorMap* ma = &P.maps[Q.map_a[seg]];
                     if (PAIR) {
                         // This CTA's share of the stage, completed on the leader's barrier: the leader uses the
@@ -703,18 +708,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                             tma_load_2d(a_dst + kAtomBytes, ma, m0 + 64, k0, full_bar(stage));
                         }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
+                        for (int h = 0; h < 2; ++h) {                                           // 64 columns of B each
                             const CUtensorMap* mb = &P.maps[Q.map_b[seg][h]];
                             const int nc = n0 + h * Q.half1_n_off;
-                            const uint32_t dst = b_dst + h * kBHalf;
-                            if (!Q.b_mn[seg]) {
-                                tma_load_2d(dst, mb, k0, nc, full_bar(stage));                  // box 64(k) x 128(n)
-                            } else if (Q.b_3d[seg]) {
-                                tma_load_3d(dst, mb, 0, k0, nc >> 6, full_bar(stage));
-                            } else {
-                                tma_load_2d(dst, mb, nc, k0, full_bar(stage));                  // box 64(n) x 64(k)
-                                tma_load_2d(dst + kAtomBytes, mb, nc + 64, k0, full_bar(stage));
-                            }
+                            const uint32_t dst = b_dst + h * kAtomBytes;
+                            if (!Q.b_mn[seg]) tma_load_2d(dst, mb, k0, nc, full_bar(stage));    // box 64(k) x 64(n)
+                            else tma_load_2d(dst, mb, nc, k0, full_bar(stage));                 // box 64(n) x 64(k)
                         }
                     }
                     }   // sub
@@ -738,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                 const uint32_t acc_phase = (it >> 1) & 1u;
                 if (!(ok = mbar_wait<PAIR>(tempty_bar(acc), acc_phase ^ 1u, abort_flag, 2, P.head.status, P.head.wait_limit_ns))) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + acc * BN;
+                const uint32_t d_tmem = tmem_base + acc * kTileN;
                 for (int seg = 0; ok && seg < kMaxSeg; ++seg) {
                 const int kb_lo = seg ? Q.kb_end[seg - 1] : 0, kb_hi = Q.kb_end[seg];
                 for (int kb0 = kb_lo; kb0 < kb_hi; kb0 += kSub) {
@@ -751,9 +750,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                         const int kb = kb0 + sub;
                         const uint32_t a_mn = Q.a_mn[seg], b_mn = Q.b_mn[seg];
                         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (a_mn << 15) | (b_mn << 16) |
-                                               (static_cast<uint32_t>(BN >> 3) << 17) | (static_cast<uint32_t>(kTileM >> 4) << 24);
+                                               (static_cast<uint32_t>(kTileN >> 3) << 17) | (static_cast<uint32_t>(kTileM >> 4) << 24);
                         const uint64_t a_desc = make_smem_desc(sA + (stage * kSub + sub) * kAStage, a_mn ? kAtomBytes : 16, 1024);
-                        const uint64_t b_desc = make_smem_desc(sB + (stage * kSub + sub) * kBLocal, b_mn ? kAtomBytes : 16, 1024);
+                        const uint64_t b_desc = make_smem_desc(sB + (stage * kSub + sub) * kBStage, b_mn ? kAtomBytes : 16, 1024);
                         const uint64_t a_step = a_mn ? (2048 >> 4) : (32 >> 4);   // per 16 k: two 8-row groups, or 32 bytes
                         const uint64_t b_step = b_mn ? (2048 >> 4) : (32 >> 4);
 #pragma unroll
@@ -811,17 +810,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             const unsigned short* Hp = static_cast<const unsigned short*>(Q.H);
             const unsigned short* Hbp = static_cast<const unsigned short*>(Q.Hb);
             uint4 hq[4], hbq[4];
-            if (need_h) staged_load32_issue(Hp, Q.ldh, m_warp, n0 + half * 128, QM, QN, hq, lane);
-            if (need_hb) staged_load32_issue(Hbp, Q.ldh, m_warp, n0 + half * 128, QM, QN, hbq, lane);
+            if (need_h) staged_load32_issue(Hp, Q.ldh, m_warp, n0 + half * kHalfN, QM, QN, hq, lane);
+            if (need_hb) staged_load32_issue(Hbp, Q.ldh, m_warp, n0 + half * kHalfN, QM, QN, hbq, lane);
             // the second slot doubles as the landing buffer of those loads: no store of an earlier tile may still read it
             if (need_h) stage_begin<0>(lane);
-            // bias of this warp's 128 columns, one column per lane and 32-column chunk (fetched while the tile is computed)
+            // bias of this warp's columns, one column per lane and 32-column chunk (fetched while the tile is computed)
             float breg[4] = {0.f, 0.f, 0.f, 0.f};
             const bool has_bias = Q.bias != nullptr;
             if (has_bias) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int col = n0 + half * 128 + 32 * j + lane;
+                for (int j = 0; j < kHalfN / 32; ++j) {
+                    const int col = n0 + half * kHalfN + 32 * j + lane;
                     if (col < QN)
                         breg[j] = Q.bias_f32 ? static_cast<const float*>(Q.bias)[col]
                                              : __uint_as_float(static_cast<uint32_t>(static_cast<const unsigned short*>(Q.bias)[col]) << 16);
@@ -829,10 +828,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             }
             if (!(ok = mbar_wait<PAIR>(tfull_bar(acc), acc_phase, abort_flag, 4, P.head.status, P.head.wait_limit_ns))) break;
             tc_fence_after();
-            const uint32_t t_row = tmem_base + acc * BN + (static_cast<uint32_t>(quad * 32) << 16);
+            const uint32_t t_row = tmem_base + acc * kTileN + (static_cast<uint32_t>(quad * 32) << 16);
             const bool warp_rows = m_warp < QM;          // any row of this warp inside the output
             if (epi == EPI_SWIGLU) {
-                // accumulator columns [0,128) = gate, [128,256) = up for hidden units n0 .. n0+127.
+                // accumulator columns: gate, then up, for hidden units n0 .. n0 + kHalfN - 1.
                 // The three outputs of a chunk alternate between the two slots, one store may stay in flight.
                 int slot = 0;
                 bool fresh = true;
@@ -845,11 +844,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     slot ^= 1;
                 };
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    const int hc = half * 64 + c * 32;
+                for (int c = 0; c < kHalfN / 64; ++c) {
+                    const int hc = half * (kHalfN / 2) + c * 32;
                     uint32_t rg[32], ru[32];
                     tc_ld32(t_row + hc, rg);
-                    tc_ld32(t_row + 128 + hc, ru);
+                    tc_ld32(t_row + kHalfN + hc, ru);
                     tc_wait_ld();
                     const int n = n0 + hc;
                     if (n >= QN || !warp_rows) continue;
@@ -866,10 +865,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     put(mc2, n, g);
                 }
             } else if (epi == EPI_STORE && !Q.out_f32) {
-                // bf16 output: two chunks of 64 columns, each one 32 x 128-byte image
+                // bf16 output: chunks of 64 columns, each one 32 x 128-byte image
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    const int col = half * 128 + c * 64;
+                for (int c = 0; c < kHalfN / 64; ++c) {
+                    const int col = half * kHalfN + c * 64;
                     uint32_t r0[32], r1[32];
                     tc_ld32(t_row + col, r0);
                     tc_ld32(t_row + col + 32, r1);
@@ -893,8 +892,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             } else if (epi == EPI_GELU_ERF || epi == EPI_GELU_TANH) {
                 // H = acc + bias and A = GELU(H), 64 columns at a time
 #pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    const int col = half * 128 + c * 64;
+                for (int c = 0; c < kHalfN / 64; ++c) {
+                    const int col = half * kHalfN + c * 64;
                     uint32_t r0[32], r1[32];
                     tc_ld32(t_row + col, r0);
                     tc_ld32(t_row + col + 32, r1);
@@ -931,8 +930,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             } else {
                 // 32 columns at a time: fp32 outputs and the derivative epilogues
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
-                    const int col = half * 128 + c * 32;
+                for (int c = 0; c < kHalfN / 32; ++c) {
+                    const int col = half * kHalfN + c * 32;
                     uint32_t r[32];
                     tc_ld32(t_row + col, r);
                     tc_wait_ld();
@@ -952,7 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     } else if (epi == EPI_DGELU_ERF || epi == EPI_DGELU_TANH) {
                         float h[32];
                         staged_load32_finish(buf_in, hq, h, lane);
-                        if (c < 3) staged_load32_issue(Hp, Q.ldh, m_warp, n + 32, QM, QN, hq, lane);
+                        if (c + 1 < kHalfN / 32) staged_load32_issue(Hp, Q.ldh, m_warp, n + 32, QM, QN, hq, lane);
 #pragma unroll
                         for (int i = 0; i < 32; ++i)
                             if (epi != EPI_DGELU_ERF) v[i] *= dgelu_tanh(h[i]);
@@ -966,7 +965,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                         float hg[32], hu[32];
                         staged_load32_finish(buf_in, hq, hg, lane);
                         staged_load32_finish(buf_in, hbq, hu, lane);
-                        if (c < 3) {
+                        if (c + 1 < kHalfN / 32) {
                             staged_load32_issue(Hp, Q.ldh, m_warp, n + 32, QM, QN, hq, lane);
                             staged_load32_issue(Hbp, Q.ldh, m_warp, n + 32, QM, QN, hbq, lane);
                         }
@@ -1360,14 +1359,19 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     }
     std::stable_sort(order, order + n_ops, [&](int a, int b) { return ktot[a] > ktot[b]; });
 
-    // CTA pairs pay off as soon as there is more than one 128-row tile to share a B tile between
+    // CTA pairs fetch a third less operand data per flop, but their 256x256 tiles leave most of the chip idle in a small
+    // product, and a lone launch then waits for one pair's main loop and for an epilogue of 128x256 outputs per CTA.  Where
+    // 128x128 tiles of single CTAs still fit one round, they take their place (320 tokens, 768 wide: the eight products of a training step took 10-19 us each and take 8-16).
     bool pair = g_pair_mode != 0 && g_max_pairs >= 1;
     if (pair) {
-        bool any_tall = false;
-        for (int i = 0; i < n_ops; ++i) any_tall = any_tall || ops[i].M > BM;
-        pair = any_tall;
+        int64_t single_tiles = 0;
+        for (int i = 0; i < n_ops; ++i) {
+            const int per_tile = ops[i].epi == EPI_SWIGLU ? TileShape<false>::kN / 2 : TileShape<false>::kN;
+            single_tiles += ceil_div(ops[i].M, BM) * ceil_div(ops[i].N, per_tile);
+        }
+        pair = single_tiles > g_num_sms;
     }
-    const int tile_m = pair ? 2 * BM : BM;
+    const int tile_m = pair ? TileShape<true>::kM : TileShape<false>::kM, tile_n = pair ? TileShape<true>::kN : TileShape<false>::kN;
 
     static thread_local LargeParams gp;
     MapTable T(gp);
@@ -1392,8 +1396,8 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
         if (op.bias && !aligned16(op.bias)) return ECOSPA_ERR_ALIGNMENT;
         Q.M = static_cast<int32_t>(op.M);
         Q.N = static_cast<int32_t>(op.N);
-        Q.n_per_tile = swiglu ? 128 : BN;
-        Q.half1_n_off = swiglu ? 0 : 128;
+        Q.n_per_tile = swiglu ? tile_n / 2 : tile_n;
+        Q.half1_n_off = swiglu ? 0 : tile_n / 2;
         Q.epi = op.epi;
         Q.out_f32 = op.out_f32;
         Q.accumulate = op.accumulate;
@@ -1418,7 +1422,7 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
             for (int h = 0; h < 2; ++h) {
                 const Stored& b = (swiglu && h == 1) ? ks.b[1] : ks.b[0];
                 if (ks.b_mn ? (b.rows < k_end || b.cols != op.N) : (b.rows != op.N || b.cols < k_end)) return ECOSPA_ERR_INVALID;
-                if ((st = operand_map(T, b, ks.b_mn, pair, 128, true, &map, &form)) != ECOSPA_OK) return st;
+                if ((st = operand_map(T, b, ks.b_mn, pair, pair ? 128 : 64, pair, &map, &form)) != ECOSPA_OK) return st;
                 Q.map_b[s][h] = static_cast<uint8_t>(map);
                 if (h == 0) {
                     Q.b_big[s] = form == FORM_BIG;
