@@ -508,10 +508,12 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
     auto pv_done = [&](uint32_t x, uint32_t buf) { return bar0 + 8u * (42 + 2 * x + buf); };
     auto s_full = [&](uint32_t x, uint32_t buf) { return bar0 + 8u * (12 + 2 * x + buf); };   // scores in buffer buf of stream x
     auto kv_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (20 + 2 * x + b); };      // the loads event G needs (b = G & 1) landed
+    auto k2_full = [&](uint32_t x) { return bar0 + 8u * (48 + x); };                          // the third K slice of stream x landed
     const uint32_t merge_a = bar0 + 8u * 40, merge_b = bar0 + 8u * 41;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        for (uint32_t x = 0; x < NS; ++x) mbar_init(k2_full(x), 1);
         for (uint32_t s = 0; s < 2; ++s) {
             mbar_init(q_full(s), 1);
             mbar_init(q_empty(s), NS);
@@ -552,8 +554,8 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
             const uint32_t sKx = sK + x * ST * kSliceB, sVx = sV + x * ST * kSliceB;
             const uint64_t dq0 = make_smem_desc(sQ, 16, 1024), dk0 = make_smem_desc(sKx, 16, 1024),
                            dv0 = make_smem_desc(sVx, kBlockBytes, 1024);
-            // meta bits: 0 valid, 1 first slice of its item, 2 last, 3 Q buffer, 4 phase of that buffer, 5-7 contraction
-            // steps of the scores, 8-11 output width / 16, 12-.. items skipped just before (first slices and the end mark)
+            // meta bits: 0 valid (clear: the end mark), 1 first slice of its item, 2 last, 3 Q buffer, 4 phase of that buffer,
+            // 5-7 contraction steps of the scores, 8-11 output width / 16
             struct SD {
                 int row;            // first key row of the slice in the K / V tensors
                 int qrow;           // first row of the item's query tile
@@ -570,13 +572,12 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                     for (;;) {
                         g_it += gridDim.x;
                         ++g_qi;
-                        if (g_it >= P.n_items) {   // end mark; it carries the Q buffers still to hand back
+                        if (g_it >= P.n_items) {   // end mark
                             d.row = 0;
                             d.cols = 0;
                             d.qcol = 0;
-                            d.meta = ((g_qi & 1u) << 3) | (g_skip << 12);
-                            g_skip = 0;
-                            g_it -= gridDim.x;      // stay at the end: later calls give the mark again, with no count
+                            d.meta = 0;
+                            g_it -= gridDim.x;      // stay at the end: later calls give the mark again
                             --g_qi;
                             g_J = g_n = 0;
                             d.qrow = 0;
@@ -602,8 +603,7 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                 d.qrow = g_qrow;
                 d.qcol = g_qcol;
                 d.cols = g_cols;
-                d.meta = g_meta | (g_J == 0 ? 2u | (g_skip << 12) : 0u) | (g_J == g_n - 1 ? 4u : 0u);
-                if (g_J == 0) g_skip = 0;
+                d.meta = g_meta | (g_J == 0 ? 2u : 0u) | (g_J == g_n - 1 ? 4u : 0u);
                 ++g_J;
                 return d;
             };
@@ -622,19 +622,11 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
             auto load_v = [&](const SD& d, uint32_t st, uint32_t bar) {
                 tma_load_2d(sVx + st * kSliceB, &P.map_v, d.cols >> 16, d.row, bar);
             };
-            auto hand_back = [&](uint32_t qs_of_item, uint32_t n) {   // Q buffers of the n items before the one whose buffer is given
-                for (uint32_t k = 1; k <= n; ++k) tc_commit(q_empty((qs_of_item + k) & 1u));
-            };
             // S_x of slice d (its K slice in stage st) into score buffer buf
-            auto scores = [&](SD& d, uint32_t st, uint32_t buf) -> bool {
+            auto scores = [&](const SD& d, uint32_t st, uint32_t buf) -> bool {
                 const uint32_t qs = (d.meta >> 3) & 1u;
-                if (!(d.meta & 1u)) {               // the end mark: only the hand-backs, once
-                    hand_back(qs, d.meta >> 12);
-                    d.meta &= 0xfffu;
-                    return true;
-                }
+                if (!(d.meta & 1u)) return true;
                 if (d.meta & 2u) {
-                    hand_back(qs, d.meta >> 12);
                     if (!mbar_wait(q_full(qs), (d.meta >> 4) & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
                     tc_fence_after();
                 }
@@ -649,18 +641,22 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                 return true;
             };
             SD d0 = next(), d1 = next(), d2 = next(), d3;
-            {   // start: K slices 0..2 and V slice 0 on the barrier event 0 waits on
-                const uint32_t nk = (d0.meta & 1u) + (d1.meta & 1u) + (d2.meta & 1u);
+            {   // start: K slices 0 and 1 and V slice 0, and their score products; then K slice 2, on a barrier of its own.  (Where
+                // every item is one slice long, slice 2 brings the third Q tile, whose buffer is free only after slice 0's product.)
+                const uint32_t nk = (d0.meta & 1u) + (d1.meta & 1u);
                 if (nk) mbar_expect_tx(kv_full(x, 0), (nk + 1) * kSliceB);
                 if (d0.meta & 1u) {
                     ok = load_k(d0, 0, kv_full(x, 0));
                     load_v(d0, 0, kv_full(x, 0));
                 }
                 if (ok && (d1.meta & 1u)) ok = load_k(d1, 1, kv_full(x, 0));
-                if (ok && (d2.meta & 1u)) ok = load_k(d2, 2, kv_full(x, 0));
                 if (ok && nk) ok = mbar_wait(kv_full(x, 0), 0u, abort_flag, 12, P.status, P.wait_limit_ns);
                 tc_fence_after();
                 ok = ok && scores(d0, 0, 0) && scores(d1, 1, 1);
+                if (ok && (d2.meta & 1u)) {
+                    mbar_expect_tx(k2_full(x), kSliceB);
+                    ok = load_k(d2, 2, k2_full(x));
+                }
             }
             uint32_t G = 0, st0 = 0;                // st0 = G % 3
             while (ok && (d0.meta & 1u)) {
@@ -668,6 +664,7 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                 const uint32_t st1 = st0 == 2 ? 0 : st0 + 1, st2 = st1 == 2 ? 0 : st1 + 1;
                 if (!(ok = mbar_wait(p_full(x, buf), ph, abort_flag, 12, P.status, P.wait_limit_ns))) break;
                 if (G > 0 && !(ok = mbar_wait(kv_full(x, buf), ph, abort_flag, 12, P.status, P.wait_limit_ns))) break;
+                if (G == 0 && (d2.meta & 1u) && !(ok = mbar_wait(k2_full(x), 0u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
                 tc_fence_after();
                 {   // O_x += P_x V_x over the slice's 64 keys
                     const uint32_t idesc_o = make_idesc(kTile, ((d0.meta >> 8) & 15u) << 4, 0, 1);
@@ -692,6 +689,14 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                 d2 = d3;
                 st0 = st1;
                 ++G;
+            }
+            // The items without a visible key for this stream are the last ones of the CTA's list (what an item sees never grows
+            // along it).  Their Q buffers are handed back one by one, each once it has been filled: a hand-back ahead of that
+            // would count towards the phase of an earlier item, and with several of them the buffer's phases run away from the
+            // loader, which then waits for good.
+            for (uint32_t k = g_qi + 1 - g_skip; ok && k != g_qi + 1; ++k) {
+                if (!(ok = mbar_wait(q_full(k & 1u), (k >> 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
+                mbar_arrive(q_empty(k & 1u));
             }
         }
     } else {

@@ -85,14 +85,16 @@ def _rel(got, want):
     return float(np.linalg.norm(got.double().cpu().numpy() - want) / max(np.linalg.norm(want), 1e-30))
 
 
-@pytest.mark.parametrize("T,d_m,k", [(1, 64, 1), (127, 72, 31), (128, 128, 64), (129, 136, 65), (300, 264, 129), (1100, 512, 1032), (1664, 1536, 1408)])
+@pytest.mark.parametrize("T,d_m,k", [(1, 64, 40), (33, 64, 1), (127, 72, 31), (128, 128, 64), (129, 136, 65), (300, 264, 129), (1100, 512, 1032), (1664, 1536, 1408)])
 @pytest.mark.parametrize("act", [B.ACT_GELU_ERF, B.ACT_SWIGLU])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("lin", [False, True])
 def test_ffn_tiles(T, d_m, k, act, dtype, lin):
     """Forward and backward of products from less than one 128 x 128 tile to more tiles than SMs (where the launch changes from
     single CTAs to pairs); the fp32 operands also come with a pitch that is not a multiple of four.  Bound: bf16 operands,
-    fp32 sums, saved activations rounded to bf16 (2e-2, as in test_gpu_layers)."""
+    fp32 sums, saved activations rounded to bf16 (2e-2, as in test_gpu_layers).  (An output of one or two numbers has no such
+    bound: a single sum of n rounded products is off by up to 2^-8 of the sum of their magnitudes, sqrt(n) times its own size or
+    more, so the smallest cases have one token or one hidden index, not both.)"""
     g = torch.Generator(device=DEV).manual_seed(T)
     sw = act == B.ACT_SWIGLU
     odd = 1 if dtype == torch.float32 else 0
@@ -126,3 +128,32 @@ def test_ffn_tiles(T, d_m, k, act, dtype, lin):
     else:
         errs["db1"], errs["db2"] = _rel(buf["db1"], dH.sum(0).cpu().numpy()), _rel(buf["db2"], dy.sum(0).cpu().numpy())
     assert max(errs.values()) <= 2e-2, errs
+
+
+@pytest.mark.parametrize("batch,seq,heads,w,causal", [(60, 48, 32, 32, False), (60, 48, 32, 64, True), (40, 130, 32, 16, True),
+                                                      (40, 130, 32, 48, True), (24, 64, 16, 32, False), (75, 65, 8, 64, False)])
+def test_attention_many_short_items(batch, seq, heads, w, causal):
+    """More work items per CTA than Q buffers, all or the last of them without a visible key for some of the streams."""
+    g = torch.Generator(device=DEV).manual_seed(seq)
+    T, off = batch * seq, [w * h for h in range(heads)]
+    q, k, v, do = (torch.randn(T, heads * w, generator=g, device=DEV).to(torch.bfloat16) for _ in range(4))
+    ctx, dq, dk, dv = (torch.zeros_like(q) for _ in range(4))
+    lse = torch.zeros(heads * T, device=DEV)
+    ws = torch.empty(B.ecospa_attn_workspace_bytes(batch, seq, heads), dtype=torch.uint8, device=DEV)
+    hd = B.heads(off, [w] * heads, off, [w] * heads)
+    B.ecospa_coupled_attn_fwd(q, k, v, batch, seq, hd, w ** -0.5, causal, ctx, lse)
+    B.ecospa_coupled_attn_bwd(q, k, v, ctx, do, lse, batch, seq, hd, w ** -0.5, causal, dq, dk, dv, ws)
+    B.ecospa_device_status()
+    split = lambda t: t.double().view(batch, seq, heads, w).transpose(1, 2)
+    Q, K, V, D = map(split, (q, k, v, do))
+    z = Q @ K.transpose(2, 3) * w ** -0.5
+    if causal:
+        z = z.masked_fill(torch.ones(seq, seq, device=DEV, dtype=torch.bool).triu(1), -float("inf"))
+    want_lse = torch.logsumexp(z, 3)
+    p = torch.exp(z - want_lse[..., None])
+    C = p @ V
+    ds = p * (D @ V.transpose(2, 3) - (D * C).sum(3, keepdim=True)) * w ** -0.5
+    assert (lse.view(heads, batch, seq).transpose(0, 1).double() - want_lse).abs().max() <= 2e-3
+    for got, want in ((ctx, C), (dq, ds @ K), (dk, ds.transpose(2, 3) @ Q), (dv, p.transpose(2, 3) @ D)):
+        err = (split(got) - want).flatten(2).norm(dim=2) / want.flatten(2).norm(dim=2)
+        assert float(err.max()) <= 2e-2
