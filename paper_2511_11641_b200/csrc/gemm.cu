@@ -91,6 +91,7 @@ struct GemmHead {
     int32_t n_problems, total_tiles, rounds, use_order;
     int* status;
     unsigned long long wait_limit_ns;   // every mbarrier wait of the launch gives up after this long
+    SideSums side;
 };
 // Kernel parameters in two sizes: what a launch costs the host grows with them (measured with an idle queue, a call of the
 // score kernels with 29 KB took 43-79 us for three launches and takes 16 with 1.7 KB).  Most launches fit the small form (a call's operands, one map each); the large one is for
@@ -535,6 +536,62 @@ __device__ __forceinline__ const DevProblem& find_problem(const Params& P, int t
     return P.prob[pi];
 }
 
+// Column sums that the launch takes along: the epilogue warps have nothing to do until the first tile's main loop is over
+// (0.3 us per 64-deep k-block), and a matrix of 8192 x 1024 is 14 KB per warp of the chip.  A warp takes a unit of kSumRows
+// rows x 64 columns: 8 lanes cover a row's 128 bytes, eight loads of four rows in flight; the four rows of an instruction are
+// added as a shuffle tree, so a unit's sum does not depend on which warp takes it.
+// As a launch of its own between the products and the finishing launch this cost 9-15 us of every
+// backward call on 8192 tokens, 1024 wide, sums and finishing launch together; now 4-5.
+__device__ __forceinline__ void side_sums(const SideSums& S, int first, int stride, int lane) {
+    int tiles = 0;
+    for (int j = 0; j < S.n_jobs; ++j) tiles += S.col_tiles[j];
+    for (int unit = first; unit < tiles * S.chunks; unit += stride) {
+        int j = 0, ct = unit % tiles;
+        const int chunk = unit / tiles;
+        while (ct >= S.col_tiles[j]) ct -= S.col_tiles[j++];
+        const int cols = S.cols[j], c0 = ct * 64 + (lane & 7) * 8;
+        const int64_t ld = S.ld[j], r0 = static_cast<int64_t>(chunk) * kSumRows;
+        const int nr = static_cast<int>(min(static_cast<int64_t>(kSumRows), S.rows - r0));
+        const uint16_t* p = S.M[j] + r0 * ld + c0;
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        if (S.vec_ok[j] && c0 + 8 <= cols) {
+#pragma unroll 1
+            for (int r = lane >> 3; r < nr; r += 32) {
+                uint4 v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    v[u] = r + 4 * u < nr ? *reinterpret_cast<const uint4*>(p + (r + 4 * u) * ld) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    acc[0] += bf16_lo(v[u].x); acc[1] += bf16_hi(v[u].x);
+                    acc[2] += bf16_lo(v[u].y); acc[3] += bf16_hi(v[u].y);
+                    acc[4] += bf16_lo(v[u].z); acc[5] += bf16_hi(v[u].z);
+                    acc[6] += bf16_lo(v[u].w); acc[7] += bf16_hi(v[u].w);
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int r = lane >> 3; r < nr; r += 4)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (c0 + e < cols) acc[e] += __uint_as_float(static_cast<uint32_t>(p[r * ld + e]) << 16);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 8);
+            acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+        }
+        float* out = S.partial[j] + static_cast<int64_t>(chunk) * cols;
+        if (lane < 8) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (c0 + e < cols) out[c0 + e] = acc[e];
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
@@ -788,6 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         const int quad = warp & 3;            // TMEM lanes this warp may read: [32*quad, 32*quad + 32)
         const int half = ew >> 2;             // which half of the tile's columns
         const uint32_t buf_out = sEpi + ew * 2 * kEpiSlotBytes, buf_in = buf_out + kEpiSlotBytes;
+        if (P.head.side.n_jobs > 0) side_sums(P.head.side, blockIdx.x + gridDim.x * ew, gridDim.x * kEpiWarps, lane);
         int it = 0;
         bool ok = true;
         for (int round = 0; ok && round < P.head.rounds; ++round) {
@@ -1342,7 +1400,7 @@ ecospa_status_t validate_gemm_ops(const GemmOp* ops, int n_ops) {
     return ECOSPA_OK;
 }
 
-ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t stream) {
+ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t stream, const SideSums* side) {
     ecospa_status_t st = validate_gemm_ops(ops, n_ops);
     if (st != ECOSPA_OK) return st;
     DeviceState* dev = gemm_setup(&st);
@@ -1458,6 +1516,8 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     gp.head.n_problems = n_ops;
     gp.head.total_tiles = tiles;
     gp.head.status = dev->status_ptr;
+    gp.head.side.n_jobs = 0;
+    if (side && side->n_jobs > 0) gp.head.side = *side;
     gp.head.wait_limit_ns = g_wait_limit_ns.load(std::memory_order_relaxed);
     const int workers = pair ? std::min(tiles, g_max_pairs) : std::min(tiles, g_num_sms);
     build_schedule(gp, workers);

@@ -56,9 +56,22 @@ struct GemmOp {
 
 constexpr int kMaxGemmOps = 16;
 
+// Column sums (bias gradients) that a launch takes along: up to three bf16 matrices with the same number of rows, none of
+// them written by the launch itself.  partial[chunk][col] = sum over the chunk's kSumRows rows.
+constexpr int kSumRows = 128;
+struct SideSums {
+    const uint16_t* M[3];
+    float* partial[3];
+    int64_t ld[3];
+    int32_t cols[3], col_tiles[3];   // col_tiles: tiles of 64 columns
+    int32_t vec_ok[3];               // rows may be read 16 bytes at a time
+    int32_t n_jobs, chunks;
+    int64_t rows;
+};
+
 // Enqueues one persistent launch that computes every op (tiles of the ops with the longest
 // contraction are scheduled first).  Operands must be 16-byte aligned with 16-byte pitches.
-ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t stream);
+ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t stream, const SideSums* side = nullptr);
 
 // The host-only checks launch_grouped_gemm starts with (shapes, null pointers, 16-byte alignment of every base and
 // pitch); makes no CUDA call.  Calls that enqueue several launches check all of them before the first.

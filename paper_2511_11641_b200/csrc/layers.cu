@@ -1,6 +1,6 @@
 // Forward / backward of the compacted coupled pairs (Eq. 2, 3, 5 after aligned removal), expressed as
-// grouped launches of the tcgen05 GEMM engine plus two small helper kernels (fp32 -> bf16 staging for
-// fp32 models, and column sums for the bias gradients).
+// grouped launches of the tcgen05 GEMM engine (which takes the column sums of the bias gradients along) plus two
+// small helper kernels (fp32 -> bf16 staging for fp32 models, and the launch that finishes split sums).
 //
 // Storage: every compacted weight is accepted as d_m x n (ECOSPA_SHARED_COLS) or n x d_m (ECOSPA_SHARED_ROWS),
 // row-major; the equations' orientation is d_m x n for W_Q^c, W_K^c, W_V^c, W_1^c (gate/up) and n x d_m for
@@ -70,81 +70,6 @@ __global__ void __launch_bounds__(kThreads) cast_f32_bf16_kernel(const __grid_co
     }
 }
 
-// Column sums (bias gradients) of up to two bf16 matrices with the same number of rows, two launches:
-// partial[chunk][c] over tiles of kSumRows rows x 64 columns (8 lanes cover a row's 128 bytes with
-// 16-byte loads, the block covers 32 rows per pass, all 4 passes in flight at once: the kernel is one round
-// of loads deep and its grid is large), then a fixed-order sum of the chunks.
-constexpr int kSumRows = 128;
-constexpr int kSumCols = 64;
-struct ColsumJob {
-    const uint16_t* M;
-    float* partial;
-    void* out;
-    int64_t ld, cols;
-    int32_t col_tiles, vec_ok;
-};
-struct ColsumParams {
-    ColsumJob job[3];
-    int64_t rows;
-    int32_t n_jobs, chunks, out_f32;
-};
-
-__global__ void __launch_bounds__(kThreads) colsum_partial_kernel(const __grid_constant__ ColsumParams P) {
-    __shared__ float red[32][kSumCols + 1];
-    pdl_start();
-    pdl_wait();
-    int ji = 0, ct = blockIdx.x;
-    while (ji + 1 < P.n_jobs && ct >= P.job[ji].col_tiles) {
-        ct -= P.job[ji].col_tiles;
-        ++ji;
-    }
-    const ColsumJob& J = P.job[ji];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rowoff = (lane >> 3) + 4 * warp;              // 0..31
-    const int64_t c0 = static_cast<int64_t>(ct) * kSumCols + (lane & 7) * 8;
-    const int64_t r0 = static_cast<int64_t>(blockIdx.y) * kSumRows;
-    const int64_t r1 = r0 + kSumRows < P.rows ? r0 + kSumRows : P.rows;
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    if (c0 < J.cols) {
-        if (J.vec_ok && c0 + 8 <= J.cols) {
-            const uint16_t* p = J.M + c0;
-            for (int64_t r = r0 + rowoff; r < r1; r += 128) {
-                uint4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int64_t rr = r + 32 * u;
-                    v[u] = rr < r1 ? ldg_stream16(p + rr * J.ld) : make_uint4(0, 0, 0, 0);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    acc[0] += bf16_lo(v[u].x); acc[1] += bf16_hi(v[u].x);
-                    acc[2] += bf16_lo(v[u].y); acc[3] += bf16_hi(v[u].y);
-                    acc[4] += bf16_lo(v[u].z); acc[5] += bf16_hi(v[u].z);
-                    acc[6] += bf16_lo(v[u].w); acc[7] += bf16_hi(v[u].w);
-                }
-            }
-        } else {
-            for (int64_t r = r0 + rowoff; r < r1; r += 32)
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (c0 + e < J.cols) acc[e] += __uint_as_float(static_cast<uint32_t>(J.M[r * J.ld + c0 + e]) << 16);
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) red[rowoff][(lane & 7) * 8 + e] = acc[e];
-    __syncthreads();
-    if (threadIdx.x < kSumCols) {
-        const int64_t c = static_cast<int64_t>(ct) * kSumCols + threadIdx.x;
-        if (c < J.cols) {
-            float s = 0.f;
-#pragma unroll
-            for (int w = 0; w < 32; ++w) s += red[w][threadIdx.x];
-            J.partial[static_cast<int64_t>(blockIdx.y) * J.cols + c] = s;
-        }
-    }
-}
 // One launch that finishes a call: out[r][c] = sum over s of partial[s][r][c] for up to three split-K weight
 // gradients (summed in split order), and the fixed-order sum of the column-sum chunks.
 struct ReduceJob {
@@ -152,6 +77,15 @@ struct ReduceJob {
     void* out;
     int64_t rows, cols, ldp, ld_out;
     int32_t splits, blk_start, n_blk, pad_;
+};
+struct ColsumFinal {
+    const float* partial;      // [chunks][cols], from the launch that took the sums along
+    void* out;
+    int64_t cols;
+};
+struct ColsumParams {
+    ColsumFinal job[4];
+    int32_t n_jobs, chunks;
 };
 struct PostParams {
     ReduceJob red[3];
@@ -289,56 +223,38 @@ Stored scratch_bf16(Ctx& cx, int64_t rows, int64_t cols) {
 }
 
 // The launch of a call's (first) products, after the staging of its operands.
-ecospa_status_t run_ops(Ctx& cx, const GemmOp* ops, int n_ops) {
+ecospa_status_t run_ops(Ctx& cx, const GemmOp* ops, int n_ops, const SideSums* side = nullptr) {
     if (cx.casts.n_jobs > 0) {
         const ecospa_status_t st = launch_pdl(cast_f32_bf16_kernel, dim3(cx.cast_blocks), kThreads, cx.stream, cx.casts,
                                               "cast_f32_bf16_kernel");
         cx.casts.n_jobs = cx.cast_blocks = 0;
         if (st != ECOSPA_OK) return st;
     }
-    return launch_grouped_gemm(ops, n_ops, cx.stream);
+    return launch_grouped_gemm(ops, n_ops, cx.stream, side);
 }
 
-// Column sums of up to three bf16 matrices with the same row count.  colsum_plan takes the scratch of the chunk
-// partials from the workspace (so that a short workspace is reported before anything is launched) and returns the
-// description that colsum_begin (launch of the chunk-partial kernel) and the finishing launch need.  A null output
-// skips that matrix.
-ColsumParams colsum_plan(Ctx& cx, const Stored& M1, void* out1, const Stored& M2 = Stored(), void* out2 = nullptr,
-                         const Stored& M3 = Stored(), void* out3 = nullptr) {
-    ColsumParams P = {};
-    if (cx.st != ECOSPA_OK) return P;
-    const Stored* mats[3] = {&M1, &M2, &M3};
-    void* outs[3] = {out1, out2, out3};
-    for (int i = 0; i < 3; ++i) {
-        if (!outs[i] || !mats[i]->ptr) continue;
-        ColsumJob& J = P.job[P.n_jobs++];
-        J.M = static_cast<const uint16_t*>(mats[i]->ptr);
-        J.out = outs[i];
-        J.ld = mats[i]->ld;
-        J.cols = mats[i]->cols;
-        J.col_tiles = static_cast<int32_t>(ceil_div(J.cols, kSumCols));
-        J.vec_ok = aligned16(J.M) && J.ld % 8 == 0;
-        P.rows = mats[i]->rows;
+// Asks for the column sums of a bf16 matrix: `side` describes the reading (done by a product launch, which must not be the one
+// that writes the matrix), `fin` what the finishing launch adds up.  All matrices of a call have the same row count.  The
+// scratch of the chunk partials comes from the workspace here, so that a short workspace is reported before anything is
+// launched.  A null output skips the matrix.
+void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, void* out) {
+    if (cx.st != ECOSPA_OK || !out || !M.ptr) return;
+    const int chunks = static_cast<int>(ceil_div(M.rows, kSumRows));
+    float* partial = static_cast<float*>(cx.arena.take(static_cast<size_t>(chunks) * M.cols * 4));
+    if (!partial) {
+        cx.st = ECOSPA_ERR_WORKSPACE;
+        return;
     }
-    if (P.n_jobs == 0) return P;
-    P.chunks = static_cast<int32_t>(ceil_div(P.rows, kSumRows));
-    P.out_f32 = cx.dtype == ECOSPA_F32;
-    for (int i = 0; i < P.n_jobs; ++i) {
-        P.job[i].partial = static_cast<float*>(cx.arena.take(static_cast<size_t>(P.chunks) * P.job[i].cols * 4));
-        if (!P.job[i].partial) {
-            cx.st = ECOSPA_ERR_WORKSPACE;
-            P.n_jobs = 0;
-            return P;
-        }
-    }
-    return P;
-}
-const ColsumParams& colsum_begin(Ctx& cx, const ColsumParams& P) {
-    if (cx.st != ECOSPA_OK || P.n_jobs == 0) return P;
-    int tiles = 0;
-    for (int i = 0; i < P.n_jobs; ++i) tiles += P.job[i].col_tiles;
-    cx.st = launch_pdl(colsum_partial_kernel, dim3(tiles, P.chunks), kThreads, cx.stream, P, "colsum_partial_kernel");
-    return P;
+    const int i = side.n_jobs++;
+    side.M[i] = static_cast<const uint16_t*>(M.ptr);
+    side.partial[i] = partial;
+    side.ld[i] = M.ld;
+    side.cols[i] = static_cast<int32_t>(M.cols);
+    side.col_tiles[i] = static_cast<int32_t>(ceil_div(M.cols, 64));
+    side.vec_ok[i] = aligned16(M.ptr) && M.ld % 8 == 0;
+    side.rows = M.rows;
+    side.chunks = fin.chunks = chunks;
+    fin.job[fin.n_jobs++] = ColsumFinal{partial, out, M.cols};
 }
 
 // Compacted weight with n real shared indices, as stored: shared-cols d_m x n, or shared-rows n x d_m.  Either
@@ -589,10 +505,13 @@ extern "C" ecospa_status_t ecospa_coupled_qk_bwd(const void* X, int64_t ldx, int
         dx.seg[1].a = dKs; dx.seg[1].b[0] = Wk; dx.seg[1].b_mn = mn_over_shared(wk_c); dx.seg[1].K = n;
     }
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
-    const ColsumParams cs = colsum_plan(cx, dQs, dbq_c, dKs, wk_c ? dbk_c : nullptr);
+    SideSums side = {};
+    ColsumParams cs = {};
+    want_colsum(cx, side, cs, dQs, dbq_c);
+    want_colsum(cx, side, cs, dKs, wk_c ? dbk_c : nullptr);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
-    finish(cx, red, 2, colsum_begin(cx, cs));
+    if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
+    finish(cx, red, 2, cs);
     return cx.st;
 }
 
@@ -661,10 +580,13 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd(const void* X, int64_t ldx, con
     dx.M = T; dx.N = d_m; dx.n_kseg = 1;
     dx.seg[0].a = dVs; dx.seg[0].b[0] = Wv; dx.seg[0].b_mn = mn_over_shared(wv_c); dx.seg[0].K = n;
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
-    const ColsumParams cs = colsum_plan(cx, dVs, dbv_c, dOs, dbo);
+    SideSums side = {};
+    ColsumParams cs = {};
+    want_colsum(cx, side, cs, dVs, dbv_c);
+    want_colsum(cx, side, cs, dOs, dbo);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
-    finish(cx, red, 2, colsum_begin(cx, cs));
+    if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
+    finish(cx, red, 2, cs);
     return cx.st;
 }
 
@@ -730,10 +652,14 @@ extern "C" ecospa_status_t ecospa_coupled_qkv_bwd(const void* X, int64_t ldx, in
     dx.seg[1].a = dKs; dx.seg[1].b[0] = Wk; dx.seg[1].b_mn = mn_over_shared(wk_c); dx.seg[1].K = n_qk;
     dx.seg[2].a = dVs; dx.seg[2].b[0] = Wv; dx.seg[2].b_mn = mn_over_shared(wv_c); dx.seg[2].K = n_vo;
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = cx.dtype == ECOSPA_F32; dx.accumulate = accumulate_dX != 0;
-    const ColsumParams cs = colsum_plan(cx, dQs, dbq_c, dKs, dbk_c, dVs, dbv_c);
+    SideSums side = {};
+    ColsumParams cs = {};
+    want_colsum(cx, side, cs, dQs, dbq_c);
+    want_colsum(cx, side, cs, dKs, dbk_c);
+    want_colsum(cx, side, cs, dVs, dbv_c);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
-    finish(cx, red, 3, colsum_begin(cx, cs));
+    if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
+    finish(cx, red, 3, cs);
     return cx.st;
 }
 
@@ -761,10 +687,12 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd_o(const void* Ctxm, int64_t ld_
     dc.M = T; dc.N = n; dc.n_kseg = 1;
     dc.seg[0].a = dOs; dc.seg[0].b[0] = Wo; dc.seg[0].b_mn = mn_over_other(wo_c); dc.seg[0].K = d_m;
     dc.epi = EPI_STORE; dc.C = dCtx; dc.ldc = ld_dctx; dc.out_f32 = cx.dtype == ECOSPA_F32;
-    const ColsumParams cs = colsum_plan(cx, dOs, dbo);
+    SideSums side = {};
+    ColsumParams cs = {};
+    want_colsum(cx, side, cs, dOs, dbo);
     if (cx.st != ECOSPA_OK) return cx.st;
-    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
-    finish(cx, &red, 1, colsum_begin(cx, cs));
+    if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
+    finish(cx, &red, 1, cs);
     return cx.st;
 }
 
@@ -883,11 +811,14 @@ extern "C" ecospa_status_t ecospa_coupled_ffn_bwd(const void* X, int64_t ldx, in
         dx.seg[1].a = dHb; dx.seg[1].b[0] = W1b; dx.seg[1].b_mn = mn_over_shared(w1b_c); dx.seg[1].K = k;
     }
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32;
-    const ColsumParams cs = colsum_plan(cx, dYs, db2, dH, sw ? nullptr : db1_c);
+    SideSums side1 = {}, side2 = {};                       // db_2 = column sums of dY; db_1 = those of dH, which the first launch writes
+    ColsumParams cs = {};
+    want_colsum(cx, side1, cs, dYs, db2);
+    want_colsum(cx, side2, cs, dH, sw ? nullptr : db1_c);
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = validate_gemm_ops(ops, n_ops)) != ECOSPA_OK || (st = validate_gemm_ops(ops2, n_ops2)) != ECOSPA_OK) return st;
-    if ((st = run_ops(cx, ops, n_ops)) != ECOSPA_OK) return st;
-    if ((st = run_ops(cx, ops2, n_ops2)) != ECOSPA_OK) return st;
-    finish(cx, red, 3, colsum_begin(cx, cs));
+    if ((st = run_ops(cx, ops, n_ops, &side1)) != ECOSPA_OK) return st;
+    if ((st = run_ops(cx, ops2, n_ops2, &side2)) != ECOSPA_OK) return st;
+    finish(cx, red, 3, cs);
     return cx.st;
 }
