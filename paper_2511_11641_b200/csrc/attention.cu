@@ -8,8 +8,8 @@
 // Q K^T, and a zero column of V^c gives a zero column of Ctx) and off_h a multiple of 8, so that every tile load starts
 // on a 16-byte boundary and every contraction is a whole number of 16-deep MMA steps.
 //
-// Two forward kernels, one CTA per SM.  Output heads up to 32 wide (with Q/K heads up to 64) take the kernel of
-// independent key streams further down (attn_fwd_ms_kernel); wider heads take the kernel described here, 320 threads.
+// Two forward kernels, one CTA per SM.  Heads up to 64 wide take the kernel of independent key streams further down
+// (attn_fwd_ms_kernel); wider heads take the kernel described here, 320 threads.
 // A work item is (sequence b, head h, two neighbouring tiles of 128 query rows); a CTA walks a static list of items
 // (for causal attention the long ones first).  The two query tiles are two streams that share the K / V tiles and run
 // half a step apart.
@@ -89,23 +89,21 @@ __device__ __forceinline__ Item decode_item(int it, int n_qt, int n_heads, int b
     return I;
 }
 
-template <int NB>   // 64-column blocks per tile: 1 (every head at most 64 wide) or 2
 struct FwdCfg {
+    static constexpr int NB = 2;                                    // 64-column blocks per tile
     static constexpr int kTileBytes = NB * kBlockBytes;
-    static constexpr int QS = NB == 1 ? 2 : 1;                     // buffers of the pair of Q tiles
+    static constexpr int QS = 1;                                    // buffers of the pair of Q tiles
     static constexpr int kSmem = (2 * QS + 4) * kTileBytes + 1024 + 256;
     static constexpr int kOCols = NB * 64;                          // columns of an output tile
-    static constexpr int CH = NB == 1 ? 32 : 16;                    // score columns a thread holds at a time (two such buffers)
-    // TMEM columns of stream x: scores, output tile, probabilities (narrow heads: a region of their own, so that the
-    // next score tile never waits for the second product; wide heads: over the scores they were made from)
+    static constexpr int CH = 16;                                   // score columns a thread holds at a time (two such buffers)
+    // TMEM columns of stream x: scores, output tile, probabilities (over the scores they were made from)
     static __device__ __forceinline__ uint32_t col_s(uint32_t x) { return 128u * x; }
     static __device__ __forceinline__ uint32_t col_o(uint32_t x) { return 256u + kOCols * x; }
-    static __device__ __forceinline__ uint32_t col_p(uint32_t x) { return NB == 1 ? 384u + 64u * x : 128u * x; }
+    static __device__ __forceinline__ uint32_t col_p(uint32_t x) { return 128u * x; }
 };
 
-template <int NB>
 __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_constant__ AttnFwdParams P) {
-    using Cfg = FwdCfg<NB>;
+    using Cfg = FwdCfg;
     constexpr int kTileBytes = Cfg::kTileBytes;
     constexpr int QS = Cfg::QS;
     extern __shared__ uint8_t smem_raw[];
@@ -1516,11 +1514,13 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     int* status = engine_status_ptr(&st);
     if (!status) return st;
     const int64_t T = batch * seq;
-    // output heads up to 32 wide (and Q/K heads up to 64): the stream kernel (K / V tiles as slices of 64 keys); wider
-    // heads: two query tiles per CTA, with one or two 64-column blocks per tile
+    // heads up to 64 wide: the stream kernel (K / V tiles as slices of 64 keys), with three streams while the output heads
+    // are at most 32 wide and the two that fit the tensor memory beyond (against two query tiles per CTA with two passes over
+    // the scores, the form of the wide heads: 10.7 -> 7.5 us at 2 x 160 positions, 12 heads; 67.7 -> 64.9 at 4 x 1000, 32
+    // heads); wider heads: two query tiles per CTA
     int max_vo = 0;
     for (int h = 0; h < heads->n_heads; ++h) max_vo = std::max<int>(max_vo, heads->vo_w[h]);
-    const bool streams = max_w <= 64 && max_vo <= 32;
+    const bool streams = max_w <= 64;
     if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk)) != ECOSPA_OK) return st;
     if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk, streams ? 64 : kTile)) != ECOSPA_OK) return st;
     if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v, streams ? 64 : kTile)) != ECOSPA_OK) return st;
@@ -1543,9 +1543,9 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     cudaGetDevice(&dev);
     cudaError_t e = cudaSuccess;
     std::call_once(once[dev & 63], [&] {
-        e = cudaFuncSetAttribute(attn_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<1>::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<2>::kSmem);
+        e = cudaFuncSetAttribute(attn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<2, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<2, 64>::kSmem);
     });
     if (e != cudaSuccess) {
         set_cuda_error(e, "attention setup");
@@ -1554,9 +1554,9 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     }
     const int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (streams) attn_fwd_ms_kernel<3, 32><<<grid, MsCfg<3, 32>::kThreads, MsCfg<3, 32>::kSmem, cs>>>(P);
-    else if (max_w <= 64) attn_fwd_kernel<1><<<grid, kFwdThreads, FwdCfg<1>::kSmem, cs>>>(P);
-    else attn_fwd_kernel<2><<<grid, kFwdThreads, FwdCfg<2>::kSmem, cs>>>(P);
+    if (streams && max_vo <= 32) attn_fwd_ms_kernel<3, 32><<<grid, MsCfg<3, 32>::kThreads, MsCfg<3, 32>::kSmem, cs>>>(P);
+    else if (streams) attn_fwd_ms_kernel<2, 64><<<grid, MsCfg<2, 64>::kThreads, MsCfg<2, 64>::kSmem, cs>>>(P);
+    else attn_fwd_kernel<<<grid, kFwdThreads, FwdCfg::kSmem, cs>>>(P);
     return check_launch("attn_fwd_kernel");
 }
 
