@@ -159,11 +159,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         prefetch_tensormap(&P.map_k);
         prefetch_tensormap(&P.map_v);
     }
+    pdl_start();
     if (warp == 1) tmem_alloc(smem_u32(tmem_holder), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
@@ -539,11 +541,13 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
         prefetch_tensormap(&P.map_k);
         prefetch_tensormap(&P.map_v);
     }
+    pdl_start();
     if (warp == 0) tmem_alloc(smem_u32(tmem_holder), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();
 
     if (warp < NS) {
         // ------------------------------------------------------------------ loader and MMA issuer of stream x
@@ -881,9 +885,14 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
 // owns key blocks (dK and dV accumulate in TMEM over the query blocks) and one that owns query blocks (dQ accumulates
 // over the key blocks).  Nothing is added across CTAs, so the results do not depend on timing.
 
-// D[h][t] for every head: a warp takes a row, every lane multiplies 16-byte vectors (8 columns, which never straddle a
-// head because offsets and widths are multiples of 8), and the per-vector partial sums are added per head in order.
-constexpr int kDotWarps = 4;
+// A block takes kDotPos neighbouring positions of the padded sequences, a warp two of them at a time: every lane multiplies
+// 16-byte vectors (8 columns, which never straddle a head because offsets and widths are multiples of 8), and the per-vector
+// partial sums are added per head in order.  The row dots D_t = sum_c dCtx[t, c] Ctx[t, c] and the log-sum-exp in the form the
+// backward kernels use are written in a layout whose 128-position blocks are whole, 512-byte aligned runs (so that a block's
+// vectors can be copied to shared memory in bulk).  The head-major reads of the log-sum-exp and the
+// writes go through whole 64-byte runs of positions.  (A warp per position touched a 32-byte sector for every 4-byte value;
+// from the previous kernel's end to this one's 9.6 us at 8192 positions, 512 columns, launched on its own; now 5.7.)
+constexpr int kDotWarps = 8, kDotPos = 2 * kDotWarps;
 constexpr int kDotMaxVecs = 2048;      // 16384 columns
 struct DotParams {
     HeadLayout heads;
@@ -894,48 +903,62 @@ struct DotParams {
     int64_t ld_ctx, ld_dctx, T;
     int32_t n_heads, n_vecs, batch, seq, seq_pad;
 };
-// One warp per position of the padded sequences: the per-head row dots D_t = sum_c dCtx[t, c] Ctx[t, c] and the
-// log-sum-exp in the form the backward kernels use, in a layout whose 128-position blocks are whole, 512-byte aligned
-// runs (so that a block's vectors can be copied to shared memory in bulk).
+inline size_t dot_smem(int n_vecs, int n_heads) { return (static_cast<size_t>(kDotWarps) * 2 * n_vecs + static_cast<size_t>(n_heads) * (kDotPos + 1)) * 4; }
+__device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
+    float s = bf16_lo(x.x) * bf16_lo(y.x);
+    s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
+    s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s);
+    s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
+    s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s);
+    s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
+    s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s);
+    return fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
+}
 __global__ void __launch_bounds__(32 * kDotWarps) attn_rowdot_kernel(const __grid_constant__ DotParams P) {
-    __shared__ float part[kDotWarps][kDotMaxVecs];
+    extern __shared__ float dot_smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t tp = static_cast<int64_t>(blockIdx.x) * kDotWarps + warp;      // position in the padded layout
-    if (tp >= static_cast<int64_t>(P.batch) * P.seq_pad) return;
-    const int b = static_cast<int>(tp / P.seq_pad), pos = static_cast<int>(tp % P.seq_pad);
-    const int64_t per_arr = static_cast<int64_t>(P.n_heads) * P.batch * P.seq_pad;
-    if (pos >= P.seq) {
-        for (int h = lane; h < P.n_heads; h += 32) {
-            const int64_t o = (static_cast<int64_t>(h) * P.batch + b) * P.seq_pad + pos;
-            P.vecs[o] = 0.f;
-            P.vecs[per_arr + o] = 0.f;
+    float* part = dot_smem_raw + warp * 2 * P.n_vecs;                 // [position][vector] of this warp
+    float* dots = dot_smem_raw + kDotWarps * 2 * P.n_vecs;            // [head][kDotPos + 1]
+    const int64_t tp = static_cast<int64_t>(blockIdx.x) * kDotPos;    // (whole blocks: the padded length is a multiple of 128)
+    const int b = static_cast<int>(tp / P.seq_pad), pos0 = static_cast<int>(tp % P.seq_pad);
+    pdl_start();
+    pdl_wait();
+    const int p0 = pos0 + 2 * warp;                                   // positions p0 and p0 + 1
+    if (p0 < P.seq) {
+        const int64_t t0 = static_cast<int64_t>(b) * P.seq + p0, t1 = static_cast<int64_t>(b) * P.seq + min(p0 + 1, P.seq - 1);
+        const uint16_t* a0 = P.ctx + t0 * P.ld_ctx;
+        const uint16_t* a1 = P.ctx + t1 * P.ld_ctx;
+        const uint16_t* d0 = P.dctx + t0 * P.ld_dctx;
+        const uint16_t* d1 = P.dctx + t1 * P.ld_dctx;
+#pragma unroll 1
+        for (int v = lane; v < P.n_vecs; v += 64) {                   // eight loads in flight
+            const int v1 = min(v + 32, P.n_vecs - 1);                 // (past the end: the last vector again)
+            const uint4 x0 = ld_stream16(a0 + 8 * v), y0 = ld_stream16(d0 + 8 * v), x1 = ld_stream16(a1 + 8 * v), y1 = ld_stream16(d1 + 8 * v);
+            const uint4 x2 = ld_stream16(a0 + 8 * v1), y2 = ld_stream16(d0 + 8 * v1), x3 = ld_stream16(a1 + 8 * v1), y3 = ld_stream16(d1 + 8 * v1);
+            part[v] = dot8(x0, y0);
+            part[P.n_vecs + v] = dot8(x1, y1);
+            if (v + 32 < P.n_vecs) {
+                part[v + 32] = dot8(x2, y2);
+                part[P.n_vecs + v + 32] = dot8(x3, y3);
+            }
         }
-        return;
+        __syncwarp();
+        for (int i = lane; i < 2 * P.n_heads; i += 32) {
+            const int h = i >> 1, p = i & 1;
+            const int v0 = P.heads.vo_off[h] >> 3, nv = P.heads.vo_w[h] >> 3;
+            float s = 0.f;
+            for (int k = 0; k < nv; ++k) s += part[p * P.n_vecs + v0 + k];
+            dots[h * (kDotPos + 1) + 2 * warp + p] = s;
+        }
     }
-    const int64_t t = static_cast<int64_t>(b) * P.seq + pos;
-    const uint16_t* a = P.ctx + t * P.ld_ctx;
-    const uint16_t* bb = P.dctx + t * P.ld_dctx;
-    for (int v = lane; v < P.n_vecs; v += 32) {
-        const uint4 x = *reinterpret_cast<const uint4*>(a + 8 * v);
-        const uint4 y = *reinterpret_cast<const uint4*>(bb + 8 * v);
-        float s = bf16_lo(x.x) * bf16_lo(y.x);
-        s = fmaf(bf16_hi(x.x), bf16_hi(y.x), s);
-        s = fmaf(bf16_lo(x.y), bf16_lo(y.y), s);
-        s = fmaf(bf16_hi(x.y), bf16_hi(y.y), s);
-        s = fmaf(bf16_lo(x.z), bf16_lo(y.z), s);
-        s = fmaf(bf16_hi(x.z), bf16_hi(y.z), s);
-        s = fmaf(bf16_lo(x.w), bf16_lo(y.w), s);
-        s = fmaf(bf16_hi(x.w), bf16_hi(y.w), s);
-        part[warp][v] = s;
-    }
-    __syncwarp();
-    for (int h = lane; h < P.n_heads; h += 32) {
-        const int v0 = P.heads.vo_off[h] >> 3, nv = P.heads.vo_w[h] >> 3;
-        float s = 0.f;
-        for (int i = 0; i < nv; ++i) s += part[warp][v0 + i];
+    __syncthreads();
+    const int64_t per_arr = static_cast<int64_t>(P.n_heads) * P.batch * P.seq_pad;
+    for (int i = threadIdx.x; i < P.n_heads * kDotPos; i += 32 * kDotWarps) {
+        const int h = i / kDotPos, p = i % kDotPos, pos = pos0 + p;
         const int64_t o = (static_cast<int64_t>(h) * P.batch + b) * P.seq_pad + pos;
-        P.vecs[o] = -P.lse[static_cast<int64_t>(h) * P.T + t] * 1.4426950408889634f;
-        P.vecs[per_arr + o] = s;
+        const bool live = pos < P.seq;
+        P.vecs[o] = live ? -P.lse[static_cast<int64_t>(h) * P.T + static_cast<int64_t>(b) * P.seq + pos] * 1.4426950408889634f : 0.f;
+        P.vecs[per_arr + o] = live ? dots[h * (kDotPos + 1) + p] : 0.f;
     }
 }
 
@@ -1065,11 +1088,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         prefetch_tensormap(&P.map_v);
         prefetch_tensormap(&P.map_do);
     }
+    pdl_start();
     if (warp == 1) tmem_alloc(smem_u32(tmem_holder), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
+    pdl_wait();
 
     // item -> (sequence, head, owned block, steps, first streamed block).  MODE 0 owns a key block of a K/V head and
     // walks the query blocks of every query head that reads it, one head after the other (h = the first of them).
@@ -1561,10 +1586,9 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     }
     const int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (streams && max_vo <= 32) attn_fwd_ms_kernel<3, 32><<<grid, MsCfg<3, 32>::kThreads, MsCfg<3, 32>::kSmem, cs>>>(P);
-    else if (streams) attn_fwd_ms_kernel<2, 64><<<grid, MsCfg<2, 64>::kThreads, MsCfg<2, 64>::kSmem, cs>>>(P);
-    else attn_fwd_kernel<<<grid, kFwdThreads, FwdCfg::kSmem, cs>>>(P);
-    return check_launch("attn_fwd_kernel");
+    if (streams && max_vo <= 32) return launch_pdl(attn_fwd_ms_kernel<3, 32>, grid, MsCfg<3, 32>::kThreads, cs, P, "attn_fwd_kernel", MsCfg<3, 32>::kSmem);
+    if (streams) return launch_pdl(attn_fwd_ms_kernel<2, 64>, grid, MsCfg<2, 64>::kThreads, cs, P, "attn_fwd_kernel", MsCfg<2, 64>::kSmem);
+    return launch_pdl(attn_fwd_kernel, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg::kSmem);
 }
 
 extern "C" size_t ecospa_attn_workspace_bytes(int64_t batch, int64_t seq, int32_t n_heads) {
@@ -1636,6 +1660,8 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 0>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 1>::kSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(attn_rowdot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem(kDotMaxVecs, kMaxHeads)));
     });
     if (e != cudaSuccess) {
         set_cuda_error(e, "attention backward setup");
@@ -1656,27 +1682,28 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
     D.T = T;
     D.n_heads = heads->n_heads;
     D.n_vecs = static_cast<int32_t>(n_vo / 8);
-    attn_rowdot_kernel<<<static_cast<unsigned>(ceil_div(batch * D.seq_pad, static_cast<int64_t>(kDotWarps))), 32 * kDotWarps, 0, stream>>>(D);
-    if ((st = check_launch("attn_rowdot_kernel")) != ECOSPA_OK) return st;
+    if ((st = launch_pdl(attn_rowdot_kernel, static_cast<unsigned>(batch * D.seq_pad / kDotPos), 32 * kDotWarps, stream, D, "attn_rowdot_kernel",
+                         dot_smem(D.n_vecs, D.n_heads))) != ECOSPA_OK)
+        return st;
     const int nb = max_w > 64 ? 2 : 1;
     // dK, dV: one item per (sequence, K/V head, key block); dQ: one per (sequence, query head, query block)
     const int items_q = P.n_items;
     P.n_items = items_q / P.heads.rep;
     int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     if (nb == 1) {
-        if (max_w <= 32) attn_bwd_kernel<1, 0, 2><<<grid, kBwdThreads, BwdCfg<1, 0>::kSmem, stream>>>(P);
-        else attn_bwd_kernel<1, 0><<<grid, kBwdThreads, BwdCfg<1, 0>::kSmem, stream>>>(P);
+        st = launch_pdl(max_w <= 32 ? attn_bwd_kernel<1, 0, 2> : attn_bwd_kernel<1, 0, 1>, grid, kBwdThreads, stream, P,
+                        "attn_bwd_kernel (dK, dV)", BwdCfg<1, 0>::kSmem);
     } else {   // wide heads: the streamed query blocks are half blocks
         AttnBwdParams P0 = P;
         if ((st = encode_tile_map(&P0.map_q, Qc, T, n_qk, ld_qk, BwdCfg<2, 0>::kStep)) != ECOSPA_OK) return st;
         if ((st = encode_tile_map(&P0.map_do, dCtx, T, n_vo, ld_dctx, BwdCfg<2, 0>::kStep)) != ECOSPA_OK) return st;
-        attn_bwd_kernel<2, 0><<<grid, kBwdThreads, BwdCfg<2, 0>::kSmem, stream>>>(P0);
+        st = launch_pdl(attn_bwd_kernel<2, 0, 1>, grid, kBwdThreads, stream, P0, "attn_bwd_kernel (dK, dV)", BwdCfg<2, 0>::kSmem);
     }
-    if ((st = check_launch("attn_bwd_kernel (dK, dV)")) != ECOSPA_OK) return st;
+    if (st != ECOSPA_OK) return st;
     P.n_items = items_q;
     grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
-    if (nb == 1 && max_w <= 32) attn_bwd_kernel<1, 1, 2><<<grid, kBwdThreads, BwdCfg<1, 1>::kSmem, stream>>>(P);
-    else if (nb == 1) attn_bwd_kernel<1, 1><<<grid, kBwdThreads, BwdCfg<1, 1>::kSmem, stream>>>(P);
-    else attn_bwd_kernel<2, 1><<<grid, kBwdThreads, BwdCfg<2, 1>::kSmem, stream>>>(P);
-    return check_launch("attn_bwd_kernel (dQ)");
+    if (nb == 1)
+        return launch_pdl(max_w <= 32 ? attn_bwd_kernel<1, 1, 2> : attn_bwd_kernel<1, 1, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)",
+                          BwdCfg<1, 1>::kSmem);
+    return launch_pdl(attn_bwd_kernel<2, 1, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)", BwdCfg<2, 1>::kSmem);
 }
