@@ -671,29 +671,28 @@ struct AttnBwdParams {
 // Heads up to 64 wide (NB = 1): warp 1 issues the score products; warps 18 and 19 the accumulating ones: dV and dK in the
 // key-block kernel, the two halves of the contraction of dQ (into two accumulators that are added at the end) in the
 // query-block kernel; their A operands go through TMEM as packed bf16; three stages of streamed tiles.
-// Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products, whose A operands go through shared
-// memory; the key-block kernel takes the queries 64 at a time (three stages of half-size tiles, two buffers of score
-// tiles and of operands), the query-block kernel has two stages.
+// Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products.  The accumulators leave no TMEM columns
+// for P^T and dS^T beside the score tiles, so the key-block kernel takes the queries 64 at a time, in two buffers of score tiles,
+// and every thread writes its packed operands over the scores it has made them from; the buffer is free for the scores of the
+// step after next when the products that read the operands are done.  (Operands in shared memory, where they
+// take two writes and reads of 16 KB a step from the port that feeds the products: both kernels 1080 us at 2 x 4096 positions,
+// 32 heads 96 wide; now 950.)  The query-block kernel has one accumulator and two buffers of dS beside it.
 // Wait codes: 14 / 15 / 16 (MODE 0 loads, products, compute) and 17 / 18 / 19 (MODE 1).
 template <int NB, int MODE>
 struct BwdCfg {
     static constexpr int kTileBytes = NB * kBlockBytes;
-    // rows of a streamed block.  The key-block kernel on wide heads walks the queries in half blocks: its two wide
-    // accumulators fill the tensor memory beside the score tiles, so P^T and dS^T go through shared memory, and only with
-    // half-size streamed tiles and operands is there room for more than one stage
+    // rows of a streamed block: the key-block kernel on wide heads walks the queries in half blocks
     static constexpr int kStep = (NB == 2 && MODE == 0) ? 64 : kTile;
     static constexpr int kStrBlockBytes = kStep * 128;                         // 64 columns of a streamed block
     static constexpr int kStrTileBytes = NB * kStrBlockBytes;
     static constexpr int kResStages = NB == 1 ? 2 : 1;                         // buffers of the resident pair of tiles
-    // stages of the streamed pair of tiles.  Three where they fit (a fourth changes nothing): a stage is free again only when the accumulating
-    // products that read it are done, a whole step after the score products, and the next load must be under way by then
-    static constexpr int kStrStages = (NB == 1 || MODE == 0) ? 3 : 2;
-    static constexpr int kOutTileBytes = (kStep / 64) * kBlockBytes;            // 128 rows x kStep columns of bf16
-    static constexpr int kOutTiles = NB == 1 ? 0 : (MODE == 0 ? 2 : 1);        // P^T and dS^T, or dS (narrow heads: in TMEM)
-    static constexpr int kOutBufs = kStep == 64 ? 2 : 1;                       // half-block steps: room for two sets of them
+    // stages of the streamed pair of tiles, as many as fit up to four (a stage is free again only when the accumulating products
+    // that read it are done, a whole step after the score products, and the next load must be under way by then)
+    static constexpr int kStrStages = NB == 1 ? 3 : (MODE == 0 ? 4 : 2);
+    static constexpr bool kOverlay = NB == 2 && MODE == 0;                      // operands over the scores
+    static constexpr int kOutBufs = NB == 2 ? 2 : 1;                            // buffers of the packed operands
     static constexpr int kVecBytes = MODE == 0 ? kStrStages * 2 * kStep * 4 : 0;   // -lse2 and D of a query block, per streamed stage
-    static constexpr int kSmem = 2 * kTileBytes * kResStages + 2 * kStrTileBytes * kStrStages + kOutBufs * kOutTiles * kOutTileBytes +
-                                 kVecBytes + 1024 + 256;
+    static constexpr int kSmem = 2 * kTileBytes * kResStages + 2 * kStrTileBytes * kStrStages + kVecBytes + 1024 + 256;
     static_assert(kSmem <= 232448, "shared memory of a block");
 };
 
@@ -701,22 +700,26 @@ template <int NB, int MODE, int NACC = 1>   // NACC = 2: every head at most 32 w
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ AttnBwdParams P) {
     using Cfg = BwdCfg<NB, MODE>;
     constexpr int kTileBytes = Cfg::kTileBytes, kStrTileBytes = Cfg::kStrTileBytes, kStrBlockBytes = Cfg::kStrBlockBytes;
-    constexpr int kStep = Cfg::kStep, kOutTileBytes = Cfg::kOutTileBytes;
+    constexpr int kStep = Cfg::kStep;
     constexpr int RS = Cfg::kResStages, SS = Cfg::kStrStages;
-    // TMEM columns.  Heads up to 64 wide: the accumulators take 64 columns each and the bf16 operands of the
-    // accumulating products (P^T and dS^T, or dS) live in TMEM too, two values per column; wider heads: accumulators of
-    // 128 columns, those operands in shared memory.
-    constexpr bool kOpsInTmem = NB == 1;
+    // TMEM columns: score tiles X and Y, accumulators (64 columns each on heads up to 64 wide, else 128), packed bf16 operands of
+    // the accumulating products (P^T and dS^T, or dS), two values per column
     constexpr uint32_t kAccIssuers = NB == 1 ? 2 : 1, kScoreIssuers = NB == 1 ? 1 : 2;
-    constexpr uint32_t kColX = 0, kColY = 128, kColAcc1 = 256, kColAcc2 = kOpsInTmem ? 320 : 384, kColP = 384, kColDS = 448;
+    constexpr uint32_t kColX = 0, kColY = 128, kColAcc1 = 256, kColAcc2 = NB == 1 ? 320 : 384;
+    // operand `which` (0: P^T, 1: dS^T or dS) of 16 contraction steps from 16 ks on, in operand buffer ob
+    auto col_op = [](int which, uint32_t ob, uint32_t ks) -> uint32_t {
+        if (Cfg::kOverlay) return (which == 0 ? kColX : kColY) + 64 * ob + 16 * ks;
+        if (NB == 2) return 384 + 64 * ob + 8 * ks;
+        return (which == 0 ? 384 : 448) + 8 * ks;
+    };
     constexpr int kCodeBase = MODE == 0 ? 14 : 17;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw_addr);
-    // resident: [stage][a | b], streamed: [stage][a | b], out tiles, vectors, barriers
-    const uint32_t sRes = base, sStr = sRes + 2 * kTileBytes * RS, sOut = sStr + 2 * kStrTileBytes * SS;
-    uint8_t* vec_raw = smem + 2 * kTileBytes * RS + 2 * kStrTileBytes * SS + Cfg::kOutBufs * Cfg::kOutTiles * kOutTileBytes;
+    // resident: [stage][a | b], streamed: [stage][a | b], vectors, barriers
+    const uint32_t sRes = base, sStr = sRes + 2 * kTileBytes * RS;
+    uint8_t* vec_raw = smem + 2 * kTileBytes * RS + 2 * kStrTileBytes * SS;
     float* vec = reinterpret_cast<float*>(vec_raw);                               // [stage][-lse2 | D][128]
     uint8_t* tail = vec_raw + Cfg::kVecBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
@@ -732,7 +735,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     auto acc_empty = [&](uint32_t a) { return bar0 + 8u * (a ? 23 : 16); };
     constexpr uint32_t n_acc = NACC;
     static_assert(NACC == 1 || NB == 1, "two sets of accumulators need the narrow layout");
-    constexpr uint32_t kOB = Cfg::kOutBufs, kOutSetBytes = Cfg::kOutTiles * kOutTileBytes;
+    constexpr uint32_t kOB = Cfg::kOutBufs;
     auto out_full = [&](uint32_t b) { return bar0 + 8u * (b ? 20 : 13); };
     auto out_empty = [&](uint32_t b) { return bar0 + 8u * (b ? 21 : 14); };
     // score tiles: one buffer of 128 columns each, or (half-block steps) two of 64, each with its own pair of barriers
@@ -821,7 +824,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                            d_rb = make_smem_desc(sRes + (2 * rs + 1) * kTileBytes, 16, 1024);
             for (int i = 0; ok && i < I.n_steps; ++i, ++g) {
                 const uint32_t use = g / kXY, st = g % SS, xb = g % kXY;
-                if (use > 0 && !(ok = mbar_wait(xy_free(xb), (use - 1) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
+                if (use > 0 && !(ok = mbar_wait(Cfg::kOverlay ? out_empty(xb) : xy_free(xb), (use - 1) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 if (!(ok = mbar_wait(t_full(st), (g / SS) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 tc_fence_after();
                 const uint64_t d_sa = make_smem_desc(sStr + (2 * st) * kStrTileBytes, 16, 1024),
@@ -863,18 +866,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 for (int which = w0; which < w1; ++which) {
                     const int wn = (MODE == 0 && which == 0) ? P.heads.vo_w[I.h] : P.heads.qk_w[I.h];
                     const uint32_t idesc = make_idesc(kTile, wn, 0, 1);
-                    const uint32_t acc_col = (MODE == 0) == (which == 0) ? acc1 : acc2;
-                    const uint32_t a_col = (MODE == 0 && which == 0) ? kColP : kColDS;                 // narrow heads: A operand in TMEM
-                    const uint32_t sA = sOut + ob * kOutSetBytes + ((MODE == 0 && which == 1) ? kOutTileBytes : 0);   // wide heads: in shared memory
+                    constexpr bool kOneAcc = NB == 2 && MODE == 1;      // (one thread issues both halves of the contraction)
+                    const uint32_t acc_col = kOneAcc || (MODE == 0) == (which == 0) ? acc1 : acc2;
                     const int ks0 = MODE == 0 ? 0 : 4 * which, ks1 = MODE == 0 ? kStep / 16 : 4 * which + 4;
                     const uint64_t db = make_smem_desc(sStr + (2 * st + ((MODE == 0 && which == 0) ? 1 : 0)) * kStrTileBytes, kStrBlockBytes, 1024);
-                    for (int ks = ks0; ks < ks1; ++ks) {
-                        if (kOpsInTmem)
-                            tc_mma_bf16_ts(tmem_base + acc_col, tmem_base + a_col + 8 * ks, db + 128 * ks, idesc, (i != 0 || ks != ks0) ? 1u : 0u);
-                        else
-                            tc_mma_bf16(tmem_base + acc_col, make_smem_desc(sA + (ks >> 2) * kBlockBytes + (ks & 3) * 32, 16, 1024),
-                                        db + 128 * ks, idesc, (i != 0 || ks != ks0) ? 1u : 0u);
-                    }
+                    for (int ks = ks0; ks < ks1; ++ks)
+                        tc_mma_bf16_ts(tmem_base + acc_col, tmem_base + col_op(MODE == 0 ? which : 1, ob, ks), db + 128 * ks, idesc,
+                                       (i != 0 || ks != (kOneAcc ? 0 : ks0)) ? 1u : 0u);
                 }
                 tc_commit(out_empty(ob));
                 tc_commit(t_empty(st));
@@ -945,13 +943,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         constexpr int kHalves = kStep / 64;                            // 16-column halves of this thread's columns
         const int col0 = part * (kStep / 4);                           // this thread's columns of the streamed block
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        // 32 columns = four 16-byte chunks of block col0 / 64 of the row's image
-        const uint32_t out_row = sOut + (col0 >> 6) * kBlockBytes + row * 128;
-        const int chunk0 = (col0 & 63) >> 3;
-        const int swz = row & 7;
         uint32_t g = 0, ri = 0;
         bool ok = true;
-        const int64_t T = static_cast<int64_t>(P.batch) * P.seq;
         struct Pend {
             int h, b, own;
             uint32_t ri;
@@ -1002,7 +995,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 write_acc(acc1, P.heads.vo_w[d.h], P.dv + t * P.ld_dv + P.heads.v_off[d.h], 1.f);
                 write_acc(acc2, P.heads.qk_w[d.h], P.dk + t * P.ld_dqk + P.heads.k_off[d.h], P.scale);
             } else {
-                write_acc(acc2, P.heads.qk_w[d.h], P.dq + t * P.ld_dqk + P.heads.qk_off[d.h], P.scale, true, acc1);
+                write_acc(NB == 2 ? acc1 : acc2, P.heads.qk_w[d.h], P.dq + t * P.ld_dqk + P.heads.qk_off[d.h], P.scale, NB == 1, acc1);
             }
             tc_fence_before();
             __syncwarp();
@@ -1032,7 +1025,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 const int q0 = MODE == 0 ? other0 : I.own * kTile, k0 = MODE == 0 ? I.own * kTile : other0;
                 const bool masked = q0 + (MODE == 0 ? kStep : kTile) > P.seq || k0 + kTile > P.seq || (P.causal && q0 < k0 + kTile);
                 // two halves of 16 columns: probabilities and dS are packed to bf16 pairs as soon as they exist
-                uint32_t pk_p[16], pk_ds[16];
+                uint32_t pk_p[8 * kHalves], pk_ds[8 * kHalves];
                 const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), neg1 = pack2(-1.f, -1.f);
 #pragma unroll
                 for (int hh = 0; hh < kHalves; ++hh) {
@@ -1040,7 +1033,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     tc_ld16(t_lane + kColX + xb * kStep + col0 + 16 * hh, rx);
                     tc_ld16(t_lane + kColY + xb * kStep + col0 + 16 * hh, ry);
                     tc_wait_ld();
-                    if (hh == kHalves - 1) {                          // this thread's last read of the step's score tiles
+                    if (!Cfg::kOverlay && hh == kHalves - 1) {        // this thread's last read of the step's score tiles
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(xy_free(xb));
@@ -1078,25 +1071,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                         pk_ds[8 * hh + (e >> 1) + 1] = pack_bf16(d2, d3);
                     }
                 }
-                // the products that read the previous step's tiles from shared memory are done
+                // the products that read the operands last in this buffer are done (over the scores: the score products waited for that)
                 const uint32_t ob = g % kOB;
-                if (!(ok = mbar_wait(out_empty(ob), ((g / kOB) & 1u) ^ 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
-                if (kOpsInTmem) {   // this thread's 32 columns = 16 packed columns of its TMEM lane
-                    if (MODE == 0) tc_st(t_lane + kColP + 16 * part, pk_p);
-                    tc_st(t_lane + kColDS + 16 * part, pk_ds);
-                    tc_wait_st();
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 2 * kHalves; ++q) {
-                        const int chunk = chunk0 + q;
-                        if (MODE == 0)
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(out_row + ob * kOutSetBytes + ((chunk ^ swz) << 4)),
-                                         "r"(pk_p[4 * q + 0]), "r"(pk_p[4 * q + 1]), "r"(pk_p[4 * q + 2]), "r"(pk_p[4 * q + 3]) : "memory");
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(out_row + ob * kOutSetBytes + (MODE == 0 ? kOutTileBytes : 0) + ((chunk ^ swz) << 4)),
-                                     "r"(pk_ds[4 * q + 0]), "r"(pk_ds[4 * q + 1]), "r"(pk_ds[4 * q + 2]), "r"(pk_ds[4 * q + 3]) : "memory");
-                    }
-                    fence_async_smem();
-                }
+                if (!Cfg::kOverlay && !(ok = mbar_wait(out_empty(ob), ((g / kOB) & 1u) ^ 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
+                // this thread's columns, packed, in its TMEM lane
+                if (MODE == 0) tc_st(t_lane + col_op(0, ob, part * kHalves), pk_p);
+                tc_st(t_lane + col_op(1, ob, part * kHalves), pk_ds);
+                tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(out_full(ob));
