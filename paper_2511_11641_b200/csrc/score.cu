@@ -51,6 +51,11 @@ struct SumsqParams {
     SumsqJob jobs[CAP];
 };
 
+// What the scores of a pair are taken from: single indices, rotation pairs of indices, indices summed over grouped heads, or
+// single indices whose row-chunk partials have not been added yet.  A compile-time choice in the kernel, so that the loads of
+// an unrolled loop stand free of branches and go out together.
+enum : int { kSingle = 0, kRotation = 1, kGrouped = 2, kChunked = 3 };
+
 struct PairDesc {
     const float* c1;
     const float* c2;
@@ -63,8 +68,8 @@ struct PairDesc {
     int32_t blk_start;  // first block of this launch that is the pair's
     float inv_numel1, inv_numel2;
     int32_t rope;       // ecospa_rope_t: the scored unit is a rotation pair of shared indices
-    int16_t rep1, rep2; // heads stacked per segment on the W_1 / W_2 side (grouped-query attention); 1 = ordinary pair
-    int32_t pad_;
+    int16_t rep1, rep2; // kGrouped: heads stacked per segment on the W_1 / W_2 side; kChunked: row-chunk partials of a statistic
+    int32_t mode;       // how a statistic is read (kSingle ... kChunked)
 };
 static_assert(sizeof(PairDesc) == 80, "pair descriptor size");
 
@@ -278,26 +283,34 @@ constexpr int kFinWarps = kFinThreads / 32;
 constexpr int kNarrow = 256;
 constexpr int kFinPass = 22 * kFinThreads;        // scores of a wide segment that shared memory holds at a time
 
-// What the scores of a pair are taken from: single indices, rotation pairs of indices, or indices summed over grouped heads.
-// A compile-time choice, so that the loads of an unrolled loop stand free of branches and go out together.
-enum : int { kSingle = 0, kRotation = 1, kGrouped = 2 };
-
-// The statistic of index j of segment seg (grouped heads: over the `rep` heads that the segment stacks, in head order).
+// The statistic of index j of segment seg (grouped heads: over the `rep` heads that the segment stacks, in head order; chunked:
+// over its `rep` row chunks, D apart, in their order).
+constexpr int kMaxChunks = 4;
 template <int MODE>
-__device__ __forceinline__ float stat_of(const float* v, int rep, int64_t seg, int n, int j) {
+__device__ __forceinline__ float stat_of(const float* v, int rep, int64_t D, int64_t seg, int n, int j) {
+    if (MODE == kChunked) {
+        const float* p = v + seg * n + j;
+        float x[kMaxChunks], t = 0.f;
+#pragma unroll
+        for (int c = 0; c < kMaxChunks; ++c) x[c] = c < rep ? p[c * D] : 0.f;
+#pragma unroll
+        for (int c = 0; c < kMaxChunks; ++c) t += x[c];
+        return t;
+    }
     if (MODE != kGrouped) return v[seg * n + j];
     float t = 0.f;
     for (int r = 0; r < rep; ++r) t += v[(seg * rep + r) * n + j];
     return t;
 }
+__device__ __forceinline__ int64_t extent(const PairDesc& Q) { return static_cast<int64_t>(Q.n_seg) * Q.seg_len; }
 // The two sums of squares behind the raw score of index j: its own column's / row's, or those of its rotation pair (both
 // members get the pair's value; the pair is counted once in the normaliser).  raw = sqrt(x) * sqrt(y); kept apart from the
 // square roots, whose branches would hold back the loads of an unrolled loop.
 template <int MODE>
 __device__ __forceinline__ void norms_of(const PairDesc& Q, int64_t seg, int n, int j, float& x, float& y) {
     if (MODE != kRotation) {
-        x = stat_of<MODE>(Q.c1, Q.rep1, seg, n, j);
-        y = stat_of<MODE>(Q.c2, Q.rep2, seg, n, j);
+        x = stat_of<MODE>(Q.c1, Q.rep1, extent(Q), seg, n, j);
+        y = stat_of<MODE>(Q.c2, Q.rep2, extent(Q), seg, n, j);
         return;
     }
     const int half = n >> 1;
@@ -326,9 +339,9 @@ __device__ __forceinline__ void finalize_narrow(const FinalizeOut& P, const Pair
     for (int i = 0; i < TREES; ++i) {
         const int j = min(32 * i + lane, n - 1);          // (lanes past the end read the last index and add nothing)
         norms_of<MODE>(Q, seg, n, j, r[i], y[i]);
-        g1[i] = with_fisher ? stat_of<MODE>(Q.gs1, Q.rep1, seg, n, j) : 0.f;
-        g1b[i] = with_fisher && with_up ? Q.gs1b[static_cast<int64_t>(seg) * n + j] : 0.f;
-        g2[i] = with_fisher ? stat_of<MODE>(Q.gs2, Q.rep2, seg, n, j) : 0.f;
+        g1[i] = with_fisher ? stat_of<MODE>(Q.gs1, Q.rep1, extent(Q), seg, n, j) : 0.f;
+        g1b[i] = with_fisher && with_up ? stat_of<MODE>(Q.gs1b, Q.rep1, extent(Q), seg, n, j) : 0.f;
+        g2[i] = with_fisher ? stat_of<MODE>(Q.gs2, Q.rep2, extent(Q), seg, n, j) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < TREES; ++i) {
@@ -419,13 +432,13 @@ __device__ __forceinline__ void scores_wide(const FinalizeOut& P, const PairDesc
 }
 // Virtual thread vt's sum of a statistic.
 template <int MODE>
-__device__ __forceinline__ float virtual_sum(const float* v, int rep, int seg, int n, int vt) {
+__device__ __forceinline__ float virtual_sum(const float* v, int rep, int64_t D, int seg, int n, int vt) {
     float s = 0.f;
 #pragma unroll 1
     for (int j0 = vt; j0 < n; j0 += 8 * 256) {
         float x[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = stat_of<MODE>(v, rep, seg, n, min(j0 + 256 * i, n - 1));
+        for (int i = 0; i < 8; ++i) x[i] = stat_of<MODE>(v, rep, D, seg, n, min(j0 + 256 * i, n - 1));
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (j0 + 256 * i < n) s += x[i];
@@ -437,8 +450,8 @@ __device__ __forceinline__ void importance_wide(const FinalizeOut& P, const Pair
     // threads 0-255: W_1's sum, then the up projection's; threads 256-511: W_2's
     const int n = Q.seg_len, tid = threadIdx.x;
     const bool first = tid < 256;
-    const float s = virtual_sum<MODE>(first ? Q.gs1 : Q.gs2, first ? Q.rep1 : Q.rep2, seg, n, tid & 255);
-    const float s_up = first && Q.gs1b ? virtual_sum<kSingle>(Q.gs1b, 1, seg, n, tid) : 0.f;
+    const float s = virtual_sum<MODE>(first ? Q.gs1 : Q.gs2, first ? Q.rep1 : Q.rep2, extent(Q), seg, n, tid & 255);
+    const float s_up = first && Q.gs1b ? virtual_sum<MODE>(Q.gs1b, Q.rep1, extent(Q), seg, n, tid) : 0.f;
     const float a = end_wide_sum(s, 0, scratch);
     const float b = end_wide_sum(s, 256, scratch);
     const float ab = end_wide_sum(s_up, 0, scratch);
@@ -471,9 +484,14 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(const __grid_cons
     const PairDesc& Q = P.pairs[pi];
     const int local = blk - Q.blk_start;
     pdl_wait();
-    if (Q.rep1 > 1 || Q.rep2 > 1) finalize_pair<kGrouped>(P.out, Q, local, buf, scratch);
-    else if (Q.rope != ECOSPA_ROPE_NONE) finalize_pair<kRotation>(P.out, Q, local, buf, scratch);
-    else finalize_pair<kSingle>(P.out, Q, local, buf, scratch);
+    switch (Q.mode) {
+        case kSingle: finalize_pair<kSingle>(P.out, Q, local, buf, scratch); break;
+        case kRotation: finalize_pair<kRotation>(P.out, Q, local, buf, scratch); break;
+        case kGrouped: finalize_pair<kGrouped>(P.out, Q, local, buf, scratch); break;
+        case kChunked:
+            if (CAP == kFewPairs) finalize_pair<kChunked>(P.out, Q, local, buf, scratch);
+            break;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -490,7 +508,7 @@ struct StatPlan {        // one per-index statistic of one pair
 
 int chunks_for(const ecospa_mat_t& m) {
     if (m.layout != ECOSPA_SHARED_COLS) return 1;
-    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(4, m.other_dim / 64)));
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(kMaxChunks, m.other_dim / 64)));
 }
 
 ecospa_status_t validate_mat(const ecospa_mat_t& m, int64_t D, int want_dtype, int want_layout, int64_t want_other) {
@@ -611,6 +629,13 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
     if (workspace_bytes < need) return ECOSPA_ERR_WORKSPACE;
     float* ws = static_cast<float*>(workspace);
 
+    // A block or two of a model with segments of moderate width: the row-chunk partials are added by the finalisation itself,
+    // a launch less where launches are what such a call costs (one fp32 block: 28.2 -> 26.3 us a pass).  A wide segment would read four times as much
+    // through one block's loads.
+    bool fold = stats.size() <= kFewJobs && n_pairs <= kFewPairs;
+    for (int i = 0; i < n_pairs && fold; ++i)
+        fold = pairs[i].seg_len <= 4096 && pairs[i].rope == ECOSPA_ROPE_NONE && pairs[i].w1_rep <= 1 && pairs[i].w2_rep <= 1;
+
     // --- sumsq + reduce, in launches of at most kMaxJobs jobs
     static thread_local SumsqParams<kMaxJobs> sp;
     size_t si = 0;
@@ -646,6 +671,7 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             if (J.n_chunks > 1) red += static_cast<int>(ceil_div(J.D, kThreads));
         }
         sp.n_jobs = nj;
+        if (fold) red = 0;
         ecospa_status_t st;
         if (nj <= kFewJobs) {
             SumsqParams<kFewJobs> few;
@@ -671,12 +697,14 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             const bool sw = pr.kind == ECOSPA_PAIR_SWIGLU;
             PairDesc& Q = fp.pairs[np];
             Q = PairDesc{};
-            Q.c1 = ws + stats[stat_i++].stat_off;
-            Q.c2 = ws + stats[stat_i++].stat_off;
+            auto stat = [&]() { const StatPlan& t = stats[stat_i++]; return ws + (fold ? t.partial_off : t.stat_off); };
+            const int chunks1 = stats[stat_i].n_chunks, chunks2 = stats[stat_i + 1].n_chunks;   // (the gradients have their weight's)
+            Q.c1 = stat();
+            Q.c2 = stat();
             if (grads) {
-                Q.gs1 = ws + stats[stat_i++].stat_off;
-                if (sw) Q.gs1b = ws + stats[stat_i++].stat_off;
-                Q.gs2 = ws + stats[stat_i++].stat_off;
+                Q.gs1 = stat();
+                if (sw) Q.gs1b = stat();
+                Q.gs2 = stat();
             }
             Q.n_seg = pr.n_seg;
             Q.seg_len = pr.seg_len;
@@ -689,6 +717,12 @@ extern "C" ecospa_status_t ecospa_score_pairs(const ecospa_pair_t* pairs, int32_
             Q.rep2 = static_cast<int16_t>(std::max(1, pr.w2_rep));
             Q.inv_numel1 = static_cast<float>(1.0 / (static_cast<double>(pr.w1.other_dim) * pr.seg_len * Q.rep1));
             Q.inv_numel2 = static_cast<float>(1.0 / (static_cast<double>(pr.w2.other_dim) * pr.seg_len * Q.rep2));
+            Q.mode = Q.rep1 > 1 || Q.rep2 > 1 ? kGrouped : pr.rope != ECOSPA_ROPE_NONE ? kRotation : kSingle;
+            if (fold) {
+                Q.mode = kChunked;
+                Q.rep1 = static_cast<int16_t>(chunks1);
+                Q.rep2 = static_cast<int16_t>(chunks2);
+            }
             d_off += pr.n_seg * pr.seg_len;
             segs += pr.n_seg;
             seg_off += pr.n_seg;
