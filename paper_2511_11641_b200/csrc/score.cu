@@ -26,7 +26,8 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxJobs = 400, kFewJobs = 24;      // 72 B each
 constexpr int kMaxPairs = 256, kFewPairs = 16;    // 80 B each
 constexpr int kRowTile = 32;       // shared-rows tile: rows per CTA
-constexpr int kUnroll = 4;
+constexpr int kUnroll = 4;       // loads of a tensor in flight per thread
+constexpr int kProd = 4;         // ... of each factor of a product
 
 struct SumsqJob {
     const void* a;       // tensor
@@ -124,29 +125,42 @@ __device__ __forceinline__ void cols_tile(const SumsqJob& J, int local, float* s
             const char* pa = static_cast<const char*>(J.a) + static_cast<int64_t>(col) * EB;
             const char* pb = has_b ? static_cast<const char*>(J.b) + static_cast<int64_t>(col) * EB : nullptr;
             const int64_t sa = static_cast<int64_t>(J.lda) * EB, sb = static_cast<int64_t>(J.ldb) * EB;  // bytes per row
-            for (int r = r0 + warp; r < r1; r += kWarps * kUnroll) {
-                uint4 va[kUnroll], vb[kUnroll];
+            // (the sums do not depend on how many rows are fetched ahead)
+            if (!has_b) {
+                for (int r = r0 + warp; r < r1; r += kWarps * kUnroll) {
+                    uint4 va[kUnroll];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int rr = r + u * kWarps;
-                    va[u] = make_uint4(0, 0, 0, 0);
-                    vb[u] = make_uint4(0, 0, 0, 0);
-                    if (rr < r1) {
-                        va[u] = ldg_stream16(pa + rr * sa);
-                        if (has_b) vb[u] = ldg_stream16(pb + rr * sb);
+                    for (int u = 0; u < kUnroll; ++u) {
+                        const int rr = r + u * kWarps;
+                        va[u] = rr < r1 ? ldg_stream16(pa + rr * sa) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u) {
+                        float fa[V];
+                        TR::unpack(va[u], fa);
+#pragma unroll
+                        for (int e = 0; e < V; ++e) acc[e] = fmaf(fa[e], fa[e], acc[e]);
                     }
                 }
+            } else {
+                for (int r = r0 + warp; r < r1; r += kWarps * kProd) {
+                    uint4 va[kProd], vb[kProd];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    float fa[V], fb[V];
-                    TR::unpack(va[u], fa);
-                    if (has_b) {
+                    for (int u = 0; u < kProd; ++u) {
+                        const int rr = r + u * kWarps;
+                        va[u] = rr < r1 ? ldg_stream16(pa + rr * sa) : make_uint4(0, 0, 0, 0);
+                        vb[u] = rr < r1 ? ldg_stream16(pb + rr * sb) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kProd; ++u) {
+                        float fa[V], fb[V];
+                        TR::unpack(va[u], fa);
                         TR::unpack(vb[u], fb);
 #pragma unroll
                         for (int e = 0; e < V; ++e) fa[e] *= fb[e];
-                    }
 #pragma unroll
-                    for (int e = 0; e < V; ++e) acc[e] = fmaf(fa[e], fa[e], acc[e]);
+                        for (int e = 0; e < V; ++e) acc[e] = fmaf(fa[e], fa[e], acc[e]);
+                    }
                 }
             }
         } else {
@@ -196,29 +210,41 @@ __device__ __forceinline__ void rows_tile(const SumsqJob& J, int local) {
             const int nvec = J.other / V;
             const uint4* pa = reinterpret_cast<const uint4*>(static_cast<const char*>(J.a) + static_cast<int64_t>(j) * J.lda * (16 / V));
             const uint4* pb = has_b ? reinterpret_cast<const uint4*>(static_cast<const char*>(J.b) + static_cast<int64_t>(j) * J.ldb * (16 / V)) : nullptr;
-            for (int v = lane; v < nvec; v += 32 * kUnroll) {
-                uint4 va[kUnroll], vb[kUnroll];
+            if (!has_b) {
+                for (int v = lane; v < nvec; v += 32 * kUnroll) {
+                    uint4 va[kUnroll];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int vv = v + u * 32;
-                    va[u] = make_uint4(0, 0, 0, 0);
-                    vb[u] = make_uint4(0, 0, 0, 0);
-                    if (vv < nvec) {
-                        va[u] = ldg_stream16(pa + vv);
-                        if (has_b) vb[u] = ldg_stream16(pb + vv);
+                    for (int u = 0; u < kUnroll; ++u) {
+                        const int vv = v + u * 32;
+                        va[u] = vv < nvec ? ldg_stream16(pa + vv) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u) {
+                        float fa[V];
+                        TR::unpack(va[u], fa);
+#pragma unroll
+                        for (int e = 0; e < V; ++e) acc = fmaf(fa[e], fa[e], acc);
                     }
                 }
+            } else {
+                for (int v = lane; v < nvec; v += 32 * kProd) {
+                    uint4 va[kProd], vb[kProd];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    float fa[V], fb[V];
-                    TR::unpack(va[u], fa);
-                    if (has_b) {
+                    for (int u = 0; u < kProd; ++u) {
+                        const int vv = v + u * 32;
+                        va[u] = vv < nvec ? ldg_stream16(pa + vv) : make_uint4(0, 0, 0, 0);
+                        vb[u] = vv < nvec ? ldg_stream16(pb + vv) : make_uint4(0, 0, 0, 0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kProd; ++u) {
+                        float fa[V], fb[V];
+                        TR::unpack(va[u], fa);
                         TR::unpack(vb[u], fb);
 #pragma unroll
                         for (int e = 0; e < V; ++e) fa[e] *= fb[e];
-                    }
 #pragma unroll
-                    for (int e = 0; e < V; ++e) acc = fmaf(fa[e], fa[e], acc);
+                        for (int e = 0; e < V; ++e) acc = fmaf(fa[e], fa[e], acc);
+                    }
                 }
             }
             for (int i = nvec * V + lane; i < J.other; i += 32) {  // ragged tail of the row
@@ -238,8 +264,12 @@ __device__ __forceinline__ void rows_tile(const SumsqJob& J, int local) {
     }
 }
 
+// Bound by memory; every block starts with the search for its job, a microsecond or so in which it loads nothing, so what counts
+// beside the loads in flight per thread is how many blocks an SM holds: 64 registers and four blocks took 198 us on a 24-layer
+// GELU model (1.2 GB) and 661 on a 22-layer SwiGLU one (4.5 GB), 48 registers and five blocks take 178 and 632; six blocks with
+// half the loads of a product in flight 183 and 655.
 template <int CAP>
-__global__ void __launch_bounds__(kThreads) sumsq_kernel(const __grid_constant__ SumsqParams<CAP> P) {
+__global__ void __launch_bounds__(kThreads, 5) sumsq_kernel(const __grid_constant__ SumsqParams<CAP> P) {
     __shared__ float smem[kWarps * (256 + 4)];
     pdl_start();
     const int tile = blockIdx.x;
