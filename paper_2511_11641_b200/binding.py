@@ -92,11 +92,16 @@ def _dtype_code(t: torch.Tensor) -> int:
 # stays out of the interpreter: integer lists go through array.array, descriptor lists through one bytes.join (measured on
 # lists of a 24-layer model: 768 segments 0.67 -> 0.05 ms, 480 gather jobs 0.18 -> 0.026 ms).
 
-def _i32(v) -> array.array:
-    try:
-        return array.array("i", v)
-    except TypeError:                      # (values that are not integers by type)
-        return array.array("i", [int(x) for x in v])
+def _i32(v, n: Optional[int] = None) -> array.array:
+    """Integer list of n (default len(v)) elements, by the rules of a ctypes array: floats are refused, wider integers wrap,
+    a list that is too long is refused and one that is too short ends in zeros."""
+    n = len(v) if n is None else n
+    if len(v) == n:
+        try:
+            return array.array("i", v if isinstance(v, (list, tuple)) else iter(v))
+        except (TypeError, OverflowError):
+            pass
+    return array.array("i", (C.c_int32 * n)(*v))
 
 
 def _addr(a: array.array) -> int:
@@ -179,8 +184,7 @@ def ecospa_select_aligned_topk(upsilon: torch.Tensor, n_seg: Sequence[int], seg_
                                k_per_seg: Sequence[int], kept: torch.Tensor,
                                seg_offsets: Optional[torch.Tensor] = None, stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
-    assert len(a_slen) == n_pairs
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len, n_pairs)
     a_k = _i32(k_per_seg)
     assert len(k_per_seg) == sum(n_seg)
     assert kept.dtype == torch.int32 and kept.numel() >= sum(k_per_seg)
@@ -194,8 +198,7 @@ def ecospa_select_rotation_pairs(upsilon: torch.Tensor, n_seg: Sequence[int], se
                                  k_per_seg: Sequence[int], rope: Sequence[int], kept: torch.Tensor,
                                  seg_offsets: Optional[torch.Tensor] = None, stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
-    assert len(a_slen) == n_pairs
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len, n_pairs)
     a_rope = _i32(rope)
     a_k = _i32(k_per_seg)
     assert len(k_per_seg) == sum(n_seg) and len(rope) == n_pairs
@@ -232,10 +235,8 @@ def ecospa_select_aligned_threshold(upsilon: torch.Tensor, n_seg: Sequence[int],
                                     chosen: Optional[torch.Tensor] = None, rope: Optional[Sequence[int]] = None,
                                     stream=None) -> None:
     n_pairs = len(n_seg)
-    a_nseg, a_slen = _i32(n_seg), _i32(seg_len)
-    assert len(a_slen) == n_pairs
-    a_rope = _i32(rope) if rope is not None else None
-    assert a_rope is None or len(a_rope) == n_pairs
+    a_nseg, a_slen = _i32(n_seg), _i32(seg_len, n_pairs)
+    a_rope = _i32(rope, n_pairs) if rope is not None else None
     assert kept.dtype == torch.int32 and kept.numel() >= sum(a * b for a, b in zip(n_seg, seg_len))
     assert k_out.dtype == torch.int32 and k_out.numel() >= sum(n_seg)
     fn = _fn("ecospa_select_aligned_threshold")
@@ -583,7 +584,7 @@ def ecospa_pad_kept(kept: torch.Tensor, src: Sequence[int], dst: Sequence[int], 
                     k_padded: Sequence[int], out: torch.Tensor, stream=None) -> None:
     n = len(src)
     assert len(dst) == n and len(k) == n and len(k_padded) == n and kept.dtype == torch.int32 and out.dtype == torch.int32
-    a_src, a_dst, a_k, a_kp = _i32(src), _i32(dst), _i32(k), _i32(k_padded)
+    a_src, a_dst, a_k, a_kp = (_i32(list(map(int, v))) for v in (src, dst, k, k_padded))
     fn = _fn("ecospa_pad_kept")
     _check(fn(_ptr(kept), _addr(a_src), _addr(a_dst), _addr(a_k), _addr(a_kp), n, _ptr(out),
               _stream(stream)), "ecospa_pad_kept")
@@ -640,7 +641,7 @@ def ecospa_alg1_apply(groups: Sequence[Group], k: Sequence[int], out: Optional[S
                       in_place: bool = False, stream=None) -> None:
     arr = _structs(Group, groups)
     oarr = _structs(Group, out) if out is not None else None
-    ka = _i32(k)
+    ka = _i32(list(map(int, k)))
     f = _fn("ecospa_alg1_apply")
     _check(f(arr, len(groups), _addr(ka), oarr,
              int(bool(in_place)), workspace.data_ptr(), workspace.numel(), _stream(stream)), "ecospa_alg1_apply")

@@ -4,6 +4,7 @@ import ctypes as C
 import os
 import re
 
+import numpy as np
 import pytest
 
 from paper_2511_11641_b200 import binding as B
@@ -457,3 +458,19 @@ def test_attention_calls_reject_bad_arguments_without_launching(lib):
 
     assert g(good, ws=None) == 6 and g(good, ws_bytes=16) == 6 and g(good, ws=0x90004) == 2
     assert g(good, dq=None) == 1 and g(good, dctx=None) == 1 and g(good, ld_dqk=62) == 1 and g(good, ld_dv=68) == 2
+
+
+@pytest.mark.parametrize("v, n", [([3, 1, 2], None), ((3, 1), 4), (range(5), 5), (bytes([1, 200, 3]), None), ([True, False], 2),
+                                  ([2 ** 31, -2 ** 31 - 1, 2 ** 32 + 5], None), ([], None), ([], 2), (np.arange(4), 4)])
+def test_integer_lists_are_marshalled_as_ctypes_arrays_are(v, n):
+    want = list((C.c_int32 * (len(v) if n is None else n))(*v))
+    assert B._i32(v, n).tolist() == want
+
+
+@pytest.mark.parametrize("v, n, error", [([1.0, 2], None, TypeError), (["1"], None, TypeError), ([1, None], None, TypeError),
+                                         ([1, 2, 3], 2, IndexError), (np.ones(2), None, TypeError)])
+def test_integer_lists_refuse_what_ctypes_arrays_refuse(v, n, error):
+    with pytest.raises(error):
+        (C.c_int32 * (len(v) if n is None else n))(*v)
+    with pytest.raises(error):
+        B._i32(v, n)
