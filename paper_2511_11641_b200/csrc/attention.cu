@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t g = 0, qi = 0;
             bool ok = true;
             for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++qi)) {
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t g = 0, qi = 0, cp[2] = {0, 0};       // cp[x]: probability tiles of stream x consumed so far
             bool ok = true;
             for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++qi)) {
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
         // issued before S(G), whose completion signal covers it.  Both loads report to the barrier event G + 1 waits on.
         // This thread shares its scheduler with the stream's softmax warps, so the loop is kept short: slices are
         // described by a few registers produced once (next()) and handed from stage to stage.
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t x = warp;
             const uint32_t tS = tmem_base + Cfg::col_s(x, 0), tO = tmem_base + Cfg::col_o(x);
             const uint32_t idesc_s = make_idesc(kTile, 64, 0, 0);
@@ -1207,7 +1207,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t g = 0, ri = 0;
             bool ok = true;
             for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++ri)) {
@@ -1249,10 +1249,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ issuer of the score products
-        if (lane == 0) score_role(true, NB == 1);
+        if (elect_one()) score_role(true, NB == 1);
     } else if (warp >= 2 + kBwdComputeWarps) {
         // ------------------------------------------------------------------ issuers of the accumulating products (wide heads: of Y, and of all accumulating products)
-        if (lane == 0) {
+        if (elect_one()) {
             const int which = warp - (2 + kBwdComputeWarps);
             if (NB == 1) acc_role(which, which + 1);
             else if (which == 0) score_role(false, true);

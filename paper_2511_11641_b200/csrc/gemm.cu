@@ -119,6 +119,15 @@ __device__ int g_gemm_status = 0;
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
+// True in one lane (always the same) of a converged warp.  The branches whose thread issues loads, stores and products are
+// entered through this and not through a comparison of the lane number: these instructions take their operands from registers
+// that a warp shares, and behind elect.sync the compiler knows that one thread is active (see tc.cuh).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
@@ -410,13 +419,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // (KEEP = stores that may stay in flight because they read the other slot).
 template <int KEEP>
 __device__ __forceinline__ void stage_begin(int lane) {
-    if (lane == 0) bulk_wait_read<KEEP>();
+    bulk_wait_read<KEEP>();                // (nothing to wait for in the lanes that issued none)
     __syncwarp();
 }
 __device__ __forceinline__ void stage_commit(const CUtensorMap* map, uint32_t buf, int x, int y, int lane, bool add = false) {
     fence_async_smem();
     __syncwarp();
-    if (lane == 0) {
+    if (elect_one()) {
         if (add) tma_reduce_add_2d(map, buf, x, y);
         else tma_store_2d(map, buf, x, y);
         bulk_commit();
@@ -669,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer (both CTAs of a pair)
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -793,7 +802,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && leader) {
+        if (leader && elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
@@ -1064,7 +1073,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             }
             ++it;
         }
-        if (lane == 0) bulk_wait_all();            // this warp's tile stores have landed
+        bulk_wait_all();                           // this warp's tile stores have landed
     }
 
     // ---------------------------------------------------------------------- teardown
