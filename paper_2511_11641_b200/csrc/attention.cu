@@ -214,7 +214,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 const uint32_t idesc_o = make_idesc(kTile, wv, 0, 1);
                 // S_x = Q_x K^T with the K tile in ring stage st
                 auto scores = [&](uint32_t x, uint32_t st) {
-                    for (int ks = 0; ks < (wq >> 4); ++ks) {
+#pragma unroll
+                    for (int ks = 0; ks < 4 * NB; ++ks) {
+                        if (ks >= (wq >> 4)) break;
                         const uint32_t o = (ks >> 2) * kBlockBytes + (ks & 3) * 32;
                         tc_mma_bf16(tmem_base + Cfg::col_s(x), make_smem_desc(sQ + (2 * qs + x) * kTileBytes + o, 16, 1024),
                                     make_smem_desc(sK + st * kTileBytes + o, 16, 1024), idesc_s, ks != 0 ? 1u : 0u);
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                     if (!mbar_wait(p_full(x), cp[x] & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
                     ++cp[x];
                     tc_fence_after();
+#pragma unroll
                     for (int ks = 0; ks < kTile / 16; ++ks)
                         tc_mma_bf16_ts(tmem_base + Cfg::col_o(x), tmem_base + Cfg::col_p(x) + 8 * ks,
                                        make_smem_desc(sV + st * kTileBytes + ks * 2048, kBlockBytes, 1024), idesc_o, ks != 0 ? 1u : 0u);
@@ -1154,15 +1157,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 const uint64_t d_sa = make_smem_desc(sStr + (2 * st) * kStrTileBytes, 16, 1024),
                                d_sb = make_smem_desc(sStr + (2 * st + 1) * kStrTileBytes, 16, 1024);
                 if (do_x) {
-                    for (int ks = 0; ks < (wa >> 4); ++ks) {
+#pragma unroll
+                    for (int ks = 0; ks < 4 * NB; ++ks) {
                         const uint32_t o = ((ks >> 2) * kBlockBytes + (ks & 3) * 32) >> 4, os = ((ks >> 2) * kStrBlockBytes + (ks & 3) * 32) >> 4;
-                        tc_mma_bf16(tmem_base + kColX + xb * kStep, d_ra + o, d_sa + os, idesc_x, ks != 0 ? 1u : 0u);
+                        if (ks < (wa >> 4)) tc_mma_bf16(tmem_base + kColX + xb * kStep, d_ra + o, d_sa + os, idesc_x, ks != 0 ? 1u : 0u);
                     }
                 }
                 if (do_y) {
-                    for (int ks = 0; ks < (wb >> 4); ++ks) {
+#pragma unroll
+                    for (int ks = 0; ks < 4 * NB; ++ks) {
                         const uint32_t o = ((ks >> 2) * kBlockBytes + (ks & 3) * 32) >> 4, os = ((ks >> 2) * kStrBlockBytes + (ks & 3) * 32) >> 4;
-                        tc_mma_bf16(tmem_base + kColY + xb * kStep, d_rb + o, d_sb + os, idesc_x, ks != 0 ? 1u : 0u);
+                        if (ks < (wb >> 4)) tc_mma_bf16(tmem_base + kColY + xb * kStep, d_rb + o, d_sb + os, idesc_x, ks != 0 ? 1u : 0u);
                     }
                 }
                 tc_commit(x_full(xb));
@@ -1192,11 +1197,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     const uint32_t idesc = make_idesc(kTile, wn, 0, 1);
                     constexpr bool kOneAcc = NB == 2 && MODE == 1;      // (one thread issues both halves of the contraction)
                     const uint32_t acc_col = kOneAcc || (MODE == 0) == (which == 0) ? acc1 : acc2;
-                    const int ks0 = MODE == 0 ? 0 : 4 * which, ks1 = MODE == 0 ? kStep / 16 : 4 * which + 4;
+                    const int ks0 = MODE == 0 ? 0 : 4 * which;
+                    constexpr int kSteps = MODE == 0 ? kStep / 16 : 4;
                     const uint64_t db = make_smem_desc(sStr + (2 * st + ((MODE == 0 && which == 0) ? 1 : 0)) * kStrTileBytes, kStrBlockBytes, 1024);
-                    for (int ks = ks0; ks < ks1; ++ks)
-                        tc_mma_bf16_ts(tmem_base + acc_col, tmem_base + col_op(MODE == 0 ? which : 1, ob, ks), db + 128 * ks, idesc,
-                                       (i != 0 || ks != (kOneAcc ? 0 : ks0)) ? 1u : 0u);
+                    const uint32_t op = tmem_base + col_op(MODE == 0 ? which : 1, ob, ks0);
+                    const bool fresh = i == 0 && (!kOneAcc || ks0 == 0);
+#pragma unroll
+                    for (int k = 0; k < kSteps; ++k)
+                        tc_mma_bf16_ts(tmem_base + acc_col, op + (Cfg::kOverlay ? 16 : 8) * k, db + 128 * (ks0 + k), idesc, k == 0 && fresh ? 0u : 1u);
                 }
                 tc_commit(out_empty(ob));
                 tc_commit(t_empty(st));
