@@ -991,53 +991,53 @@ struct AttnBwdParams {
 // MODE 1: a CTA owns a query block and walks the key blocks: Q, dCtx resident, K_j and V_j streamed; X = S = Q K_j^T and
 //         Y = dP = dCtx V_j^T (thread = query row); dS is the A operand of dQ += dS K_j, which accumulates in TMEM.
 // Streamed tiles serve twice: as K-major B operands of the score products and as MN-major B operands of the
-// accumulating ones (same bytes, other descriptor).  Warp 0 loads, warps 2..17 compute (thread = row, quarter of the
-// columns), and three threads issue products: a thread gets a tcgen05 instruction (product or commit) accepted every
-// 70-130 clocks, so the 25-40 of a step are spread evenly over them, and the score products of a step are issued as soon
-// as every compute thread has the previous score tiles in registers.
-// Heads up to 64 wide (NB = 1): warp 1 issues the score products; warps 18 and 19 the accumulating ones: dV and dK in the
-// key-block kernel, the two halves of the contraction of dQ (into two accumulators that are added at the end) in the
-// query-block kernel; their A operands go through TMEM as packed bf16; three stages of streamed tiles.
-// Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products.  The accumulators leave no TMEM columns
-// for P^T and dS^T beside the score tiles, so the key-block kernel takes the queries 64 at a time, in two buffers of score tiles,
-// and every thread writes its packed operands over the scores it has made them from; the buffer is free for the scores of the
-// step after next when the products that read the operands are done.  (Operands in shared memory, where they
-// take two writes and reads of 16 KB a step from the port that feeds the products: both kernels 1080 us at 2 x 4096 positions,
-// 32 heads 96 wide; now 950.)  The query-block kernel has one accumulator and two buffers of dS beside it.
+// accumulating ones (same bytes, other descriptor).  A step is a streamed block of 64 rows.  Warp 0 loads, warps 2..17 compute, in
+// two groups of eight that take the steps in turn, each with score tiles and packed operands of its own: while one waits
+// for its products the other keeps the exponential unit busy.  What a step costs is a chain of short waits (scores, TMEM loads,
+// exponentials, operands, products), not a pipe: the exponentials of 128 x 128 scores take 1024 clocks, a pair of steps 2200.
+// Before (all warps on one block of 128, or on half blocks in turn) / now, us: 109.4 / 65.0 (60 x 48 positions, 32 heads 64
+// wide), 125.5 / 108.9 (4 x 1000, 32 heads 48 wide on 8), 42.0 / 36.1 (32 x 197, 6 heads 48 wide), 104.8 / 101.3 (8 x 1024, 16
+// heads 32 wide), 1205 / 1088 (2 x 4096, 32 heads 128 wide).
+// The products are issued by separate threads.  Heads up to 64 wide (NB = 1): warp 1 issues the score products; warps 18 and 19
+// the accumulating ones (dV and dK; the query-block kernel needs only the second), whose A operands go through TMEM as
+// packed bf16 beside the scores.  Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products.  The
+// accumulators of the key-block kernel then leave no TMEM columns beside the score tiles: every thread writes its packed P^T and
+// dS^T over the scores it has made them from, and the buffer is free for the next scores when the products that read the
+// operands are done.  The query-block kernel has one accumulator (on heads up to 64 wide two, which the items take in turn).
 // Wait codes: 14 / 15 / 16 (MODE 0 loads, products, compute) and 17 / 18 / 19 (MODE 1).
+constexpr int kStep = 64;                  // rows of a streamed block (queries in the key-block kernel, keys in the query-block kernel)
 template <int NB, int MODE>
 struct BwdCfg {
     static constexpr int kTileBytes = NB * kBlockBytes;
-    // rows of a streamed block: the key-block kernel on wide heads walks the queries in half blocks
-    static constexpr int kStep = (NB == 2 && MODE == 0) ? 64 : kTile;
     static constexpr int kStrBlockBytes = kStep * 128;                         // 64 columns of a streamed block
     static constexpr int kStrTileBytes = NB * kStrBlockBytes;
     static constexpr int kResStages = NB == 1 ? 2 : 1;                         // buffers of the resident pair of tiles
-    // stages of the streamed pair of tiles, as many as fit up to four (a stage is free again only when the accumulating products
-    // that read it are done, a whole step after the score products, and the next load must be under way by then)
-    static constexpr int kStrStages = NB == 1 ? 3 : (MODE == 0 ? 4 : 2);
+    static constexpr int kStrStages = NB == 1 ? 6 : 4;                         // stages of the streamed pair of tiles
     static constexpr bool kOverlay = NB == 2 && MODE == 0;                      // operands over the scores
-    static constexpr int kOutBufs = NB == 2 ? 2 : 1;                            // buffers of the packed operands
     static constexpr int kVecBytes = MODE == 0 ? kStrStages * 2 * kStep * 4 : 0;   // -lse2 and D of a query block, per streamed stage
-    static constexpr int kSmem = 2 * kTileBytes * kResStages + 2 * kStrTileBytes * kStrStages + kVecBytes + 1024 + 256;
+    static constexpr int kSmem = 2 * kTileBytes * kResStages + 2 * kStrTileBytes * kStrStages + kVecBytes + 1024 + 512;
     static_assert(kSmem <= 232448, "shared memory of a block");
 };
 
-template <int NB, int MODE, int NACC = 1>   // NACC = 2: every head at most 32 wide, the accumulators of two items side by side
+template <int NB, int MODE, int NACC = 1>   // NACC = 2: the accumulators of two items side by side (of the key-block kernel: heads at most 32 wide)
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ AttnBwdParams P) {
     using Cfg = BwdCfg<NB, MODE>;
     constexpr int kTileBytes = Cfg::kTileBytes, kStrTileBytes = Cfg::kStrTileBytes, kStrBlockBytes = Cfg::kStrBlockBytes;
-    constexpr int kStep = Cfg::kStep;
     constexpr int RS = Cfg::kResStages, SS = Cfg::kStrStages;
-    // TMEM columns: score tiles X and Y, accumulators (64 columns each on heads up to 64 wide, else 128), packed bf16 operands of
-    // the accumulating products (P^T and dS^T, or dS), two values per column
-    constexpr uint32_t kAccIssuers = NB == 1 ? 2 : 1, kScoreIssuers = NB == 1 ? 1 : 2;
-    constexpr uint32_t kColX = 0, kColY = 128, kColAcc1 = 256, kColAcc2 = NB == 1 ? 320 : 384;
-    // operand `which` (0: P^T, 1: dS^T or dS) of 16 contraction steps from 16 ks on, in operand buffer ob
+    // TMEM columns: two buffers of the score tiles X and Y, accumulators, two buffers of the packed bf16 operands of the
+    // accumulating products (P^T and dS^T, or dS), two values per column
+    constexpr uint32_t kAccIssuers = NB == 1 && MODE == 0 ? 2 : 1, kScoreIssuers = NB == 1 ? 1 : 2;
+    constexpr uint32_t kColX = 0, kColY = 128, kColAcc = 256;
+    // accumulator `which` (0: dV or dQ, 1: dK) of set as
+    auto col_acc = [](int which, uint32_t as) -> uint32_t {
+        if (MODE == 1) return kColAcc + 64 * as;
+        return kColAcc + (NACC == 2 ? 64 * as + 32 * which : (NB == 1 ? 64 : 128) * which);
+    };
+    // operand `which` (0: P^T, 1: dS^T or dS) of 16 contraction steps from 16 ks on, in operand buffer ob.  (Over the scores a
+    // thread's 32 columns become its first 16.)
     auto col_op = [](int which, uint32_t ob, uint32_t ks) -> uint32_t {
-        if (Cfg::kOverlay) return (which == 0 ? kColX : kColY) + 64 * ob + 16 * ks;
-        if (NB == 2) return 384 + 64 * ob + 8 * ks;
-        return (which == 0 ? 384 : 448) + 8 * ks;
+        if (Cfg::kOverlay) return (which == 0 ? kColX : kColY) + 64 * ob + 32 * (ks >> 1) + 8 * (ks & 1);
+        return 384 + (MODE == 0 ? 64 * which : 0) + 32 * ob + 8 * ks;
     };
     constexpr int kCodeBase = MODE == 0 ? 14 : 17;
     extern __shared__ uint8_t smem_raw[];
@@ -1050,25 +1050,23 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     float* vec = reinterpret_cast<float*>(vec_raw);                               // [stage][-lse2 | D][128]
     uint8_t* tail = vec_raw + Cfg::kVecBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 24 * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 24 * 8 + 8);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 32 * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 32 * 8 + 8);
     const uint32_t bar0 = smem_u32(bars);
     auto r_full = [&](uint32_t s) { return bar0 + 8u * s; };
     auto r_empty = [&](uint32_t s) { return bar0 + 8u * (2 + s); };
     auto t_full = [&](uint32_t s) { return bar0 + 8u * (4 + s); };
-    auto t_empty = [&](uint32_t s) { return bar0 + 8u * (8 + s); };
-    // accumulators: one set, or two (heads at most 32 wide) that the items take in turn, each with its own pair of barriers
-    auto acc_full = [&](uint32_t a) { return bar0 + 8u * (a ? 22 : 15); };
-    auto acc_empty = [&](uint32_t a) { return bar0 + 8u * (a ? 23 : 16); };
+    auto t_empty = [&](uint32_t s) { return bar0 + 8u * (10 + s); };
+    // per group of compute warps: scores complete; scores in registers; operands written; operands read
+    auto x_full = [&](uint32_t b) { return bar0 + 8u * (16 + b); };
+    auto xy_free = [&](uint32_t b) { return bar0 + 8u * (18 + b); };
+    auto out_full = [&](uint32_t b) { return bar0 + 8u * (20 + b); };
+    auto out_empty = [&](uint32_t b) { return bar0 + 8u * (22 + b); };
+    // accumulators: one set, or two that the items take in turn, each with its own pair of barriers
+    auto acc_full = [&](uint32_t a) { return bar0 + 8u * (24 + a); };
+    auto acc_empty = [&](uint32_t a) { return bar0 + 8u * (26 + a); };
     constexpr uint32_t n_acc = NACC;
     static_assert(NACC == 1 || NB == 1, "two sets of accumulators need the narrow layout");
-    constexpr uint32_t kOB = Cfg::kOutBufs;
-    auto out_full = [&](uint32_t b) { return bar0 + 8u * (b ? 20 : 13); };
-    auto out_empty = [&](uint32_t b) { return bar0 + 8u * (b ? 21 : 14); };
-    // score tiles: one buffer of 128 columns each, or (half-block steps) two of 64, each with its own pair of barriers
-    constexpr uint32_t kXY = kStep == 64 ? 2 : 1;
-    auto x_full = [&](uint32_t b) { return bar0 + 8u * (b ? 18 : 12); };
-    auto xy_free = [&](uint32_t b) { return bar0 + 8u * (b ? 19 : 17); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -1076,14 +1074,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             mbar_init(r_full(s), 1);
             mbar_init(r_empty(s), kScoreIssuers);
         }
-        for (uint32_t s = 0; s < 4; ++s) {
+        for (uint32_t s = 0; s < SS; ++s) {
             mbar_init(t_full(s), 1);
             mbar_init(t_empty(s), kAccIssuers);
         }
         for (uint32_t b = 0; b < 2; ++b) {
             mbar_init(x_full(b), kScoreIssuers);
-            mbar_init(xy_free(b), kBwdComputeWarps);
-            mbar_init(out_full(b), kBwdComputeWarps);     // barriers the compute threads arrive on: one arrival per warp (its lanes meet first)
+            mbar_init(xy_free(b), kBwdComputeWarps / 2);  // barriers the compute threads arrive on: one arrival per warp (its lanes meet first)
+            mbar_init(out_full(b), kBwdComputeWarps / 2);
             mbar_init(out_empty(b), kAccIssuers);
         }
         for (uint32_t a = 0; a < 2; ++a) {
@@ -1124,7 +1122,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             I.n_per = (P.seq + kStep - 1) / kStep - I.first;
         } else {
             I.first = 0;
-            I.n_per = P.causal ? I.own + 1 : P.n_t;            // key blocks up to the query block
+            I.n_per = (P.seq + kStep - 1) / kStep;             // key blocks (of kStep keys) up to the end of the query block
+            if (P.causal) I.n_per = min(I.n_per, (I.own + 1) * (kTile / kStep));
         }
         I.n_steps = I.n_per * grp;
         return I;
@@ -1150,7 +1149,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             const uint64_t d_ra = make_smem_desc(sRes + (2 * rs) * kTileBytes, 16, 1024),
                            d_rb = make_smem_desc(sRes + (2 * rs + 1) * kTileBytes, 16, 1024);
             for (int i = 0; ok && i < I.n_steps; ++i, ++g) {
-                const uint32_t use = g / kXY, st = g % SS, xb = g % kXY;
+                const uint32_t use = g >> 1, st = g % SS, xb = g & 1;
                 if (use > 0 && !(ok = mbar_wait(Cfg::kOverlay ? out_empty(xb) : xy_free(xb), (use - 1) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 if (!(ok = mbar_wait(t_full(st), (g / SS) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 tc_fence_after();
@@ -1176,35 +1175,27 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         }
     };
     // The accumulating products number w0 .. w1 - 1 of every step.  Key-block kernel: 0 is dV += P^T dCtx_i (B = streamed b
-    // tile), 1 is dK += dS^T Q_i (B = streamed a tile), all steps of the contraction over the step's queries; query-block
-    // kernel: dQ += dS K_j (B = streamed a tile), 0 is steps 0-3 of the contraction, 1 is steps 4-7 (two accumulators).
+    // tile), 1 is dK += dS^T Q_i (B = streamed a tile); query-block kernel: 1 is dQ += dS K_j (B = streamed a tile).
     auto acc_role = [&](int w0, int w1) {
         uint32_t g = 0, ri = 0;
         bool ok = true;
         for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++ri)) {
             const BItem I = decode(it);
             const uint32_t as = ri % n_acc;
-            const uint32_t acc1 = n_acc == 2 ? kColAcc1 + 64 * as : kColAcc1, acc2 = n_acc == 2 ? kColAcc1 + 64 * as + 32 : kColAcc2;
             for (int i = 0; i < I.n_steps; ++i, ++g) {
-                const uint32_t st = g % SS;
+                const uint32_t st = g % SS, ob = g & 1;
                 if (!(ok = mbar_wait(t_full(st), (g / SS) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
-                const uint32_t ob = g % kOB;
-                if (!(ok = mbar_wait(out_full(ob), (g / kOB) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
+                if (!(ok = mbar_wait(out_full(ob), (g >> 1) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 if (i == 0 && !(ok = mbar_wait(acc_empty(as), ((ri / n_acc) & 1u) ^ 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 tc_fence_after();
                 for (int which = w0; which < w1; ++which) {
-                    const int wn = (MODE == 0 && which == 0) ? P.heads.vo_w[I.h] : P.heads.qk_w[I.h];
+                    const int wn = which == 0 ? P.heads.vo_w[I.h] : P.heads.qk_w[I.h];
                     const uint32_t idesc = make_idesc(kTile, wn, 0, 1);
-                    constexpr bool kOneAcc = NB == 2 && MODE == 1;      // (one thread issues both halves of the contraction)
-                    const uint32_t acc_col = kOneAcc || (MODE == 0) == (which == 0) ? acc1 : acc2;
-                    const int ks0 = MODE == 0 ? 0 : 4 * which;
-                    constexpr int kSteps = MODE == 0 ? kStep / 16 : 4;
-                    const uint64_t db = make_smem_desc(sStr + (2 * st + ((MODE == 0 && which == 0) ? 1 : 0)) * kStrTileBytes, kStrBlockBytes, 1024);
-                    const uint32_t op = tmem_base + col_op(MODE == 0 ? which : 1, ob, ks0);
-                    const bool fresh = i == 0 && (!kOneAcc || ks0 == 0);
+                    const uint32_t acc = tmem_base + col_acc(MODE == 0 ? which : 0, as), op = tmem_base + col_op(which, ob, 0);
+                    const uint64_t db = make_smem_desc(sStr + (2 * st + (which == 0 ? 1 : 0)) * kStrTileBytes, kStrBlockBytes, 1024);
 #pragma unroll
-                    for (int k = 0; k < kSteps; ++k)
-                        tc_mma_bf16_ts(tmem_base + acc_col, op + (Cfg::kOverlay ? 16 : 8) * k, db + 128 * (ks0 + k), idesc, k == 0 && fresh ? 0u : 1u);
+                    for (int ks = 0; ks < kStep / 16; ++ks)
+                        tc_mma_bf16_ts(acc, op + (Cfg::kOverlay ? 32 * (ks >> 1) + 8 * (ks & 1) : 8 * ks), db + 128 * ks, idesc, (i | ks) != 0 ? 1u : 0u);
                 }
                 tc_commit(out_empty(ob));
                 tc_commit(t_empty(st));
@@ -1228,10 +1219,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 const uint32_t rs = ri % RS;
                 if (!(ok = mbar_wait(r_empty(rs), ((ri / RS) & 1u) ^ 1u, abort_flag, kCodeBase, P.status, P.wait_limit_ns))) break;
                 mbar_expect_tx(r_full(rs), (nba + nbb) * kBlockBytes);
-                for (int blk = 0; blk < nba; ++blk)
-                    tma_load_2d(sRes + (2 * rs) * kTileBytes + blk * kBlockBytes, map_ra, ra_off + 64 * blk, row0 + I.own * kTile, r_full(rs));
-                for (int blk = 0; blk < nbb; ++blk)
-                    tma_load_2d(sRes + (2 * rs + 1) * kTileBytes + blk * kBlockBytes, map_rb, rb_off + 64 * blk, row0 + I.own * kTile, r_full(rs));
+                for (int half = 0; half < 2; ++half) {              // (all boxes are 64 rows high)
+                    const uint32_t dst = sRes + (2 * rs) * kTileBytes + half * kStep * 128;
+                    const int y = row0 + I.own * kTile + half * kStep;
+                    for (int blk = 0; blk < nba; ++blk) tma_load_2d(dst + blk * kBlockBytes, map_ra, ra_off + 64 * blk, y, r_full(rs));
+                    for (int blk = 0; blk < nbb; ++blk) tma_load_2d(dst + kTileBytes + blk * kBlockBytes, map_rb, rb_off + 64 * blk, y, r_full(rs));
+                }
                 for (int i = 0; i < I.n_steps; ++i, ++g) {
                     const uint32_t st = g % SS;
                     if (!(ok = mbar_wait(t_empty(st), ((g / SS) & 1u) ^ 1u, abort_flag, kCodeBase, P.status, P.wait_limit_ns))) break;
@@ -1262,18 +1255,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         // ------------------------------------------------------------------ issuers of the accumulating products (wide heads: of Y, and of all accumulating products)
         if (elect_one()) {
             const int which = warp - (2 + kBwdComputeWarps);
-            if (NB == 1) acc_role(which, which + 1);
-            else if (which == 0) score_role(false, true);
-            else acc_role(0, 2);
+            if (MODE == 0 && NB == 1) acc_role(which, which + 1);
+            else if (which == 1) acc_role(MODE, 2);
+            else if (NB == 2) score_role(false, true);
         }
     } else {
         // ------------------------------------------------------------------ compute
-        // Thread = (row of the owned block = TMEM lane, quarter of the streamed block's 128 columns): warps 2..5 take
-        // columns [0, 32), warps 6..9 [32, 64), and so on, so every scheduler has four compute warps to interleave.
-        const int part = (warp - 2) >> 2;
+        // Two groups of eight warps take the steps in turn (group = score buffer); thread = (row of the owned block = TMEM lane, half
+        // of the streamed block's 64 columns), so every scheduler has two warps of each group.
+        const int part = (warp - 2) >> 2, group = part >> 1;
         const int row = (warp & 3) * 32 + lane;
-        constexpr int kHalves = kStep / 64;                            // 16-column halves of this thread's columns
-        const int col0 = part * (kStep / 4);                           // this thread's columns of the streamed block
+        constexpr int kHalves = 2;                                     // 16-column halves of this thread's columns
+        const int col0 = (part & 1) * 32;                              // this thread's columns of the streamed block
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         uint32_t g = 0, ri = 0;
         bool ok = true;
@@ -1283,30 +1276,22 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             bool on;
         };
         Pend pend = {0, 0, 0, 0, false};
-        // writes an item's accumulators out once they are complete (every thread its quarter of the columns) and releases them
+        // writes an item's accumulators out once they are complete (every thread a quarter of the columns) and releases them
         auto flush = [&](const Pend& d) -> bool {
             const uint32_t as = d.ri % n_acc;
-            const uint32_t acc1 = n_acc == 2 ? kColAcc1 + 64 * as : kColAcc1, acc2 = n_acc == 2 ? kColAcc1 + 64 * as + 32 : kColAcc2;
             if (!mbar_wait(acc_full(as), (d.ri / n_acc) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns)) return false;
             tc_fence_after();
             const int pos = d.own * kTile + row;
             const bool live = pos < P.seq;
             const int64_t t = static_cast<int64_t>(d.b) * P.seq + pos;
-            auto write_acc = [&](uint32_t colbase, int w, uint16_t* dst, float mul, bool two = false, uint32_t colbase2 = 0) {
+            auto write_acc = [&](uint32_t colbase, int w, uint16_t* dst, float mul) {
 #pragma unroll
                 for (int c = 0; c < NB; ++c) {
                     const int col = part * (NB * 16) + c * 16;
                     if (col < w) {
                         uint32_t r[16];
                         tc_ld16(t_lane + colbase + col, r);
-                        tc_wait_ld();
-                        if (two) {                               // the contraction was split over two accumulators
-                            uint32_t r2[16];
-                            tc_ld16(t_lane + colbase2 + col, r2);
-                            tc_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(r2[e]));
-                        }
+                        tc_wait_ld(r);
                         if (live) {
                             uint4 v0, v1;
                             v0.x = pack_bf16(__uint_as_float(r[0]) * mul, __uint_as_float(r[1]) * mul);
@@ -1324,10 +1309,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 }
             };
             if (MODE == 0) {
-                write_acc(acc1, P.heads.vo_w[d.h], P.dv + t * P.ld_dv + P.heads.v_off[d.h], 1.f);
-                write_acc(acc2, P.heads.qk_w[d.h], P.dk + t * P.ld_dqk + P.heads.k_off[d.h], P.scale);
+                write_acc(col_acc(0, as), P.heads.vo_w[d.h], P.dv + t * P.ld_dv + P.heads.v_off[d.h], 1.f);
+                write_acc(col_acc(1, as), P.heads.qk_w[d.h], P.dk + t * P.ld_dqk + P.heads.k_off[d.h], P.scale);
             } else {
-                write_acc(NB == 2 ? acc1 : acc2, P.heads.qk_w[d.h], P.dq + t * P.ld_dqk + P.heads.qk_off[d.h], P.scale, NB == 1, acc1);
+                write_acc(col_acc(0, as), P.heads.qk_w[d.h], P.dq + t * P.ld_dqk + P.heads.qk_off[d.h], P.scale);
             }
             tc_fence_before();
             __syncwarp();
@@ -1345,17 +1330,26 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                 lse_r = P.vecs[o];
                 d_r = P.vecs[static_cast<int64_t>(P.n_heads) * P.batch * P.seq_pad + o];
             }
-            for (int i = 0; i < I.n_steps; ++i, ++g) {
-                const int other0 = (I.first + i % I.n_per) * kStep;  // first position of the streamed block
+            const int i0 = (g & 1) == static_cast<uint32_t>(group) ? 0 : 1;
+            const uint32_t g_next = g + I.n_steps;
+            g += i0;
+            int blk = i0;                                            // step i of its query head (MODE 0: the heads of a group follow one another)
+            for (int i = i0; i < I.n_steps; i += 2, g += 2, blk += 2) {
+                while (MODE == 0 && blk >= I.n_per) blk -= I.n_per;
+                const int other0 = (I.first + blk) * kStep;          // first position of the streamed block
                 const float* vb = vec + (g % SS) * 2 * kStep;
-                const uint32_t xb = g % kXY;
-                if (!(ok = mbar_wait(x_full(xb), (g / kXY) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
-                tc_fence_after();
+                const uint32_t xb = g & 1, ob = xb;
                 // (the step's loads landed long ago; this thread reads the vectors among them, so it looks at their barrier itself)
                 if (MODE == 0 && !(ok = mbar_wait(t_full(g % SS), (g / SS) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
+                if (!(ok = mbar_wait(x_full(xb), (g >> 1) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
+                tc_fence_after();
                 // (query position, key position) of element (row, column c): MODE 0 rows are keys, MODE 1 rows are queries
                 const int q0 = MODE == 0 ? other0 : I.own * kTile, k0 = MODE == 0 ? I.own * kTile : other0;
-                const bool masked = q0 + (MODE == 0 ? kStep : kTile) > P.seq || k0 + kTile > P.seq || (P.causal && q0 < k0 + kTile);
+                const bool masked = q0 + (MODE == 0 ? kStep : kTile) > P.seq || k0 + (MODE == 0 ? kTile : kStep) > P.seq ||
+                                    (P.causal && q0 < k0 + (MODE == 0 ? kTile : kStep));
+                // this thread's visible columns (MODE 0: queries at or after the row's key, MODE 1: keys up to the row's query)
+                const int vis_lo = MODE == 0 && P.causal ? own_pos - q0 - col0 : 0;
+                const int vis_hi = own_pos >= P.seq ? 0 : (MODE == 1 && P.causal ? min(P.seq, own_pos + 1) : P.seq) - other0 - col0;
                 // two halves of 16 columns: probabilities and dS are packed to bf16 pairs as soon as they exist
                 uint32_t pk_p[8 * kHalves], pk_ds[8 * kHalves];
                 const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), neg1 = pack2(-1.f, -1.f);
@@ -1372,12 +1366,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     }
                     if (masked) {                                     // pairs outside the mask count as -inf (p = 0)
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const int c = col0 + 16 * hh + e;
-                            const int qp = MODE == 0 ? q0 + c : own_pos;
-                            const int kp = MODE == 0 ? own_pos : k0 + c;
-                            if (!(qp < P.seq && kp < P.seq && (!P.causal || kp <= qp))) rx[e] = 0xff800000u;
-                        }
+                        for (int e = 0; e < 16; ++e)
+                            if (16 * hh + e < vis_lo || 16 * hh + e >= vis_hi) rx[e] = 0xff800000u;
                     }
 #pragma unroll
                     for (int e = 0; e < 16; e += 4) {
@@ -1404,26 +1394,23 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     }
                 }
                 // the products that read the operands last in this buffer are done (over the scores: the score products waited for that)
-                const uint32_t ob = g % kOB;
-                if (!Cfg::kOverlay && !(ok = mbar_wait(out_empty(ob), ((g / kOB) & 1u) ^ 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
+                if (!Cfg::kOverlay && !(ok = mbar_wait(out_empty(ob), ((g >> 1) & 1u) ^ 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns))) break;
                 // this thread's columns, packed, in its TMEM lane
-                if (MODE == 0) tc_st(t_lane + col_op(0, ob, part * kHalves), pk_p);
-                tc_st(t_lane + col_op(1, ob, part * kHalves), pk_ds);
+                if (MODE == 0) tc_st(t_lane + col_op(0, ob, (part & 1) * kHalves), pk_p);
+                tc_st(t_lane + col_op(1, ob, (part & 1) * kHalves), pk_ds);
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(out_full(ob));
-                if (i == 0 && pend.on) {   // the previous item's accumulators, now that this item's first step is on its way
+                if (pend.on) {   // the previous item's accumulators, now that this item's first step is on its way
                     if (!(ok = flush(pend))) break;
                     pend.on = false;
                 }
             }
             if (!ok) break;
-            // the accumulators of this item: written out now, or (two sets) after the first step of the CTA's next item, when
-            // the last products into them have long landed
-            const Pend cur = {I.h, I.b, I.own, ri, true};
-            if (n_acc == 2) pend = cur;
-            else if (!(ok = flush(cur))) break;
+            if (pend.on && !(ok = flush(pend))) break;         // (an item without a step for this group)
+            g = g_next;
+            pend = {I.h, I.b, I.own, ri, true};                // written out after the first step of the next item, when the last products into them have long landed
         }
         if (ok && pend.on) flush(pend);
     }
@@ -1619,10 +1606,10 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
     int* status = engine_status_ptr(&st);
     if (!status) return st;
     const int64_t T = batch * seq;
-    if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk)) != ECOSPA_OK) return st;
-    if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk)) != ECOSPA_OK) return st;
-    if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v)) != ECOSPA_OK) return st;
-    if ((st = encode_tile_map(&P.map_do, dCtx, T, n_vo, ld_dctx)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk, kStep)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk, kStep)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v, kStep)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_do, dCtx, T, n_vo, ld_dctx, kStep)) != ECOSPA_OK) return st;
     float* vecs = static_cast<float*>(workspace);
     P.batch = static_cast<int32_t>(batch);
     P.seq = static_cast<int32_t>(seq);
@@ -1652,7 +1639,6 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 0>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 0>::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 1>::kSmem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(attn_rowdot_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dot_smem(kDotMaxVecs, kMaxHeads)));
@@ -1684,20 +1670,15 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
     const int items_q = P.n_items;
     P.n_items = items_q / P.heads.rep;
     int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
-    if (nb == 1) {
+    if (nb == 1)
         st = launch_pdl(max_w <= 32 ? attn_bwd_kernel<1, 0, 2> : attn_bwd_kernel<1, 0, 1>, grid, kBwdThreads, stream, P,
                         "attn_bwd_kernel (dK, dV)", BwdCfg<1, 0>::kSmem);
-    } else {   // wide heads: the streamed query blocks are half blocks
-        AttnBwdParams P0 = P;
-        if ((st = encode_tile_map(&P0.map_q, Qc, T, n_qk, ld_qk, BwdCfg<2, 0>::kStep)) != ECOSPA_OK) return st;
-        if ((st = encode_tile_map(&P0.map_do, dCtx, T, n_vo, ld_dctx, BwdCfg<2, 0>::kStep)) != ECOSPA_OK) return st;
-        st = launch_pdl(attn_bwd_kernel<2, 0, 1>, grid, kBwdThreads, stream, P0, "attn_bwd_kernel (dK, dV)", BwdCfg<2, 0>::kSmem);
-    }
+    else
+        st = launch_pdl(attn_bwd_kernel<2, 0, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dK, dV)", BwdCfg<2, 0>::kSmem);
     if (st != ECOSPA_OK) return st;
     P.n_items = items_q;
     grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     if (nb == 1)
-        return launch_pdl(max_w <= 32 ? attn_bwd_kernel<1, 1, 2> : attn_bwd_kernel<1, 1, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)",
-                          BwdCfg<1, 1>::kSmem);
+        return launch_pdl(attn_bwd_kernel<1, 1, 2>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)", BwdCfg<1, 1>::kSmem);
     return launch_pdl(attn_bwd_kernel<2, 1, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)", BwdCfg<2, 1>::kSmem);
 }
