@@ -8,24 +8,28 @@
 // Q K^T, and a zero column of V^c gives a zero column of Ctx) and off_h a multiple of 8, so that every tile load starts
 // on a 16-byte boundary and every contraction is a whole number of 16-deep MMA steps.
 //
-// Two forward kernels, one CTA per SM.  Output heads up to 32 wide (with Q/K heads up to 64) take the kernel of
-// independent key streams further down (attn_fwd_ms_kernel); wider heads take the kernel described here, 320 threads.
-// A work item is (sequence b, head h, two neighbouring tiles of 128 query rows); a CTA walks a static list of items
-// (for causal attention the long ones first).  The two query tiles are two streams that share the K / V tiles and run
-// half a step apart.
-//   warp 0      producer: one lane issues the TMA loads of the item's two Q tiles and of every K / V tile (rings of 2
-//               stages); a tile is one or two 64-column blocks of 128 rows x 128 bytes, 128-byte swizzle
-//   warp 1      owns TMEM (512 columns: a 128-column score tile and an output tile per stream, and the probabilities as
-//               packed bf16); one lane issues S = Q K^T (K-major operands from shared memory) and O_tile = P V (P read
-//               from TMEM, V as stored = MN-major) for both streams
-//   warps 2..5  softmax of stream 0, warps 6..9 of stream 1; thread = query row = TMEM lane, all 128 key columns, so
-//               nothing is exchanged between threads.  Per key block: pass 1 reads the score tile for the row maximum,
-//               folds the previous output tile (O = O * 2^(m_old - m_new) + O_tile, in registers); pass 2 reads the
-//               scores again, p = 2^(s*c - m), packs P to bf16 and writes it to TMEM for the second product.
-// Pass 2 is bound by the exponential unit, pass 1 and the waits on the tensor pipe are not: a token (two mbarriers)
-// lets only one stream at a time through pass 2, so one stream exponentiates while the other reads maxima, folds and
-// waits for its products.  Every mbarrier wait is bounded; on expiry the CTA records a code (11 producer, 12 MMA
-// issuer, 13 softmax) in the device status word, lets copies land, frees TMEM and returns.
+// Two forward kernels, one CTA per SM.  Output heads up to 32 wide (with Q/K heads up to 64) on sequences above two tiles take
+// the kernel of independent key streams further down (attn_fwd_ms_kernel); all others the kernel described here, 640 threads.
+// A work item is one or two tiles of 128 query rows, one per stream (see FwdItems); a CTA walks a static list of items (for
+// causal attention the long ones first).  Two neighbouring query tiles of a sequence and head share the K / V tiles.
+//   warp 0       one lane issues the TMA loads of the streams' Q tiles and of the K / V tiles (rings of 4 or 2 stages); a tile
+//                is one or two 64-column blocks of 128 rows x 128 bytes, 128-byte swizzle
+//   warps 1, 2   one lane each issues the products of its stream: S = Q K^T (K-major operands from shared memory) and
+//                O += P V (P read from TMEM, V as stored = MN-major), accumulating in TMEM
+//   warps 4..11  scaling, four warps per stream: where a key block raises a row's maximum, the output row so far is multiplied by
+//                2^(m_old - m_new) while the softmax warps exponentiate; at the end of an item times 1 / l and to memory
+//   warps 12..19 softmax, four warps per stream; thread = query row = TMEM lane, all 128 key columns, so nothing is exchanged
+//                between threads.  A first pass over the scores takes the row maximum, a second one p = 2^(s*c - m), which it
+//                packs to bf16 and writes to TMEM for the second product.  Every probability is taken against the row's running
+//                maximum, so the largest one of a row is exactly 1.
+// Both passes are rolled loops of 64 columns: holding a block's 128 scores in registers, unrolled, was slower (163 -> 233 us at
+// 4 x 2048 positions, 32 heads 32 wide: warps waited for instructions, 4.0 of 15 cycles per issue, now 1.0).  Columns that
+// no row of a warp sees are skipped, keys past the end of the sequence also in the products.
+// Before (two streams in one thread's registers, a token between them) / now, us: 420 / 370 (2 x 4096, 32 heads 96 wide),
+// 59.3 / 53.1 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 8.5 (2 x 160, 12 heads 48 wide), 60.9 / 28.2 (60 x 48, 32 heads 64
+// wide), 41.8 / 18.9 (30 x 48, 32 heads 128 wide), 24.9 / 27.2 (8 x 512, 16 heads 64 wide, no mask).
+// Every mbarrier wait is bounded; on expiry the CTA records a code (11 loads, 12 products, 13 softmax and scaling) in the device
+// status word, lets copies land, frees TMEM and returns.
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -48,7 +52,7 @@ using namespace tc;
 constexpr int kTile = 128;                  // query rows and key rows per tile
 constexpr int kBlockBytes = kTile * 128;    // one 64-column block of a 128-row tile
 constexpr int kMaxHeads = 128;
-constexpr int kFwdThreads = 64 + 2 * 128;   // producer warp, MMA warp, two streams of four softmax warps
+constexpr int kFwdThreads = 640;              // four service warps; per stream four scaling and four softmax warps
 constexpr int kBwdComputeWarps = 16;
 constexpr int kBwdThreads = 64 + 4 * 128 + 64;   // producer warp, MMA warp, four sets of four compute warps, two more MMA warps
 constexpr int kTmemCols = 512;
@@ -63,6 +67,7 @@ struct AttnFwdParams {
     alignas(64) CUtensorMap map_q, map_k, map_v;
     HeadLayout heads;
     int32_t batch, seq, n_heads, n_qt, causal, n_items;
+    int32_t items;                          // FwdItems
     float scale_log2e;                      // scale * log2(e): scores are exponentiated in base 2
     uint16_t* ctx;
     int64_t ld_ctx;
@@ -79,81 +84,113 @@ __device__ __forceinline__ int dealt_item(uint32_t round) {
     return (r & 1) ? (r + 1) * G - 1 - c : r * G + c;
 }
 
-struct Item {
-    int b, h, qp, n_a, n_b, n;   // query tiles 2 qp and 2 qp + 1 with n_a and n_b key blocks (0: no such tile), n = the larger
+// A work item is one or two tiles of 128 query rows, one per stream.
+enum FwdItems {
+    ITEMS_SHARED = 0,   // two neighbouring query tiles of a (sequence, head); both streams read the same K / V tiles
+    ITEMS_SOLO = 1,     // sequences of one tile: two (sequence, head) units, each with a K / V tile of its own
+    ITEMS_SINGLE = 2,   // one query tile (few of them: each gets an SM to itself)
 };
-__device__ __forceinline__ Item decode_item(int it, int n_qt, int n_heads, int batch, int n_kt, int causal) {
-    Item I;
-    const int per = n_heads * batch;
-    const int n_qp = (n_qt + 1) >> 1;
-    I.qp = n_qp - 1 - it / per;             // long (late) query tiles first
-    const int rem = it % per;
-    I.h = rem / batch;
-    I.b = rem % batch;
-    const int qa = 2 * I.qp, qb = qa + 1;
-    I.n_a = causal ? min(n_kt, qa + 1) : n_kt;
-    I.n_b = qb < n_qt ? (causal ? min(n_kt, qb + 1) : n_kt) : 0;
-    I.n = max(I.n_a, I.n_b);
+struct FwdItem {
+    int h0, b0, qt0, n0, h1, b1, qt1, n1;   // of stream 0 and 1: head, sequence, query tile, key blocks (0: no such tile)
+};
+__device__ __forceinline__ FwdItem decode_item(int it, const AttnFwdParams& P) {
+    FwdItem I;
+    const int per = P.n_heads * P.batch;
+    if (P.items == ITEMS_SOLO) {
+        const int u0 = 2 * it, u1 = min(u0 + 1, per - 1);
+        I.h0 = u0 / P.batch;
+        I.b0 = u0 % P.batch;
+        I.h1 = u1 / P.batch;
+        I.b1 = u1 % P.batch;
+        I.qt0 = I.qt1 = 0;
+        I.n0 = 1;
+        I.n1 = u0 + 1 < per ? 1 : 0;
+        return I;
+    }
+    const int rem = it % per, a = it / per;
+    I.h0 = I.h1 = rem / P.batch;
+    I.b0 = I.b1 = rem % P.batch;
+    if (P.items == ITEMS_SINGLE) {
+        I.qt0 = I.qt1 = P.n_qt - 1 - a;                            // long (late) query tiles first
+        I.n1 = 0;
+    } else {                                                       // (an odd one out is the first, the shortest)
+        const int qa = 2 * ((P.n_qt + 1) / 2 - 1 - a) - (P.n_qt & 1);
+        I.qt0 = max(qa, 0);
+        I.qt1 = qa + 1;
+        I.n1 = qa < 0 ? 0 : (P.causal ? qa + 2 : P.n_qt);
+    }
+    I.n0 = P.causal ? I.qt0 + 1 : P.n_qt;
     return I;
 }
 
 template <int NB>   // 64-column blocks per tile: 1 (every head at most 64 wide) or 2
 struct FwdCfg {
     static constexpr int kTileBytes = NB * kBlockBytes;
-    static constexpr int QS = NB == 1 ? 2 : 1;                     // buffers of the pair of Q tiles
-    static constexpr int kSmem = (2 * QS + 4) * kTileBytes + 1024 + 256;
+    static constexpr int QS = NB == 1 ? 2 : 1;                     // buffers of a stream's Q tile
+    static constexpr int ST = NB == 1 ? 4 : 2;                     // stages of the K and of the V tiles
+    static constexpr int kRowBytes = (2 * 2 + 2 * 2) * kTile * 4;  // [buffer][stream][row]: factor of the outputs, then 1 / sum
+    static constexpr int kSmem = (2 * QS + 2 * ST) * kTileBytes + kRowBytes + 1024 + 512;
     static constexpr int kOCols = NB * 64;                          // columns of an output tile
-    static constexpr int CH = NB == 1 ? 32 : 16;                    // score columns a thread holds at a time (two such buffers)
-    // TMEM columns of stream x: scores, output tile, probabilities (narrow heads: a region of their own, so that the
-    // next score tile never waits for the second product; wide heads: over the scores they were made from)
+    // TMEM columns of stream x: scores, output, probabilities (narrow heads: a region of their own, so that the scores of the
+    // next key block are computed while these are made; wide heads: over the scores they were made from)
     static __device__ __forceinline__ uint32_t col_s(uint32_t x) { return 128u * x; }
     static __device__ __forceinline__ uint32_t col_o(uint32_t x) { return 256u + kOCols * x; }
     static __device__ __forceinline__ uint32_t col_p(uint32_t x) { return NB == 1 ? 384u + 64u * x : 128u * x; }
+    static constexpr bool kEarly = NB == 1;                         // scores one block ahead of the probabilities
+    static_assert(kSmem <= 232448, "shared memory of a block");
 };
 
 template <int NB>
 __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_constant__ AttnFwdParams P) {
     using Cfg = FwdCfg<NB>;
-    constexpr int kTileBytes = Cfg::kTileBytes;
-    constexpr int QS = Cfg::QS;
+    constexpr int kTileBytes = Cfg::kTileBytes, QS = Cfg::QS, ST = Cfg::ST;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - raw_addr);
-    const uint32_t sQ = base, sK = sQ + 2 * QS * kTileBytes, sV = sK + 2 * kTileBytes;
-    uint8_t* tail = smem + (2 * QS + 4) * kTileBytes;
+    const uint32_t sQ = base, sK = sQ + 2 * QS * kTileBytes, sV = sK + ST * kTileBytes;   // Q: [stage][stream]
+    float* row_factor = reinterpret_cast<float*>(smem + (2 * QS + 2 * ST) * kTileBytes);    // [buffer][stream][row]
+    float* row_inv = row_factor + 4 * kTile;                                                // [buffer][stream][row]
+    uint8_t* tail = smem + (2 * QS + 2 * ST) * kTileBytes + Cfg::kRowBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 24 * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 24 * 8 + 8);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 48 * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 48 * 8 + 8);
     const uint32_t bar0 = smem_u32(bars);
-    auto q_full = [&](uint32_t s) { return bar0 + 8u * s; };
-    auto q_empty = [&](uint32_t s) { return bar0 + 8u * (2 + s); };
-    // K and V tiles have rings of their own: a K stage is free as soon as the score products that read it are done
-    // (one step earlier than the V stage), so the load of the next K tile is not held up by the second products
-    auto k_full = [&](uint32_t s) { return bar0 + 8u * (4 + s); };
-    auto k_empty = [&](uint32_t s) { return bar0 + 8u * (6 + s); };
-    auto v_full = [&](uint32_t s) { return bar0 + 8u * (8 + s); };
-    auto v_empty = [&](uint32_t s) { return bar0 + 8u * (10 + s); };
-    // per stream: score tile complete, probabilities written, output tile complete, pass-2 token
-    auto s_full = [&](uint32_t x) { return bar0 + 8u * (12 + x); };
-    auto p_full = [&](uint32_t x) { return bar0 + 8u * (14 + x); };
-    auto o_full = [&](uint32_t x) { return bar0 + 8u * (16 + x); };
-    auto token = [&](uint32_t x) { return bar0 + 8u * (18 + x); };
+    auto q_full = [&](uint32_t x, uint32_t s) { return bar0 + 8u * (2 * x + s); };
+    auto q_empty = [&](uint32_t x, uint32_t s) { return bar0 + 8u * (4 + 2 * x + s); };
+    auto k_full = [&](uint32_t s) { return bar0 + 8u * (8 + s); };
+    auto k_empty = [&](uint32_t s) { return bar0 + 8u * (12 + s); };
+    auto v_full = [&](uint32_t s) { return bar0 + 8u * (16 + s); };
+    auto v_empty = [&](uint32_t s) { return bar0 + 8u * (20 + s); };
+    // per stream: scores complete; scores in registers; product with the probabilities done.  In pairs, used alternately, where
+    // a warp may arrive for one step before every other has looked at the step before: probabilities and rescaled output ready,
+    // factors of the rows written, sums of the rows written.
+    auto s_full = [&](uint32_t x) { return bar0 + 8u * (24 + x); };
+    auto s_read = [&](uint32_t x) { return bar0 + 8u * (26 + x); };
+    auto pv_done = [&](uint32_t x) { return bar0 + 8u * (28 + x); };
+    auto p_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (30 + 2 * x + b); };
+    auto f_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (34 + 2 * x + b); };
+    auto l_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (38 + 2 * x + b); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_kt = (P.seq + kTile - 1) / kTile;
     if (threadIdx.x == 0) {
-        for (uint32_t s = 0; s < 2; ++s) {
-            mbar_init(q_full(s), 1);
-            mbar_init(q_empty(s), 1);
+        for (uint32_t x = 0; x < 2; ++x) {
+            for (uint32_t s = 0; s < 2; ++s) {
+                mbar_init(q_full(x, s), 1);
+                mbar_init(q_empty(x, s), 1);
+                mbar_init(p_full(x, s), 8);       // (one arrival per softmax warp and per scaling warp of the stream)
+                mbar_init(f_full(x, s), 4);
+                mbar_init(l_full(x, s), 4);
+            }
+            mbar_init(s_full(x), 1);
+            mbar_init(s_read(x), 4);
+            mbar_init(pv_done(x), 1);
+        }
+        for (uint32_t s = 0; s < 4; ++s) {
             mbar_init(k_full(s), 1);
-            mbar_init(k_empty(s), 1);
+            mbar_init(k_empty(s), 2);             // both streams
             mbar_init(v_full(s), 1);
-            mbar_init(v_empty(s), 1);
-            mbar_init(s_full(s), 1);
-            mbar_init(p_full(s), 128);
-            mbar_init(o_full(s), 1);
-            mbar_init(token(s), 128);
+            mbar_init(v_empty(s), 2);
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -169,232 +206,330 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     const uint32_t tmem_base = *tmem_holder;
     pdl_wait();
 
+    // K / V stage and phase of a tile (solo: tiles and stages are numbered per stream)
+    const bool solo = P.items == ITEMS_SOLO;
+    auto stage = [&](uint32_t tile, uint32_t x) -> uint32_t { return solo ? 2 * (tile % (ST / 2)) + x : tile % ST; };
+    auto phase = [&](uint32_t tile) -> uint32_t { return (solo ? tile / (ST / 2) : tile / ST) & 1u; };
+
     if (warp == 0) {
-        // ------------------------------------------------------------------ producer
+        // ------------------------------------------------------------------ loads
         if (elect_one()) {
-            uint32_t g = 0, qi = 0;
+            uint32_t t = 0, round = 0;                              // K / V tiles (solo: of a stream) and items before this item
             bool ok = true;
-            for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++qi)) {
-                const Item I = decode_item(it, P.n_qt, P.n_heads, P.batch, n_kt, P.causal);
-                const int qoff = P.heads.qk_off[I.h], koff = P.heads.k_off[I.h], voff = P.heads.v_off[I.h];
-                const int nbq = (P.heads.qk_w[I.h] + 63) >> 6, nbv = (P.heads.vo_w[I.h] + 63) >> 6;
-                const int row0 = I.b * P.seq;
-                const uint32_t qs = qi % QS;
-                if (!(ok = mbar_wait(q_empty(qs), ((qi / QS) & 1u) ^ 1u, abort_flag, 11, P.status, P.wait_limit_ns))) break;
-                const int n_tiles = I.n_b > 0 ? 2 : 1;
-                mbar_expect_tx(q_full(qs), n_tiles * nbq * kBlockBytes);
-                for (int x = 0; x < n_tiles; ++x)
-                    for (int blk = 0; blk < nbq; ++blk)
-                        tma_load_2d(sQ + (2 * qs + x) * kTileBytes + blk * kBlockBytes, &P.map_q, qoff + 64 * blk,
-                                    row0 + (2 * I.qp + x) * kTile, q_full(qs));
-                for (int j = 0; j < I.n; ++j, ++g) {
-                    const uint32_t st = g & 1;
-                    if (!(ok = mbar_wait(k_empty(st), ((g >> 1) & 1u) ^ 1u, abort_flag, 11, P.status, P.wait_limit_ns))) break;
+            auto load_q = [&](uint32_t x, uint32_t n, int h, int row) -> bool {
+                const uint32_t qs = n % QS;
+                if (!mbar_wait(q_empty(x, qs), ((n / QS) & 1u) ^ 1u, abort_flag, 11, P.status, P.wait_limit_ns)) return false;
+                const int nb = (P.heads.qk_w[h] + 63) >> 6;
+                mbar_expect_tx(q_full(x, qs), nb * kBlockBytes);
+                for (int blk = 0; blk < nb; ++blk)
+                    tma_load_2d(sQ + (2 * qs + x) * kTileBytes + blk * kBlockBytes, &P.map_q, P.heads.qk_off[h] + 64 * blk, row, q_full(x, qs));
+                return true;
+            };
+            uint32_t nq0 = 0, nq1 = 0;
+            for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++round)) {
+                const FwdItem I = decode_item(it, P);
+                ok = load_q(0, nq0++, I.h0, I.b0 * P.seq + I.qt0 * kTile);
+                if (ok && I.n1 > 0) ok = load_q(1, nq1++, I.h1, I.b1 * P.seq + I.qt1 * kTile);
+                const int tiles = solo ? 1 + I.n1 : max(I.n0, I.n1);
+                for (int j = 0; ok && j < tiles; ++j) {
+                    const bool second = solo && j == 1;
+                    const uint32_t tile = solo ? t : t + j, st = stage(tile, second), ph = phase(tile) ^ 1u;
+                    const int h = second ? I.h1 : I.h0, y = (second ? I.b1 : I.b0) * P.seq + (solo ? 0 : j * kTile);
+                    const int nbq = (P.heads.qk_w[h] + 63) >> 6, nbv = (P.heads.vo_w[h] + 63) >> 6;
+                    if (!(ok = mbar_wait(k_empty(st), ph, abort_flag, 11, P.status, P.wait_limit_ns))) break;
                     mbar_expect_tx(k_full(st), nbq * kBlockBytes);
                     for (int blk = 0; blk < nbq; ++blk)
-                        tma_load_2d(sK + st * kTileBytes + blk * kBlockBytes, &P.map_k, koff + 64 * blk, row0 + j * kTile, k_full(st));
-                    if (!(ok = mbar_wait(v_empty(st), ((g >> 1) & 1u) ^ 1u, abort_flag, 11, P.status, P.wait_limit_ns))) break;
+                        tma_load_2d(sK + st * kTileBytes + blk * kBlockBytes, &P.map_k, P.heads.k_off[h] + 64 * blk, y, k_full(st));
+                    if (!(ok = mbar_wait(v_empty(st), ph, abort_flag, 11, P.status, P.wait_limit_ns))) break;
                     mbar_expect_tx(v_full(st), nbv * kBlockBytes);
                     for (int blk = 0; blk < nbv; ++blk)
-                        tma_load_2d(sV + st * kTileBytes + blk * kBlockBytes, &P.map_v, voff + 64 * blk, row0 + j * kTile, v_full(st));
+                        tma_load_2d(sV + st * kTileBytes + blk * kBlockBytes, &P.map_v, P.heads.v_off[h] + 64 * blk, y, v_full(st));
                 }
+                t += solo ? 1 : tiles;
             }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
-        if (elect_one()) {
-            uint32_t g = 0, qi = 0, cp[2] = {0, 0};       // cp[x]: probability tiles of stream x consumed so far
+    } else if (warp < 3) {
+        // ------------------------------------------------------------------ products of stream x
+        // The stream goes through all the tiles of its CTA, also those that only the other one uses (it hands them back unused).
+        const uint32_t x = warp - 1;
+        if (!(P.items == ITEMS_SINGLE && x == 1) && elect_one()) {
+            uint32_t nq = 0, ns = 0, np = 0;                        // items, score tiles and probability tiles of this stream so far
             bool ok = true;
-            for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++qi)) {
-                const Item I = decode_item(it, P.n_qt, P.n_heads, P.batch, n_kt, P.causal);
-                const int wq = P.heads.qk_w[I.h], wv = P.heads.vo_w[I.h];
-                const uint32_t qs = qi % QS;
-                if (!(ok = mbar_wait(q_full(qs), (qi / QS) & 1u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
-                const uint32_t idesc_s = make_idesc(kTile, kTile, 0, 0);
-                const uint32_t idesc_o = make_idesc(kTile, wv, 0, 1);
-                // S_x = Q_x K^T with the K tile in ring stage st
-                auto scores = [&](uint32_t x, uint32_t st) {
-#pragma unroll
-                    for (int ks = 0; ks < 4 * NB; ++ks) {
-                        if (ks >= (wq >> 4)) break;
-                        const uint32_t o = (ks >> 2) * kBlockBytes + (ks & 3) * 32;
-                        tc_mma_bf16(tmem_base + Cfg::col_s(x), make_smem_desc(sQ + (2 * qs + x) * kTileBytes + o, 16, 1024),
-                                    make_smem_desc(sK + st * kTileBytes + o, 16, 1024), idesc_s, ks != 0 ? 1u : 0u);
-                    }
-                    tc_commit(s_full(x));
-                };
-                // O_tile_x = P_x V over the 128 keys of the block in ring stage st
-                auto outputs = [&](uint32_t x, uint32_t st) -> bool {
-                    if (!mbar_wait(p_full(x), cp[x] & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
-                    ++cp[x];
-                    tc_fence_after();
-#pragma unroll
-                    for (int ks = 0; ks < kTile / 16; ++ks)
-                        tc_mma_bf16_ts(tmem_base + Cfg::col_o(x), tmem_base + Cfg::col_p(x) + 8 * ks,
-                                       make_smem_desc(sV + st * kTileBytes + ks * 2048, kBlockBytes, 1024), idesc_o, ks != 0 ? 1u : 0u);
-                    tc_commit(o_full(x));
+            // the tile a step works on: tile number, widths of the head, key block, and how many of the item's key blocks are this stream's
+            struct Slot {
+                uint32_t tile;
+                int wq, wv, j, n, n_max;
+                bool valid;
+            };
+            uint32_t round = 0;
+            auto item_start = [&](Slot& d) {
+                const int it = dealt_item(round);
+                d.valid = it < P.n_items;
+                if (!d.valid) return;
+                const FwdItem I = decode_item(it, P);
+                d.wq = P.heads.qk_w[x ? I.h1 : I.h0];
+                d.wv = P.heads.vo_w[x ? I.h1 : I.h0];
+                d.j = 0;
+                d.n = x ? I.n1 : I.n0;
+                d.n_max = solo ? 1 : max(I.n0, I.n1);
+                if (solo && d.n == 0) d.valid = false;               // (the odd unit out is the last item's)
+            };
+            auto release = [&](uint32_t bar) {                      // once the products issued so far are done
+                tc_commit(bar);
+                if (P.items != ITEMS_SHARED) tc_commit(bar);         // (in the other stream's place)
+            };
+            // S_x = Q_x K^T.  On narrow heads the scores of the step before must be in registers; on wide heads this comes after the
+            // product that read the probabilities made from them.
+            auto scores = [&](const Slot& d) -> bool {
+                const uint32_t st = stage(d.tile, x);
+                if (!mbar_wait(k_full(st), phase(d.tile), abort_flag, 12, P.status, P.wait_limit_ns)) return false;
+                if (d.j >= d.n) {
+                    mbar_arrive(k_empty(st));
                     return true;
-                };
-                if (!(ok = mbar_wait(k_full(g & 1), (g >> 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
-                tc_fence_after();
-                scores(0, g & 1);
-                if (I.n_b > 0) scores(1, g & 1);
-                tc_commit(k_empty(g & 1));
-                for (int j = 0; j < I.n; ++j, ++g) {
-                    const uint32_t st = g & 1, nx = (g + 1) & 1;
-                    if (!(ok = mbar_wait(v_full(st), (g >> 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
-                    if (j + 1 < I.n && !(ok = mbar_wait(k_full(nx), ((g + 1) >> 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns))) break;
-                    tc_fence_after();
-                    if (j < I.n_a && !(ok = outputs(0, st))) break;
-                    if (j + 1 < I.n_a) scores(0, nx);
-                    if (j < I.n_b && !(ok = outputs(1, st))) break;
-                    tc_commit(v_empty(st));
-                    if (j + 1 < I.n_b) scores(1, nx);
-                    if (j + 1 < I.n) tc_commit(k_empty(nx));
                 }
-                if (ok) tc_commit(q_empty(qs));
+                const uint32_t qs = nq % QS;
+                if (d.j == 0 && !mbar_wait(q_full(x, qs), (nq / QS) & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
+                const int steps = d.wq >> 4, cols = min(kTile, P.seq - d.j * kTile);     // keys of the tile, in whole steps of 16
+                const uint32_t idesc = make_idesc(kTile, (cols + 15) & ~15, 0, 0);
+                const uint64_t dq = make_smem_desc(sQ + (2 * qs + x) * kTileBytes, 16, 1024), dk = make_smem_desc(sK + st * kTileBytes, 16, 1024);
+                // (the wait that decides when the products can go comes last, with all their operands at hand)
+                if (Cfg::kEarly && ns > 0 && !mbar_wait(s_read(x), (ns - 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
+                ++ns;
+                tc_fence_after();
+#pragma unroll
+                for (int ks = 0; ks < 4 * NB; ++ks) {
+                    const uint32_t o = ((ks >> 2) * kBlockBytes + (ks & 3) * 32) >> 4;
+                    if (ks < steps) tc_mma_bf16(tmem_base + Cfg::col_s(x), dq + o, dk + o, idesc, ks != 0 ? 1u : 0u);
+                }
+                tc_commit(s_full(x));
+                release(k_empty(st));
+                if (d.j == d.n - 1) {
+                    tc_commit(q_empty(x, qs));
+                    ++nq;
+                }
+                return true;
+            };
+            // O_x (+)= P_x V over the keys of the tile
+            auto outputs = [&](const Slot& d) -> bool {
+                const uint32_t st = stage(d.tile, x);
+                if (!mbar_wait(v_full(st), phase(d.tile), abort_flag, 12, P.status, P.wait_limit_ns)) return false;
+                if (d.j >= d.n) {
+                    mbar_arrive(v_empty(st));
+                    return true;
+                }
+                const int steps = (min(kTile, P.seq - d.j * kTile) + 15) >> 4;
+                const uint32_t idesc = make_idesc(kTile, d.wv, 0, 1);
+                const uint64_t dv = make_smem_desc(sV + st * kTileBytes, kBlockBytes, 1024);
+                if (!mbar_wait(p_full(x, np & 1u), (np >> 1) & 1u, abort_flag, 12, P.status, P.wait_limit_ns)) return false;
+                ++np;
+                tc_fence_after();
+#pragma unroll
+                for (int ks = 0; ks < kTile / 16; ++ks)
+                    if (ks < steps) tc_mma_bf16_ts(tmem_base + Cfg::col_o(x), tmem_base + Cfg::col_p(x) + 8 * ks, dv + 128 * ks, idesc, (d.j | ks) != 0 ? 1u : 0u);
+                tc_commit(pv_done(x));
+                release(v_empty(st));
+                return true;
+            };
+            Slot cur, nxt;
+            cur.valid = false;
+            nxt.tile = 0;
+            item_start(nxt);
+            while (ok && (cur.valid || nxt.valid)) {
+                if (Cfg::kEarly && nxt.valid) ok = scores(nxt);
+                if (ok && cur.valid) ok = outputs(cur);
+                if (ok && !Cfg::kEarly && nxt.valid) ok = scores(nxt);
+                cur = nxt;
+                if (nxt.valid) {
+                    ++nxt.tile;
+                    if (++nxt.j == nxt.n_max) {
+                        ++round;
+                        item_start(nxt);
+                    }
+                }
             }
         }
-    } else {
-        // ------------------------------------------------------------------ softmax
-        const uint32_t x = static_cast<uint32_t>(warp - 2) >> 2;           // stream
+    } else if (warp >= 4 && warp < 12) {
+        // ------------------------------------------------------------------ scaling of the outputs of stream x
+        const uint32_t x = static_cast<uint32_t>(warp - 4) >> 2;
         const int row = (warp & 3) * 32 + lane;
-        const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        const uint32_t tS = t_lane + Cfg::col_s(x), tO = t_lane + Cfg::col_o(x), tP = t_lane + Cfg::col_p(x);
-        constexpr int CH = Cfg::CH, NC = kTile / CH;
-        constexpr int kOwn = Cfg::kOCols;
-        uint32_t cs = 0, turn = 0;                                          // tiles of this stream so far; turns of the token
+        const uint32_t tO = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + Cfg::col_o(x);
+        uint32_t ns = 0, nf = 0, nl = 0, round = 0;                  // steps, factors, items of this stream so far
         bool ok = true;
-        const int64_t T = static_cast<int64_t>(P.batch) * P.seq;
-        uint32_t round = 0;
         for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++round)) {
-            const Item I = decode_item(it, P.n_qt, P.n_heads, P.batch, n_kt, P.causal);
-            const int n_own = x == 0 ? I.n_a : I.n_b;
-            const int wv = P.heads.vo_w[I.h];
-            const int q_pos = (2 * I.qp + static_cast<int>(x)) * kTile + row;   // position of this row in its sequence
-            const int limit = P.causal ? min(P.seq, q_pos + 1) : P.seq;     // keys [0, limit) are visible
-            float m = -INFINITY, l = 0.f, alpha_prev = 0.f;
-            float o[kOwn];
-#pragma unroll
-            for (int i = 0; i < kOwn; ++i) o[i] = 0.f;
-            // O = O * a + O_tile (the output tile of the previous key block)
-            auto fold_output = [&](float a) {
-                const f32x2 a2 = pack2(a, a);
-#pragma unroll
-                for (int c = 0; c < kOwn / 16; ++c) {
-                    if (c * 16 < wv) {
-                        uint32_t r[16];
-                        tc_ld16(tO + c * 16, r);
-                        tc_wait_ld(r);
-#pragma unroll
-                        for (int i = 0; i < 16; i += 2)     // (packed fp32: half the issue slots)
-                            unpack2(fma2(pack2(o[c * 16 + i], o[c * 16 + i + 1]), a2, pack2(r[i], r[i + 1])), o[c * 16 + i], o[c * 16 + i + 1]);
-                    }
-                }
-            };
-            for (int j = 0; j < I.n; ++j, ++turn) {
-                const bool active = j < n_own;
-                const int kv_base = j * kTile;
-                const bool masked = kv_base + kTile > limit;               // keys past the limit count as -inf
-                float m_new = m, alpha = 1.f;
-                if (active) {
-                    if (!(ok = mbar_wait(s_full(x), cs & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
-                    tc_fence_after();
-                    // pass 1: row maximum (four independent chains); the next chunk is in flight while one is reduced
-                    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    uint32_t ra[CH], rb[CH];
-                    tc_ld(tS, ra);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        uint32_t(&cur)[CH] = (c & 1) ? rb : ra;
-                        uint32_t(&nxt)[CH] = (c & 1) ? ra : rb;
-                        tc_wait_ld(cur);
-                        if (c + 1 < NC) tc_ld(tS + (c + 1) * CH, nxt);
-                        if (masked) {
-#pragma unroll
-                            for (int i = 0; i < CH; ++i)
-                                if (kv_base + c * CH + i >= limit) cur[i] = 0xff800000u;
-                        }
-#pragma unroll
-                        for (int i = 0; i < CH; i += 2) mx4[(i >> 1) & 3] = max3(mx4[(i >> 1) & 3], __uint_as_float(cur[i]), __uint_as_float(cur[i + 1]));
-                    }
-                    const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                    m_new = fmaxf(m, mx * P.scale_log2e);
-                    alpha = ex2(m - m_new);
-                    if (j > 0) {
-                        if (!(ok = mbar_wait(o_full(x), (cs - 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+            const FwdItem I = decode_item(it, P);
+            const int n_own = x ? I.n1 : I.n0, h = x ? I.h1 : I.h0, wv = P.heads.vo_w[h];
+            if (n_own == 0) continue;
+            for (int j = 0; j < n_own; ++j, ++ns) {
+                if (j > 0) {
+                    if (!(ok = mbar_wait(f_full(x, nf & 1u), (nf >> 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+                    const float a = row_factor[((nf & 1u) * 2 + x) * kTile + row];
+                    ++nf;
+                    if (__any_sync(0xffffffffu, a != 1.f)) {         // some row of the warp has a new maximum
+                        if (!(ok = mbar_wait(pv_done(x), (ns - 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
                         tc_fence_after();
-                        fold_output(alpha_prev);
+                        const f32x2 a2 = pack2(a, a);
+#pragma unroll 1
+                        for (int c = 0; c < wv; c += 16) {
+                            uint32_t r[16];
+                            tc_ld16(tO + c, r);
+                            tc_wait_ld(r);
+#pragma unroll
+                            for (int i = 0; i < 16; i += 2) {
+                                float u, v;
+                                unpack2(mul2(pack2(r[i], r[i + 1]), a2), u, v);
+                                r[i] = __float_as_uint(u);
+                                r[i + 1] = __float_as_uint(v);
+                            }
+                            tc_st(tO + c, r);
+                        }
+                        tc_wait_st();
+                        tc_fence_before();
                     }
                 }
-                // the token: stream 0 goes first, then the streams alternate
-                if (!(ok = mbar_wait(token(x), x == 0 ? (turn & 1u) ^ 1u : turn & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
-                float rs4[4] = {0.f, 0.f, 0.f, 0.f};
-                if (active) {
-                    // pass 2: p = 2^(s * c - m_new) (2^-inf = 0 for the masked keys), row sum, P as packed bf16 into TMEM
-                    uint32_t ra[CH], rb[CH];
-                    const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), nm2 = pack2(-m_new, -m_new);
-                    f32x2 acc2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
-                    tc_ld(tS, ra);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        uint32_t(&cur)[CH] = (c & 1) ? rb : ra;
-                        uint32_t(&nxt)[CH] = (c & 1) ? ra : rb;
-                        tc_wait_ld(cur);
-                        if (c + 1 < NC) tc_ld(tS + (c + 1) * CH, nxt);
-                        if (masked) {
-#pragma unroll
-                            for (int i = 0; i < CH; ++i)
-                                if (kv_base + c * CH + i >= limit) cur[i] = 0xff800000u;
-                        }
-                        uint32_t pk[CH / 2];
-#pragma unroll
-                        for (int i = 0; i < CH; i += 2) {
-                            float x0, x1;
-                            unpack2(fma2(pack2(cur[i], cur[i + 1]), c2, nm2), x0, x1);
-                            const float p0 = ex2(x0), p1 = ex2(x1);
-                            acc2[(i >> 1) & 1] = add2(acc2[(i >> 1) & 1], pack2(p0, p1));
-                            pk[i >> 1] = pack_bf16(p0, p1);
-                        }
-                        tc_st(tP + c * (CH / 2), pk);
-                    }
-                    unpack2(acc2[0], rs4[0], rs4[1]);
-                    unpack2(acc2[1], rs4[2], rs4[3]);
-                }
-                mbar_arrive(token(x ^ 1u));
-                if (active) {
-                    tc_wait_st();
-                    tc_fence_before();
-                    mbar_arrive(p_full(x));
-                    l = fmaf(l, alpha, (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]));
-                    m = m_new;
-                    alpha_prev = alpha;
-                    ++cs;
-                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_full(x, ns & 1u));
             }
             if (!ok) break;
-            if (n_own > 0) {
-                if (!(ok = mbar_wait(o_full(x), (cs - 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
-                tc_fence_after();
-                fold_output(alpha_prev);
+            // the item's output rows: times 1 / sum, to memory
+            if (!(ok = mbar_wait(l_full(x, nl & 1u), (nl >> 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+            if (!(ok = mbar_wait(pv_done(x), (ns - 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+            tc_fence_after();
+            const float inv = row_inv[((nl & 1u) * 2 + x) * kTile + row];
+            ++nl;
+            const int q_pos = (x ? I.qt1 : I.qt0) * kTile + row;
+            uint16_t* dst = P.ctx + (static_cast<int64_t>(x ? I.b1 : I.b0) * P.seq + q_pos) * P.ld_ctx + P.heads.vo_off[h];
+#pragma unroll 1
+            for (int c = 0; c < wv; c += 16) {
+                uint32_t r[16];
+                tc_ld16(tO + c, r);
+                tc_wait_ld(r);
                 if (q_pos < P.seq) {
-                    const int64_t t = static_cast<int64_t>(I.b) * P.seq + q_pos;
-                    const float inv = 1.f / l;
-                    uint16_t* dst = P.ctx + t * P.ld_ctx + P.heads.vo_off[I.h];
-#pragma unroll
-                    for (int c = 0; c < kOwn / 8; ++c) {
-                        if (c * 8 < wv) {
-                            uint4 v;
-                            v.x = pack_bf16(o[c * 8 + 0] * inv, o[c * 8 + 1] * inv);
-                            v.y = pack_bf16(o[c * 8 + 2] * inv, o[c * 8 + 3] * inv);
-                            v.z = pack_bf16(o[c * 8 + 4] * inv, o[c * 8 + 5] * inv);
-                            v.w = pack_bf16(o[c * 8 + 6] * inv, o[c * 8 + 7] * inv);
-                            *reinterpret_cast<uint4*>(dst + c * 8) = v;
-                        }
-                    }
-                    P.lse[static_cast<int64_t>(I.h) * T + t] = m * 0.6931471805599453f + logf(l);
+                    uint4 v0, v1;
+                    v0.x = pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv);
+                    v0.y = pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv);
+                    v0.z = pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv);
+                    v0.w = pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv);
+                    v1.x = pack_bf16(__uint_as_float(r[8]) * inv, __uint_as_float(r[9]) * inv);
+                    v1.y = pack_bf16(__uint_as_float(r[10]) * inv, __uint_as_float(r[11]) * inv);
+                    v1.z = pack_bf16(__uint_as_float(r[12]) * inv, __uint_as_float(r[13]) * inv);
+                    v1.w = pack_bf16(__uint_as_float(r[14]) * inv, __uint_as_float(r[15]) * inv);
+                    *reinterpret_cast<uint4*>(dst + c) = v0;
+                    *reinterpret_cast<uint4*>(dst + c + 8) = v1;
                 }
             }
+            tc_fence_before();
+        }
+    } else if (warp >= 12) {
+        // ------------------------------------------------------------------ softmax of stream x
+        const uint32_t x = static_cast<uint32_t>(warp - 12) >> 2;
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t tS = t_lane + Cfg::col_s(x), tP = t_lane + Cfg::col_p(x);
+        uint32_t ns = 0, nf = 0, nl = 0, round = 0;                         // steps, factors, items of this stream so far
+        bool ok = true;
+        for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++round)) {
+            const FwdItem I = decode_item(it, P);
+            const int n_own = x ? I.n1 : I.n0;
+            if (n_own == 0) continue;
+            const int q_base = (x ? I.qt1 : I.qt0) * kTile, q_pos = q_base + row;   // position of this row in its sequence
+            const int limit = P.causal ? min(P.seq, q_pos + 1) : P.seq;     // keys [0, limit) are visible to the row,
+            const int w_limit = P.causal ? min(P.seq, q_base + ((warp & 3) + 1) * 32) : P.seq;   // and these to some row of the warp
+            const int w_first = P.causal ? min(P.seq, q_base + (warp & 3) * 32 + 1) : P.seq;     // every row of the warp sees these
+            float m = -INFINITY, l = 0.f;
+            for (int j = 0; j < n_own; ++j, ++ns) {
+                const int kv_base = j * kTile;
+                // columns with a visible key, and those that the product reads (zeros beyond the first)
+                const int n_vis = min(kTile, w_limit - kv_base), n_pv = min(kTile, P.seq - kv_base);
+                if (!(ok = mbar_wait(s_full(x), ns & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+                tc_fence_after();
+                // row maximum, 64 columns at a time; keys past the limit count as -inf (and are left so for the second pass)
+                float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+                for (int c = 0; c < n_vis; c += 64) {
+                    uint32_t a[32], b[32];
+                    tc_ld32(tS + c, a);
+                    tc_ld32(tS + c + 32, b);
+                    tc_wait_ld(a);
+                    tc_wait_ld(b);
+                    if (kv_base + c + 64 > w_first) {
+                        const int vis = limit - kv_base - c;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            if (i >= vis) a[i] = 0xff800000u;
+                            if (i + 32 >= vis) b[i] = 0xff800000u;
+                        }
+                        tc_st32(tS + c, a);
+                        tc_st32(tS + c + 32, b);
+                        tc_wait_st();
+                    }
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        mx4[(i >> 1) & 1] = max3(mx4[(i >> 1) & 1], __uint_as_float(a[i]), __uint_as_float(a[i + 1]));
+                        mx4[2 + ((i >> 1) & 1)] = max3(mx4[2 + ((i >> 1) & 1)], __uint_as_float(b[i]), __uint_as_float(b[i + 1]));
+                    }
+                }
+                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+                const float m_new = fmaxf(m, mx * P.scale_log2e), alpha = ex2(m - m_new);
+                if (j > 0) {                                                // the output row is rescaled while this thread exponentiates
+                    row_factor[((nf & 1u) * 2 + x) * kTile + row] = alpha;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(f_full(x, nf & 1u));
+                    ++nf;
+                }
+                // p = 2^(s * c - m_new), packed to bf16, and the row sum
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};
+                auto exponentiate = [&](uint32_t (&a)[32]) {               // 32 scores -> 16 packed pairs, in place
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) {
+                        const float p0 = ex2(fmaf(__uint_as_float(a[i]), P.scale_log2e, -m_new)), p1 = ex2(fmaf(__uint_as_float(a[i + 1]), P.scale_log2e, -m_new));
+                        sum[i & 2] += p0;
+                        sum[(i & 2) + 1] += p1;
+                        a[i >> 1] = pack_bf16(p0, p1);
+                    }
+                };
+                int c = 0;
+#pragma unroll 1
+                for (; c < n_vis; c += 64) {
+                    uint32_t a[32], b[32];
+                    tc_ld32(tS + c, a);
+                    tc_ld32(tS + c + 32, b);
+                    tc_wait_ld(a);
+                    tc_wait_ld(b);
+                    if (Cfg::kEarly && c + 64 >= n_vis) {                   // the last of the scores are in registers
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(s_read(x));
+                    }
+                    exponentiate(a);
+                    if (Cfg::kEarly && c == 0 && ns > 0) {                  // the last probabilities have been read (wide heads: the scores came after that product)
+                        ok = mbar_wait(pv_done(x), (ns - 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns);
+                        tc_fence_after();
+                    }
+                    tc_st16(tP + (c >> 1), a);
+                    exponentiate(b);
+                    tc_st16(tP + (c >> 1) + 16, b);
+                }
+                if (c < n_pv) {                                             // (at most 64 columns that only later rows see)
+                    uint32_t z[32];
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) z[i] = 0u;
+                    tc_st32(tP + (c >> 1), z);
+                }
+                if (!ok) break;
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_full(x, ns & 1u));
+                l = fmaf(l, alpha, (sum[0] + sum[1]) + (sum[2] + sum[3]));
+                m = m_new;
+            }
+            if (!ok) break;
+            row_inv[((nl & 1u) * 2 + x) * kTile + row] = 1.f / l;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(l_full(x, nl & 1u));
+            ++nl;
+            if (q_pos < P.seq)
+                P.lse[(static_cast<int64_t>(x ? I.h1 : I.h0) * P.batch + (x ? I.b1 : I.b0)) * P.seq + q_pos] = m * 0.6931471805599453f + logf(l);
         }
     }
 
@@ -413,7 +548,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 }
 
 // ------------------------------------------------------------------------------------------------
-// forward, output heads up to 32 wide: NS independent streams per CTA
+// forward, output heads up to 32 wide, longer sequences: NS independent streams per CTA
 // ------------------------------------------------------------------------------------------------
 // A work item is (sequence b, head h, one tile of 128 query rows).  A K / V tile holds NS slices of 64 keys; stream x
 // (four warps, thread = query row) owns slice x of every tile and keeps a softmax of its own over its keys: reference
@@ -1525,16 +1660,16 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     int* status = engine_status_ptr(&st);
     if (!status) return st;
     const int64_t T = batch * seq;
-    // Output heads up to 32 wide (and Q/K heads up to 64): the stream kernel (K / V tiles as slices of 64 keys); wider
-    // heads: two query tiles per CTA, with one or two 64-column blocks per tile.  The line is one of precision: the stream kernel
-    // rounds a row's probabilities to bf16 against a reference up to 2^32 below the row's largest, the kernel of wider heads
-    // against the largest itself, which is then exactly 1.  On rows that few keys dominate (scores of deviation 4, 1000
-    // positions, 64 wide) the outputs are 1.7e-3 off the values in 64 bits, all of it their own rounding; two streams
-    // per CTA for the wider heads too were 2.3e-3 off (and took 57 instead of 67 us at 4 x 1000 positions, 32 heads 48 wide on 8
-    // K/V heads, 467 instead of 495 at 2 x 4096, 32 heads 96 wide, but 31 instead of 27 at 8 x 512, 16 heads 64 wide).
+    // Output heads up to 32 wide (and Q/K heads up to 64) on sequences above two tiles: the kernel of key streams (K / V tiles as
+    // slices of 64 keys); everything else: two query tiles per CTA, with one or two 64-column blocks per tile.  The width is a
+    // line of precision: the stream kernel rounds a row's probabilities to bf16 against a reference up to 2^32 below the row's
+    // largest, the other kernel against the largest itself, which is then exactly 1.  On rows that few keys dominate (scores of
+    // deviation 4, 1000 positions, 64 wide) the outputs are 1.7e-3 off the values in 64 bits, all of it their own rounding;
+    // streams for the wider heads too were 2.3e-3 off.  The length is one of time (32 wide, 16 heads, 8192 positions,
+    // causal; streams / tiles, us): 25.6 / 18.4 in sequences of 128, 29.4 / 27.5 of 256, 34.2 / 36.2 of 512, 44.8 / 51 of 1024.
     int max_vo = 0;
     for (int h = 0; h < heads->n_heads; ++h) max_vo = std::max<int>(max_vo, heads->vo_w[h]);
-    const bool streams = max_w <= 64 && max_vo <= 32;
+    const bool streams = max_w <= 64 && max_vo <= 32 && seq > 2 * kTile;
     if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk)) != ECOSPA_OK) return st;
     if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk, streams ? 64 : kTile)) != ECOSPA_OK) return st;
     if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v, streams ? 64 : kTile)) != ECOSPA_OK) return st;
@@ -1543,7 +1678,10 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     P.n_heads = heads->n_heads;
     P.n_qt = static_cast<int32_t>(ceil_div(seq, kTile));
     P.causal = causal != 0;
-    const int64_t items = static_cast<int64_t>(streams ? P.n_qt : (P.n_qt + 1) / 2) * P.n_heads * batch;
+    const int64_t units = static_cast<int64_t>(P.n_heads) * batch, sms = std::max(1, engine_num_sms());
+    // Few query tiles: one per SM (2 x 160 positions, 12 heads: 10.4 -> 8.1 us)
+    P.items = units * P.n_qt <= sms ? ITEMS_SINGLE : P.n_qt == 1 ? ITEMS_SOLO : ITEMS_SHARED;
+    const int64_t items = streams || P.items == ITEMS_SINGLE ? units * P.n_qt : P.items == ITEMS_SOLO ? (units + 1) / 2 : units * ((P.n_qt + 1) / 2);
     if (items > INT32_MAX) return ECOSPA_ERR_UNSUPPORTED;
     P.n_items = static_cast<int32_t>(items);
     P.scale_log2e = scale * 1.4426950408889634f;

@@ -122,7 +122,21 @@ def test_forward_llama1b_sized_sampled_heads(causal):
         np.testing.assert_allclose(got_lse[h, rows], ref["lse"][0], rtol=0, atol=2e-3)
 
 
-NARROW = [20, 21, 25, 26, 30, 16, 32]      # output heads at most 32 wide take the kernel with independent key streams
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("batch,seq,k_qk,k_vo", [
+    (151, 40, [48], [40]),                  # sequences of one tile, two units to an item, an odd unit out
+    (51, 128, [100, 32, 70], [17, 128, 80]),   # the same on wide heads, tiles full
+    (3, 129, [64, 20], [64, 37]),           # few query tiles: one to an item; one key past a tile
+    (40, 257, [64, 37, 20], [48, 64, 33]),  # three query tiles: the odd one out is the first; one key past two tiles
+    (40, 352, [96, 128, 40], [72, 128, 100]),  # the same on wide heads, a last tile of 96 keys
+    (80, 250, [30, 20, 64], [32, 16, 25]),  # narrow output heads below the line of the stream kernel
+])
+def test_forward_item_forms(batch, seq, k_qk, k_vo, causal):
+    """Every way of pairing query tiles into work items, at the edges of tiles, with more items than blocks and fewer."""
+    run_forward(batch, seq, k_qk, k_vo, causal, seed=seq, d_h=max(64, max(k_qk + k_vo)))
+
+
+NARROW = [20, 21, 25, 26, 30, 16, 32]      # output heads at most 32 wide take the kernel with independent key streams (above 256 positions)
 
 
 @pytest.mark.parametrize("causal", [False, True])
