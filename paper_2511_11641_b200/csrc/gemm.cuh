@@ -57,15 +57,18 @@ struct GemmOp {
 constexpr int kMaxGemmOps = 16;
 
 // Column sums (bias gradients) that a launch takes along: up to three bf16 matrices with the same number of rows, none of
-// them written by the launch itself.  partial[chunk][col] = sum over the chunk's kSumRows rows.
-constexpr int kSumRows = 128;
+// them written by the launch itself.  Up to kSumWholeRows rows the launch writes the sums themselves (out); above, a finishing
+// launch adds the chunks: partial[chunk][col] = sum over the chunk's kSumRows rows.
+constexpr int kSumRows = 128, kSumWholeRows = 2048;
 struct SideSums {
     const uint16_t* M[3];
     float* partial[3];
+    void* out[3];
     int64_t ld[3];
     int32_t cols[3], col_tiles[3];   // col_tiles: tiles of 64 columns
     int32_t vec_ok[3];               // rows may be read 16 bytes at a time
     int32_t n_jobs, chunks;
+    int32_t whole, out_f32;          // write the sums themselves, as fp32 or bf16
     int64_t rows;
 };
 

@@ -234,7 +234,7 @@ ecospa_status_t run_ops(Ctx& cx, const GemmOp* ops, int n_ops, const SideSums* s
 }
 
 // Asks for the column sums of a bf16 matrix: `side` describes the reading (done by a product launch, which must not be the one
-// that writes the matrix), `fin` what the finishing launch adds up.  All matrices of a call have the same row count.  The
+// that writes the matrix), `fin` what the finishing launch adds up, where one is needed (see SideSums).  All matrices of a call have the same row count.  The
 // scratch of the chunk partials comes from the workspace here, so that a short workspace is reported before anything is
 // launched.  A null output skips the matrix.
 void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, void* out) {
@@ -254,7 +254,10 @@ void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, vo
     side.vec_ok[i] = aligned16(M.ptr) && M.ld % 8 == 0;
     side.rows = M.rows;
     side.chunks = fin.chunks = chunks;
-    fin.job[fin.n_jobs++] = ColsumFinal{partial, out, M.cols};
+    side.out[i] = out;
+    side.out_f32 = cx.dtype == ECOSPA_F32;
+    side.whole = M.rows <= kSumWholeRows;
+    if (!side.whole) fin.job[fin.n_jobs++] = ColsumFinal{partial, out, M.cols};
 }
 
 // Compacted weight with n real shared indices, as stored: shared-cols d_m x n, or shared-rows n x d_m.  Either

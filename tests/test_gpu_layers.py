@@ -418,3 +418,28 @@ def test_full_size_ffn_sampled(name, sparsity):
 @pytest.mark.parametrize("name,sparsity", [("gpt2m", 0.5), ("llama1b", 0.5), ("llama7b_layer", 0.75)])
 def test_full_size_qk_sampled(name, sparsity):
     run_qk_sampled(WL.WORKLOADS[name], sparsity)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("T", [1, 31, 33, 256, 257, 2048, 2049])
+def test_bias_gradient_row_counts(T, dtype):
+    """Column sums on both sides of the row count up to which the product launch writes them itself, and at the edges of the
+    rows a warp takes.  A sum goes through fewer than 84 fp32 additions (2^-24 each, of at most sum |x|), then the output's
+    rounding; an fp32 model's operands are rounded to bf16 first, on both sides."""
+    n, d_m = 24, 200
+    g = torch.Generator().manual_seed(T)
+    r = lambda *s: torch.randn(s, generator=g).to(dtype).to(DEV)
+    ctx, wo, dout = r(T, n), r(n, d_m), r(T, d_m)
+    dctx, dwo, dbo = torch.empty_like(ctx), torch.empty_like(wo), torch.full((d_m + 8,), 7.0, dtype=dtype, device=DEV)
+    code = B.BF16 if dtype == torch.bfloat16 else B.F32
+    ws = torch.empty(B.ecospa_proj_workspace_bytes(T, d_m, n, code) + 16, dtype=torch.uint8, device=DEV)
+    B.ecospa_coupled_vo_bwd_o(ctx, wo, n, dout, dctx, dwo, dbo, workspace=ws)
+    B.ecospa_device_status()
+    x = dout.bfloat16().double()
+    ref, mag = x.sum(0), x.abs().sum(0)
+    bound = 84 * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if dtype == torch.bfloat16 else 0.0)
+    assert torch.all((dbo[:d_m].double() - ref).abs() <= bound)
+    assert torch.all(dbo[d_m:] == 7.0)
+    first = dbo.clone()
+    B.ecospa_coupled_vo_bwd_o(ctx, wo, n, dout, dctx, dwo, dbo, workspace=ws)
+    assert torch.equal(first, dbo)
