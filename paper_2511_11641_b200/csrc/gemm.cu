@@ -1,7 +1,8 @@
 // Grouped persistent bf16 GEMM for sm_100a: TMA -> shared memory ring -> tcgen05.mma (fp32 accumulators
-// in TMEM, double buffered) -> fused epilogues.  Three forms of the same kernel:
-//   single  cta_group::1, one CTA per SM computes 128x128 tiles (3 stages of 2 x (16 KB A + 16 KB B)): launches that
+// in TMEM, double buffered) -> fused epilogues.  Four forms of the same kernel:
+//   slim    cta_group::1, one CTA per SM computes 128x64 tiles (4 stages of 2 x (16 KB A + 8 KB B)): launches that
 //           such tiles cover in one round
+//   single  the same with 128x128 tiles (3 stages of 2 x (16 KB A + 16 KB B)): launches that such tiles cover in one round
 //   wide    the same with 128x256 tiles (2 stages of 2 x (16 KB A + 32 KB B)): longer launches of at most 128 rows, where
 //           the second CTA of a pair would compute nothing
 //   pair    cta_group::2, a cluster of two CTAs computes 256x256 tiles: each CTA loads its 128 rows of A
@@ -43,16 +44,16 @@ namespace {
 constexpr int BM = 128, BK = 64;
 constexpr int kAStage = BM * BK * 2;        // 16 KB: 128 rows of A
 constexpr int kSub = 2;                     // 64-deep k-blocks per pipeline stage
-constexpr int kMaxStages = 3;
+constexpr int kMaxStages = 4;
 constexpr int kRingBytes = 192 * 1024;
 // Tile of a worker, by form: rows and columns, and the ring that brings its operands.
-enum TileForm { TILE_SINGLE = 0, TILE_PAIR = 1, TILE_WIDE = 2 };
+enum TileForm { TILE_SINGLE = 0, TILE_PAIR = 1, TILE_WIDE = 2, TILE_SLIM = 3 };
 template <int FORM>
 struct TileShape {
-    static constexpr int kM = FORM == TILE_PAIR ? 2 * BM : BM, kN = FORM == TILE_SINGLE ? 128 : 256;
+    static constexpr int kM = FORM == TILE_PAIR ? 2 * BM : BM, kN = FORM == TILE_SLIM ? 64 : FORM == TILE_SINGLE ? 128 : 256;
     static constexpr int kTmemCols = 2 * kN;               // two accumulators
     static constexpr int kBStage = (FORM == TILE_PAIR ? kN / 2 : kN) * BK * 2;   // B bytes of a CTA per k-block (a pair's holds half the tile's columns)
-    static constexpr int kStages = FORM == TILE_WIDE ? 2 : kMaxStages;
+    static constexpr int kStages = FORM == TILE_WIDE ? 2 : FORM == TILE_SLIM ? 4 : 3;
     static_assert(kStages * kSub * (kAStage + kBStage) == kRingBytes, "ring of a CTA");
 };
 constexpr int kAtomBytes = 64 * 64 * 2;     // one 64x64 bf16 swizzle atom of an MN-major operand
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     constexpr bool PAIR = FORM == TILE_PAIR;
     constexpr int kTileM = TileShape<FORM>::kM, kTileN = TileShape<FORM>::kN;
     constexpr int kTmemCols = TileShape<FORM>::kTmemCols, kStages = TileShape<FORM>::kStages, kBStage = TileShape<FORM>::kBStage;
-    constexpr int kHalfN = kTileN / 2;                       // columns of an epilogue warp
+    constexpr int kHalfN = FORM == TILE_SLIM ? 64 : kTileN / 2;   // columns of an epilogue warp (64-wide tiles: of the first four)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;       // 1024-byte aligned stage memory
@@ -712,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull_bar(a), 1);
-            mbar_init(tempty_bar(a), PAIR ? 2 * kEpiWarps : kEpiWarps);
+            mbar_init(tempty_bar(a), PAIR ? 2 * kEpiWarps : FORM == TILE_SLIM ? kEpiWarps / 2 : kEpiWarps);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -845,7 +846,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                             tma_load_2d(a_dst + kAtomBytes, ma, m0 + 64, k0, full_bar(stage));
                         }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {                                           // half of the tile's columns of B each
+                        for (int h = 0; h < (FORM == TILE_SLIM ? 1 : 2); ++h) {                 // half of the tile's columns of B each (64-wide tiles: all)
                             const CUtensorMap* mb = &P.maps[Q.map_b[seg][h]];
                             const int nc = n0 + h * Q.half1_n_off;
                             const uint32_t dst = b_dst + h * (kBStage / 2);
@@ -935,7 +936,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         else if (P.head.side.n_jobs > 0) side_sums(P.head.side, blockIdx.x + gridDim.x * ew, gridDim.x * kEpiWarps, lane);
         int it = 0;
         bool ok = true;
-        for (int round = 0; ok && round < P.head.rounds; ++round) {
+        const int rounds = FORM == TILE_SLIM && half == 1 ? 0 : P.head.rounds;
+        for (int round = 0; ok && round < rounds; ++round) {
             const int tile = scheduled_tile(P, worker, n_workers, round);
             if (tile < 0) continue;
             const DevProblem& Q = find_problem(P, tile);
@@ -1300,6 +1302,8 @@ DeviceState* gemm_setup(ecospa_status_t* st_out) {
         cudaError_t e = cudaDeviceGetAttribute(&D.num_sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_SINGLE, SmallParams>);
         if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_SINGLE, LargeParams>);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_SLIM, SmallParams>);
+        if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_SLIM, LargeParams>);
         if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_WIDE, SmallParams>);
         if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_WIDE, LargeParams>);
         if (e == cudaSuccess) e = allow_smem(gemm_kernel<TILE_PAIR, SmallParams>);
@@ -1512,17 +1516,21 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     // Beyond one round pairs need rows for both CTAs: launches of at most 128 rows (few tokens) take single CTAs with 128x256
     // tiles (Q/K/V of an 8192-wide model, 16 to 128 tokens: pairs 99-103 us, 128x128 tiles 86-89, 128x256 80-82; up to 4 tokens, where
     // every tile waits for the same few lines of X, 117, 120 and 123).
-    int64_t single_tiles = 0;
+    // Where tiles of half that width fit one round too, they take it: an SM then fetches 24 KB instead of 32 per 64-deep k-block, twice
+    // as many SMs fetch, and a tile's epilogue is half as long: 113 -> 103 us for the training step of 320 tokens, 768 wide.  (Not for
+    // the gated epilogue, whose tile is two operands side by side.)
+    int64_t single_tiles = 0, slim_tiles = 0;
     bool any_tall = false;
     for (int i = 0; i < n_ops; ++i) {
         const int per_tile = ops[i].epi == EPI_SWIGLU ? TileShape<TILE_SINGLE>::kN / 2 : TileShape<TILE_SINGLE>::kN;
         single_tiles += ceil_div(ops[i].M, BM) * ceil_div(ops[i].N, per_tile);
+        slim_tiles += ops[i].epi == EPI_SWIGLU ? g_num_sms + 1 : ceil_div(ops[i].M, BM) * ceil_div(ops[i].N, TileShape<TILE_SLIM>::kN);
         any_tall = any_tall || ops[i].M > BM;
     }
     const bool pairs = g_pair_mode != 0 && g_max_pairs >= 1 && any_tall;
-    const int form = single_tiles <= g_num_sms ? TILE_SINGLE : pairs ? TILE_PAIR : TILE_WIDE;
+    const int form = slim_tiles <= g_num_sms ? TILE_SLIM : single_tiles <= g_num_sms ? TILE_SINGLE : pairs ? TILE_PAIR : TILE_WIDE;
     const bool pair = form == TILE_PAIR;
-    const int tile_m = pair ? 2 * BM : BM, tile_n = form == TILE_SINGLE ? TileShape<TILE_SINGLE>::kN : TileShape<TILE_PAIR>::kN;
+    const int tile_m = pair ? 2 * BM : BM, tile_n = form == TILE_SLIM ? TileShape<TILE_SLIM>::kN : form == TILE_SINGLE ? TileShape<TILE_SINGLE>::kN : TileShape<TILE_PAIR>::kN;
 
     static thread_local LargeParams gp;
     MapTable T(gp);
@@ -1573,7 +1581,7 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
             for (int h = 0; h < 2; ++h) {
                 const Stored& b = (swiglu && h == 1) ? ks.b[1] : ks.b[0];
                 if (ks.b_mn ? (b.rows < k_end || b.cols != op.N) : (b.rows != op.N || b.cols < k_end)) return ECOSPA_ERR_INVALID;
-                if ((st = operand_map(T, b, ks.b_mn, pair, tile_n / 2, tile_n == 256, &map, &how)) != ECOSPA_OK) return st;
+                if ((st = operand_map(T, b, ks.b_mn, pair, std::max(64, tile_n / 2), tile_n == 256, &map, &how)) != ECOSPA_OK) return st;
                 Q.map_b[s][h] = static_cast<uint8_t>(map);
                 if (h == 0) {
                     Q.b_big[s] = how == FORM_BIG;
@@ -1615,6 +1623,7 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     const int workers = pair ? std::min(tiles, g_max_pairs) : std::min(tiles, g_num_sms);
     build_schedule(gp, workers);
     const cudaError_t e = pair ? launch_smallest_form<TILE_PAIR>(gp, T.n, workers, stream)
+                          : form == TILE_SLIM ? launch_smallest_form<TILE_SLIM>(gp, T.n, workers, stream)
                           : form == TILE_SINGLE ? launch_smallest_form<TILE_SINGLE>(gp, T.n, workers, stream)
                                                 : launch_smallest_form<TILE_WIDE>(gp, T.n, workers, stream);
     if (e != cudaSuccess) {

@@ -440,6 +440,9 @@ def test_bias_gradient_row_counts(T, dtype):
     bound = 84 * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if dtype == torch.bfloat16 else 0.0)
     assert torch.all((dbo[:d_m].double() - ref).abs() <= bound)
     assert torch.all(dbo[d_m:] == 7.0)
+    off = lambda got, want: float((got.double() - want).norm() / want.norm())     # the products beside the sums, in narrow tiles
+    assert off(dctx, dout.double() @ wo.double().t()) <= TOL
+    assert off(dwo, ctx.double().t() @ dout.double()) <= TOL
     first = dbo.clone()
     B.ecospa_coupled_vo_bwd_o(ctx, wo, n, dout, dctx, dwo, dbo, workspace=ws)
     assert torch.equal(first, dbo)
