@@ -25,8 +25,8 @@
 // Both passes are rolled loops of 64 columns: holding a block's 128 scores in registers, unrolled, was slower (163 -> 233 us at
 // 4 x 2048 positions, 32 heads 32 wide: warps waited for instructions, 4.0 of 15 cycles per issue, now 1.0).  Columns that
 // no row of a warp sees are skipped, keys past the end of the sequence also in the products.
-// Before (two streams in one thread's registers, a token between them) / now, us: 420 / 370 (2 x 4096, 32 heads 96 wide),
-// 59.3 / 53.1 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 8.5 (2 x 160, 12 heads 48 wide), 60.9 / 28.2 (60 x 48, 32 heads 64
+// Before (two streams in one thread's registers, a token between them) / now, us: 420 / 335 (2 x 4096, 32 heads 96 wide),
+// 59.3 / 53.0 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 7.9 (2 x 160, 12 heads 48 wide), 60.9 / 28.2 (60 x 48, 32 heads 64
 // wide), 41.8 / 18.9 (30 x 48, 32 heads 128 wide), 24.9 / 27.2 (8 x 512, 16 heads 64 wide, no mask).
 // Every mbarrier wait is bounded; on expiry the CTA records a code (11 loads, 12 products, 13 softmax and scaling) in the device
 // status word, lets copies land, frees TMEM and returns.
@@ -68,6 +68,7 @@ struct AttnFwdParams {
     HeadLayout heads;
     int32_t batch, seq, n_heads, n_qt, causal, n_items;
     int32_t items;                          // FwdItems
+    int32_t turns;                          // wide heads: the two streams exponentiate in turn
     float scale_log2e;                      // scale * log2(e): scores are exponentiated in base 2
     uint16_t* ctx;
     int64_t ld_ctx;
@@ -153,8 +154,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     float* row_inv = row_factor + 4 * kTile;                                                // [buffer][stream][row]
     uint8_t* tail = smem + (2 * QS + 2 * ST) * kTileBytes + Cfg::kRowBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 48 * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 48 * 8 + 8);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 52 * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 52 * 8 + 8);
     const uint32_t bar0 = smem_u32(bars);
     auto q_full = [&](uint32_t x, uint32_t s) { return bar0 + 8u * (2 * x + s); };
     auto q_empty = [&](uint32_t x, uint32_t s) { return bar0 + 8u * (4 + 2 * x + s); };
@@ -171,6 +172,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     auto p_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (30 + 2 * x + b); };
     auto f_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (34 + 2 * x + b); };
     auto l_full = [&](uint32_t x, uint32_t b) { return bar0 + 8u * (38 + 2 * x + b); };
+    // whose turn it is to exponentiate, per scheduler: warp q of stream 0 and warp q of stream 1 share one
+    auto turn_of = [&](uint32_t x, uint32_t q) { return bar0 + 8u * (42 + 4 * x + q); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -185,6 +188,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
             mbar_init(s_full(x), 1);
             mbar_init(s_read(x), 4);
             mbar_init(pv_done(x), 1);
+            for (uint32_t q = 0; q < 4; ++q) mbar_init(turn_of(x, q), 1);
         }
         for (uint32_t s = 0; s < 4; ++s) {
             mbar_init(k_full(s), 1);
@@ -425,12 +429,26 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
         const int row = (warp & 3) * 32 + lane;
         const uint32_t t_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t tS = t_lane + Cfg::col_s(x), tP = t_lane + Cfg::col_p(x);
+        // Wide heads: the streams exponentiate in turn, warp by warp.  Both at once they take as long for it, and then wait for their
+        // products at the same time too; the scores of narrow heads come a block ahead, and the turns cost more than they give.  (2 x
+        // 4096, 32 heads 96 wide 358 -> 335 us, 16 x 512, 80 wide, no mask 99 -> 88; 8 x 1024, 48 wide: 100 -> 120.)
+        const bool turns = NB == 2 && P.turns;
+        uint32_t turn = 0;
+        auto take_turn = [&]() -> bool {
+            return !turns || mbar_wait(turn_of(x, warp & 3), x == 0 ? (turn & 1u) ^ 1u : turn & 1u, abort_flag, 13, P.status, P.wait_limit_ns);
+        };
+        auto pass_turn = [&]() {
+            if (!turns) return;
+            ++turn;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(turn_of(x ^ 1u, warp & 3));
+        };
         uint32_t ns = 0, nf = 0, nl = 0, round = 0;                         // steps, factors, items of this stream so far
         bool ok = true;
         for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++round)) {
             const FwdItem I = decode_item(it, P);
             const int n_own = x ? I.n1 : I.n0;
-            if (n_own == 0) continue;
+            if (n_own == 0 && !turns) continue;
             const int q_base = (x ? I.qt1 : I.qt0) * kTile, q_pos = q_base + row;   // position of this row in its sequence
             const int limit = P.causal ? min(P.seq, q_pos + 1) : P.seq;     // keys [0, limit) are visible to the row,
             const int w_limit = P.causal ? min(P.seq, q_base + ((warp & 3) + 1) * 32) : P.seq;   // and these to some row of the warp
@@ -476,6 +494,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                     if (lane == 0) mbar_arrive(f_full(x, nf & 1u));
                     ++nf;
                 }
+                ok = take_turn();
+                if (!ok) break;
                 // p = 2^(s * c - m_new), packed to bf16, and the row sum
                 float sum[4] = {0.f, 0.f, 0.f, 0.f};
                 auto exponentiate = [&](uint32_t (&a)[32]) {               // 32 scores -> 16 packed pairs, in place
@@ -516,6 +536,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                     tc_st32(tP + (c >> 1), z);
                 }
                 if (!ok) break;
+                pass_turn();
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
@@ -523,7 +544,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
                 l = fmaf(l, alpha, (sum[0] + sum[1]) + (sum[2] + sum[3]));
                 m = m_new;
             }
+            for (int j = n_own; turns && ok && j < max(I.n0, I.n1); ++j) {   // (a stream without a tile left lets the other one go on)
+                ok = take_turn();
+                pass_turn();
+            }
             if (!ok) break;
+            if (n_own == 0) continue;
             row_inv[((nl & 1u) * 2 + x) * kTile + row] = 1.f / l;
             __syncwarp();
             if (lane == 0) mbar_arrive(l_full(x, nl & 1u));
@@ -1681,6 +1707,8 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     const int64_t units = static_cast<int64_t>(P.n_heads) * batch, sms = std::max(1, engine_num_sms());
     // Few query tiles: one per SM (2 x 160 positions, 12 heads: 10.4 -> 8.1 us)
     P.items = units * P.n_qt <= sms ? ITEMS_SINGLE : P.n_qt == 1 ? ITEMS_SOLO : ITEMS_SHARED;
+    // (Causal sequences of up to two tiles: 200 positions, 80 wide, 63 us without turns, 67 with; 768: 93 and 90.)
+    P.turns = P.items == ITEMS_SHARED && (!P.causal || P.n_qt > 2);
     const int64_t items = streams || P.items == ITEMS_SINGLE ? units * P.n_qt : P.items == ITEMS_SOLO ? (units + 1) / 2 : units * ((P.n_qt + 1) / 2);
     if (items > INT32_MAX) return ECOSPA_ERR_UNSUPPORTED;
     P.n_items = static_cast<int32_t>(items);
