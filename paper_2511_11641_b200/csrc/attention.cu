@@ -1164,7 +1164,9 @@ struct AttnBwdParams {
 // packed bf16 beside the scores.  Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products.  The
 // accumulators of the key-block kernel then leave no TMEM columns beside the score tiles: every thread writes its packed P^T and
 // dS^T over the scores it has made them from, and the buffer is free for the next scores when the products that read the
-// operands are done.  The query-block kernel has one accumulator (on heads up to 64 wide two, which the items take in turn).
+// operands are done.  On heads up to 64 wide the query-block kernel adds the products of even and of odd steps up in accumulators
+// of their own, which are added at the end: a sum in one accumulator would be twice as long (and 0.3 us per item shorter to write
+// out: 109.3 against 112.7 us at 4 x 1000, 32 heads 48 wide on 8, 98.3 against 99.4 at 8 x 1024, 16 heads 32 wide).
 // Wait codes: 14 / 15 / 16 (MODE 0 loads, products, compute) and 17 / 18 / 19 (MODE 1).
 constexpr int kStep = 64;                  // rows of a streamed block (queries in the key-block kernel, keys in the query-block kernel)
 template <int NB, int MODE>
@@ -1180,7 +1182,9 @@ struct BwdCfg {
     static_assert(kSmem <= 232448, "shared memory of a block");
 };
 
-template <int NB, int MODE, int NACC = 1>   // NACC = 2: the accumulators of two items side by side (of the key-block kernel: heads at most 32 wide)
+// NACC: accumulators.  Key-block kernel: 2 = those of two items side by side (heads at most 32 wide).  Query-block kernel: 3 or 4 (heads
+// at most 64 or 32 wide) that the halves of the items' sums take in turn, 64 or 32 columns each.
+template <int NB, int MODE, int NACC = 1>
 __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_constant__ AttnBwdParams P) {
     using Cfg = BwdCfg<NB, MODE>;
     constexpr int kTileBytes = Cfg::kTileBytes, kStrTileBytes = Cfg::kStrTileBytes, kStrBlockBytes = Cfg::kStrBlockBytes;
@@ -1189,16 +1193,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     // accumulating products (P^T and dS^T, or dS), two values per column
     constexpr uint32_t kAccIssuers = NB == 1 && MODE == 0 ? 2 : 1, kScoreIssuers = NB == 1 ? 1 : 2;
     constexpr uint32_t kColX = 0, kColY = 128, kColAcc = 256;
-    // accumulator `which` (0: dV or dQ, 1: dK) of set as
+    // accumulator `which` (0: dV, 1: dK) of set as, or accumulator as of the query-block kernel
     auto col_acc = [](int which, uint32_t as) -> uint32_t {
-        if (MODE == 1) return kColAcc + 64 * as;
+        if (MODE == 1) return kColAcc + (NACC == 4 ? 32 : 64) * as;
         return kColAcc + (NACC == 2 ? 64 * as + 32 * which : (NB == 1 ? 64 : 128) * which);
     };
     // operand `which` (0: P^T, 1: dS^T or dS) of 16 contraction steps from 16 ks on, in operand buffer ob.  (Over the scores a
     // thread's 32 columns become its first 16.)
     auto col_op = [](int which, uint32_t ob, uint32_t ks) -> uint32_t {
         if (Cfg::kOverlay) return (which == 0 ? kColX : kColY) + 64 * ob + 32 * (ks >> 1) + 8 * (ks & 1);
-        return 384 + (MODE == 0 ? 64 * which : 0) + 32 * ob + 8 * ks;
+        return (MODE == 0 ? 384 + 64 * which : 448) + 32 * ob + 8 * ks;
     };
     constexpr int kCodeBase = MODE == 0 ? 14 : 17;
     extern __shared__ uint8_t smem_raw[];
@@ -1223,11 +1227,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     auto xy_free = [&](uint32_t b) { return bar0 + 8u * (18 + b); };
     auto out_full = [&](uint32_t b) { return bar0 + 8u * (20 + b); };
     auto out_empty = [&](uint32_t b) { return bar0 + 8u * (22 + b); };
-    // accumulators: one set, or two that the items take in turn, each with its own pair of barriers
+    // accumulators: one set, or several that the items (or the halves of their sums) take in turn, each with its own pair of barriers
     auto acc_full = [&](uint32_t a) { return bar0 + 8u * (24 + a); };
-    auto acc_empty = [&](uint32_t a) { return bar0 + 8u * (26 + a); };
+    auto acc_empty = [&](uint32_t a) { return bar0 + 8u * (28 + a); };
     constexpr uint32_t n_acc = NACC;
-    static_assert(NACC == 1 || NB == 1, "two sets of accumulators need the narrow layout");
+    constexpr bool kHalfSums = MODE == 1 && NB == 1;             // sum 2 ri + (step & 1) of the item number ri, in accumulator (2 ri + (step & 1)) % n_acc
+    static_assert(kHalfSums ? NACC == 3 || NACC == 4 : NACC == 1 || (NACC == 2 && NB == 1), "several accumulators need the narrow layout");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -1245,7 +1250,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             mbar_init(out_full(b), kBwdComputeWarps / 2);
             mbar_init(out_empty(b), kAccIssuers);
         }
-        for (uint32_t a = 0; a < 2; ++a) {
+        for (uint32_t a = 0; a < 4; ++a) {
             mbar_init(acc_full(a), kAccIssuers);
             mbar_init(acc_empty(a), kBwdComputeWarps);
         }
@@ -1336,18 +1341,22 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         }
     };
     // The accumulating products number w0 .. w1 - 1 of every step.  Key-block kernel: 0 is dV += P^T dCtx_i (B = streamed b
-    // tile), 1 is dK += dS^T Q_i (B = streamed a tile); query-block kernel: 1 is dQ += dS K_j (B = streamed a tile).
+    // tile), 1 is dK += dS^T Q_i (B = streamed a tile); query-block kernel: 1 is dQ += dS K_j (B = streamed a tile), on heads up to
+    // 64 wide in two sums, over the even and over the odd steps.
     auto acc_role = [&](int w0, int w1) {
         uint32_t g = 0, ri = 0;
         bool ok = true;
         for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++ri)) {
             const BItem I = decode(it);
-            const uint32_t as = ri % n_acc;
+            auto wait_acc = [&](uint32_t n) -> bool {                // the accumulator that takes sum number n has been written out
+                return mbar_wait(acc_empty(n % n_acc), ((n / n_acc) & 1u) ^ 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns);
+            };
             for (int i = 0; i < I.n_steps; ++i, ++g) {
-                const uint32_t st = g % SS, ob = g & 1;
+                const uint32_t st = g % SS, ob = g & 1, n = kHalfSums ? 2 * ri + (i & 1) : ri, as = n % n_acc;
+                const int i_sum = kHalfSums ? i >> 1 : i;             // step of its sum
                 if (!(ok = mbar_wait(t_full(st), (g / SS) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
                 if (!(ok = mbar_wait(out_full(ob), (g >> 1) & 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
-                if (i == 0 && !(ok = mbar_wait(acc_empty(as), ((ri / n_acc) & 1u) ^ 1u, abort_flag, kCodeBase + 1, P.status, P.wait_limit_ns))) break;
+                if (i_sum == 0 && !(ok = wait_acc(n))) break;
                 tc_fence_after();
                 for (int which = w0; which < w1; ++which) {
                     const int wn = which == 0 ? P.heads.vo_w[I.h] : P.heads.qk_w[I.h];
@@ -1356,12 +1365,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     const uint64_t db = make_smem_desc(sStr + (2 * st + (which == 0 ? 1 : 0)) * kStrTileBytes, kStrBlockBytes, 1024);
 #pragma unroll
                     for (int ks = 0; ks < kStep / 16; ++ks)
-                        tc_mma_bf16_ts(acc, op + (Cfg::kOverlay ? 32 * (ks >> 1) + 8 * (ks & 1) : 8 * ks), db + 128 * ks, idesc, (i | ks) != 0 ? 1u : 0u);
+                        tc_mma_bf16_ts(acc, op + (Cfg::kOverlay ? 32 * (ks >> 1) + 8 * (ks & 1) : 8 * ks), db + 128 * ks, idesc, (i_sum | ks) != 0 ? 1u : 0u);
                 }
                 tc_commit(out_empty(ob));
                 tc_commit(t_empty(st));
             }
-            if (ok) tc_commit(acc_full(as));
+            if (kHalfSums) {                                         // (one step: the second sum is empty, its turn is taken all the same)
+                if (ok && I.n_steps == 1) ok = wait_acc(2 * ri + 1);
+                if (ok) {
+                    tc_commit(acc_full((2 * ri) % n_acc));
+                    tc_commit(acc_full((2 * ri + 1) % n_acc));
+                }
+            } else if (ok) {
+                tc_commit(acc_full(ri % n_acc));
+            }
         }
     };
 
@@ -1434,13 +1451,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
         struct Pend {
             int h, b, own;
             uint32_t ri;
-            bool on;
+            bool on, two;                                              // two: both halves of the sum have products
         };
-        Pend pend = {0, 0, 0, 0, false};
+        Pend pend = {0, 0, 0, 0, false, false};
         // writes an item's accumulators out once they are complete (every thread a quarter of the columns) and releases them
         auto flush = [&](const Pend& d) -> bool {
-            const uint32_t as = d.ri % n_acc;
-            if (!mbar_wait(acc_full(as), (d.ri / n_acc) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns)) return false;
+            const uint32_t n = kHalfSums ? 2 * d.ri : d.ri, as = n % n_acc, as2 = (n + 1) % n_acc;   // (as2: the second half's)
+            if (!mbar_wait(acc_full(as), (n / n_acc) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns)) return false;
+            if (kHalfSums && !mbar_wait(acc_full(as2), ((n + 1) / n_acc) & 1u, abort_flag, kCodeBase + 2, P.status, P.wait_limit_ns)) return false;
             tc_fence_after();
             const int pos = d.own * kTile + row;
             const bool live = pos < P.seq;
@@ -1452,7 +1470,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
                     if (col < w) {
                         uint32_t r[16];
                         tc_ld16(t_lane + colbase + col, r);
-                        tc_wait_ld(r);
+                        if (kHalfSums && d.two) {
+                            uint32_t r2[16];
+                            tc_ld16(t_lane + col_acc(0, as2) + col, r2);
+                            tc_wait_ld(r2);
+                            tc_wait_ld(r);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(r2[e]));
+                        } else {
+                            tc_wait_ld(r);
+                        }
                         if (live) {
                             uint4 v0, v1;
                             v0.x = pack_bf16(__uint_as_float(r[0]) * mul, __uint_as_float(r[1]) * mul);
@@ -1477,7 +1504,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty(as));
+            if (lane == 0) {
+                mbar_arrive(acc_empty(as));
+                if (kHalfSums) mbar_arrive(acc_empty(as2));
+            }
             return true;
         };
         for (int it = dealt_item(0); ok && it < P.n_items; it = dealt_item(++ri)) {
@@ -1571,7 +1601,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             if (!ok) break;
             if (pend.on && !(ok = flush(pend))) break;         // (an item without a step for this group)
             g = g_next;
-            pend = {I.h, I.b, I.own, ri, true};                // written out after the first step of the next item, when the last products into them have long landed
+            pend = {I.h, I.b, I.own, ri, true, I.n_steps > 1};                // written out after the first step of the next item, when the last products into them have long landed
         }
         if (ok && pend.on) flush(pend);
     }
@@ -1803,7 +1833,8 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
     std::call_once(once[dev & 63], [&] {
         e = cudaFuncSetAttribute(attn_bwd_kernel<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 0>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 0>::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<1, 1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<1, 1>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 0>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_bwd_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<2, 1>::kSmem);
         if (e == cudaSuccess)
@@ -1845,6 +1876,7 @@ extern "C" ecospa_status_t ecospa_coupled_attn_bwd(const void* Qc, const void* K
     P.n_items = items_q;
     grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     if (nb == 1)
-        return launch_pdl(attn_bwd_kernel<1, 1, 2>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)", BwdCfg<1, 1>::kSmem);
+        return launch_pdl(max_w <= 32 ? attn_bwd_kernel<1, 1, 4> : attn_bwd_kernel<1, 1, 3>, grid, kBwdThreads, stream, P,
+                          "attn_bwd_kernel (dQ)", BwdCfg<1, 1>::kSmem);
     return launch_pdl(attn_bwd_kernel<2, 1, 1>, grid, kBwdThreads, stream, P, "attn_bwd_kernel (dQ)", BwdCfg<2, 1>::kSmem);
 }

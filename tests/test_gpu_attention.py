@@ -355,6 +355,27 @@ def test_backward_block_config_in_full_and_bit_identical_reruns():
             assert torch.equal(x.view(torch.int16), y.view(torch.int16))
 
 
+@pytest.mark.parametrize("batch", [1, 40])
+@pytest.mark.parametrize("w", [16, 32, 48, 64])
+def test_query_gradient_sums_even_and_odd_key_blocks_apart(w, batch):
+    """Heads up to 64 wide: dQ is the sum over the even blocks of 64 keys plus the one over the odd blocks.  All dS are 2^-8 here (equal
+    scores over 256 keys, dP = 1, D = 0), the even blocks cancel at 2^38 and the odd ones add up to 1/2: exact in two sums, while one
+    fp32 sum over all blocks in order loses the first odd one."""
+    seq, H = 256, 8
+    T, off = batch * seq, [w * h for h in range(H)]
+    z = lambda: torch.zeros((T, H * w), dtype=torch.bfloat16, device=DEV)
+    Q, K, V, Ctx, dCtx, dQ, dK, dV = (z() for _ in range(8))
+    K.view(batch, 4, 64, H, w)[:, :, :, :, 3] = torch.tensor([2.0 ** 40, 1.0, -(2.0 ** 40), 1.0], device=DEV).view(1, 4, 1, 1)
+    V[:, ::w] = 1.0
+    dCtx[:, ::w] = 1.0
+    lse = torch.full((H * T,), float(np.log(seq)), device=DEV)
+    ws = torch.empty(B.ecospa_attn_workspace_bytes(batch, seq, H), dtype=torch.uint8, device=DEV)
+    B.ecospa_coupled_attn_bwd(Q, K, V, Ctx, dCtx, lse, batch, seq, B.heads(off, [w] * H, off, [w] * H), 1.0, False, dQ, dK, dV, ws)
+    B.ecospa_device_status()
+    got = dQ.view(T, H, w)
+    assert torch.all(got[:, :, 3] == 0.5) and int((got != 0).sum()) == T * H
+
+
 @pytest.mark.parametrize("causal", [False, True])
 def test_backward_llama1b_sized_sampled_heads(causal):
     batch, seq, H = 4, 2048, 32
