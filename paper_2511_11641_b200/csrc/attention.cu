@@ -8,8 +8,9 @@
 // Q K^T, and a zero column of V^c gives a zero column of Ctx) and off_h a multiple of 8, so that every tile load starts
 // on a 16-byte boundary and every contraction is a whole number of 16-deep MMA steps.
 //
-// Two forward kernels, one CTA per SM.  Output heads up to 32 wide (with Q/K heads up to 64) on sequences above two tiles take
-// the kernel of independent key streams further down (attn_fwd_ms_kernel); all others the kernel described here, 640 threads.
+// Two forward kernels, one CTA per SM.  Output heads up to 32 wide (with Q/K heads up to 64) take the kernel of independent key
+// streams further down (attn_fwd_ms_kernel) unless there are many sequences of up to two tiles (the rule stands in
+// ecospa_coupled_attn_fwd); all others take the kernel described here, 640 threads.
 // A work item is one or two tiles of 128 query rows, one per stream (see FwdItems); a CTA walks a static list of items (for
 // causal attention the long ones first).  Two neighbouring query tiles of a sequence and head share the K / V tiles.
 //   warp 0       one lane issues the TMA loads of the streams' Q tiles and of the K / V tiles (rings of 4 or 2 stages); a tile
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 }
 
 // ------------------------------------------------------------------------------------------------
-// forward, output heads up to 32 wide, longer sequences: NS independent streams per CTA
+// forward, output heads up to 32 wide, not many short sequences: NS independent streams per CTA
 // ------------------------------------------------------------------------------------------------
 // A work item is (sequence b, head h, one tile of 128 query rows).  A K / V tile holds NS slices of 64 keys; stream x
 // (four warps, thread = query row) owns slice x of every tile and keeps a softmax of its own over its keys: reference
@@ -1716,19 +1717,6 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     int* status = engine_status_ptr(&st);
     if (!status) return st;
     const int64_t T = batch * seq;
-    // Output heads up to 32 wide (and Q/K heads up to 64) on sequences above two tiles: the kernel of key streams (K / V tiles as
-    // slices of 64 keys); everything else: two query tiles per CTA, with one or two 64-column blocks per tile.  The width is a
-    // line of precision: the stream kernel rounds a row's probabilities to bf16 against a reference up to 2^32 below the row's
-    // largest, the other kernel against the largest itself, which is then exactly 1.  On rows that few keys dominate (scores of
-    // deviation 4, 1000 positions, 64 wide) the outputs are 1.7e-3 off the values in 64 bits, all of it their own rounding;
-    // streams for the wider heads too were 2.3e-3 off.  The length is one of time (32 wide, 16 heads, 8192 positions,
-    // causal; streams / tiles, us): 25.6 / 18.4 in sequences of 128, 29.4 / 27.5 of 256, 34.2 / 36.2 of 512, 44.8 / 51 of 1024.
-    int max_vo = 0;
-    for (int h = 0; h < heads->n_heads; ++h) max_vo = std::max<int>(max_vo, heads->vo_w[h]);
-    const bool streams = max_w <= 64 && max_vo <= 32 && seq > 2 * kTile;
-    if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk)) != ECOSPA_OK) return st;
-    if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk, streams ? 64 : kTile)) != ECOSPA_OK) return st;
-    if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v, streams ? 64 : kTile)) != ECOSPA_OK) return st;
     P.batch = static_cast<int32_t>(batch);
     P.seq = static_cast<int32_t>(seq);
     P.n_heads = heads->n_heads;
@@ -1739,7 +1727,26 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     P.items = units * P.n_qt <= sms ? ITEMS_SINGLE : P.n_qt == 1 ? ITEMS_SOLO : ITEMS_SHARED;
     // (Causal sequences of up to two tiles: 200 positions, 80 wide, 63 us without turns, 67 with; 768: 93 and 90.)
     P.turns = P.items == ITEMS_SHARED && (!P.causal || P.n_qt > 2);
-    const int64_t items = streams || P.items == ITEMS_SINGLE ? units * P.n_qt : P.items == ITEMS_SOLO ? (units + 1) / 2 : units * ((P.n_qt + 1) / 2);
+    const int64_t tile_items = P.items == ITEMS_SINGLE ? units * P.n_qt : P.items == ITEMS_SOLO ? (units + 1) / 2 : units * ((P.n_qt + 1) / 2);
+    // Output heads up to 32 wide (and Q/K heads up to 64): the kernel of key streams (K / V tiles as slices of 64 keys), but for
+    // many short sequences; everything else: the kernel of tiles, with one or two 64-column blocks per tile.  The width is a
+    // line of precision: the stream kernel rounds a row's probabilities to bf16 against a reference up to 2^32 below the row's
+    // largest, the other kernel against the largest itself, which is then exactly 1.  On rows that few keys dominate (scores of
+    // deviation 4, 1000 positions, 64 wide) the outputs are 1.7e-3 off the values in 64 bits, all of it their own rounding;
+    // streams for the wider heads too were 2.3e-3 off.  The length is one of time, in rounds of items over the SMs: an item of the
+    // stream kernel is a query tile, one of the tile kernel up to two.  With sequences of one tile a round takes about as long in
+    // both, with two tiles half as long again in the tile kernel; longer ones are always faster as streams.  Streams / tiles, us, 8
+    // heads 32 wide, no mask and causal: 5.5 / 6.0, 5.6 / 6.1 (16 units of 128 positions), 5.7 / 6.5, 5.7 / 6.6 (144), 9.3 / 7.3, 9.5 / 7.4
+    // (200), 11.9 / 9.8, 12.3 / 10.2 (320); 6.7 / 7.5, 6.9 / 7.6 (16 of 256), 6.7 / 8.2, 6.8 / 8.1 (72), 11.8 / 9.9, 9.4 / 9.2 (96), 14.2 / 15.4, 13.5 /
+    // 14.9 (200), 23.9 / 20.6, 22.5 / 19.2 (320); 16 heads, 8192 positions, causal: 34.2 / 36.2 (sequences of 512), 44.8 / 51 (1024).
+    int max_vo = 0;
+    for (int h = 0; h < heads->n_heads; ++h) max_vo = std::max<int>(max_vo, heads->vo_w[h]);
+    const int64_t stream_rounds = ceil_div(units * P.n_qt, sms), tile_rounds = ceil_div(tile_items, sms);
+    const bool streams = max_w <= 64 && max_vo <= 32 && (P.n_qt > 2 || (P.n_qt == 2 ? 2 * stream_rounds <= 3 * tile_rounds : stream_rounds <= tile_rounds));
+    if ((st = encode_tile_map(&P.map_q, Qc, T, n_qk, ld_qk)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_k, Kc, T, n_k, ld_qk, streams ? 64 : kTile)) != ECOSPA_OK) return st;
+    if ((st = encode_tile_map(&P.map_v, Vc, T, n_v, ld_v, streams ? 64 : kTile)) != ECOSPA_OK) return st;
+    const int64_t items = streams ? units * P.n_qt : tile_items;
     if (items > INT32_MAX) return ECOSPA_ERR_UNSUPPORTED;
     P.n_items = static_cast<int32_t>(items);
     P.scale_log2e = scale * 1.4426950408889634f;

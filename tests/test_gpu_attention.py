@@ -5,6 +5,8 @@ probabilities on the tensor cores, fp32 accumulation and softmax; the oracle wor
 the log-sum-exp within 2e-3 absolute.  Small cases are compared in full; the LLaMA-1B-sized case on sampled
 (sequence, head) pairs, each of which is an independent sub-problem.
 """
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -129,14 +131,37 @@ def test_forward_llama1b_sized_sampled_heads(causal):
     (3, 129, [64, 20], [64, 37]),           # few query tiles: one to an item; one key past a tile
     (40, 257, [64, 37, 20], [48, 64, 33]),  # three query tiles: the odd one out is the first; one key past two tiles
     (40, 352, [96, 128, 40], [72, 128, 100]),  # the same on wide heads, a last tile of 96 keys
-    (80, 250, [30, 20, 64], [32, 16, 25]),  # narrow output heads below the line of the stream kernel
+    (80, 250, [30, 20, 64], [32, 16, 25]),  # narrow output heads, too many short sequences for the stream kernel
 ])
 def test_forward_item_forms(batch, seq, k_qk, k_vo, causal):
     """Every way of pairing query tiles into work items, at the edges of tiles, with more items than blocks and fewer."""
     run_forward(batch, seq, k_qk, k_vo, causal, seed=seq, d_h=max(64, max(k_qk + k_vo)))
 
 
-NARROW = [20, 21, 25, 26, 30, 16, 32]      # output heads at most 32 wide take the kernel with independent key streams (above 256 positions)
+NARROW = [20, 21, 25, 26, 30, 16, 32]      # output heads at most 32 wide take the kernel with independent key streams, but for many short sequences
+
+
+@pytest.mark.parametrize("seq,rounds,streams", [(128, 1.0, True), (128, 1.01, False), (64, 2.01, False), (129, 0.5, True), (256, 0.51, False), (256, 1.0, False),
+                                                (192, 1.01, True), (256, 1.5, True), (256, 1.51, False), (257, 3.0, True)])
+def test_forward_narrow_heads_kernel_by_rounds(seq, rounds, streams):
+    """Heads of 16 columns, `rounds` (sequence, head) units per SM: which of the two forward kernels takes them, on both sides of
+    each line of the rule (one tile: as many rounds of query tiles as of pairs; two tiles: at most 3 : 2; more: always streams)."""
+    units = int(torch.cuda.get_device_properties(0).multi_processor_count * rounds)
+    T, w = units * seq, 16
+    Q, K, V, Ctx = (torch.zeros((T, w), dtype=torch.bfloat16, device=DEV) for _ in range(4))
+    lse = torch.zeros(T, device=DEV)
+    call = lambda: B.ecospa_coupled_attn_fwd(Q, K, V, units, seq, B.heads([0], [w], [0], [w]), 0.25, True, Ctx, lse)
+    call()
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    names = [e.name for e in prof.events() if "attn_fwd" in e.name]
+    del prof
+    gc.collect()
+    if not names:
+        pytest.skip("no kernel records from the profiler")
+    assert ["attn_fwd_ms_kernel" in x for x in names] == [streams], names
 
 
 @pytest.mark.parametrize("causal", [False, True])

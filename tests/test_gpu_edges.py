@@ -263,6 +263,14 @@ def test_attention_many_short_items(batch, seq, heads, w, causal):
         assert float(err.max()) <= 2e-2
 
 
+@pytest.mark.parametrize("batch,seq,heads,w,causal", [(25, 130, 8, 16, True), (25, 192, 8, 32, True), (25, 160, 8, 32, False), (25, 256, 8, 32, True),
+                                                      (40, 257, 32, 16, True), (40, 257, 32, 32, False), (40, 300, 32, 32, True), (40, 384, 16, 16, True)])
+def test_attention_many_short_stream_items(batch, seq, heads, w, causal):
+    """The same in the forward kernel of key streams: blocks that walk three or more items, of one slice per stream each (up to 192
+    positions) or the last several of them without a visible key for the third stream (above 256 positions, causal)."""
+    test_attention_many_short_items(batch, seq, heads, w, causal)
+
+
 @pytest.mark.parametrize("batch,seq,heads,w,causal", [(60, 48, 32, 96, False), (60, 48, 32, 128, True), (40, 130, 32, 96, True), (40, 130, 32, 128, False),
                                                       (75, 65, 8, 112, False)])
 def test_attention_many_short_wide_items(batch, seq, heads, w, causal):
