@@ -131,7 +131,8 @@ struct FwdCfg {
     static constexpr int QS = NB == 1 ? 2 : 1;                     // buffers of a stream's Q tile
     static constexpr int ST = NB == 1 ? 4 : 2;                     // stages of the K and of the V tiles
     static constexpr int kRowBytes = (2 * 2 + 2 * 2) * kTile * 4;  // [buffer][stream][row]: factor of the outputs, then 1 / sum
-    static constexpr int kSmem = (2 * QS + 2 * ST) * kTileBytes + kRowBytes + 1024 + 512;
+    static constexpr int kOutBytes = 8 * 32 * 64;                  // output rows on their way out: [scaling warp][row][32 columns]
+    static constexpr int kSmem = (2 * QS + 2 * ST) * kTileBytes + kRowBytes + kOutBytes + 1024 + 512;
     static constexpr int kOCols = NB * 64;                          // columns of an output tile
     // TMEM columns of stream x: scores, output, probabilities (narrow heads: a region of their own, so that the scores of the
     // next key block are computed while these are made; wide heads: over the scores they were made from)
@@ -153,7 +154,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
     const uint32_t sQ = base, sK = sQ + 2 * QS * kTileBytes, sV = sK + ST * kTileBytes;   // Q: [stage][stream]
     float* row_factor = reinterpret_cast<float*>(smem + (2 * QS + 2 * ST) * kTileBytes);    // [buffer][stream][row]
     float* row_inv = row_factor + 4 * kTile;                                                // [buffer][stream][row]
-    uint8_t* tail = smem + (2 * QS + 2 * ST) * kTileBytes + Cfg::kRowBytes;
+    const uint32_t sOut = base + (2 * QS + 2 * ST) * kTileBytes + Cfg::kRowBytes;
+    uint8_t* tail = smem + (2 * QS + 2 * ST) * kTileBytes + Cfg::kRowBytes + Cfg::kOutBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 52 * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 52 * 8 + 8);
@@ -401,25 +403,39 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
             tc_fence_after();
             const float inv = row_inv[((nl & 1u) * 2 + x) * kTile + row];
             ++nl;
-            const int q_pos = (x ? I.qt1 : I.qt0) * kTile + row;
-            uint16_t* dst = P.ctx + (static_cast<int64_t>(x ? I.b1 : I.b0) * P.seq + q_pos) * P.ld_ctx + P.heads.vo_off[h];
+            // 32 columns at a time, through shared memory, eight rows to a store instruction.  Stored straight from the threads, each
+            // with a row of its own, 64 columns of both streams took 2400 to 2900 clocks, which nothing hides at the end of a CTA's last
+            // items.  Direct / through shared memory, us: 10.9 / 10.4 (96 heads of 256 positions, 64 wide, no mask), 17.4 / 16.1 (192 of 197,
+            // ragged), 26.0 / 24.9 (128 of 512), 12.5 / 11.2 (96 of 256, 96 wide), 166.5 / 164.3 (64 of 2048); causal 53.1 / 52.4 (128 of 1024, 48
+            // wide), 17.4 / 16.5 (72 of 512, 96 wide), but 20.4 / 20.8 (128 of 512, 64 wide), 16.4 / 17.0 (256 of 200, 80 wide).
+            const int q_warp = (x ? I.qt1 : I.qt0) * kTile + (warp & 3) * 32;
+            uint16_t* dst = P.ctx + (static_cast<int64_t>(x ? I.b1 : I.b0) * P.seq + q_warp) * P.ld_ctx + P.heads.vo_off[h];
+            const uint32_t buf = sOut + (warp - 4) * 2048;                // [row][4 chunks of 8 columns], chunk c of row r in place c ^ (r / 2 % 4)
+            const int r_in = lane >> 2, chunk = lane & 3;                 // on the way out: eight rows to an instruction, four lanes to a row
 #pragma unroll 1
-            for (int c = 0; c < wv; c += 16) {
-                uint32_t r[16];
+            for (int c = 0; c < wv; c += 32) {
+                uint32_t r[16], q[16];                                     // (columns past the head's width are not stored)
                 tc_ld16(tO + c, r);
+                tc_ld16(tO + c + 16, q);
                 tc_wait_ld(r);
-                if (q_pos < P.seq) {
-                    uint4 v0, v1;
-                    v0.x = pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv);
-                    v0.y = pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv);
-                    v0.z = pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv);
-                    v0.w = pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv);
-                    v1.x = pack_bf16(__uint_as_float(r[8]) * inv, __uint_as_float(r[9]) * inv);
-                    v1.y = pack_bf16(__uint_as_float(r[10]) * inv, __uint_as_float(r[11]) * inv);
-                    v1.z = pack_bf16(__uint_as_float(r[12]) * inv, __uint_as_float(r[13]) * inv);
-                    v1.w = pack_bf16(__uint_as_float(r[14]) * inv, __uint_as_float(r[15]) * inv);
-                    *reinterpret_cast<uint4*>(dst + c) = v0;
-                    *reinterpret_cast<uint4*>(dst + c + 8) = v1;
+                tc_wait_ld(q);
+                __syncwarp();                                              // the columns before these have left
+                auto put = [&](const uint32_t (&v)[16], int at, int k) {
+                    st_shared_v4(buf + lane * 64 + 16 * (k ^ ((lane >> 1) & 3)), pack_bf16(__uint_as_float(v[at]) * inv, __uint_as_float(v[at + 1]) * inv),
+                                 pack_bf16(__uint_as_float(v[at + 2]) * inv, __uint_as_float(v[at + 3]) * inv),
+                                 pack_bf16(__uint_as_float(v[at + 4]) * inv, __uint_as_float(v[at + 5]) * inv),
+                                 pack_bf16(__uint_as_float(v[at + 6]) * inv, __uint_as_float(v[at + 7]) * inv));
+                };
+                put(r, 0, 0);
+                put(r, 8, 1);
+                put(q, 0, 2);
+                put(q, 8, 3);
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int rr = 8 * u + r_in;
+                    if (q_warp + rr < P.seq && c + 8 * chunk < wv)
+                        *reinterpret_cast<uint4*>(dst + rr * P.ld_ctx + c + 8 * chunk) = ld_shared_v4(buf + rr * 64 + 16 * (chunk ^ ((rr >> 1) & 3)));
                 }
             }
             tc_fence_before();
