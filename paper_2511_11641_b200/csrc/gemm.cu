@@ -1519,16 +1519,27 @@ ecospa_status_t launch_grouped_gemm(const GemmOp* ops, int n_ops, cudaStream_t s
     // Where tiles of half that width fit one round too, they take it: an SM then fetches 24 KB instead of 32 per 64-deep k-block, twice
     // as many SMs fetch, and a tile's epilogue is half as long: 113 -> 103 us for the training step of 320 tokens, 768 wide.  (Not for
     // the gated epilogue, whose tile is two operands side by side.)
+    // But not many of them on few rows: all tiles then wait for the same few lines of X, k-block by k-block, and twice as many wait
+    // twice as long.  Measured, this holds while X takes less than 128 KB and there are more than 48 tiles, or with contractions
+    // above 4096 more than 32.  128 x 64 / 128 x 128 tiles, us: Q/K/V of 4096 / 2048 (96 narrow tiles) 28.6 / 20.9 at 8 tokens, 13.9 / 15 at 16
+    // (128 KB); of 2048 / 2048 17.9 / 11.6 at one, 14.8 / 10.3 at 24, 8.7 / 11 at 32; 1024 / 6144 (96) 9.6 / 7.0 at one, 6.1 / 7.5 at 64; 2048 /
+    // 2560 (40) 10.3 / 10.6; 768 / 3072 (48) 5.5 / 6.4; 8192 / 2688 (42) 32.8 / 27.4 at one, 23.9 / 31.8 at 8.
     int64_t single_tiles = 0, slim_tiles = 0;
     bool any_tall = false;
+    int64_t x_bytes = 0, k_max = 0;                            // X: operand A
     for (int i = 0; i < n_ops; ++i) {
+        int64_t k = 0;
+        for (int s = 0; s < ops[i].n_kseg; ++s) k += ops[i].seg[s].K;
+        k_max = std::max(k_max, k);
+        x_bytes = std::max(x_bytes, 2 * std::min<int64_t>(ops[i].M, BM) * k);
         const int per_tile = ops[i].epi == EPI_SWIGLU ? TileShape<TILE_SINGLE>::kN / 2 : TileShape<TILE_SINGLE>::kN;
         single_tiles += ceil_div(ops[i].M, BM) * ceil_div(ops[i].N, per_tile);
         slim_tiles += ops[i].epi == EPI_SWIGLU ? g_num_sms + 1 : ceil_div(ops[i].M, BM) * ceil_div(ops[i].N, TileShape<TILE_SLIM>::kN);
         any_tall = any_tall || ops[i].M > BM;
     }
     const bool pairs = g_pair_mode != 0 && g_max_pairs >= 1 && any_tall;
-    const int form = slim_tiles <= g_num_sms ? TILE_SLIM : single_tiles <= g_num_sms ? TILE_SINGLE : pairs ? TILE_PAIR : TILE_WIDE;
+    const bool crowded = !any_tall && x_bytes < 128 * 1024 && slim_tiles > (k_max > 4096 ? 32 : 48);
+    const int form = slim_tiles <= g_num_sms && !crowded ? TILE_SLIM : single_tiles <= g_num_sms ? TILE_SINGLE : pairs ? TILE_PAIR : TILE_WIDE;
     const bool pair = form == TILE_PAIR;
     const int tile_m = pair ? 2 * BM : BM, tile_n = form == TILE_SLIM ? TileShape<TILE_SLIM>::kN : form == TILE_SINGLE ? TileShape<TILE_SINGLE>::kN : TileShape<TILE_PAIR>::kN;
 

@@ -70,3 +70,25 @@ def test_cta_pairs_need_more_than_128_rows(T, pairs):
     if not names:
         pytest.skip("no kernel records from the profiler")
     assert [("gemm_kernel<1," in x or "gemm_kernel<true," in x) for x in names] == [pairs], names
+
+
+@pytest.mark.parametrize("T,d_m,n,slim", [(1, 3072, 768, True), (1, 3136, 768, False), (1, 2048, 4160, True), (1, 2112, 4160, False), (1, 3072, 4096, True),
+                                          (31, 4096, 2048, False), (32, 4096, 2048, True), (128, 4096, 504, False), (128, 4096, 512, True), (129, 4096, 256, True)])
+def test_narrow_tiles_on_few_rows(T, d_m, n, slim):
+    """Which of the two single-CTA tiles a product of few rows takes, on both sides of each line of the rule (48 tiles of 64 columns, 32 on
+    contractions above 4096, 128 KB of X, 128 rows), and its values.  Bound: bf16 operands, fp32 sums, the output's rounding."""
+    g = torch.Generator(device=DEV).manual_seed(T)
+    x, w = torch.randn(T, n, generator=g, device=DEV).bfloat16(), (torch.randn(n, d_m, generator=g, device=DEV) * 0.05).bfloat16()
+    out = torch.zeros(T, d_m, dtype=torch.bfloat16, device=DEV)
+    B.ecospa_coupled_vo_fwd_o(x, w, n, out)
+    B.ecospa_device_status()
+    assert _rel(out, (x.double() @ w.double()).cpu().numpy()) <= 4e-3
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        B.ecospa_coupled_vo_fwd_o(x, w, n, out)
+        torch.cuda.synchronize()
+    names = [e.name for e in prof.events() if "gemm_kernel" in e.name]
+    del prof
+    gc.collect()
+    if not names:
+        pytest.skip("no kernel records from the profiler")
+    assert ["gemm_kernel<3," in s for s in names] == [slim], names
