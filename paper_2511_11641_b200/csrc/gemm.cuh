@@ -57,8 +57,10 @@ struct GemmOp {
 constexpr int kMaxGemmOps = 16;
 
 // Column sums (bias gradients) that a launch takes along: up to three bf16 matrices with the same number of rows, none of
-// them written by the launch itself.  Up to kSumWholeRows rows the launch writes the sums themselves (out); above, a finishing
-// launch adds the chunks: partial[chunk][col] = sum over the chunk's kSumRows rows.
+// them written by the launch itself.  Up to kSumWholeRows rows, and unless the call has a finishing launch anyway, the launch
+// writes the sums themselves (out); otherwise the finishing launch adds the chunks: partial[chunk][col] = sum over the chunk's
+// kSumRows rows.  (Whole / chunks and a finishing launch, us, output projection backward with bias: 7.3 / 10.1 at 1024 rows, 768 wide, 11.1
+// / 14.5 at 2047.)
 constexpr int kSumRows = 128, kSumWholeRows = 2048;
 struct SideSums {
     const uint16_t* M[3];

@@ -234,10 +234,12 @@ ecospa_status_t run_ops(Ctx& cx, const GemmOp* ops, int n_ops, const SideSums* s
 }
 
 // Asks for the column sums of a bf16 matrix: `side` describes the reading (done by a product launch, which must not be the one
-// that writes the matrix), `fin` what the finishing launch adds up, where one is needed (see SideSums).  All matrices of a call have the same row count.  The
-// scratch of the chunk partials comes from the workspace here, so that a short workspace is reported before anything is
-// launched.  A null output skips the matrix.
-void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, void* out) {
+// that writes the matrix), `fin` what the finishing launch adds up, where one is needed (see SideSums): the call has one anyway if
+// `finishing`, and adding the chunks there is then the cheaper way (2048 rows, products with a split weight gradient, whole sums / chunks:
+// 11.0 / 8.7 us, 256 wide; 12.6 / 11.4, 768; 13.5 / 11.7, 1024; no split, 2048 wide: 15.8 / 17.9).  All matrices of a call have the same
+// row count.  The scratch of the chunk partials comes from the workspace here, so that a short workspace is reported before anything
+// is launched, and in either case, so that what a call needs does not depend on how it forms its sums.  A null output skips the matrix.
+void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, void* out, bool finishing) {
     if (cx.st != ECOSPA_OK || !out || !M.ptr) return;
     const int chunks = static_cast<int>(ceil_div(M.rows, kSumRows));
     float* partial = static_cast<float*>(cx.arena.take(static_cast<size_t>(chunks) * M.cols * 4));
@@ -256,7 +258,7 @@ void want_colsum(Ctx& cx, SideSums& side, ColsumParams& fin, const Stored& M, vo
     side.chunks = fin.chunks = chunks;
     side.out[i] = out;
     side.out_f32 = cx.dtype == ECOSPA_F32;
-    side.whole = M.rows <= kSumWholeRows;
+    side.whole = M.rows <= kSumWholeRows && !finishing;
     if (!side.whole) fin.job[fin.n_jobs++] = ColsumFinal{partial, out, M.cols};
 }
 
@@ -406,6 +408,12 @@ int add_wgrad_w(Ctx& cx, GemmOp* ops, int n_ops, const ecospa_mat_t* w, const St
     return add_wgrad(cx, ops, n_ops, shared_act, other_act, n, d_m, T, out, ld_out, red, reserve, launch_cost);
 }
 
+// Whether a call has a finishing launch for its split weight gradients.
+bool any_split(const PendingReduce* red, int n_red) {
+    bool any = false;
+    for (int i = 0; i < n_red; ++i) any = any || red[i].splits > 0;
+    return any;
+}
 // The finishing launch of a call: split-K reductions and column-sum finals together.
 void finish(Ctx& cx, const PendingReduce* red, int n_red, const ColsumParams& cs) {
     if (cx.st != ECOSPA_OK) return;
@@ -510,8 +518,8 @@ extern "C" ecospa_status_t ecospa_coupled_qk_bwd(const void* X, int64_t ldx, int
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
     SideSums side = {};
     ColsumParams cs = {};
-    want_colsum(cx, side, cs, dQs, dbq_c);
-    want_colsum(cx, side, cs, dKs, wk_c ? dbk_c : nullptr);
+    want_colsum(cx, side, cs, dQs, dbq_c, any_split(red, 2));
+    want_colsum(cx, side, cs, dKs, wk_c ? dbk_c : nullptr, any_split(red, 2));
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
     finish(cx, red, 2, cs);
@@ -585,8 +593,8 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd(const void* X, int64_t ldx, con
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32; dx.accumulate = accumulate_dX != 0;
     SideSums side = {};
     ColsumParams cs = {};
-    want_colsum(cx, side, cs, dVs, dbv_c);
-    want_colsum(cx, side, cs, dOs, dbo);
+    want_colsum(cx, side, cs, dVs, dbv_c, any_split(red, 2));
+    want_colsum(cx, side, cs, dOs, dbo, any_split(red, 2));
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
     finish(cx, red, 2, cs);
@@ -657,9 +665,9 @@ extern "C" ecospa_status_t ecospa_coupled_qkv_bwd(const void* X, int64_t ldx, in
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = cx.dtype == ECOSPA_F32; dx.accumulate = accumulate_dX != 0;
     SideSums side = {};
     ColsumParams cs = {};
-    want_colsum(cx, side, cs, dQs, dbq_c);
-    want_colsum(cx, side, cs, dKs, dbk_c);
-    want_colsum(cx, side, cs, dVs, dbv_c);
+    want_colsum(cx, side, cs, dQs, dbq_c, any_split(red, 3));
+    want_colsum(cx, side, cs, dKs, dbk_c, any_split(red, 3));
+    want_colsum(cx, side, cs, dVs, dbv_c, any_split(red, 3));
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
     finish(cx, red, 3, cs);
@@ -692,7 +700,7 @@ extern "C" ecospa_status_t ecospa_coupled_vo_bwd_o(const void* Ctxm, int64_t ld_
     dc.epi = EPI_STORE; dc.C = dCtx; dc.ldc = ld_dctx; dc.out_f32 = cx.dtype == ECOSPA_F32;
     SideSums side = {};
     ColsumParams cs = {};
-    want_colsum(cx, side, cs, dOs, dbo);
+    want_colsum(cx, side, cs, dOs, dbo, any_split(&red, 1));
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = run_ops(cx, ops, n_ops, &side)) != ECOSPA_OK) return st;
     finish(cx, &red, 1, cs);
@@ -816,8 +824,8 @@ extern "C" ecospa_status_t ecospa_coupled_ffn_bwd(const void* X, int64_t ldx, in
     dx.epi = EPI_STORE; dx.C = dX; dx.ldc = ld_dx; dx.out_f32 = f32;
     SideSums side1 = {}, side2 = {};                       // db_2 = column sums of dY; db_1 = those of dH, which the first launch writes
     ColsumParams cs = {};
-    want_colsum(cx, side1, cs, dYs, db2);
-    want_colsum(cx, side2, cs, dH, sw ? nullptr : db1_c);
+    want_colsum(cx, side1, cs, dYs, db2, any_split(red, 3));
+    want_colsum(cx, side2, cs, dH, sw ? nullptr : db1_c, any_split(red, 3));
     if (cx.st != ECOSPA_OK) return cx.st;
     if ((st = validate_gemm_ops(ops, n_ops)) != ECOSPA_OK || (st = validate_gemm_ops(ops2, n_ops2)) != ECOSPA_OK) return st;
     if ((st = run_ops(cx, ops, n_ops, &side1)) != ECOSPA_OK) return st;

@@ -446,3 +446,18 @@ def test_bias_gradient_row_counts(T, dtype):
     first = dbo.clone()
     B.ecospa_coupled_vo_bwd_o(ctx, wo, n, dout, dctx, dwo, dbo, workspace=ws)
     assert torch.equal(first, dbo)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_bias_gradient_beside_split_weight_gradients(dtype):
+    """2048 rows, weight gradient split over them: the finishing launch of that call adds the bias gradient's chunks of 128 rows, chunk k to
+    chunk k + 8 first.  2^30 in chunk 0 and -2^30 in chunk 8 cancel there exactly; a sum that runs through the rows loses the 1 between them."""
+    T, n, d_m = 2048, 128, 256
+    z = lambda *s: torch.zeros(s, dtype=dtype, device=DEV)
+    ctx, wo, dout, dctx, dwo, dbo = z(T, n), z(n, d_m), z(T, d_m), z(T, n), z(n, d_m), z(d_m)
+    dout[0], dout[256], dout[1024] = 2.0 ** 30, 1.0, -(2.0 ** 30)
+    code = B.BF16 if dtype == torch.bfloat16 else B.F32
+    ws = torch.empty(B.ecospa_proj_workspace_bytes(T, d_m, n, code) + 16, dtype=torch.uint8, device=DEV)
+    B.ecospa_coupled_vo_bwd_o(ctx, wo, n, dout, dctx, dwo, dbo, workspace=ws)
+    B.ecospa_device_status()
+    assert torch.all(dbo == 1.0)
