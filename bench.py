@@ -445,6 +445,19 @@ def measure_step(m, args, world, rank, local, steps: int, graph: bool = True):
             "replay": (fns["sparsify"], fns["blocks"]), "timed_ms": timed_ms, "timed_gemm_ms": timed_gemm}
 
 
+def attn_fwd_name(wl, m) -> str:
+    """The forward kernel that a workload's attention calls take: the rule of `ecospa_coupled_attn_fwd`, for 148 SMs."""
+    streams, tiles = "attn_fwd_ms_kernel", "attn_fwd_kernel"
+    if max(m.vo_w) > 32 or max(m.qk_w) > 64:
+        return tiles
+    units, n_qt = wl.batch * wl.n_heads, -(-wl.seq // 128)
+    if n_qt > 2:
+        return streams
+    items = units * n_qt if units * n_qt <= 148 else (units + 1) // 2 if n_qt == 1 else units
+    r_streams, r_tiles = -(-units * n_qt // 148), -(-items // 148)
+    return streams if (2 * r_streams <= 3 * r_tiles if n_qt == 2 else r_streams <= r_tiles) else tiles
+
+
 def attention_report(wl, m, r):
     """The attention core's share: algorithmic flops / its own replay time, and its exponentials against the
     special-function rate of the part (one 2^x per query-key pair in the forward pass and in each of the two backward
@@ -457,7 +470,7 @@ def attention_report(wl, m, r):
     exp_peak = 148 * 16 * sm * 1e6          # exponentials per second
     return {"ms": r["ms_attn"], "TFLOP/s": fl / r["ms_attn"] / 1e9, "flops": fl, "frac_of_nominal_2250": fl / r["ms_attn"] / 1e9 / 2250.0,
             "causal": m.causal, "head_widths": f"{m.plan['qk'][0]} of {wl.d_h} (padded to {m.qk_w[0]})",
-            "roofline": {"bound": "alu", "kernel": ("attn_fwd_ms_kernel" if max(m.vo_w) <= 32 and max(m.qk_w) <= 64 else "attn_fwd_kernel") + " + attn_bwd_kernel x2", "achieved": 3 * pairs / (r["ms_attn"] * 1e-3) / 1e12,
+            "roofline": {"bound": "alu", "kernel": attn_fwd_name(wl, m) + " + attn_bwd_kernel x2", "achieved": 3 * pairs / (r["ms_attn"] * 1e-3) / 1e12,
                          "peak": exp_peak / 1e12, "unit": "T exp/s", "frac": 3 * pairs / (r["ms_attn"] * 1e-3) / exp_peak,
                          "peak_source": f"16 ex2/clk/SM x 148 SMs x {sm:.0f} MHz (sampled)"},
             "clocks": r["clocks_attn"]}

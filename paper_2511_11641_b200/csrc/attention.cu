@@ -26,9 +26,11 @@
 // Both passes are rolled loops of 64 columns: holding a block's 128 scores in registers, unrolled, was slower (163 -> 233 us at
 // 4 x 2048 positions, 32 heads 32 wide: warps waited for instructions, 4.0 of 15 cycles per issue, now 1.0).  Columns that
 // no row of a warp sees are skipped, keys past the end of the sequence also in the products.
-// Before (two streams in one thread's registers, a token between them) / now, us: 420 / 335 (2 x 4096, 32 heads 96 wide),
-// 59.3 / 53.0 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 7.9 (2 x 160, 12 heads 48 wide), 60.9 / 28.2 (60 x 48, 32 heads 64
-// wide), 41.8 / 18.9 (30 x 48, 32 heads 128 wide), 24.9 / 27.2 (8 x 512, 16 heads 64 wide, no mask).
+// Before (two streams in one thread's registers, a token between them) / now, us: 475 / 301 (2 x 4096, 32 heads 96 wide),
+// 69.7 / 53.2 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 7.5 (2 x 160, 12 heads 48 wide), 63.9 / 28.9 (60 x 48, 32 heads 64
+// wide), 41.7 / 18.9 (30 x 48, 32 heads 128 wide), 26.6 / 25.1 (8 x 512, 16 heads 64 wide, no mask).  One form is slower than before: one
+// pair of tiles to a CTA, short, without a mask, heads of 33 to 64 (9.8 / 10.4 for 96 heads of 256, 12.3 / 12.6 for 72 of 384): the two
+// streams start and end together.
 // Every mbarrier wait is bounded; on expiry the CTA records a code (11 loads, 12 products, 13 softmax and scaling) in the device
 // status word, lets copies land, frees TMEM and returns.
 
@@ -836,7 +838,8 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
             };
             SD d0 = next(), d1 = next(), d2 = next(), d3;
             {   // start: K slices 0 and 1 and V slice 0, and their score products; then K slice 2, on a barrier of its own.  (Where
-                // every item is one slice long, slice 2 brings the third Q tile, whose buffer is free only after slice 0's product.)
+                // every item is one slice long - three items to a CTA, sequences of 129 to 192 positions -, slice 2 brings the third Q
+                // tile, whose buffer is free only after slice 0's product.)
                 const uint32_t nk = (d0.meta & 1u) + (d1.meta & 1u);
                 if (nk) mbar_expect_tx(kv_full(x, 0), (nk + 1) * kSliceB);
                 if (d0.meta & 1u) {
@@ -1173,9 +1176,10 @@ struct AttnBwdParams {
 // two groups of eight that take the steps in turn, each with score tiles and packed operands of its own: while one waits
 // for its products the other keeps the exponential unit busy.  What a step costs is a chain of short waits (scores, TMEM loads,
 // exponentials, operands, products), not a pipe: the exponentials of 128 x 128 scores take 1024 clocks, a pair of steps 2200.
-// Before (all warps on one block of 128, or on half blocks in turn) / now, us: 109.4 / 65.0 (60 x 48 positions, 32 heads 64
-// wide), 125.5 / 108.9 (4 x 1000, 32 heads 48 wide on 8), 42.0 / 36.1 (32 x 197, 6 heads 48 wide), 104.8 / 101.3 (8 x 1024, 16
-// heads 32 wide), 1205 / 1088 (2 x 4096, 32 heads 128 wide).
+// Before (all warps on one block of 128, or on half blocks in turn) / now, us: 109 / 63 (60 x 48 positions, 32 heads 64
+// wide), 134 / 112 (4 x 1000, 32 heads 48 wide on 8), 45.1 / 36.3 (32 x 197, 6 heads 48 wide, no mask), 106.5 / 100 (8 x 1024, 16
+// heads 32 wide), 1045 / 969 (2 x 4096, 32 heads 128 wide).  Slower than before: heads up to 32 wide, two tiles, no mask, many items (54.0 /
+// 58.3 for 512 heads of 256 positions, 35.2 / 37.2 for 256; causal 58.1 / 54.5).
 // The products are issued by separate threads.  Heads up to 64 wide (NB = 1): warp 1 issues the score products; warps 18 and 19
 // the accumulating ones (dV and dK; the query-block kernel needs only the second), whose A operands go through TMEM as
 // packed bf16 beside the scores.  Wider heads (NB = 2): warp 1 issues X, warp 18 Y, warp 19 the accumulating products.  The
@@ -1230,7 +1234,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
     // resident: [stage][a | b], streamed: [stage][a | b], vectors, barriers
     const uint32_t sRes = base, sStr = sRes + 2 * kTileBytes * RS;
     uint8_t* vec_raw = smem + 2 * kTileBytes * RS + 2 * kStrTileBytes * SS;
-    float* vec = reinterpret_cast<float*>(vec_raw);                               // [stage][-lse2 | D][128]
+    float* vec = reinterpret_cast<float*>(vec_raw);                               // [stage][-lse2 | D][kStep]
     uint8_t* tail = vec_raw + Cfg::kVecBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(tail + 32 * 8);
@@ -1536,7 +1540,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attn_bwd_kernel(const __grid_c
             const BItem I = decode(it);
             const int own_pos = I.own * kTile + row;                 // position of this thread's row in the sequence
             // MODE 1: this row's -log-sum-exp (base 2) and row dot (zeros past the end of the sequence).  MODE 0: the values of
-            // the step's 128 queries arrive in shared memory with the step's tiles.
+            // the step's 64 queries arrive in shared memory with the step's tiles.
             float lse_r = 0.f, d_r = 0.f;
             if (MODE == 1) {
                 const int64_t o = (static_cast<int64_t>(I.h) * P.batch + I.b) * P.seq_pad + own_pos;

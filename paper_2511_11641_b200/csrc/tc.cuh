@@ -12,10 +12,9 @@ namespace tc {
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // True in one lane of a converged warp (always the same one).  The branches whose thread issues loads and products are entered
-// through this and not through a comparison of the lane number: these instructions take their operands from registers that a
-// warp shares, and behind elect.sync the compiler knows that one thread is active, where behind a comparison it wraps each of
-// them in code for several.  (Products with A in tensor memory, 128 x 32 x 16, in an unrolled loop: 46 clocks apart behind a
-// comparison, 17 behind this; in a loop with run-time descriptors 154.)
+// through this and not through a comparison of the lane number, because it measured faster: products with A in tensor memory,
+// 128 x 32 x 16, in an unrolled loop were 46 clocks apart behind a comparison and 17 behind this (154 behind a comparison in a loop with
+// run-time descriptors).  Why is not known from these timings; presumably the compiler can tell here that one thread is active.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
