@@ -594,6 +594,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
 
 // ------------------------------------------------------------------------------------------------
 // forward, output heads up to 32 wide, not many short sequences: NS independent streams per CTA
+// (EXACT: a slice's maximum is taken before its exponentials and the reference is the stream's running maximum; see the rule in
+// ecospa_coupled_attn_fwd.  Otherwise one pass over the scores, against a reference that moves when a score exceeds it by 2^32.)
 // ------------------------------------------------------------------------------------------------
 // A work item is (sequence b, head h, one tile of 128 query rows).  A K / V tile holds NS slices of 64 keys; stream x
 // (four warps, thread = query row) owns slice x of every tile and keeps a softmax of its own over its keys: reference
@@ -678,7 +680,7 @@ __device__ __forceinline__ RowState rescale_row(RowState s, float cm, uint32_t t
     return o;
 }
 
-template <int NS, int OC>
+template <int NS, int OC, bool EXACT>
 __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel(const __grid_constant__ AttnFwdParams P) {
     using Cfg = MsCfg<NS, OC>;
     constexpr int kSliceB = Cfg::kSliceBytes, kKeys = Cfg::kKeys, ST = Cfg::kStages;
@@ -923,55 +925,109 @@ __global__ void __launch_bounds__(MsCfg<NS, OC>::kThreads, 1) attn_fwd_ms_kernel
                 const bool masked = kv_base + 64 > limit;                   // keys past the limit count as -inf
                 float rs4[4] = {0.f, 0.f, 0.f, 0.f};
                 uint32_t ra[CH], rb[CH];
-                tc_ld(tS, ra);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    uint32_t(&cur)[CH] = (c & 1) ? rb : ra;
-                    uint32_t(&nxt)[CH] = (c & 1) ? ra : rb;
-                    tc_wait_ld(cur);
-                    if (c + 1 < NC) tc_ld(tS + (c + 1) * CH, nxt);
-                    if (masked) {
-#pragma unroll
-                        for (int i = 0; i < CH; ++i)
-                            if (kv_base + c * CH + i >= limit) cur[i] = 0xff800000u;
-                    }
-                    // The chunk's maximum and its exponentials (with the reference the row has) have no dependence on one
-                    // another, so they can be interleaved; only if some score exceeds the reference by more than 32 (rare) is
-                    // the row rescaled and the chunk exponentiated again.
+                if constexpr (EXACT) {
+                    // the slice's maximum before its exponentials: the reference is the stream's running maximum, so that the
+                    // largest probability of a row is exactly 1 in the stream that has its key
+                    tc_ld(tS, ra);
+                    tc_ld(tS + CH, rb);
+                    tc_wait_ld(ra);
+                    tc_wait_ld(rb);
                     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                    for (int i = 0; i < CH; i += 2) mx4[(i >> 1) & 3] = max3(mx4[(i >> 1) & 3], __uint_as_float(cur[i]), __uint_as_float(cur[i + 1]));
-                    const float cm = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * P.scale_log2e;
-                    uint32_t pk[CH / 2];
-                    float cs4[4] = {0.f, 0.f, 0.f, 0.f};
-                    auto exponentiate = [&](float neg_m) {   // (packed fp32 multiply-adds and sums: half the issue slots)
-                        const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), nm2 = pack2(neg_m, neg_m);
-                        f32x2 acc2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+                    for (int i = 0; i < CH; ++i) {
+                        if (masked && kv_base + i >= limit) ra[i] = 0xff800000u;
+                        if (masked && kv_base + CH + i >= limit) rb[i] = 0xff800000u;
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH; i += 2) {
+                        mx4[(i >> 1) & 1] = max3(mx4[(i >> 1) & 1], __uint_as_float(ra[i]), __uint_as_float(ra[i + 1]));
+                        mx4[2 + ((i >> 1) & 1)] = max3(mx4[2 + ((i >> 1) & 1)], __uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
+                    }
+                    const float m_new = fmaxf(rsx.m, fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * P.scale_log2e);
+                    const float f = ex2(rsx.m - m_new);
+                    if (j > 0 && __any_sync(0xffffffffu, m_new > rsx.m)) {
+                        if (!(ok = mbar_wait(pv_done(x, (cs - 1) & 1), ((cs - 1) >> 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+                        tc_fence_after();
+                        for (int g = 0; g < (wv >> 4); ++g) {
+                            uint32_t r[16];
+                            tc_ld16(tO + 16 * g, r);
+                            tc_wait_ld(r);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f);
+                            tc_st(tO + 16 * g, r);
+                        }
+                    }
+                    rsx.m = m_new;
+                    rsx.l *= f;
+                    const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), nm2 = pack2(-m_new, -m_new);
+                    f32x2 acc2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+                    auto exponentiate = [&](const uint32_t (&v)[CH], uint32_t t) {
+                        uint32_t pk[CH / 2];
 #pragma unroll
                         for (int i = 0; i < CH; i += 2) {
                             float x0, x1;
-                            unpack2(fma2(pack2(cur[i], cur[i + 1]), c2, nm2), x0, x1);
+                            unpack2(fma2(pack2(v[i], v[i + 1]), c2, nm2), x0, x1);
                             const float p0 = ex2(x0), p1 = ex2(x1);
                             acc2[(i >> 1) & 1] = add2(acc2[(i >> 1) & 1], pack2(p0, p1));
                             pk[i >> 1] = pack_bf16(p0, p1);
                         }
-                        unpack2(acc2[0], cs4[0], cs4[1]);
-                        unpack2(acc2[1], cs4[2], cs4[3]);
+                        tc_st(t, pk);
                     };
-                    exponentiate(-rsx.m);
-                    if (__any_sync(0xffffffffu, cm - rsx.m > 32.f)) {
-                        // the output row is touched: the product of the previous slice must have landed
-                        if (j > 0 && !(ok = mbar_wait(pv_done(x, (cs - 1) & 1), ((cs - 1) >> 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
-                        tc_fence_after();
-                        rsx.rs = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
-                        rsx = rescale_row(rsx, cm, tO, j > 0 ? wv >> 4 : 0, tP, c);
-                        rs4[0] = rsx.rs;
-                        rs4[1] = rs4[2] = rs4[3] = 0.f;
-                        exponentiate(-rsx.m);
-                    }
+                    exponentiate(ra, tP);
+                    exponentiate(rb, tP + CH / 2);
+                    unpack2(acc2[0], rs4[0], rs4[1]);
+                    unpack2(acc2[1], rs4[2], rs4[3]);
+                } else {
+                    tc_ld(tS, ra);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) rs4[q] += cs4[q];
-                    tc_st(tP + c * (CH / 2), pk);
+                    for (int c = 0; c < NC; ++c) {
+                        uint32_t(&cur)[CH] = (c & 1) ? rb : ra;
+                        uint32_t(&nxt)[CH] = (c & 1) ? ra : rb;
+                        tc_wait_ld(cur);
+                        if (c + 1 < NC) tc_ld(tS + (c + 1) * CH, nxt);
+                        if (masked) {
+#pragma unroll
+                            for (int i = 0; i < CH; ++i)
+                                if (kv_base + c * CH + i >= limit) cur[i] = 0xff800000u;
+                        }
+                        // The chunk's maximum and its exponentials (with the reference the row has) have no dependence on one
+                        // another, so they can be interleaved; only if some score exceeds the reference by more than 32 (rare) is
+                        // the row rescaled and the chunk exponentiated again.
+                        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                        for (int i = 0; i < CH; i += 2) mx4[(i >> 1) & 3] = max3(mx4[(i >> 1) & 3], __uint_as_float(cur[i]), __uint_as_float(cur[i + 1]));
+                        const float cm = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * P.scale_log2e;
+                        uint32_t pk[CH / 2];
+                        float cs4[4] = {0.f, 0.f, 0.f, 0.f};
+                        auto exponentiate = [&](float neg_m) {   // (packed fp32 multiply-adds and sums: half the issue slots)
+                            const f32x2 c2 = pack2(P.scale_log2e, P.scale_log2e), nm2 = pack2(neg_m, neg_m);
+                            f32x2 acc2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+#pragma unroll
+                            for (int i = 0; i < CH; i += 2) {
+                                float x0, x1;
+                                unpack2(fma2(pack2(cur[i], cur[i + 1]), c2, nm2), x0, x1);
+                                const float p0 = ex2(x0), p1 = ex2(x1);
+                                acc2[(i >> 1) & 1] = add2(acc2[(i >> 1) & 1], pack2(p0, p1));
+                                pk[i >> 1] = pack_bf16(p0, p1);
+                            }
+                            unpack2(acc2[0], cs4[0], cs4[1]);
+                            unpack2(acc2[1], cs4[2], cs4[3]);
+                        };
+                        exponentiate(-rsx.m);
+                        if (__any_sync(0xffffffffu, cm - rsx.m > 32.f)) {
+                            // the output row is touched: the product of the previous slice must have landed
+                            if (j > 0 && !(ok = mbar_wait(pv_done(x, (cs - 1) & 1), ((cs - 1) >> 1) & 1u, abort_flag, 13, P.status, P.wait_limit_ns))) break;
+                            tc_fence_after();
+                            rsx.rs = (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
+                            rsx = rescale_row(rsx, cm, tO, j > 0 ? wv >> 4 : 0, tP, c);
+                            rs4[0] = rsx.rs;
+                            rs4[1] = rs4[2] = rs4[3] = 0.f;
+                            exponentiate(-rsx.m);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) rs4[q] += cs4[q];
+                        tc_st(tP + c * (CH / 2), pk);
+                    }
                 }
                 if (!ok) break;
                 tc_wait_st();
@@ -1758,12 +1814,14 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     // line of precision: the stream kernel rounds a row's probabilities to bf16 against a reference up to 2^32 below the row's
     // largest, the other kernel against the largest itself, which is then exactly 1.  On rows that few keys dominate (scores of
     // deviation 4, 1000 positions, 64 wide) the outputs are 1.7e-3 off the values in 64 bits, all of it their own rounding;
-    // streams for the wider heads too were 2.3e-3 off.  The length is one of time, in rounds of items over the SMs: an item of the
+    // streams for the wider heads too were 2.3e-3 off.  Up to two tiles the streams take exact maxima too (one or two slices each, so
+    // that the second look at the scores costs up to 0.6 us of 6.7): 1.74e-3 off there on such rows, the tile kernel 1.77e-3, streams without
+    // exact maxima 1.95e-3 (72 heads of 256 positions, 32 wide, causal).  The length is one of time, in rounds of items over the SMs: an item of the
     // stream kernel is a query tile, one of the tile kernel up to two.  With sequences of one tile a round takes about as long in
     // both, with two tiles half as long again in the tile kernel; longer ones are always faster as streams.  Streams / tiles, us, 8
-    // heads 32 wide, no mask and causal: 5.5 / 6.0, 5.6 / 6.1 (16 units of 128 positions), 5.7 / 6.5, 5.7 / 6.6 (144), 9.3 / 7.3, 9.5 / 7.4
-    // (200), 11.9 / 9.8, 12.3 / 10.2 (320); 6.7 / 7.5, 6.9 / 7.6 (16 of 256), 6.7 / 8.2, 6.8 / 8.1 (72), 11.8 / 9.9, 9.4 / 9.2 (96), 14.2 / 15.4, 13.5 /
-    // 14.9 (200), 23.9 / 20.6, 22.5 / 19.2 (320); 16 heads, 8192 positions, causal: 34.2 / 36.2 (sequences of 512), 44.8 / 51 (1024).
+    // heads 32 wide, no mask and causal: 5.5 / 6.0, 5.5 / 6.0 (16 units of 128 positions), 5.8 / 6.6, 5.8 / 6.7 (144), 9.3 / 7.3, 9.5 / 7.4
+    // (200), 11.9 / 9.8, 12.3 / 10.2 (320); 7.3 / 7.5, 7.3 / 7.6 (16 of 256), 7.4 / 8.2, 7.3 / 8.2 (72), 11.8 / 9.9, 9.4 / 9.2 (96), 15.8 / 15.4, 14.4 /
+    // 14.9 (200), 23.9 / 20.6, 22.5 / 19.2 (320); 13.2 / 13.8, 12.3 / 13.7 (200 of 160); 16 heads, 8192 positions, causal: 34.2 / 36.2 (sequences of 512), 44.8 / 51 (1024).
     int max_vo = 0;
     for (int h = 0; h < heads->n_heads; ++h) max_vo = std::max<int>(max_vo, heads->vo_w[h]);
     const int64_t stream_rounds = ceil_div(units * P.n_qt, sms), tile_rounds = ceil_div(tile_items, sms);
@@ -1787,7 +1845,8 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     std::call_once(once[dev & 63], [&] {
         e = cudaFuncSetAttribute(attn_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<1>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<2>::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
     });
     if (e != cudaSuccess) {
         set_cuda_error(e, "attention setup");
@@ -1796,7 +1855,7 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     }
     const int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (streams) return launch_pdl(attn_fwd_ms_kernel<3, 32>, grid, MsCfg<3, 32>::kThreads, cs, P, "attn_fwd_kernel", MsCfg<3, 32>::kSmem);
+    if (streams) return launch_pdl(P.n_qt <= 2 ? attn_fwd_ms_kernel<3, 32, true> : attn_fwd_ms_kernel<3, 32, false>, grid, MsCfg<3, 32>::kThreads, cs, P, "attn_fwd_kernel", MsCfg<3, 32>::kSmem);
     if (max_w <= 64) return launch_pdl(attn_fwd_kernel<1>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<1>::kSmem);
     return launch_pdl(attn_fwd_kernel<2>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<2>::kSmem);
 }

@@ -260,7 +260,8 @@ def test_forward_scores_that_grow_wider_heads(w_qk, w_vo, causal):
 def test_forward_row_with_one_key_returns_its_value(w_qk, w_vo, at):
     """One key outweighs all others by 2^24 to 2^31 (a different exponent, hence a different fraction, in every row), so a row's
     output is that key's value times 1 - 200 * 2^-24: its entries, bf16 numbers of magnitude 0.5 to 2, come back bit for bit if
-    the largest probability of a row is not rounded (output heads up to 32 wide with Q/K heads up to 64 have no such promise)."""
+    the largest probability of a row is not rounded (output heads up to 32 wide with Q/K heads up to 64 have no such promise above 256
+    positions)."""
     batch, seq, H = 2, 200, 3
     T = batch * seq
     g = torch.Generator().manual_seed(at)
@@ -278,6 +279,13 @@ def test_forward_row_with_one_key_returns_its_value(w_qk, w_vo, at):
         for b in range(batch):
             rows = Ctx[b * seq + (at if causal else 0): (b + 1) * seq].cpu()
             assert torch.equal(rows, V[b * seq + at].expand_as(rows))
+
+
+@pytest.mark.parametrize("w_qk,w_vo", [(32, 32), (64, 16), (16, 32)])
+@pytest.mark.parametrize("at", [3, 40, 150, 199])
+def test_forward_row_with_one_key_narrow_heads_short_sequences(w_qk, w_vo, at):
+    """The same promise on narrow output heads, where the sequence has at most 256 positions."""
+    test_forward_row_with_one_key_returns_its_value(w_qk, w_vo, at)
 
 
 @pytest.mark.parametrize("w_qk,w_vo", [(32, 32), (64, 16), (64, 64), (16, 48), (96, 128), (128, 16)])
