@@ -145,7 +145,7 @@ struct FwdCfg {
     static_assert(kSmem <= 232448, "shared memory of a block");
 };
 
-template <int NB>
+template <int NB, bool STAGED>   // STAGED: output rows leave through shared memory
 __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_constant__ AttnFwdParams P) {
     using Cfg = FwdCfg<NB>;
     constexpr int kTileBytes = Cfg::kTileBytes, QS = Cfg::QS, ST = Cfg::ST;
@@ -405,39 +405,58 @@ __global__ void __launch_bounds__(kFwdThreads, 1) attn_fwd_kernel(const __grid_c
             tc_fence_after();
             const float inv = row_inv[((nl & 1u) * 2 + x) * kTile + row];
             ++nl;
-            // 32 columns at a time, through shared memory, eight rows to a store instruction.  Stored straight from the threads, each
-            // with a row of its own, 64 columns of both streams took 2400 to 2900 clocks, which nothing hides at the end of a CTA's last
-            // items.  Direct / through shared memory, us: 10.9 / 10.4 (96 heads of 256 positions, 64 wide, no mask), 17.4 / 16.1 (192 of 197,
-            // ragged), 26.0 / 24.9 (128 of 512), 12.5 / 11.2 (96 of 256, 96 wide), 166.5 / 164.3 (64 of 2048); causal 53.1 / 52.4 (128 of 1024, 48
-            // wide), 17.4 / 16.5 (72 of 512, 96 wide), but 20.4 / 20.8 (128 of 512, 64 wide), 16.4 / 17.0 (256 of 200, 80 wide).
             const int q_warp = (x ? I.qt1 : I.qt0) * kTile + (warp & 3) * 32;
             uint16_t* dst = P.ctx + (static_cast<int64_t>(x ? I.b1 : I.b0) * P.seq + q_warp) * P.ld_ctx + P.heads.vo_off[h];
-            const uint32_t buf = sOut + (warp - 4) * 2048;                // [row][4 chunks of 8 columns], chunk c of row r in place c ^ (r / 2 % 4)
-            const int r_in = lane >> 2, chunk = lane & 3;                 // on the way out: eight rows to an instruction, four lanes to a row
+            if constexpr (STAGED) {
+                // 32 columns at a time, eight rows to a store instruction
+                const uint32_t buf = sOut + (warp - 4) * 2048;                // [row][4 chunks of 8 columns], chunk c of row r in place c ^ (r / 2 % 4)
+                const int r_in = lane >> 2, chunk = lane & 3;                 // on the way out: eight rows to an instruction, four lanes to a row
 #pragma unroll 1
-            for (int c = 0; c < wv; c += 32) {
-                uint32_t r[16], q[16];                                     // (columns past the head's width are not stored)
-                tc_ld16(tO + c, r);
-                tc_ld16(tO + c + 16, q);
-                tc_wait_ld(r);
-                tc_wait_ld(q);
-                __syncwarp();                                              // the columns before these have left
-                auto put = [&](const uint32_t (&v)[16], int at, int k) {
-                    st_shared_v4(buf + lane * 64 + 16 * (k ^ ((lane >> 1) & 3)), pack_bf16(__uint_as_float(v[at]) * inv, __uint_as_float(v[at + 1]) * inv),
-                                 pack_bf16(__uint_as_float(v[at + 2]) * inv, __uint_as_float(v[at + 3]) * inv),
-                                 pack_bf16(__uint_as_float(v[at + 4]) * inv, __uint_as_float(v[at + 5]) * inv),
-                                 pack_bf16(__uint_as_float(v[at + 6]) * inv, __uint_as_float(v[at + 7]) * inv));
-                };
-                put(r, 0, 0);
-                put(r, 8, 1);
-                put(q, 0, 2);
-                put(q, 8, 3);
-                __syncwarp();
+                for (int c = 0; c < wv; c += 32) {
+                    uint32_t r[16], q[16];                                     // (columns past the head's width are not stored)
+                    tc_ld16(tO + c, r);
+                    tc_ld16(tO + c + 16, q);
+                    tc_wait_ld(r);
+                    tc_wait_ld(q);
+                    __syncwarp();                                              // the columns before these have left
+                    auto put = [&](const uint32_t (&v)[16], int at, int k) {
+                        st_shared_v4(buf + lane * 64 + 16 * (k ^ ((lane >> 1) & 3)), pack_bf16(__uint_as_float(v[at]) * inv, __uint_as_float(v[at + 1]) * inv),
+                                     pack_bf16(__uint_as_float(v[at + 2]) * inv, __uint_as_float(v[at + 3]) * inv),
+                                     pack_bf16(__uint_as_float(v[at + 4]) * inv, __uint_as_float(v[at + 5]) * inv),
+                                     pack_bf16(__uint_as_float(v[at + 6]) * inv, __uint_as_float(v[at + 7]) * inv));
+                    };
+                    put(r, 0, 0);
+                    put(r, 8, 1);
+                    put(q, 0, 2);
+                    put(q, 8, 3);
+                    __syncwarp();
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int rr = 8 * u + r_in;
-                    if (q_warp + rr < P.seq && c + 8 * chunk < wv)
-                        *reinterpret_cast<uint4*>(dst + rr * P.ld_ctx + c + 8 * chunk) = ld_shared_v4(buf + rr * 64 + 16 * (chunk ^ ((rr >> 1) & 3)));
+                    for (int u = 0; u < 4; ++u) {
+                        const int rr = 8 * u + r_in;
+                        if (q_warp + rr < P.seq && c + 8 * chunk < wv)
+                            *reinterpret_cast<uint4*>(dst + rr * P.ld_ctx + c + 8 * chunk) = ld_shared_v4(buf + rr * 64 + 16 * (chunk ^ ((rr >> 1) & 3)));
+                    }
+                }
+            } else {
+                const int q_pos = q_warp + lane;
+#pragma unroll 1
+                for (int c = 0; c < wv; c += 16) {
+                    uint32_t r[16];
+                    tc_ld16(tO + c, r);
+                    tc_wait_ld(r);
+                    if (q_pos < P.seq) {
+                        uint4 v0, v1;
+                        v0.x = pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv);
+                        v0.y = pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv);
+                        v0.z = pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv);
+                        v0.w = pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv);
+                        v1.x = pack_bf16(__uint_as_float(r[8]) * inv, __uint_as_float(r[9]) * inv);
+                        v1.y = pack_bf16(__uint_as_float(r[10]) * inv, __uint_as_float(r[11]) * inv);
+                        v1.z = pack_bf16(__uint_as_float(r[12]) * inv, __uint_as_float(r[13]) * inv);
+                        v1.w = pack_bf16(__uint_as_float(r[14]) * inv, __uint_as_float(r[15]) * inv);
+                        *reinterpret_cast<uint4*>(dst + lane * P.ld_ctx + c) = v0;
+                        *reinterpret_cast<uint4*>(dst + lane * P.ld_ctx + c + 8) = v1;
+                    }
                 }
             }
             tc_fence_before();
@@ -1843,8 +1862,10 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     cudaGetDevice(&dev);
     cudaError_t e = cudaSuccess;
     std::call_once(once[dev & 63], [&] {
-        e = cudaFuncSetAttribute(attn_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<1>::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<2>::kSmem);
+        e = cudaFuncSetAttribute(attn_fwd_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<1>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<1>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<2>::kSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<2>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_fwd_ms_kernel<3, 32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MsCfg<3, 32>::kSmem);
     });
@@ -1856,8 +1877,15 @@ extern "C" ecospa_status_t ecospa_coupled_attn_fwd(const void* Qc, const void* K
     const int grid = std::min<int>(P.n_items, std::max(1, engine_num_sms()));
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (streams) return launch_pdl(P.n_qt <= 2 ? attn_fwd_ms_kernel<3, 32, true> : attn_fwd_ms_kernel<3, 32, false>, grid, MsCfg<3, 32>::kThreads, cs, P, "attn_fwd_kernel", MsCfg<3, 32>::kSmem);
-    if (max_w <= 64) return launch_pdl(attn_fwd_kernel<1>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<1>::kSmem);
-    return launch_pdl(attn_fwd_kernel<2>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<2>::kSmem);
+    // Output rows through shared memory: stored straight from the threads, each with a row of its own, 64 columns of both streams take
+    // 2400 to 2900 clocks, which nothing hides at the end of a CTA's last items (and all end together without a mask); items of one
+    // key block, and causal ones on heads up to 64, rather wait for the longer way.  Direct / through shared memory, us: no mask 10.9 / 10.4 (96
+    // heads of 256 positions, 64 wide), 17.4 / 16.1 (192 of 197, ragged), 26.0 / 24.9 (128 of 512), 12.5 / 11.2 (96 of 256, 96 wide), 166.5 / 164.3 (64
+    // of 2048); causal 17.4 / 16.5 (72 of 512, 96 wide), 91.8 / 90.2 (64 of 2048), 16.4 / 17.0 (256 of 200, 80 wide), 20.4 / 20.8 (128 of 512, 64
+    // wide); one key block 26.7 / 28.3 (1920 of 48, 48 wide), 8.7 / 9.2 (320 of 64, 32 wide).
+    const bool staged = P.items != ITEMS_SOLO && (!P.causal || max_w > 64);
+    if (max_w <= 64) return launch_pdl(staged ? attn_fwd_kernel<1, true> : attn_fwd_kernel<1, false>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<1>::kSmem);
+    return launch_pdl(staged ? attn_fwd_kernel<2, true> : attn_fwd_kernel<2, false>, grid, kFwdThreads, cs, P, "attn_fwd_kernel", FwdCfg<2>::kSmem);
 }
 
 extern "C" size_t ecospa_attn_workspace_bytes(int64_t batch, int64_t seq, int32_t n_heads) {
