@@ -27,9 +27,9 @@
 // 4 x 2048 positions, 32 heads 32 wide: warps waited for instructions, 4.0 of 15 cycles per issue, now 1.0).  Columns that
 // no row of a warp sees are skipped, keys past the end of the sequence also in the products.
 // Before (two streams in one thread's registers, a token between them) / now, us: 475 / 301 (2 x 4096, 32 heads 96 wide),
-// 69.7 / 53.2 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 7.5 (2 x 160, 12 heads 48 wide), 63.9 / 28.9 (60 x 48, 32 heads 64
-// wide), 41.7 / 18.9 (30 x 48, 32 heads 128 wide), 26.6 / 25.1 (8 x 512, 16 heads 64 wide, no mask).  One form is slower than before: one
-// pair of tiles to a CTA, short, without a mask, heads of 33 to 64 (9.8 / 10.4 for 96 heads of 256, 12.3 / 12.6 for 72 of 384): the two
+// 69.7 / 53.2 (4 x 1000, 32 heads 48 wide on 8), 10.5 / 7.5 (2 x 160, 12 heads 48 wide), 63.3 / 26.8 (60 x 48, 32 heads 64
+// wide), 41.7 / 18.3 (30 x 48, 32 heads 128 wide), 26.4 / 24.7 (8 x 512, 16 heads 64 wide, no mask).  One form is slower than before: one
+// pair of tiles to a CTA, short, without a mask, heads of 33 to 64 (9.7 / 10.3 for 96 heads of 256, 12.2 / 12.6 for 72 of 384): the two
 // streams start and end together.
 // Every mbarrier wait is bounded; on expiry the CTA records a code (11 loads, 12 products, 13 softmax and scaling) in the device
 // status word, lets copies land, frees TMEM and returns.
